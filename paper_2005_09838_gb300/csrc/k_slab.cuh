@@ -14,13 +14,25 @@ namespace tc {
 
 enum SlabMode : int { MODE_ITER = 0, MODE_W = 1, MODE_R = 2, MODE_GRAD = 3 };
 
+// Launch flags of the slab kernels: the slab lives in shared memory (else in
+// d.scratch; k_slab only), and MODE_W writes Wout in the row-major order
+// [i1][i3][i2] (one CTA then writes whole rows; k_unpack brings it to the
+// caller's column-major order) instead of the column-major one.
+// SLAB_NOSUM: MODE_W forms no sums.
+enum SlabFlag : int { SLAB_IN_SMEM = 1, SLAB_WROWS = 2, SLAB_NOSUM = 4 };
+
 // Threads per CTA: the register transforms and the W-step sweeps need the
 // 255-register budget of two warps per scheduler (nine warps would put three
 // on one scheduler and cap a thread at 168 registers); tubes beyond the thread
 // count loop.
 __host__ __device__ constexpr int slab_max_threads(int) { return 256; }
-// Rows (inverse) or slices (forward) per item of the generic transform, by
-// default; the engine picks among 2, 4 and 8 by timing (slab_tile_candidates).
+// Rows (inverse) or slices (forward) per item of the generic transform by
+// default; every tile gives the same sums in the same order, and tc_init times
+// 2, 4 and 8 where this kernel runs the iteration.  It runs where k_slab_g does
+// not hold the slab in shared memory, and for TC_BF16: the split operands of
+// its contractions keep 16 bits, so any other rounding of the transform
+// comes back as other BF16 rounding errors in the factors (3e-5 of Y~ after
+// five iterations on 435 x 205 x 34, r = 28, as large as the form's error).
 constexpr int kTL = 4;
 
 // Odd stride between tubes in the slab (n3 values per tube).
@@ -311,11 +323,10 @@ __device__ __forceinline__ double dw_term(cx<T> rnew, cx<T> rold, cx<T> dz, int 
 // Layouts used here: G row-major [i1][n3][n2] and mask words row-major
 // [i1][n3][ceil(n2/32)] (written by k_pack), copied to shared memory.
 // ---------------------------------------------------------------------------
-// TL: rows (inverse) or slices (forward) per item of the generic transform
-// (L = 0); every TL gives the same sums in the same order.
 template <typename T, int L, int MODE, int TL = kTL>
 __global__ void __launch_bounds__(slab_max_threads(L), 1)
-    k_slab(Dev<T> d, T* __restrict__ Wout, int slabs_in_smem, int init) {
+    k_slab(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
+  const int slabs_in_smem = flags & SLAB_IN_SMEM;
   extern __shared__ __align__(16) unsigned char smem[];
   const int i1 = blockIdx.x;
   const int n1 = d.n1, n2 = d.n2;
@@ -354,7 +365,7 @@ __global__ void __launch_bounds__(slab_max_threads(L), 1)
 
   // ---- phase A: inverse transform of each tube; v = G on the mask ------------
   // (MODE_GRAD: v = Z - G on the mask, 0 elsewhere; gsum = ||v||^2)
-  double gsum = 0.0;
+  SqSum<T> gsum;
   if constexpr (L > 0) {
     constexpr int SL = L / 2 + 1;
     if (MODE == MODE_ITER || MODE == MODE_GRAD) {
@@ -411,7 +422,7 @@ __global__ void __launch_bounds__(slab_max_threads(L), 1)
         for (int l = 0; l < L; ++l) {
           const bool ob = act && ((msk[l * mwords + (ta >> 5)] >> (ta & 31)) & 1u);
           x[l] = ob ? x[l] - spat[(size_t)ta * LP + l] : T(0);
-          gsum += (double)x[l] * (double)x[l];
+          gsum.add(x[l]);
         }
       }
       if (act) {
@@ -475,7 +486,7 @@ __global__ void __launch_bounds__(slab_max_threads(L), 1)
         } else if (MODE == MODE_GRAD) {
           const bool ob = (msk[l * mwords + (t >> 5)] >> (t & 31)) & 1u;
           x = ob ? x - __ldg(Gi + (size_t)l * n2 + t) : T(0);
-          gsum += (double)x * (double)x;
+          gsum.add(x);
         }
         col[l] = x;
       }
@@ -485,21 +496,24 @@ __global__ void __launch_bounds__(slab_max_threads(L), 1)
 
   // ---- phase B: rows ------------------------------------------------------
   if (MODE == MODE_W || MODE == MODE_R) {
-    double a = 0.0, b = 0.0;
+    const bool sums = MODE == MODE_R || !(flags & SLAB_NOSUM);
+    SqSum<T> sa, sb;
     for (int e = tid; e < n2 * n3; e += nt) {
       const int j = e / n3, l = e - j * n3;
       const T v = spat[j * LP + l];
-      a += (double)v * (double)v;
+      if (sums) sa.add(v);
       if (MODE == MODE_W) {
-        if (j + 1 < n2) {
-          const double dv = (double)v - (double)spat[(j + 1) * LP + l];
-          b += dv * dv;
+        if (sums && j + 1 < n2) sb.add_diff(v, spat[(j + 1) * LP + l]);
+        if (Wout) {
+          if (flags & SLAB_WROWS) Wout[((size_t)i1 * n3 + l) * n2 + j] = v;
+          else Wout[(size_t)i1 + (size_t)n1 * ((size_t)j + (size_t)n2 * l)] = v;
         }
-        if (Wout) Wout[(size_t)i1 + (size_t)n1 * ((size_t)j + (size_t)n2 * l)] = v;
       } else {
-        if ((msk[l * mwords + (j >> 5)] >> (j & 31)) & 1u) b += (double)v * (double)v;
+        if ((msk[l * mwords + (j >> 5)] >> (j & 31)) & 1u) sb.add(v);
       }
     }
+    if (!sums) return;
+    double a = sa.total(), b = sb.total();
     block_sum2(a, b, red);
     if (tid == 0) {
       const int o = (MODE == MODE_W) ? 2 : 0;
@@ -509,9 +523,13 @@ __global__ void __launch_bounds__(slab_max_threads(L), 1)
     return;
   }
   if (wsolve) {
-    for (int l = tid; l < n3; l += nt)
-      wstep_sweeps<T>(spat + l, LP, msk + l * mwords, stw + l * mwords, n2, d.rho2, wtab);
-    __syncthreads();
+    if (n3 <= nt) {  // every thread one (row, segment)
+      wstep_sweeps_seg<T>([&](int l) { return spat + l; }, LP, msk, stw, n3, nt / n3, tid, n2, d.rho2, wtab);
+    } else {
+      for (int l = tid; l < n3; l += nt)
+        wstep_sweeps<T>(spat + l, LP, msk + l * mwords, stw + l * mwords, n2, d.rho2, wtab);
+      __syncthreads();
+    }
   }
 
   // ---- phase C: forward transform, R~ = W~ - Z~ ------------------------------
@@ -540,42 +558,49 @@ __global__ void __launch_bounds__(slab_max_threads(L), 1)
     // slices k, tube index fastest
     const cx<T>* tw = reinterpret_cast<const cx<T>*>(smem + lay.tw);
     const int nkb = (S + TL - 1) / TL;
-    for (int e = tid; e < nkb * n2; e += nt) {
-      const int kb = e / n2, t = e - kb * n2, k0 = kb * TL;
-      cx<T> acc[TL];
+    // the change of W~ (FP64) in a loop of its own: predicated into the plain one,
+    // its instructions would take their issue slots of the FP64 pipe all the same
+    auto slices = [&](auto tr) {
+      constexpr bool TRACK = decltype(tr)::value;
+      for (int e = tid; e < nkb * n2; e += nt) {
+        const int kb = e / n2, t = e - kb * n2, k0 = kb * TL;
+        cx<T> acc[TL];
 #pragma unroll
-      for (int j = 0; j < TL; ++j) acc[j] = cx<T>{T(0), T(0)};
-      int idx[TL], inc[TL];  // (k0 + j) l mod n3, advanced by (k0 + j) mod n3 (< n3)
-#pragma unroll
-      for (int j = 0; j < TL; ++j) {
-        idx[j] = 0;
-        inc[j] = (k0 + j) % n3;
-      }
-      const T* col = spat + (size_t)t * LP;
-      for (int l = 0; l < n3; ++l) {
-        const T x = col[l];
+        for (int j = 0; j < TL; ++j) acc[j] = cx<T>{T(0), T(0)};
+        int idx[TL], inc[TL];  // (k0 + j) l mod n3, advanced by (k0 + j) mod n3 (< n3)
 #pragma unroll
         for (int j = 0; j < TL; ++j) {
-          const cx<T> w = tw[idx[j]];
-          acc[j].re += x * w.re;
-          acc[j].im += x * w.im;
-          idx[j] += inc[j];
-          if (idx[j] >= n3) idx[j] -= n3;
+          idx[j] = 0;
+          inc[j] = (k0 + j) % n3;
+        }
+        const T* col = spat + (size_t)t * LP;
+        for (int l = 0; l < n3; ++l) {
+          const T x = col[l];
+#pragma unroll
+          for (int j = 0; j < TL; ++j) {
+            const cx<T> w = tw[idx[j]];
+            acc[j].re += x * w.re;
+            acc[j].im += x * w.im;
+            idx[j] += inc[j];
+            if (idx[j] >= n3) idx[j] -= n3;
+          }
+        }
+        const size_t o = (size_t)i1 * S * n2 + t;
+#pragma unroll
+        for (int j = 0; j < TL; ++j) {
+          const int k = k0 + j;
+          if (k >= S) break;
+          cx<T> a = acc[j];
+          if (k == 0 || (2 * k == n3)) a.im = T(0);
+          const size_t ok = o + (size_t)k * n2;
+          const cx<T> rn = (MODE == MODE_GRAD) ? a : a - zrow[(size_t)k * n2 + t];
+          if constexpr (TRACK) dw2 += dw_term(rn, d.Rt[ok], d.dZt[ok], k, n3);
+          d.Rt[ok] = rn;
         }
       }
-      const size_t o = (size_t)i1 * S * n2 + t;
-#pragma unroll
-      for (int j = 0; j < TL; ++j) {
-        const int k = k0 + j;
-        if (k >= S) break;
-        cx<T> a = acc[j];
-        if (k == 0 || (2 * k == n3)) a.im = T(0);
-        const size_t ok = o + (size_t)k * n2;
-        const cx<T> rn = (MODE == MODE_GRAD) ? a : a - zrow[(size_t)k * n2 + t];
-        if (track) dw2 += dw_term(rn, d.Rt[ok], d.dZt[ok], k, n3);
-        d.Rt[ok] = rn;
-      }
-    }
+    };
+    if (track) slices(BoolC<true>{});
+    else slices(BoolC<false>{});
   }
   if (track) {
     double unused = 0.0;
@@ -583,9 +608,9 @@ __global__ void __launch_bounds__(slab_max_threads(L), 1)
     if (tid == 0) d.part_dw[i1] = dw2;
   }
   if (MODE == MODE_GRAD) {
-    double unused = 0.0;
-    block_sum2(gsum, unused, red);
-    if (tid == 0) d.part[(size_t)i1 * 4] = gsum;
+    double g = gsum.total(), unused = 0.0;
+    block_sum2(g, unused, red);
+    if (tid == 0) d.part[(size_t)i1 * 4] = g;
   }
 }
 

@@ -119,7 +119,7 @@ __device__ __forceinline__ cx<T> fwd_split(cx<T> zk, cx<T> zm, int k) {
 }
 
 template <typename T, int L, int N1, int N2, int MODE>
-__global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __restrict__ Wout, int, int init) {
+__global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
   constexpr int M = L / 2;
   static_assert(L % 2 == 0 && M == N1 * N2, "n3 = 2 N1 N2");
   constexpr int LP = slab_f_stride(L);
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __rest
   // ---- A3: inverse DFT_N2 over slots N2 k1 + j -> spatial values; v = G on the mask -------
   // (the G values of the next item are loaded while the current one is computed)
   const T scale = T(1) / T(M);
-  double gsum = 0.0;  // MODE_GRAD: ||E||^2 partial
+  SqSum<T> gsum;  // MODE_GRAD: ||E||^2 partial
   {
     T gn[2 * N2];
     auto load_g = [&](int k1, int t) {
@@ -256,7 +256,8 @@ __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __rest
           const uint32_t w0 = msk[l * mw + (t >> 5)], w1 = msk[(l + 1) * mw + (t >> 5)];
           x0 = ((w0 >> (t & 31)) & 1u) ? x0 - g[2 * k2] : T(0);
           x1 = ((w1 >> (t & 31)) & 1u) ? x1 - g[2 * k2 + 1] : T(0);
-          gsum += (double)x0 * (double)x0 + (double)x1 * (double)x1;
+          gsum.add(x0);
+          gsum.add(x1);
         }
         st_slot(tb, k2, cx<T>{x0, x1});
       }
@@ -266,22 +267,25 @@ __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __rest
 
   // ---- partial sums of the read-back modes ----------------------------------------------
   if (MODE == MODE_W || MODE == MODE_R) {
-    double a = 0.0, b = 0.0;
+    const bool sums = MODE == MODE_R || !(flags & SLAB_NOSUM);
+    SqSum<T> sa, sb;
     for (int e = tid; e < L * n2; e += nt) {
       const int l = e / n2, t = e - l * n2;
       const int off = slab_f_off<N1, N2>(l);
       const T v = buf[(size_t)t * LP + off];
-      a += (double)v * (double)v;
+      if (sums) sa.add(v);
       if (MODE == MODE_W) {
-        if (t + 1 < n2) {
-          const double dv = (double)v - (double)buf[(size_t)(t + 1) * LP + off];
-          b += dv * dv;
+        if (sums && t + 1 < n2) sb.add_diff(v, buf[(size_t)(t + 1) * LP + off]);
+        if (Wout) {
+          if (flags & SLAB_WROWS) Wout[((size_t)i1 * L + l) * n2 + t] = v;
+          else Wout[(size_t)i1 + (size_t)n1 * ((size_t)t + (size_t)n2 * l)] = v;
         }
-        if (Wout) Wout[(size_t)i1 + (size_t)n1 * ((size_t)t + (size_t)n2 * l)] = v;
       } else {
-        if ((msk[l * mw + (t >> 5)] >> (t & 31)) & 1u) b += (double)v * (double)v;
+        if ((msk[l * mw + (t >> 5)] >> (t & 31)) & 1u) sb.add(v);
       }
     }
+    if (!sums) return;
+    double a = sa.total(), b = sb.total();
     block_sum2(a, b, red);
     if (tid == 0) {
       const int o = (MODE == MODE_W) ? 2 : 0;
@@ -340,31 +344,38 @@ __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __rest
   const cx<T>* dz = track ? d.dZt + (size_t)i1 * (M + 1) * n2 : nullptr;
   double dw2 = 0.0;
   {
-    ItemIter it(tid, n2);
-    for (int e = tid; e < (M / 2 + 1) * n2; e += nt, it.advance(nt, n2)) {
-      const int k = it.g, t = it.t;
-      const int kc = M - k;
-      const T* tb = buf + (size_t)t * LP;
-      const size_t ok = (size_t)k * n2 + t, oc = (size_t)kc * n2 + t;
-      const cx<T> zk0 = (MODE == MODE_GRAD) ? cx<T>{T(0), T(0)} : ldg_cx(zrow + ok);
-      const cx<T> zc0 = (MODE == MODE_GRAD) ? cx<T>{T(0), T(0)} : ldg_cx(zrow + oc);
-      cx<T> rk, rc;
-      if (k == 0) {
-        const cx<T> z0 = ld_slot(tb, 0);
-        rk = cx<T>{z0.re + z0.im - zk0.re, T(0)};
-        rc = cx<T>{z0.re - z0.im - zc0.re, T(0)};
-      } else {
-        const cx<T> zk = ld_slot(tb, k), zm = ld_slot(tb, kc);
-        rk = fwd_split<T, L>(zk, zm, k) - zk0;
-        rc = fwd_split<T, L>(zm, zk, kc) - zc0;
+    // the change of W~ (FP64) in a loop of its own: predicated into the plain one,
+    // its instructions would take their issue slots of the FP64 pipe all the same
+    auto split = [&](auto tr) {
+      constexpr bool TRACK = decltype(tr)::value;
+      ItemIter it(tid, n2);
+      for (int e = tid; e < (M / 2 + 1) * n2; e += nt, it.advance(nt, n2)) {
+        const int k = it.g, t = it.t;
+        const int kc = M - k;
+        const T* tb = buf + (size_t)t * LP;
+        const size_t ok = (size_t)k * n2 + t, oc = (size_t)kc * n2 + t;
+        const cx<T> zk0 = (MODE == MODE_GRAD) ? cx<T>{T(0), T(0)} : ldg_cx(zrow + ok);
+        const cx<T> zc0 = (MODE == MODE_GRAD) ? cx<T>{T(0), T(0)} : ldg_cx(zrow + oc);
+        cx<T> rk, rc;
+        if (k == 0) {
+          const cx<T> z0 = ld_slot(tb, 0);
+          rk = cx<T>{z0.re + z0.im - zk0.re, T(0)};
+          rc = cx<T>{z0.re - z0.im - zc0.re, T(0)};
+        } else {
+          const cx<T> zk = ld_slot(tb, k), zm = ld_slot(tb, kc);
+          rk = fwd_split<T, L>(zk, zm, k) - zk0;
+          rc = fwd_split<T, L>(zm, zk, kc) - zc0;
+        }
+        if constexpr (TRACK) {
+          dw2 += dw_term(rk, rt[ok], dz[ok], k, L);
+          if (k != kc) dw2 += dw_term(rc, rt[oc], dz[oc], kc, L);
+        }
+        rt[ok] = rk;
+        if (k != kc) rt[oc] = rc;
       }
-      if (track) {
-        dw2 += dw_term(rk, rt[ok], dz[ok], k, L);
-        if (k != kc) dw2 += dw_term(rc, rt[oc], dz[oc], kc, L);
-      }
-      rt[ok] = rk;
-      if (k != kc) rt[oc] = rc;
-    }
+    };
+    if (track) split(BoolC<true>{});
+    else split(BoolC<false>{});
   }
   if (track) {
     double unused = 0.0;
@@ -372,9 +383,9 @@ __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __rest
     if (tid == 0) d.part_dw[i1] = dw2;
   }
   if (MODE == MODE_GRAD) {
-    double unused = 0.0;
-    block_sum2(gsum, unused, red);
-    if (tid == 0) d.part[(size_t)i1 * 4] = gsum;
+    double g = gsum.total(), unused = 0.0;
+    block_sum2(g, unused, red);
+    if (tid == 0) d.part[(size_t)i1 * 4] = g;
   }
 }
 

@@ -193,21 +193,6 @@ __device__ __forceinline__ df df_rcp(df a) {
   return df_add(df{y0, 0.0f}, df_mul(df{y0, 0.0f}, e));
 }
 
-// s + c += a b with the rounding errors of the product (FMA) and of the sum
-// (Knuth's two-sum) collected in c: about twice the working precision.
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-
-template <typename T>
-__device__ __forceinline__ void dot2(T& s, T& c, T a, T b) {
-  const T p = mul_rn(a, b);  // not contracted: the FMA below recovers its rounding error
-  const T pe = fma(a, b, -p);
-  const T t = s + p;
-  const T z = t - s;
-  c += ((s - (t - z)) + (p - z)) + pe;
-  s = t;
-}
-
 // gauss_jordan_inplace on an FP64 matrix, with the arithmetic in df64 (the
 // matrix is converted, eliminated and converted back; no FP64 instruction in
 // the elimination itself).

@@ -119,6 +119,50 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+// s + c += a b with the rounding errors of the product (FMA) and of the sum
+// (Knuth's two-sum) collected in c: about twice the working precision.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+template <typename T>
+__device__ __forceinline__ void dot2(T& s, T& c, T a, T b) {
+  const T p = mul_rn(a, b);  // not contracted: the FMA below recovers its rounding error
+  const T pe = fma(a, b, -p);
+  const T t = s + p;
+  const T z = t - s;
+  c += ((s - (t - z)) + (p - z)) + pe;
+  s = t;
+}
+
+// Sum of squares of a thread's values to FP64 accuracy.  FP32 values: error-free
+// products and sums on the FP32 pipe (dot2); GB300 issues one FP64 warp
+// instruction per scheduler in about 60 clocks, and the FP64 form (a conversion
+// and a multiply-add per value) took more than half of the read-back kernels.
+template <typename T>
+struct SqSum {
+  T s = T(0), c = T(0);
+  __device__ __forceinline__ void add(T v) {
+    if constexpr (sizeof(T) == 8) s = fma(v, v, s);
+    else dot2(s, c, v, v);
+  }
+  // (a - b)^2, the difference not rounded
+  __device__ __forceinline__ void add_diff(T a, T b) {
+    const T h = a - b;
+    add(h);
+    if constexpr (sizeof(T) == 4) {
+      const T z = h - a;
+      c = fma(T(2) * h, (a - (h - z)) - (b + z), c);
+    }
+  }
+  __device__ __forceinline__ double total() const { return (double)s + (double)c; }
+};
+
+// A truth value as a type, for generic lambdas.
+template <bool B>
+struct BoolC {
+  static constexpr bool value = B;
+};
+
 constexpr int kMaxRank = 32;
 
 // Asynchronous 4-, 8- or 16-byte global -> shared copy (cp.async, L1-allocating);

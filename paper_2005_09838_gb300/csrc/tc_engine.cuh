@@ -37,12 +37,53 @@ inline void slab_table(SlabFn<T> f[3]) {
   f[MODE_R] = k_slab<T, L, MODE_R>;
 }
 
-// Generic-length slab kernels with TL rows / slices per transform item.
-template <typename T, int TL>
-inline void slab_table_tl(SlabFn<T> f[3]) {
-  f[MODE_ITER] = k_slab<T, 0, MODE_ITER, TL>;
-  f[MODE_W] = k_slab<T, 0, MODE_W, TL>;
-  f[MODE_R] = k_slab<T, 0, MODE_R, TL>;
+// Folded-transform slab kernels with TL rows / slices per item (the read-back
+// modes, one launch per call, take TL = 4).
+template <typename T, bool STAGED>
+inline SlabFn<T> pick_slab_g_st(int mode, int tl) {
+  if (mode == MODE_W) return k_slab_g<T, MODE_W, 4, STAGED>;
+  if (mode == MODE_R) return k_slab_g<T, MODE_R, 4, STAGED>;
+  return tl == 2 ? k_slab_g<T, MODE_ITER, 2, STAGED>
+                 : tl == 4 ? k_slab_g<T, MODE_ITER, 4, STAGED> : k_slab_g<T, MODE_ITER, 8, STAGED>;
+}
+template <typename T>
+inline SlabFn<T> pick_slab_g(int mode, int tl, bool staged) {
+  return staged ? pick_slab_g_st<T, true>(mode, tl) : pick_slab_g_st<T, false>(mode, tl);
+}
+
+// The iteration's slab kernel with a tile of tl.
+template <typename T>
+inline SlabFn<T> pick_slab_tile(bool folded, bool staged, int tl) {
+  if (folded) return pick_slab_g<T>(MODE_ITER, tl, staged);
+  return tl == 2 ? k_slab<T, 0, MODE_ITER, 2> : tl == 4 ? k_slab<T, 0, MODE_ITER, 4> : k_slab<T, 0, MODE_ITER, 8>;
+}
+
+// Launch shape of the folded-transform slab kernels: two CTAs of 256 threads on
+// an SM where the slab, the coefficients and a stage of one group fit half of
+// its shared memory, else one with twice the threads; as many groups per stage
+// as fit; unstaged where even one does not.  False where the slab itself does
+// not fit (k_slab keeps it in global memory).
+struct SlabGPlan {
+  int threads, sg;
+  size_t smem;
+};
+template <typename T>
+inline bool slab_g_plan(int n2, int n3, int optin, SlabGPlan& pl) {
+  if (n3 > kSlabGMaxN3) return false;
+  const int ngr = (n2 + kGTubes - 1) / kGTubes;
+  const size_t half = (size_t)(optin + kStaticSmemReserve + 1024) / 2 - 1024;  // 1 KB per CTA is the system's
+  for (int pass = 0; pass < 2; ++pass) {
+    const size_t room = pass == 0 ? half : (size_t)optin;
+    for (int sg = ngr; sg >= 1; --sg) {
+      const size_t b = slab_g_layout<T>(n2, n3, sg).total;
+      if (b <= room) {
+        pl = SlabGPlan{pass == 0 ? 256 : kSlabGThreads<T>, sg, b};
+        return true;
+      }
+    }
+  }
+  pl = SlabGPlan{kSlabGThreads<T>, 0, slab_g_layout<T>(n2, n3, 0).total};
+  return pl.smem <= (size_t)optin;
 }
 
 template <typename T, int L, int N1, int N2>
@@ -243,6 +284,16 @@ class Engine final : public EngineBase {
       slab_threads_ = cfg.threads;
       slab_smem_ = cfg.smem;
       slabs_in_smem_ = true;
+    } else if (SlabGPlan gp; p.precision != TC_BF16 && slab_g_plan<T>(n2_, n3_, optin, gp)) {
+      folded_ = true;
+      d_.fold_sg = gp.sg;
+      for (int m = 0; m < 3; ++m) slab_[m] = pick_slab_g<T>(m, 4, gp.sg > 0);
+      slab_smem_ = gp.smem;
+      slab_threads_ = gp.threads;
+      slabs_in_smem_ = true;
+      fold_ = alloc<cx<T>>(fold_table_entries(n3_), err);
+      if (!err.empty()) return TC_ERR_NOMEM;
+      d_.fold = fold_;
     } else {
       slab_table<T, 0>(slab_);
       slab_threads_ = 256;
@@ -453,7 +504,7 @@ class Engine final : public EngineBase {
         return TC_ERR_NOMEM;
       }
     }
-    k_pack<T><<<n1_ * n3_, 256, 0, stream_>>>(dG, dM, Gint, maskbits, n1_, n2_, n3_, mw_);
+    k_pack<T><<<pack_grid(n1_, n2_, n3_), kTileThreads, 0, stream_>>>(dG, dM, Gint, maskbits, n1_, n2_, n3_, mw_);
     const int fgrid = 4 * 152;
     k_factor_dft<T><<<fgrid, 256, 0, stream_>>>(dY, Yt, n2_, r_, n3_, 1, twg);
     if (dX) {
@@ -464,6 +515,7 @@ class Engine final : public EngineBase {
     k_synth_init<T><<<fgrid, 256, 0, stream_>>>(d_);                    // Z~0 = X~0 Y~0
     k_gram_tiles<T><<<dim3(S_, ytiles), 256, 0, stream_>>>(d_);         // A of the first X-step
     if (xsplit_ || apre_) xa_fn_<<<S_, xa_threads_, xa_smem_, stream_>>>(d_);  // its A^+
+    if (folded_) k_fold_tables<T><<<2 * 152, 256, 0, stream_>>>(fold_, twg, n3_);
     if (!specialised_) {
       // tile of the generic transform for this shape: each candidate runs the
       // initial slab pass (it only depends on G and Z~0, so every run writes the
@@ -603,7 +655,20 @@ class Engine final : public EngineBase {
       err = "allocation of read-back buffers failed";
       return TC_ERR_NOMEM;
     }
-    if (dW) launch_slab(MODE_W, dW, 0, stream_);
+    if (dW) {
+      // rows into a buffer of the context's own, then one transpose; straight into
+      // the caller's order where there is no room for the buffer
+      if (!wrows_) {
+        std::string full;
+        wrows_ = alloc<T>(N, full);
+      }
+      if (wrows_) {
+        launch_slab(MODE_W, wrows_, 0, stream_, SLAB_WROWS | SLAB_NOSUM);
+        k_unpack<T><<<pack_grid(n1_, n2_, n3_), kTileThreads, 0, stream_>>>(wrows_, dW, n1_, n2_, n3_);
+      } else {
+        launch_slab(MODE_W, dW, 0, stream_, SLAB_NOSUM);
+      }
+    }
     const int fgrid = 4 * 152;
     if (dXo) k_factor_idft<T><<<fgrid, 256, 0, stream_>>>(d_.Xt, dXo, n1_, r_, n3_, 0, d_.twg);
     if (dYo) k_factor_idft<T><<<fgrid, 256, 0, stream_>>>(d_.Yt, dYo, n2_, r_, n3_, 1, d_.twg);
@@ -795,10 +860,6 @@ class Engine final : public EngineBase {
 
   tc_status tune_slab_tile(std::string& err) {
     const int cand[3] = {2, 4, 8};
-    SlabFn<T> tab[3][3];
-    slab_table_tl<T, 2>(tab[0]);
-    slab_table_tl<T, 4>(tab[1]);
-    slab_table_tl<T, 8>(tab[2]);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     TC_CUDA_TRY(cudaEventCreate(&e0));
     TC_CUDA_TRY(cudaEventCreate(&e1));
@@ -806,8 +867,8 @@ class Engine final : public EngineBase {
     int pick = 1;
     cudaError_t e = cudaSuccess;
     for (int c = 0; c < 3 && e == cudaSuccess; ++c) {
-      for (int m = 0; m < 3 && e == cudaSuccess; ++m) e = allow_dynamic_smem((const void*)tab[c][m], slab_smem_);
-      for (int m = 0; m < 3; ++m) slab_[m] = tab[c][m];
+      slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[c]);
+      e = allow_dynamic_smem((const void*)slab_[MODE_ITER], slab_smem_);
       float ms = 1e30f;
       for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
         e = cudaEventRecord(e0, stream_);
@@ -831,13 +892,13 @@ class Engine final : public EngineBase {
       poisoned_ = true;
       return TC_ERR_CUDA;
     }
-    for (int m = 0; m < 3; ++m) slab_[m] = tab[pick][m];
+    slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[pick]);
     slab_tile_ = cand[pick];
     return TC_OK;
   }
 
-  void launch_slab(int mode, T* Wout, int init, cudaStream_t s) {
-    slab_[mode]<<<n1_, slab_threads_, slab_smem_, s>>>(d_, Wout, slabs_in_smem_ ? 1 : 0, init);
+  void launch_slab(int mode, T* Wout, int init, cudaStream_t s, int flags = 0) {
+    slab_[mode]<<<n1_, slab_threads_, slab_smem_, s>>>(d_, Wout, flags | (slabs_in_smem_ ? SLAB_IN_SMEM : 0), init);
   }
   void launch_qcon(cudaStream_t s) { qcon_<<<qgrid_, qthreads_, qcon_smem_, s>>>(d_, Q_); }
   // With the four-kernel X-step, A^+ (k_xa) is formed after every change of Y~
@@ -934,6 +995,9 @@ class Engine final : public EngineBase {
   int n1_ = 0, n2_ = 0, n3_ = 0, r_ = 0, S_ = 0, mw_ = 0, rp_ = 8;
   bool poisoned_ = false;
   bool specialised_ = false;
+  bool folded_ = false;  // folded-transform slab kernels (k_slab_g)
+  cx<T>* fold_ = nullptr;
+  T* wrows_ = nullptr;   // W in row-major order (allocated by the first read-back)
   bool slabs_in_smem_ = true;
   bool xarrays_in_smem_ = true;
   bool mixed_ = false;

@@ -230,7 +230,7 @@ struct GradEngine final : tc_grad {
       dG = static_cast<const T*>(tG);
       dM = static_cast<const uint8_t*>(tM);
     }
-    k_pack<T><<<n1_ * n3_, 256, 0, stream_>>>(dG, dM, Gint, maskbits, n1_, n2_, n3_, mw);
+    k_pack<T><<<pack_grid(n1_, n2_, n3_), kTileThreads, 0, stream_>>>(dG, dM, Gint, maskbits, n1_, n2_, n3_, mw);
     const cudaError_t le = cudaGetLastError();
     const cudaError_t se = cudaStreamSynchronize(stream_);
     if (tG) cudaFree(tG);

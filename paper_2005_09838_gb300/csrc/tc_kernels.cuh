@@ -44,6 +44,8 @@ struct Dev {
   const T* winv;    // [6][n2] W-step run tables (wstep_tables)
   const T* hinv;    // [2][n1] H_rho1 = I + rho1 H^T H: inverse pivots and rho1 * inverse pivots
   const cx<T>* twg; // [n3] exp(-2 pi i m / n3) for the generic transform
+  int fold_sg;       // 64-tube groups per stage of k_slab_g (0: unstaged)
+  const cx<T>* fold; // (cos, sin) tables of the folded transform (fold_table_entries)
   T* scratch;       // per-CTA slabs when shared memory is too small
   double* part;     // [n1][4] objective partial sums
   double* part_k;   // [S][kRhoChunks] rho1-term partial sums per slice
@@ -139,6 +141,7 @@ __device__ __forceinline__ void block_sum2(double& a, double& b, double* red) {
 #include "k_slab.cuh"
 #include "k_slab_f.cuh"
 #include "k_slice.cuh"
+#include "k_slab_g.cuh"
 #include "k_xsplit.cuh"
 #include "k_aux.cuh"
 #include "k_grad.cuh"

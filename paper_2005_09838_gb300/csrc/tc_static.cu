@@ -222,7 +222,7 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
       return sfail(TC_ERR_CUDA, std::string("clearing the device error flag failed: ") + cudaGetErrorString(e));
   }
   k_static_tables<T><<<3, 256, 0, st>>>(winv, hinv, twg, n1, n2, n3, p.mu, p.rho1, p.rho2);
-  k_pack<T><<<n1 * n3, 256, 0, st>>>(static_cast<const T*>(G), mask, Gint, maskbits, n1, n2, n3, mw);
+  k_pack<T><<<pack_grid(n1, n2, n3), kTileThreads, 0, st>>>(static_cast<const T*>(G), mask, Gint, maskbits, n1, n2, n3, mw);
   k_factor_dft<T><<<fgrid, 256, 0, st>>>(static_cast<const T*>(Y0), d.Yt, n2, r, n3, 1, twg);
   if (X0) {
     k_factor_dft<T><<<fgrid, 256, 0, st>>>(static_cast<const T*>(X0), d.Xt, n1, r, n3, 0, twg);
@@ -240,7 +240,7 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
     ystep<<<dim3(S, (n2 + 32 * ystep_cpl(rp) - 1) / (32 * ystep_cpl(rp))), kYThreads, ysm, st>>>(d);
     slab[MODE_ITER]<<<n1, 256, lay.total, st>>>(d, nullptr, sis, 0);
   }
-  slab[MODE_W]<<<n1, 256, lay.total, st>>>(d, static_cast<T*>(W), sis, 0);
+  slab[MODE_W]<<<n1, 256, lay.total, st>>>(d, static_cast<T*>(W), sis | (f0 ? 0 : SLAB_NOSUM), 0);
   if (f0) {
     slab[MODE_R]<<<n1, 256, lay.total, st>>>(d, nullptr, sis, 0);
     k_rho1_term<T><<<dim3(S, kRhoChunks), 256, 0, st>>>(d);
