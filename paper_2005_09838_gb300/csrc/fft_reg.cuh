@@ -1,20 +1,11 @@
-// Register-resident mode-3 DFTs of one tube per thread.
-//
-// The t-product algebra of Sec. 2.2 needs, for every tube (i1, i2, :), the
-// forward transform of Eq. (bar BA-k) restricted to the floor(n3/2)+1 slices
-// that are solved, and the inverse of Eq. (barAAk) from that half spectrum
-// (conjugate symmetry, Eq. (rcm_3-k+2)).  Here the transform is computed by a
-// mixed-radix decimation-in-time FFT whose length is a compile-time constant,
-// fully unrolled so that the tube lives in registers.
+// Small complex DFTs in registers, the passes of the shared-memory transforms
+// (k_slab_f): mixed-radix decimation in time, the length a compile-time constant,
+// fully unrolled.
 //
 // Sign convention: the forward transform uses w = exp(-2 pi i / n3).  The paper
 // writes omega = exp(+2 pi i / n3); every slice of one convention is the
 // complex conjugate of the other, the slice updates commute with conjugation
 // (all operators H, K are real), so every real quantity is unchanged.
-//
-// Real-input trick for even n3 = 2M: the even/odd samples are packed into one
-// complex sequence of length M, transformed, and split with the twiddles
-// w_n3^k.  Odd n3 runs a complex transform of length n3.
 #pragma once
 
 #include "tc_common.cuh"
@@ -22,15 +13,15 @@
 namespace tc {
 namespace fft {
 
-// Tube lengths with a specialised register kernel, and the offsets of their
+// Tube lengths with a specialised kernel, and the offsets of their
 // twiddle tables in the concatenated table.
-constexpr int kLengths[] = {7, 112, 168};
+constexpr int kLengths[] = {112, 168};
 constexpr int kNumLengths = sizeof(kLengths) / sizeof(int);
 
 __host__ __device__ constexpr int table_offset(int L) {
-  return L == 7 ? 0 : L == 112 ? 7 : L == 168 ? 7 + 112 : -1;
+  return L == 112 ? 0 : L == 168 ? 112 : -1;
 }
-constexpr int kTableSize = 7 + 112 + 168;
+constexpr int kTableSize = 112 + 168;
 
 __host__ __device__ constexpr bool supported(int L) { return table_offset(L) >= 0; }
 
@@ -41,14 +32,11 @@ constexpr int pick_radix(int N) {
 // Twiddle tables w_L^m = exp(-2 pi i m / L), m < L, for every specialised L,
 // concatenated.  Filled from the host (FP64 cos/sin) by upload_twiddles().
 static __constant__ cx<float> c_tw_f32[kTableSize];
-static __constant__ cx<double> c_tw_f64[kTableSize];
 
 template <typename T>
 __device__ __forceinline__ cx<T> tw_entry(int i);
 template <>
 __device__ __forceinline__ cx<float> tw_entry<float>(int i) { return c_tw_f32[i]; }
-template <>
-__device__ __forceinline__ cx<double> tw_entry<double>(int i) { return c_tw_f64[i]; }
 
 // w_L^m (forward); conjugated for the inverse.
 template <typename T, int L, bool INV>
@@ -139,89 +127,6 @@ struct CFFT {
   }
 };
 
-// Forward real transform of x[0..L) -> X[0..L/2] (half spectrum, L/2+1 values).
-template <typename T, int L>
-__device__ __forceinline__ void rfft(const T* x, cx<T>* X) {
-  if constexpr (L % 2 == 0) {
-    constexpr int M = L / 2;
-    cx<T> z[M];
-#pragma unroll
-    for (int m = 0; m < M; ++m) z[m] = cx<T>{x[2 * m], x[2 * m + 1]};
-    cx<T> Z[M];
-    CFFT<T, M, L, false>::run(z, 1, Z);
-#pragma unroll
-    for (int k = 0; k <= M; ++k) {
-      const cx<T> zk = Z[k % M];
-      const cx<T> zc = conj(Z[(M - k) % M]);
-      const cx<T> E = (zk + zc) * T(0.5);
-      const cx<T> D = (zk - zc) * T(0.5);  // O = D / i = (D.im, -D.re)
-      const cx<T> O = {D.im, -D.re};
-      if (k == 0) {
-        X[k] = cx<T>{E.re + O.re, T(0)};
-      } else if (k == M) {
-        X[k] = cx<T>{E.re - O.re, T(0)};
-      } else {
-        X[k] = E + cmul(O, tw<T, L, false>(k));
-      }
-    }
-  } else {
-    cx<T> z[L];
-#pragma unroll
-    for (int m = 0; m < L; ++m) z[m] = cx<T>{x[m], T(0)};
-    cx<T> Z[L];
-    CFFT<T, L, L, false>::run(z, 1, Z);
-#pragma unroll
-    for (int k = 0; k <= L / 2; ++k) X[k] = Z[k];
-    X[0].im = T(0);
-  }
-}
-
-// Inverse real transform: half spectrum X[0..L/2] -> x[0..L), including the
-// 1/L of Eq. (barAAk).  The imaginary parts of the DC (and, for even L, the
-// Nyquist) slice are ignored, as for any Hermitian-extended spectrum.
-template <typename T, int L>
-__device__ __forceinline__ void irfft(const cx<T>* X, T* x) {
-  if constexpr (L % 2 == 0) {
-    constexpr int M = L / 2;
-    cx<T> z[M];
-#pragma unroll
-    for (int k = 0; k < M; ++k) {
-      cx<T> a = X[k];
-      cx<T> b = X[M - k];
-      if (k == 0) {
-        a.im = T(0);
-        b.im = T(0);
-      }
-      const cx<T> bc = conj(b);
-      const cx<T> E = (a + bc) * T(0.5);
-      const cx<T> D = (a - bc) * T(0.5);
-      const cx<T> O = (k == 0) ? D : cmul(D, tw<T, L, true>(k));
-      z[k] = cx<T>{E.re - O.im, E.im + O.re};  // E + i O
-    }
-    cx<T> Z[M];
-    CFFT<T, M, L, true>::run(z, 1, Z);
-    const T s = T(1) / T(M);
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      x[2 * m] = Z[m].re * s;
-      x[2 * m + 1] = Z[m].im * s;
-    }
-  } else {
-    cx<T> z[L];
-    z[0] = cx<T>{X[0].re, T(0)};
-#pragma unroll
-    for (int k = 1; k <= L / 2; ++k) {
-      z[k] = X[k];
-      z[L - k] = conj(X[k]);
-    }
-    cx<T> Z[L];
-    CFFT<T, L, L, true>::run(z, 1, Z);
-    const T s = T(1) / T(L);
-#pragma unroll
-    for (int m = 0; m < L; ++m) x[m] = Z[m].re * s;
-  }
-}
-
 }  // namespace fft
 }  // namespace tc
 
@@ -231,8 +136,8 @@ namespace fft {
 // Fill this translation unit's twiddle tables on the current device (FP64
 // cos/sin rounded to the table type).  Each translation unit that launches a
 // register-FFT kernel owns its own copy of the constant tables.
-template <typename T>
 static void upload_tables() {
+  using T = float;
   cx<T> tab[kTableSize];
   for (int i = 0; i < kNumLengths; ++i) {
     const int L = kLengths[i];
@@ -242,11 +147,7 @@ static void upload_tables() {
       tab[off + m] = cx<T>{(T)cos(a), (T)(-sin(a))};
     }
   }
-  if constexpr (sizeof(T) == 4) {
-    cudaMemcpyToSymbol(c_tw_f32, tab, sizeof(tab));
-  } else {
-    cudaMemcpyToSymbol(c_tw_f64, tab, sizeof(tab));
-  }
+  cudaMemcpyToSymbol(c_tw_f32, tab, sizeof(tab));
 }
 
 }  // namespace fft

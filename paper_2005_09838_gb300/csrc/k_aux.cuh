@@ -461,12 +461,12 @@ __global__ void k_gram_tiles(Dev<T> d) {
   const int k = blockIdx.x, tile = blockIdx.y;
   const int r = d.r, n2 = d.n2, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int ntask = r * (r + 1) / 2;
-  const int j = tile * 32 + lane;
+  const int j = tile * d.ytw + lane;
   for (int task = wid; task < ntask; task += nw) {
     int s, u;
     tri_index(task, r, s, u);
     cx<T> g = {T(0), T(0)};  // the same arithmetic as the tile Grams of k_ystep
-    if (j < n2) cfmac(g, d.Yt[((size_t)k * r + s) * n2 + j], d.Yt[((size_t)k * r + u) * n2 + j]);
+    if (lane < d.ytw && j < n2) cfmac(g, d.Yt[((size_t)k * r + s) * n2 + j], d.Yt[((size_t)k * r + u) * n2 + j]);
     g.re = warp_sum(g.re);
     g.im = warp_sum(g.im);
     if (lane == 0) d.Ag[((size_t)k * d.ytiles + tile) * ntask + task] = cx<double>{(double)g.re, (double)g.im};

@@ -21,11 +21,8 @@ enum SlabMode : int { MODE_ITER = 0, MODE_W = 1, MODE_R = 2, MODE_GRAD = 3 };
 // SLAB_NOSUM: MODE_W forms no sums.
 enum SlabFlag : int { SLAB_IN_SMEM = 1, SLAB_WROWS = 2, SLAB_NOSUM = 4 };
 
-// Threads per CTA: the register transforms and the W-step sweeps need the
-// 255-register budget of two warps per scheduler (nine warps would put three
-// on one scheduler and cap a thread at 168 registers); tubes beyond the thread
-// count loop.
-__host__ __device__ constexpr int slab_max_threads(int) { return 256; }
+// Threads per CTA.
+constexpr int kSlabThreads = 256;
 // Rows (inverse) or slices (forward) per item of the generic transform by
 // default; every tile gives the same sums in the same order, and tc_init times
 // 2, 4 and 8 where this kernel runs the iteration.  It runs where k_slab_g does
@@ -44,7 +41,7 @@ struct SlabLayout {
 };
 
 template <typename T>
-__host__ __device__ inline SlabLayout slab_layout(int n2, int n3, bool specialised, bool slabs_in_smem) {
+__host__ __device__ inline SlabLayout slab_layout(int n2, int n3, bool slabs_in_smem) {
   SlabLayout L{};
   const int S = n3 / 2 + 1;
   size_t off = 0;
@@ -57,8 +54,8 @@ __host__ __device__ inline SlabLayout slab_layout(int n2, int n3, bool specialis
   L.stw = off;  // per row and mask word: start of the run of missing entries entering the word
   off = align_up(off + sizeof(int) * (size_t)n3 * ((n2 + 31) / 32), 16);
   L.tw = off;  // generic transform: the n3 twiddles exp(-2 pi i m / n3)
-  if (!specialised) off = align_up(off + sizeof(cx<T>) * (size_t)n3, 16);
-  const size_t spec_bytes = specialised ? 0 : align_up(sizeof(cx<T>) * (size_t)S * n2, 16);
+  off = align_up(off + sizeof(cx<T>) * (size_t)n3, 16);
+  const size_t spec_bytes = align_up(sizeof(cx<T>) * (size_t)S * n2, 16);
   const size_t spat_bytes = align_up(sizeof(T) * (size_t)n2 * slab_stride(n3), 16);
   L.slab_bytes = spec_bytes + spat_bytes;
   if (slabs_in_smem) {
@@ -304,6 +301,135 @@ __device__ void wstep_sweeps_seg(ColFn col_of, int LP, const uint32_t* __restric
   __syncthreads();
 }
 
+// ---------------------------------------------------------------------------
+// W-step of one segment (kWSeg entries, fewer in the last one) of one row, from
+// the slab's values v (G on the mask, Z elsewhere) as they were before any
+// segment was solved: every segment then stands alone, and the caller stores the
+// results once all segments of the row have read.  Inside the segment the sweeps
+// are those of wstep_sweeps, with the values and the backward coefficients in
+// registers.
+//   Left:  d_{base-1} of a run that enters the segment, by the forward
+//          recurrence from the run's start.
+//   Right: a run that goes on past the segment is eliminated from its other end,
+//          w_j = e w_{j-1} + f (pivots by the distance from that end: the same
+//          table), so the segment's last entry is (d + c f) / (1 - c e).
+// Fewer than half the instructions of the two sweeps over shared memory (no
+// second pass over the values, the table and the mask).  A segment is a mask
+// word in FP32; in FP64, where a warp instruction holds its scheduler's pipe for
+// 60 clocks however few lanes take part, shorter ones fill the lanes (121 x 144 x 7:
+// 7 rows are 7 lanes as rows, 126 as segments of 8).
+// ---------------------------------------------------------------------------
+template <typename T>
+constexpr int kWSeg = sizeof(T) == 8 ? 8 : 32;
+
+template <typename T, bool FULL, bool LAST>
+__device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP, const uint32_t* __restrict__ rowm,
+                                              int words, int sgm, int qn, int n2, T rho2, const T* __restrict__ wtab,
+                                              T (&v)[kWSeg<T>]) {
+  constexpr int SEG = kWSeg<T>;
+  const int base = SEG * sgm, bw = base >> 5, bb = base & 31;
+  const uint32_t word = rowm[bw], mw = word >> bb;
+#pragma unroll
+  for (int q = 0; q < SEG; ++q)
+    if (FULL || q < qn) v[q] = col[(base + q) * LP];
+  int st = 0;  // start of the run of missing entries that enters the segment
+  T d = T(0);
+  if (base > 0) {
+    uint32_t m = word & ((1u << bb) - 1u);
+    int u = bw;
+    while (m == 0u && u > 0) m = rowm[--u];
+    if (m) st = 32 * u + 32 - __clz(m);
+    if (!(mw & 1u)) {
+      if (st > 0) d = col[(st - 1) * LP];
+      const T* tb = wtab + (st == 0 ? 0 : n2);
+      for (int j = st; j < base; ++j) {
+        const T inv = tb[j - st];
+        d = fma(rho2 * inv, d, col[j * LP] * inv);
+      }
+    }
+  }
+  const int cw = ((st == 0) ? 0 : n2) + base - st;  // index base of entries without bits below
+  T c[SEG];
+#pragma unroll
+  for (int q = 0; q < SEG; ++q) {
+    if (FULL || q < qn) {
+      const bool ob = (mw >> q) & 1u;
+      const uint32_t below = mw & ((1u << q) - 1u);
+      int idx = below ? (n2 - 32 + q + __clz(below)) : (cw + q);
+      const bool end = LAST && base + q == n2 - 1;
+      if (end) idx += 4 * n2;
+      const T inv = wtab[idx];
+      // rho2 inv from its table in FP64, whose pipe is the scarce one
+      const T a = (sizeof(T) == 8 && !end) ? wtab[idx + 2 * n2] : rho2 * inv;
+      d = fma(ob ? T(0) : a, d, ob ? v[q] : v[q] * inv);
+      v[q] = d;
+      c[q] = (ob || end) ? T(0) : a;
+    }
+  }
+  T wn = T(0);
+  if (!LAST && !((mw >> (SEG - 1)) & 1u)) {
+    const int j1 = base + SEG;
+    int u = j1 >> 5;
+    uint32_t m = rowm[u] & (0xffffffffu << (j1 & 31));
+    while (m == 0u && u + 1 < words) m = rowm[++u];
+    const int k = m ? 32 * u + __ffs(m) - 1 : n2;  // next observed entry, or the row's end
+    T x = (k < n2) ? col[k * LP] : T(0), e = T(0);
+    const T* tb = wtab + (k < n2 ? n2 : 0);
+    for (int j = k - 1; j >= j1; --j) {
+      const T inv = tb[k - 1 - j];
+      e = rho2 * inv;
+      x = fma(e, x, col[j * LP] * inv);
+    }
+    wn = fma(c[SEG - 1], x, v[SEG - 1]);
+    if (k > j1) wn *= rcp_refined(fma(-c[SEG - 1], e, T(1)));
+    v[SEG - 1] = wn;
+    c[SEG - 1] = T(0);
+  }
+#pragma unroll
+  for (int q = SEG - 1; q >= 0; --q)
+    if (FULL || q < qn) {
+      wn = fma(c[q], wn, v[q]);
+      v[q] = wn;
+    }
+}
+
+// W-step of every row of the slab: a thread per (row, segment), as many whole
+// rows at a time as the block has threads for; rows at col_of(q) (stride LP
+// along j), their mask words at msk + q words.  Ends with a barrier.
+template <typename T, typename ColFn>
+__device__ __forceinline__ void wstep_segments(ColFn col_of, int LP, const uint32_t* __restrict__ msk, int nrows, int n2,
+                                               T rho2, const T* __restrict__ wtab) {
+  constexpr int SEG = kWSeg<T>;
+  const int words = (n2 + 31) >> 5, segs = (n2 + SEG - 1) / SEG, ql = n2 - SEG * (segs - 1);
+  const int rpr = blockDim.x / segs;  // rows per round (the block has at least segs threads)
+  const int row = threadIdx.x % rpr, w = threadIdx.x / rpr;
+  for (int r0 = 0; r0 < nrows; r0 += rpr) {
+    const bool work = w < segs && r0 + row < nrows;
+    T v[SEG];
+    T* col = nullptr;
+    if (work) {
+      col = col_of(r0 + row);
+      const uint32_t* rowm = msk + (size_t)(r0 + row) * words;
+      if (w < segs - 1) wstep_segment<T, true, false>(col, LP, rowm, words, w, SEG, n2, rho2, wtab, v);
+      else wstep_segment<T, false, true>(col, LP, rowm, words, w, ql, n2, rho2, wtab, v);
+    }
+    __syncthreads();
+    if (work) {
+      const int qn = (w < segs - 1) ? SEG : ql;
+      T* cb = col + SEG * w * LP;
+      if (qn == SEG) {
+#pragma unroll
+        for (int q = 0; q < SEG; ++q) cb[q * LP] = v[q];
+      } else {
+#pragma unroll
+        for (int q = 0; q < SEG; ++q)
+          if (q < qn) cb[q * LP] = v[q];
+      }
+    }
+  }
+  __syncthreads();
+}
+
 // Weighted |W~^{l+1} - W~^l|^2 of one half-spectrum entry: W~ = Z~ + R~, so the
 // change is (R~new - R~old) + (Z~new - Z~old); weight 1 for the real slices
 // (k = 0 and, for even n3, k = n3/2), 2 for the others (their mirror).
@@ -323,23 +449,19 @@ __device__ __forceinline__ double dw_term(cx<T> rnew, cx<T> rold, cx<T> dz, int 
 // Layouts used here: G row-major [i1][n3][n2] and mask words row-major
 // [i1][n3][ceil(n2/32)] (written by k_pack), copied to shared memory.
 // ---------------------------------------------------------------------------
-template <typename T, int L, int MODE, int TL = kTL>
-__global__ void __launch_bounds__(slab_max_threads(L), 1)
+template <typename T, int MODE, int TL = kTL>
+__global__ void __launch_bounds__(kSlabThreads, 1)
     k_slab(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
   const int slabs_in_smem = flags & SLAB_IN_SMEM;
   extern __shared__ __align__(16) unsigned char smem[];
   const int i1 = blockIdx.x;
   const int n1 = d.n1, n2 = d.n2;
-  const int n3 = (L > 0) ? L : d.n3;
+  const int n3 = d.n3;
   const int S = n3 / 2 + 1;
   const int LP = slab_stride(n3);
   const int tid = threadIdx.x, nt = blockDim.x;
   if (MODE == MODE_ITER && !init && converged(d)) return;
-  if (L > 0 && d.n3 != L) {
-    if (tid == 0) set_err(d.err, DEV_BAD_LAUNCH);
-    return;
-  }
-  const SlabLayout lay = slab_layout<T>(n2, n3, L > 0, slabs_in_smem != 0);
+  const SlabLayout lay = slab_layout<T>(n2, n3, slabs_in_smem != 0);
   T* wtab = reinterpret_cast<T*>(smem + lay.wtab);
   double* red = reinterpret_cast<double*>(smem + lay.red);
   uint32_t* msk = reinterpret_cast<uint32_t*>(smem + lay.msk);
@@ -366,71 +488,7 @@ __global__ void __launch_bounds__(slab_max_threads(L), 1)
   // ---- phase A: inverse transform of each tube; v = G on the mask ------------
   // (MODE_GRAD: v = Z - G on the mask, 0 elsewhere; gsum = ||v||^2)
   SqSum<T> gsum;
-  if constexpr (L > 0) {
-    constexpr int SL = L / 2 + 1;
-    if (MODE == MODE_ITER || MODE == MODE_GRAD) {
-      // G (row-major, read coalesced) is staged into the slab, transposed to the
-      // tube-major layout, with asynchronous copies issued ahead of the transforms;
-      // each tube then picks its observed values from its own column.
-      int l = tid / n2, t = tid - (tid / n2) * n2;
-      if (slabs_in_smem) {
-        for (int e = tid; e < n3 * n2; e += nt) {
-          cp_async_elem(spat + t * LP + l, Gi + e);
-          t += nt;
-          while (t >= n2) {
-            t -= n2;
-            ++l;
-          }
-        }
-        cp_async_wait_all();
-      } else {
-        for (int e = tid; e < n3 * n2; e += nt) {
-          spat[(size_t)t * LP + l] = __ldg(Gi + e);
-          t += nt;
-          while (t >= n2) {
-            t -= n2;
-            ++l;
-          }
-        }
-      }
-      __syncthreads();
-    }
-    for (int t0 = 0; t0 < n2; t0 += nt) {
-      const int t = t0 + tid;
-      if (t0 + (tid & ~31) >= n2) continue;  // whole warp past the last column (warp-uniform)
-      const bool act = t < n2;
-      cx<T> X[SL];
-#pragma unroll
-      for (int k = 0; k < SL; ++k) {
-        const size_t o = (size_t)k * n2 + (act ? t : 0);
-        if (MODE == MODE_ITER || MODE == MODE_GRAD) X[k] = ldg_cx(zrow + o);
-        else if (MODE == MODE_W) X[k] = ldg_cx(zrow + o) + ldg_cx(rrow + o);
-        else X[k] = ldg_cx(rrow + o);
-      }
-      T x[L];
-      fft::irfft<T, L>(X, x);
-      if (MODE == MODE_ITER) {
-        const int ta = act ? t : 0;
-#pragma unroll
-        for (int l = 0; l < L; ++l) {
-          const bool ob = act && ((msk[l * mwords + (ta >> 5)] >> (ta & 31)) & 1u);
-          x[l] = ob ? spat[(size_t)ta * LP + l] : x[l] * zfac;
-        }
-      } else if (MODE == MODE_GRAD) {
-        const int ta = act ? t : 0;
-#pragma unroll
-        for (int l = 0; l < L; ++l) {
-          const bool ob = act && ((msk[l * mwords + (ta >> 5)] >> (ta & 31)) & 1u);
-          x[l] = ob ? x[l] - spat[(size_t)ta * LP + l] : T(0);
-          gsum.add(x[l]);
-        }
-      }
-      if (act) {
-#pragma unroll
-        for (int l = 0; l < L; ++l) spat[t * LP + l] = x[l];
-      }
-    }
-  } else {
+  {
     // the half spectrum of the slab ([k][n2], as stored) and the twiddles
     cx<T>* tw = reinterpret_cast<cx<T>*>(smem + lay.tw);
     for (int m = tid; m < n3; m += nt) tw[m] = d.twg[m];
@@ -535,24 +593,7 @@ __global__ void __launch_bounds__(slab_max_threads(L), 1)
   // ---- phase C: forward transform, R~ = W~ - Z~ ------------------------------
   const bool track = (MODE == MODE_ITER) && !init && d.dZt != nullptr;
   double dw2 = 0.0;
-  if constexpr (L > 0) {
-    constexpr int SL = L / 2 + 1;
-    for (int t = tid; t < n2; t += nt) {
-      T x[L];
-#pragma unroll
-      for (int l = 0; l < L; ++l) x[l] = spat[t * LP + l];
-      cx<T> X[SL];
-      fft::rfft<T, L>(x, X);
-      cx<T>* rt = d.Rt + (size_t)i1 * SL * n2 + t;
-      const cx<T>* zt = zrow + t;
-#pragma unroll
-      for (int k = 0; k < SL; ++k) {
-        const cx<T> rn = (MODE == MODE_GRAD) ? X[k] : X[k] - ldg_cx(zt + (size_t)k * n2);
-        if (track) dw2 += dw_term(rn, rt[(size_t)k * n2], d.dZt[(size_t)i1 * SL * n2 + (size_t)k * n2 + t], k, L);
-        rt[(size_t)k * n2] = rn;
-      }
-    }
-  } else {
+  {
     // Eq. (bar BA-k) for any n3, as a product of the slab with the DFT matrix:
     // X_k = sum_l x_l w_{kl} for k < S, for items of one tube and TL consecutive
     // slices k, tube index fastest

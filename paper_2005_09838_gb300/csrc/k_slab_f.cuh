@@ -118,7 +118,9 @@ __device__ __forceinline__ cx<T> fwd_split(cx<T> zk, cx<T> zm, int k) {
   return E + cmul(O, fft::tw<T, L, false>(k));
 }
 
-template <typename T, int L, int N1, int N2, int MODE>
+// SEGW: the W-step by wstep_sweeps_seg, bit for bit the sequential sweeps (the
+// TC_BF16 form, see kTL); else one thread per segment (wstep_segments).
+template <typename T, int L, int N1, int N2, int MODE, bool SEGW = false>
 __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
   constexpr int M = L / 2;
   static_assert(L % 2 == 0 && M == N1 * N2, "n3 = 2 N1 N2");
@@ -144,8 +146,12 @@ __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __rest
   const bool wsolve = (MODE == MODE_ITER) && !init && d.rho2 != T(0);
   const T zfac = init ? T(0) : ((d.rho2 == T(0)) ? T(1) / (T(1) + d.mu) : T(1));
 
+  // mask words of the rows in slab order: row q is the one at offset q of a tube
   if (MODE != MODE_W)
-    for (int j = tid; j < L * mw; j += nt) msk[j] = __ldg(d.mask + (size_t)i1 * L * mw + j);
+    for (int j = tid; j < L * mw; j += nt) {
+      const int l = j / mw;
+      msk[slab_f_off<N1, N2>(l) * mw + (j - l * mw)] = __ldg(d.mask + (size_t)i1 * L * mw + j);
+    }
   if (wsolve)
     for (int j = tid; j < 6 * n2; j += nt) wtab[j] = d.winv[j];
 
@@ -247,13 +253,13 @@ __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __rest
       for (int k2 = 0; k2 < N2; ++k2) {
         T x0 = o[k2].re * scale, x1 = o[k2].im * scale;
         if (MODE == MODE_ITER) {
-          const int l = 2 * (k1 + N1 * k2);
-          const uint32_t w0 = msk[l * mw + (t >> 5)], w1 = msk[(l + 1) * mw + (t >> 5)];
+          const int q = 2 * (N2 * k1 + k2);
+          const uint32_t w0 = msk[q * mw + (t >> 5)], w1 = msk[(q + 1) * mw + (t >> 5)];
           x0 = ((w0 >> (t & 31)) & 1u) ? g[2 * k2] : x0 * zfac;
           x1 = ((w1 >> (t & 31)) & 1u) ? g[2 * k2 + 1] : x1 * zfac;
         } else if (MODE == MODE_GRAD) {
-          const int l = 2 * (k1 + N1 * k2);
-          const uint32_t w0 = msk[l * mw + (t >> 5)], w1 = msk[(l + 1) * mw + (t >> 5)];
+          const int q = 2 * (N2 * k1 + k2);
+          const uint32_t w0 = msk[q * mw + (t >> 5)], w1 = msk[(q + 1) * mw + (t >> 5)];
           x0 = ((w0 >> (t & 31)) & 1u) ? x0 - g[2 * k2] : T(0);
           x1 = ((w1 >> (t & 31)) & 1u) ? x1 - g[2 * k2 + 1] : T(0);
           gsum.add(x0);
@@ -281,7 +287,7 @@ __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __rest
           else Wout[(size_t)i1 + (size_t)n1 * ((size_t)t + (size_t)n2 * l)] = v;
         }
       } else {
-        if ((msk[l * mw + (t >> 5)] >> (t & 31)) & 1u) sb.add(v);
+        if ((msk[off * mw + (t >> 5)] >> (t & 31)) & 1u) sb.add(v);
       }
     }
     if (!sums) return;
@@ -295,12 +301,12 @@ __global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __rest
     return;
   }
 
-  // ---- W-step (rows split into segments of mask words) ---------------------------------------
+  // ---- W-step ----------------------------------------------------------------------------------
   if (wsolve) {
-    // rows split into nseg segments so that every thread has one (row, segment)
-    const int nseg = max(1, nt / L);
-    auto col_of = [&](int l) { return buf + slab_f_off<N1, N2>(l); };
-    wstep_sweeps_seg<T>(col_of, LP, msk, stw, L, nseg, tid, n2, d.rho2, wtab);
+    auto col_of = [&](int q) { return buf + q; };
+    // SEGW: rows split into segments so that every thread has one (row, segment)
+    if (SEGW) wstep_sweeps_seg<T>(col_of, LP, msk, stw, L, max(1, nt / L), tid, n2, d.rho2, wtab);
+    else wstep_segments<T>(col_of, LP, msk, L, n2, d.rho2, wtab);
   }
 
   // ---- C1: forward DFT_N2 over slots N2 k1 + j, twiddle w_M^{k1 q} -----------------------

@@ -21,7 +21,7 @@
 // consecutive rows of a tube, both without bank conflicts.
 //
 // Tiles.  A warp computes TL rows (inverse) or slices (forward) of 64 tubes
-// (two per lane): each pair that is read feeds TL products and each
+// (two per lane; FP64: 32): each pair that is read feeds TL products and each
 // coefficient two.  tc_init times TL = 2, 4, 8 (a larger tile has fewer loads
 // per product, a smaller one fills the warps of small slabs).
 //
@@ -43,8 +43,11 @@ namespace tc {
 // two each, so half as many threads).
 template <typename T>
 constexpr int kSlabGThreads = sizeof(T) == 8 ? 256 : 512;
-constexpr int kTT = 2;                // tubes per lane
-constexpr int kGTubes = 32 * kTT;     // tubes per item
+// Tubes per lane (FP64: one, no product is worth a half-empty warp there) and per item.
+template <typename T>
+constexpr int kTT = sizeof(T) == 8 ? 1 : 2;
+template <typename T>
+constexpr int kGTubes = 32 * kTT<T>;
 constexpr int kSlabGMaxN3 = 512;      // the tables grow as n3^2
 
 // Pairs of T with packed arithmetic.
@@ -175,7 +178,8 @@ struct SlabGLayout {
 // Tubes per slot of the slab: odd, so that consecutive slots start in other banks.
 __host__ __device__ inline int slab_g_stride(int n2) { return n2 | 1; }
 // Tubes of a stage of sg groups.
-__host__ __device__ inline int slab_g_width(int n2, int sg) { return sg * kGTubes < n2 ? sg * kGTubes : n2; }
+template <typename T>
+__host__ __device__ inline int slab_g_width(int n2, int sg) { return sg * kGTubes<T> < n2 ? sg * kGTubes<T> : n2; }
 // sg: 64-tube groups per stage (0: unstaged).
 template <typename T>
 __host__ __device__ inline SlabGLayout slab_g_layout(int n2, int n3, int sg) {
@@ -196,9 +200,38 @@ __host__ __device__ inline SlabGLayout slab_g_layout(int n2, int n3, int sg) {
   L.pairs = off;
   off = align_up(off + sizeof(cx<T>) * (size_t)((n3 + 1) / 2) * slab_g_stride(n2), 16);
   L.stage = off;
-  off = align_up(off + sizeof(cx<T>) * (size_t)(n3 / 2 + 1) * slab_g_width(n2, sg), 16);
+  off = align_up(off + sizeof(cx<T>) * (size_t)(n3 / 2 + 1) * slab_g_width<T>(n2, sg), 16);
   L.total = off;
   return L;
+}
+
+// Launch shape of the folded-transform slab kernels: two CTAs of 256 threads on
+// an SM where the slab, the coefficients and a stage of one group fit half of
+// its shared memory, else one with twice the threads; as many groups per stage
+// as fit; unstaged where even one does not.  False where the slab itself does
+// not fit (k_slab keeps it in global memory).
+struct SlabGPlan {
+  int threads, sg;
+  size_t smem;
+};
+template <typename T>
+inline bool slab_g_plan(int n2, int n3, int optin, SlabGPlan& pl) {
+  // (the W-step has a thread per segment of a row)
+  if (n3 > kSlabGMaxN3 || (n2 + kWSeg<T> - 1) / kWSeg<T> > 256) return false;
+  const int ngr = (n2 + kGTubes<T> - 1) / kGTubes<T>;
+  const size_t half = (size_t)(optin + kStaticSmemReserve + 1024) / 2 - 1024;  // 1 KB per CTA is the system's
+  for (int pass = 0; pass < 2; ++pass) {
+    const size_t room = pass == 0 ? half : (size_t)optin;
+    for (int sg = ngr; sg >= 1; --sg) {
+      const size_t b = slab_g_layout<T>(n2, n3, sg).total;
+      if (b <= room) {
+        pl = SlabGPlan{pass == 0 ? 256 : kSlabGThreads<T>, sg, b};
+        return true;
+      }
+    }
+  }
+  pl = SlabGPlan{kSlabGThreads<T>, 0, slab_g_layout<T>(n2, n3, 0).total};
+  return pl.smem <= (size_t)optin;
 }
 
 // Row l of the q-th row in slab order (slot by slot), 0 <= q < n3, and the
@@ -219,17 +252,17 @@ __device__ __forceinline__ int slab_g_off(bool even, int n3, int l, int np2) {
 }
 
 // One item of the inverse transform: rows l0 .. l0 + TL - 1 (and those that
-// follow from them) of kGTubes tubes.  load(k, j) gives the spectrum pair of
+// follow from them) of kGTubes<T> tubes.  load(k, j) gives the spectrum pair of
 // slice k in tube j of the lane; E, O receive the sums over even and odd
 // slices (all slices in E for odd n3), slices 0 and n3/2 included with weight 1/2.
 template <typename T, int TL, bool EVEN, bool SH, typename LoadFn>
 __device__ __forceinline__ void fold_inverse(const FoldDims& f, const cx<T>* __restrict__ tab, int l0, LoadFn load,
-                                             typename Pk<T>::V (&E)[TL][kTT],
-                                             typename Pk<T>::V (&O)[EVEN ? TL : 1][kTT]) {
+                                             typename Pk<T>::V (&E)[TL][kTT<T>],
+                                             typename Pk<T>::V (&O)[EVEN ? TL : 1][kTT<T>]) {
   using P = Pk<T>;
   using V = typename P::V;
 #pragma unroll
-  for (int j = 0; j < kTT; ++j) {
+  for (int j = 0; j < kTT<T>; ++j) {
     const V x0 = P::mk(T(0.5) * P::un(load(0, j)).re, T(0));
 #pragma unroll
     for (int i = 0; i < TL; ++i) E[i][j] = x0;
@@ -245,46 +278,46 @@ __device__ __forceinline__ void fold_inverse(const FoldDims& f, const cx<T>* __r
     }
   }
   const cx<T>* tl = tab + l0;
-  auto step = [&](int k, const V (&x)[kTT], V (&acc)[TL][kTT]) {
+  auto step = [&](int k, const V (&x)[kTT<T>], V (&acc)[TL][kTT<T>]) {
     const cx<T>* tk = tl + (size_t)k * f.nlp;
 #pragma unroll
     for (int i = 0; i < TL; i += 2) {
       V c0, c1;
       P::template ld2<SH>(tk + i, c0, c1);
 #pragma unroll
-      for (int j = 0; j < kTT; ++j) {
+      for (int j = 0; j < kTT<T>; ++j) {
         P::fma(acc[i][j], x[j], c0);
         P::fma(acc[i + 1][j], x[j], c1);
       }
     }
   };
-  auto acc_of = [&](int odd) -> V(&)[TL][kTT] {
+  auto acc_of = [&](int odd) -> V(&)[TL][kTT<T>] {
     if constexpr (EVEN) {
       if (odd) return O;
     }
     return E;
   };
   constexpr int U = 4;  // slices whose loads are in flight together (even: parity fixed per position)
-  V xn[U][kTT];
+  V xn[U][kTT<T>];
   int k = 1;
   const int kend = 1 + f.kmax / U * U;
   if (k < kend) {
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int j = 0; j < kTT; ++j) xn[u][j] = load(k + u, j);
+      for (int j = 0; j < kTT<T>; ++j) xn[u][j] = load(k + u, j);
   }
   for (; k < kend; k += U) {
-    V x[U][kTT];
+    V x[U][kTT<T>];
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int j = 0; j < kTT; ++j) x[u][j] = xn[u][j];
+      for (int j = 0; j < kTT<T>; ++j) x[u][j] = xn[u][j];
     if (k + U < kend) {
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int j = 0; j < kTT; ++j) xn[u][j] = load(k + U + u, j);
+        for (int j = 0; j < kTT<T>; ++j) xn[u][j] = load(k + U + u, j);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) step(k + u, x[u], acc_of((u + 1) & 1));
@@ -292,27 +325,27 @@ __device__ __forceinline__ void fold_inverse(const FoldDims& f, const cx<T>* __r
 #pragma unroll
   for (int u = 0; u < U - 1; ++u) {
     if (k + u <= f.kmax) {
-      V x[kTT];
+      V x[kTT<T>];
 #pragma unroll
-      for (int j = 0; j < kTT; ++j) x[j] = load(k + u, j);
+      for (int j = 0; j < kTT<T>; ++j) x[j] = load(k + u, j);
       step(k + u, x, acc_of((u + 1) & 1));
     }
   }
 }
 
 // One item of the forward transform: columns q0 .. q0 + TL - 1 of the forward
-// table (slices of one parity for even n3) of kGTubes tubes, from the folded
+// table (slices of one parity for even n3) of kGTubes<T> tubes, from the folded
 // slab.  acc receives (sum e c, sum o s).
 template <typename T, int TL, bool EVEN, bool SH>
 __device__ __forceinline__ void fold_forward(const FoldDims& f, const cx<T>* __restrict__ tab, int q0,
-                                             const cx<T>* const (&col)[kTT], int np2,
-                                             typename Pk<T>::V (&acc)[TL][kTT]) {
+                                             const cx<T>* const (&col)[kTT<T>], int np2,
+                                             typename Pk<T>::V (&acc)[TL][kTT<T>]) {
   using P = Pk<T>;
   using V = typename P::V;
   const bool oddk = EVEN && q0 >= f.nkep;
   const int kk0 = oddk ? q0 - f.nkep : q0;  // k = 2 (kk0 + i) + oddk for even n3
 #pragma unroll
-  for (int j = 0; j < kTT; ++j) {
+  for (int j = 0; j < kTT<T>; ++j) {
     const cx<T> s0 = col[j][0];
     const V a0 = P::mk(EVEN && oddk ? s0.im : s0.re, T(0));
 #pragma unroll
@@ -333,143 +366,22 @@ __device__ __forceinline__ void fold_forward(const FoldDims& f, const cx<T>* __r
   const cx<T>* tq = tab + q0;
 #pragma unroll 4
   for (int l = 1; l <= f.lmax; ++l) {
-    V x[kTT];
+    V x[kTT<T>];
     const int so = (sl + sd * l) * np2;
 #pragma unroll
-    for (int j = 0; j < kTT; ++j) x[j] = P::lds(col[j] + so);
+    for (int j = 0; j < kTT<T>; ++j) x[j] = P::lds(col[j] + so);
     const cx<T>* tk = tq + (size_t)l * f.nkt;
 #pragma unroll
     for (int i = 0; i < TL; i += 2) {
       V c0, c1;
       P::template ld2<SH>(tk + i, c0, c1);
 #pragma unroll
-      for (int j = 0; j < kTT; ++j) {
+      for (int j = 0; j < kTT<T>; ++j) {
         P::fma(acc[i][j], x[j], c0);
         P::fma(acc[i + 1][j], x[j], c1);
       }
     }
   }
-}
-
-// W-step of one mask word (32 entries, fewer in the last word) of one row, from
-// the slab's values v (G on the mask, Z elsewhere) as they were before any word
-// was solved: every word then stands alone, and the caller stores the results
-// once all words of the row have read.  Inside the word the sweeps are those of
-// wstep_sweeps, with the values and the backward coefficients in registers.
-//   Left:  d_{base-1} of a run that enters the word, by the forward recurrence
-//          from the run's start.
-//   Right: a run that goes on past the word is eliminated from its other end,
-//          w_j = e w_{j-1} + f (pivots by the distance from that end: the same
-//          table), so the last entry of the word is (d + c f) / (1 - c e).
-// Fewer than half the instructions of the two sweeps over shared memory (no
-// second pass over the values, the table and the mask) and one thread per word.
-template <typename T, bool FULL, bool LAST>
-__device__ __forceinline__ void wstep_word(const T* __restrict__ col, int LP, const uint32_t* __restrict__ rowm, int words,
-                                           int w, int qn, int n2, T rho2, const T* __restrict__ wtab, T (&v)[32]) {
-  const int base = 32 * w;
-  const uint32_t mw = rowm[w];
-#pragma unroll
-  for (int q = 0; q < 32; ++q)
-    if (FULL || q < qn) v[q] = col[(base + q) * LP];
-  int st = 0;  // start of the run of missing entries that enters the word
-  T d = T(0);
-  if (w > 0) {
-    for (int u = w - 1; u >= 0; --u)
-      if (rowm[u]) {
-        st = 32 * u + 32 - __clz(rowm[u]);
-        break;
-      }
-    if (!(mw & 1u)) {
-      if (st > 0) d = col[(st - 1) * LP];
-      const T* tb = wtab + (st == 0 ? 0 : n2);
-      for (int j = st; j < base; ++j) {
-        const T inv = tb[j - st];
-        d = fma(rho2 * inv, d, col[j * LP] * inv);
-      }
-    }
-  }
-  const int cw = ((st == 0) ? 0 : n2) + base - st;  // index base of entries without bits below
-  T c[32];
-#pragma unroll
-  for (int q = 0; q < 32; ++q) {
-    if (FULL || q < qn) {
-      const bool ob = (mw >> q) & 1u;
-      const uint32_t below = mw & ((1u << q) - 1u);
-      int idx = below ? (n2 - 32 + q + __clz(below)) : (cw + q);
-      const bool end = LAST && base + q == n2 - 1;
-      if (end) idx += 4 * n2;
-      const T inv = wtab[idx];
-      // rho2 inv from its table in FP64, whose pipe is the scarce one
-      const T a = (sizeof(T) == 8 && !end) ? wtab[idx + 2 * n2] : rho2 * inv;
-      d = fma(ob ? T(0) : a, d, ob ? v[q] : v[q] * inv);
-      v[q] = d;
-      c[q] = (ob || end) ? T(0) : a;
-    }
-  }
-  T wn = T(0);
-  if (!LAST && !(mw >> 31)) {
-    const int j1 = base + 32;
-    int k = n2;
-    for (int u = w + 1; u < words; ++u)
-      if (rowm[u]) {
-        k = 32 * u + __ffs(rowm[u]) - 1;
-        break;
-      }
-    T x = (k < n2) ? col[k * LP] : T(0), e = T(0);
-    const T* tb = wtab + (k < n2 ? n2 : 0);
-    for (int j = k - 1; j >= j1; --j) {
-      const T inv = tb[k - 1 - j];
-      e = rho2 * inv;
-      x = fma(e, x, col[j * LP] * inv);
-    }
-    const T num = fma(c[31], x, v[31]);
-    wn = (k > j1) ? num * rcp_refined(fma(-c[31], e, T(1))) : num;
-    v[31] = wn;
-    c[31] = T(0);
-  }
-#pragma unroll
-  for (int q = 31; q >= 0; --q)
-    if (FULL || q < qn) {
-      wn = fma(c[q], wn, v[q]);
-      v[q] = wn;
-    }
-}
-
-// W-step of every row of the slab: a thread per (row, word), as many whole rows
-// at a time as the block has threads for; rows at col_of(q) (stride LP along j).
-// Ends with a barrier.
-template <typename T, typename ColFn>
-__device__ __forceinline__ void wstep_words(ColFn col_of, int LP, const uint32_t* __restrict__ msk, int nrows, int n2,
-                                            T rho2, const T* __restrict__ wtab) {
-  const int words = (n2 + 31) >> 5, ql = n2 - 32 * (words - 1);
-  const int rpr = blockDim.x / words;  // rows per round (n2 <= 4096: words <= 128 <= threads)
-  const int row = threadIdx.x % rpr, w = threadIdx.x / rpr;
-  for (int r0 = 0; r0 < nrows; r0 += rpr) {
-    const bool work = w < words && r0 + row < nrows;
-    T v[32];
-    T* col = nullptr;
-    if (work) {
-      col = col_of(r0 + row);
-      const uint32_t* rowm = msk + (size_t)(r0 + row) * words;
-      if (w < words - 1) wstep_word<T, true, false>(col, LP, rowm, words, w, 32, n2, rho2, wtab, v);
-      else if (ql == 32) wstep_word<T, true, true>(col, LP, rowm, words, w, 32, n2, rho2, wtab, v);
-      else wstep_word<T, false, true>(col, LP, rowm, words, w, ql, n2, rho2, wtab, v);
-    }
-    __syncthreads();
-    if (work) {
-      const int qn = (w < words - 1) ? 32 : ql;
-      T* cb = col + 32 * w * LP;
-      if (qn == 32) {
-#pragma unroll
-        for (int q = 0; q < 32; ++q) cb[q * LP] = v[q];
-      } else {
-#pragma unroll
-        for (int q = 0; q < 32; ++q)
-          if (q < qn) cb[q * LP] = v[q];
-      }
-    }
-  }
-  __syncthreads();
 }
 
 template <typename T, int MODE, int TL, bool EVEN, bool STAGED>
@@ -520,15 +432,15 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
 
   // ---- inverse transform; v = G on the mask, Z elsewhere (MODE_GRAD: Z - G on the
   // mask, 0 elsewhere) --------------------------------------------------------------------
-  const int ngr = (n2 + kGTubes - 1) / kGTubes;
+  const int ngr = (n2 + kGTubes<T> - 1) / kGTubes<T>;
   const int gstage = STAGED ? sg : ngr;
-  const int width = slab_g_width(n2, gstage);  // tubes of a full stage, its row stride
+  const int width = slab_g_width<T>(n2, gstage);  // tubes of a full stage, its row stride
   const T scale = T(2) / T(n3);
   SqSum<T> gsum;
   for (int g0 = 0; g0 < ngr; g0 += gstage) {
     const int gn = min(gstage, ngr - g0);
     if (STAGED) {
-      const int t0 = g0 * kGTubes, tn = min(gn * kGTubes, n2 - t0);
+      const int t0 = g0 * kGTubes<T>, tn = min(gn * kGTubes<T>, n2 - t0);
       if (g0 > 0) __syncthreads();  // the stage is read no more
       for (int k = wid; k < S; k += nw) {
         const cx<T>* zs = (MODE == MODE_R ? rrow : zrow) + (size_t)k * n2 + t0;
@@ -544,14 +456,14 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
     const int ntile = (f.nl + TL - 1) / TL;
     for (int e = wid; e < ntile * gn; e += nw) {
       const int gl = e / ntile, g = g0 + gl, l0 = (e - gl * ntile) * TL;
-      int t[kTT];
-      const cx<T>* zc[kTT];
-      const cx<T>* rc[kTT];
+      int t[kTT<T>];
+      const cx<T>* zc[kTT<T>];
+      const cx<T>* rc[kTT<T>];
 #pragma unroll
-      for (int j = 0; j < kTT; ++j) {
-        t[j] = g * kGTubes + 32 * j + lane;
+      for (int j = 0; j < kTT<T>; ++j) {
+        t[j] = g * kGTubes<T> + 32 * j + lane;
         const int tq = min(t[j], n2 - 1);
-        zc[j] = STAGED ? stg + (tq - g0 * kGTubes) : zrow + tq;
+        zc[j] = STAGED ? stg + (tq - g0 * kGTubes<T>) : zrow + tq;
         rc[j] = rrow + tq;
       }
       auto load = [&](int k, int j) -> V {
@@ -560,14 +472,14 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
         if (MODE == MODE_W) return P::add(P::ldg(zc[j] + o), P::ldg(rc[j] + o));
         return P::ldg((MODE == MODE_R ? rc[j] : zc[j]) + o);
       };
-      V E[TL][kTT], O[EVEN ? TL : 1][kTT];
+      V E[TL][kTT<T>], O[EVEN ? TL : 1][kTT<T>];
       fold_inverse<T, TL, EVEN, STAGED>(f, tabi, l0, load, E, O);
       // value of the row at slab index q (row order), half h of slot p, tube j
       auto put = [&](T x, int q, T* at, int j) {
         x *= scale;
         const bool live = t[j] < n2;
         if (NEED_G) {
-          const uint32_t w = (g * kTT + j < mw) ? msk[q * mw + g * kTT + j] : 0u;
+          const uint32_t w = (g * kTT<T> + j < mw) ? msk[q * mw + g * kTT<T> + j] : 0u;
           const bool ob = (w >> lane) & 1u;
           if (MODE == MODE_ITER) {
             if (live && !ob) *at = x * zfac;
@@ -585,7 +497,7 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
         const int l = l0 + i;
         if (l >= f.nl) break;
 #pragma unroll
-        for (int j = 0; j < kTT; ++j) {
+        for (int j = 0; j < kTT<T>; ++j) {
           T* cp = spat + 2 * (l * np2 + t[j]);
           if constexpr (EVEN) {
             const cx<T> a = P::un(E[i][j]), b = P::un(O[i][j]);
@@ -653,7 +565,7 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
 
   // ---- W-step -------------------------------------------------------------------------------
   if (wsolve)
-    wstep_words<T>([&](int q) { return spat + slab_g_off(EVEN, n3, slab_g_row(EVEN, n3, q), np2); }, 2, msk, n3, n2,
+    wstep_segments<T>([&](int q) { return spat + slab_g_off(EVEN, n3, slab_g_row(EVEN, n3, q), np2); }, 2, msk, n3, n2,
                    d.rho2, wtab);
 
   // ---- fold -----------------------------------------------------------------------------------
@@ -693,21 +605,21 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
       for (int e = wid; e < ntile * ngr; e += nw) {
         const int g = e / ntile, it = e - g * ntile;
         const int q0 = (it < nte) ? it * TL : f.nkep + (it - nte) * TL;
-        int t[kTT];
-        const cx<T>* col[kTT];
+        int t[kTT<T>];
+        const cx<T>* col[kTT<T>];
 #pragma unroll
-        for (int j = 0; j < kTT; ++j) {
-          t[j] = g * kGTubes + 32 * j + lane;
+        for (int j = 0; j < kTT<T>; ++j) {
+          t[j] = g * kGTubes<T> + 32 * j + lane;
           col[j] = pairs + min(t[j], n2 - 1);
         }
-        V acc[TL][kTT];
+        V acc[TL][kTT<T>];
         fold_forward<T, TL, EVEN, STAGED>(f, tabf, q0, col, np2, acc);
 #pragma unroll
         for (int i = 0; i < TL; ++i) {
           const int k = EVEN ? (it < nte ? 2 * (q0 + i) : 2 * (q0 - f.nkep + i) + 1) : q0 + i;
           if (k >= S) break;
 #pragma unroll
-          for (int j = 0; j < kTT; ++j) {
+          for (int j = 0; j < kTT<T>; ++j) {
             if (t[j] >= n2) continue;
             const int o = k * n2 + t[j];
             const cx<T> a = P::un(acc[i][j]);

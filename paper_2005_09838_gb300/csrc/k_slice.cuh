@@ -83,19 +83,6 @@ __device__ inline float warp_frob_lowp(const cx<T>* M, int r) {
   return sqrtf(sq) * pow2f(ex);  // infinite beyond the FP32 range
 }
 
-// 1/a.  FP64: a correctly rounded FP32 seed and two Newton steps
-// y <- y (2 - a y) (the error squares at each step); FP64 division is slow on
-// this part.  FP32: the IEEE quotient.
-__device__ __forceinline__ double rcp_refined(double a) {
-  const float af = (float)a;
-  if (!(fabsf(af) > 1e-30f && fabsf(af) < 1e30f)) return 1.0 / a;
-  double y = (double)__frcp_rn(af);
-  y = y * fma(-a, y, 2.0);
-  y = y * fma(-a, y, 2.0);
-  return y;
-}
-__device__ __forceinline__ float rcp_refined(float a) { return 1.0f / a; }
-
 // Smallest positive normal number of T, as a guard for pivots.
 template <typename T>
 __device__ __forceinline__ T tiny_pivot() {
@@ -248,6 +235,27 @@ __device__ __forceinline__ int gauss_jordan_inplace_df(cx<double>* W64, cx<doubl
   return ok;
 }
 
+// Square root of the sum of a non-negative value over the lanes of a warp, for a
+// certificate (a few digits).  FP64: exponents and FP32 mantissas, since a
+// dependent FP64 operation takes some 60 clocks and a square root twenty of them.
+__device__ __forceinline__ float warp_norm(float a) {
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return sqrtf(a);
+}
+__device__ __forceinline__ double warp_norm(double a) {
+  const int hi = __double2hiint(a), e = ((hi >> 20) & 0x7ff) - 1023;
+  int en = max(e >> 1, -500);  // a = m 2^e = 4^en sq
+  float sq = (e < -1000) ? 0.f : __int_as_float(0x3f800000 | ((hi & 0xfffff) << 3)) * ((e & 1) ? 2.f : 1.f);
+  const bool bad = __any_sync(0xffffffffu, e == 1024);
+  for (int o = 16; o > 0; o >>= 1) {
+    const int e2 = __shfl_xor_sync(0xffffffffu, en, o);
+    const float q2 = __shfl_xor_sync(0xffffffffu, sq, o);
+    nrm_merge(en, sq, e2, q2);
+  }
+  if (bad) return INFINITY;
+  return (double)sqrtf(sq) * __hiloint2double((en + 1023) << 20, 0);
+}
+
 // Gauss-Jordan inverse of the Hermitian r x r matrix A (r <= RP <= 16) by one
 // warp with [A | I] in registers: lane j holds column j of the 2r augmented
 // columns, and the pivot column reaches the other lanes by shuffles.  On
@@ -271,10 +279,8 @@ __device__ int warp_gj_inverse(const cx<T>* A, cx<T>* Ainv, int r, T& an, T& in)
   for (int i = 0; i < RP; ++i) cs += c[i].re * c[i].re + c[i].im * c[i].im;
   an = T(0);
   in = T(0);
-  T a = (lane < r) ? cs : T(0);
-  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-  an = sqrt(a);
-  if (!(a > T(0) && isfinite(a))) return 0;
+  an = warp_norm((lane < r) ? cs : T(0));
+  if (!(an > T(0) && isfinite(an))) return 0;
   // a runtime pivot loop with row p picked by selects: the body (RP rows) is
   // fetched once and stays in the instruction cache for the later pivots (the
   // code runs once per launch and CTA, so an unrolled body runs cold)
@@ -298,9 +304,7 @@ __device__ int warp_gj_inverse(const cx<T>* A, cx<T>* Ainv, int r, T& an, T& in)
   cs = T(0);
 #pragma unroll
   for (int i = 0; i < RP; ++i) cs += c[i].re * c[i].re + c[i].im * c[i].im;
-  a = (lane >= r && lane < 2 * r) ? cs : T(0);
-  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-  in = sqrt(a);
+  in = warp_norm((lane >= r && lane < 2 * r) ? cs : T(0));
   if (lane >= r && lane < 2 * r) {
 #pragma unroll
     for (int i = 0; i < RP; ++i)
@@ -1020,11 +1024,14 @@ struct Log2<1> {
 
 // ---------------------------------------------------------------------------
 // Q_k = R~_k Y~_k^H (n1 x r per slice), the W~Y~^H part of the X-gradient of
-// Eq. (hkXYDer) that involves the residual.  Grid (S, ceil(n1/32)); a warp
+// Eq. (hkXYDer) that involves the residual.  Grid (S, ceil(n1/qrows)); a warp
 // takes one or two rows at a time with coalesced loads along the rows, four
 // 32-column loads per row in flight, Y~_k staged in shared memory.  Reads R~
-// once.
+// once.  qrows is 32, fewer where that leaves SMs idle (small S n1): FP64 has
+// one row per warp, on 121 x 144 x 7 (16 CTAs of 32 rows) 30 -> 5 us.
 // ---------------------------------------------------------------------------
+template <typename T, int RP>
+constexpr int kQRR = (RP <= 8 && sizeof(T) == 4) ? 2 : 1;  // rows per pass of a warp
 template <typename T, int RP>
 __global__ void __launch_bounds__(kSliceThreads) k_qcon(Dev<T> d, cx<T>* __restrict__ Qout) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1037,14 +1044,15 @@ __global__ void __launch_bounds__(kSliceThreads) k_qcon(Dev<T> d, cx<T>* __restr
   for (int e = tid; e < r * n2; e += blockDim.x) Ys[e] = Y[e];
   __syncthreads();
   constexpr int HALF = (RP > 16) ? 16 : RP;  // complex values per reduction pass
-  constexpr int RR = (RP <= 8) ? 2 : 1;       // rows per pass of a warp
+  constexpr int RR = kQRR<T, RP>;
   constexpr int U = 4;                        // 32-column loads in flight per row
-  for (int ii = wid * RR; ii < 32; ii += nw * RR) {
+  const int rows = d.qrows;
+  for (int ii = wid * RR; ii < rows; ii += nw * RR) {
     const cx<T>* rowp[RR];
     bool live[RR];
 #pragma unroll
     for (int q = 0; q < RR; ++q) {
-      const int i = blockIdx.y * 32 + ii + q;
+      const int i = blockIdx.y * rows + ii + q;
       live[q] = i < n1;
       rowp[q] = d.Rt + ((size_t)(live[q] ? i : 0) * S + k) * n2;
     }
@@ -1080,7 +1088,7 @@ __global__ void __launch_bounds__(kSliceThreads) k_qcon(Dev<T> d, cx<T>* __restr
 #pragma unroll
     for (int q = 0; q < RR; ++q) {
       if (!live[q]) continue;
-      const int i = blockIdx.y * 32 + ii + q;
+      const int i = blockIdx.y * rows + ii + q;
 #pragma unroll
       for (int h = 0; h < RP; h += HALF) {
         T f[2 * HALF];
@@ -1543,6 +1551,54 @@ __global__ void __launch_bounds__(xstep_threads(RP), 1) k_xstep(Dev<T> d, const 
     for (int e = tid; e < r * n1; e += blockDim.x) Xg[e] = Ts[e];
     return;
   }
+  // ---- FP64, arrays resident: G = X~'^H (X~' + rho1 H^T H X~') (upper triangle) and
+  // Dg = -X~'^H ((X~' - X~) + rho1 H^T H X~'), the right factors formed once per entry
+  // (over Q and X~, both done with): four FP64 operations per product of either where
+  // the form below takes sixteen for the three sums (121 x 144 x 7, r = 4: 41 -> 30 us
+  // for the whole X-step)
+  if (sizeof(T) == 8 && arrays_in_smem) {
+    for (int e = tid; e < r * n1; e += blockDim.x) {
+      const int s = e / n1, i = e - s * n1;
+      const cx<T> x = Ts[e], h = hth_at(Ts + (size_t)s * n1, i, n1);
+      const cx<T> dx = x - Xs[e];
+      Qs[e] = cx<T>{fma(rho1, h.re, x.re), fma(rho1, h.im, x.im)};
+      Xs[e] = cx<T>{fma(rho1, h.re, dx.re), fma(rho1, h.im, dx.im)};
+    }
+    __syncthreads();
+    const int ntri = r * (r + 1) / 2, ntask = rr + ntri;
+    int tp = 1;
+    while (tp < 32 && tp * 2 * ntask <= (int)blockDim.x) tp *= 2;
+    const int q = tid & (tp - 1), per = blockDim.x / tp;
+    for (int t0 = 0; t0 < ntask; t0 += per) {
+      const int task = t0 + tid / tp;
+      int s = 0, u = 0;
+      cx<T> acc = {T(0), T(0)};
+      if (task < ntask) {
+        if (task < rr) {
+          s = task / r;
+          u = task - s * r;
+        } else {
+          tri_index(task - rr, r, s, u);
+        }
+        const cx<T>* xs = Ts + (size_t)s * n1;
+        const cx<T>* v = (task < rr ? Xs : Qs) + (size_t)u * n1;
+        for (int i = q; i < n1; i += tp) cfmaconj(acc, xs[i], v[i]);
+      }
+      for (int o = tp >> 1; o > 0; o >>= 1) {
+        acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
+        acc.im += __shfl_xor_sync(0xffffffffu, acc.im, o);
+      }
+      if (task < ntask && q == 0) {
+        if (task < rr) {
+          Dgm[s * r + u] = cx<TS>{(TS)-acc.re, realslice ? TS(0) : (TS)-acc.im};
+        } else {
+          if (s == u || realslice) acc.im = T(0);
+          Gm[s * r + u] = cvt<TS>(acc);
+          Gm[u * r + s] = cx<TS>{(TS)acc.re, -(TS)acc.im};
+        }
+      }
+    }
+  } else
   // ---- G = X~'^H H_rho1 X~' (Hermitian) and Dg = E - G ----------------------------------
   // (H X~')^H (H X~') = sum_i conj(x_i - x_{i+1}) (x_i - x_{i+1}) row by row.
   // tp adjacent threads share one (s, u) pair and split the rows; their partial
@@ -1659,16 +1715,34 @@ __global__ void __launch_bounds__(xstep_threads(RP), 1) k_xstep(Dev<T> d, const 
 // Grid (S, ceil(n2/TW)); warp w accumulates rows i = w, w + 8, ...; a lane
 // holds CPL columns (two for r <= 16, so each X~' value read from shared
 // memory feeds two columns).
+//
+// CW < 32 (FP64): tiles of CW columns, the lanes of a warp as 32 / CW row
+// groups of CW columns, their partial sums halved across the groups.  The FP64
+// pipe takes one warp instruction in 15 clocks per SM, so the work has to
+// reach every SM: 121 x 144 x 7, r = 4 is 12 CTAs of 64 columns (78 us) or 144
+// of 4.
 // ---------------------------------------------------------------------------
 constexpr int kYThreads = 256;
 
 __host__ __device__ constexpr int ystep_cpl(int rp) { return rp <= 16 ? 2 : 1; }
+// Columns per CTA of k_ystep with row groups of cw lanes.
+__host__ __device__ constexpr int ystep_tw(int rp, int cw) { return cw < 32 ? cw : 32 * ystep_cpl(rp); }
+// Lanes per row group: 32, in FP64 the most of 32, 8 and 4 that give every SM a CTA.
+template <typename T>
+inline int ystep_cw(int S, int n2, int rp) {
+  if (sizeof(T) == 4) return 32;
+  for (int cw : {32, 8}) {
+    const int tw = ystep_tw(rp, cw);
+    if (S * ((n2 + tw - 1) / tw) >= 152) return cw;
+  }
+  return 4;
+}
 
 // Shared memory of k_ystep: partial sums, D, old and new Y~ of the tile, Dg,
 // G^+, X~' of the slice (XSH), then r^2 doubles for the FP64 G^+ of a real slice.
 template <typename T>
-__host__ __device__ inline size_t ystep_gh64_offset(int n1, int r, int rp, bool x_in_smem, bool tcy) {
-  const size_t tw = 32 * (size_t)ystep_cpl(rp);
+__host__ __device__ inline size_t ystep_gh64_offset(int n1, int r, int rp, bool x_in_smem, bool tcy, int cw) {
+  const size_t tw = ystep_tw(rp, cw);
   return align_up(((size_t)((tcy ? 0 : kYThreads / 32) + 3) * rp * tw + 2 * (size_t)r * r +
                    (x_in_smem && !tcy ? (size_t)r * n1 : 0)) *
                       sizeof(cx<T>),
@@ -1678,13 +1752,14 @@ __host__ __device__ inline size_t ystep_gh64_offset(int n1, int r, int rp, bool 
 // n1 from k_dcon_tc (d.Dpart) and Z~ is formed by k_zsyn_tc afterwards.
 // XSH: X~' of the slice staged in shared memory (the compiler then sees
 // shared-memory loads in the contraction loops), else read through L1.
-template <typename T, int RP, bool TCY, bool XSH>
+template <typename T, int RP, bool TCY, bool XSH, int CW>
 __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem) {
-  constexpr int CPL = ystep_cpl(RP), TW = 32 * CPL;
+  constexpr int CPL = CW < 32 ? 1 : ystep_cpl(RP), TW = CW * CPL, NG = 32 / CW;  // NG row groups per warp
   const int k = blockIdx.x;
   const int j0 = blockIdx.y * TW;
   const int n1 = d.n1, n2 = d.n2, r = d.r, S = d.S, rr = r * r;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+  const int lc = lane & (CW - 1), row0 = wid * NG + lane / CW, nr = nw * NG;  // column, first row, row step
   cx<T>* red = reinterpret_cast<cx<T>*>(smem);  // [nw][RP][TW]
   cx<T>* Ds = red + (TCY ? 0 : nw * RP * TW);   // [RP][TW]
   cx<T>* Yo = Ds + RP * TW;                     // [RP][TW]
@@ -1701,7 +1776,7 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
   // real slices of an FP32 engine: t G^+ in FP64 (k_xstep / k_xc), applied in FP64
   const bool realslice = (k == 0) || (2 * k == d.n3);
   const bool g64 = sizeof(T) == 4 && realslice && d.Gp64 != nullptr;
-  double* gh64 = reinterpret_cast<double*>(smem + ystep_gh64_offset<T>(n1, r, RP, XSH, TCY));
+  double* gh64 = reinterpret_cast<double*>(smem + ystep_gh64_offset<T>(n1, r, RP, XSH, TCY, CW));
   for (int e = tid; e < rr; e += blockDim.x) {
     Dgs[e] = d.Dg[(size_t)k * rr + e];
     Gh[e] = d.Gp[(size_t)k * rr + e];
@@ -1719,29 +1794,29 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
     for (int s = 0; s < RP; ++s) acc[h][s] = cx<T>{T(0), T(0)};
   bool live[CPL];
 #pragma unroll
-  for (int h = 0; h < CPL; ++h) live[h] = j0 + 32 * h + lane < n2;
-  const cx<T>* rbase = d.Rt + (size_t)k * n2 + j0 + lane;  // + i * S * n2 + 32 h
+  for (int h = 0; h < CPL; ++h) live[h] = j0 + 32 * h + lc < n2;
+  const cx<T>* rbase = d.Rt + (size_t)k * n2 + j0 + lc;  // + i * S * n2 + 32 h
   const size_t rstride = (size_t)S * n2;
   if constexpr (!TCY) {
-    int i = wid;
-    for (; i + nw < n1; i += 2 * nw) {
+    int i = row0;
+    for (; i + nr < n1; i += 2 * nr) {
       cx<T> v[2][CPL];
 #pragma unroll
       for (int q = 0; q < 2; ++q)
 #pragma unroll
         for (int h = 0; h < CPL; ++h)
-          v[q][h] = live[h] ? ldg_cx(rbase + (size_t)(i + q * nw) * rstride + 32 * h) : cx<T>{T(0), T(0)};
+          v[q][h] = live[h] ? ldg_cx(rbase + (size_t)(i + q * nr) * rstride + 32 * h) : cx<T>{T(0), T(0)};
 #pragma unroll
       for (int q = 0; q < 2; ++q)
 #pragma unroll
         for (int s = 0; s < RP; ++s)
           if (s < r) {
-            const cx<T> x = Xs[(size_t)s * n1 + i + q * nw];
+            const cx<T> x = Xs[(size_t)s * n1 + i + q * nr];
 #pragma unroll
             for (int h = 0; h < CPL; ++h) cfmaconj(acc[h][s], x, v[q][h]);
           }
     }
-    for (; i < n1; i += nw) {
+    for (; i < n1; i += nr) {
       cx<T> v[CPL];
 #pragma unroll
       for (int h = 0; h < CPL; ++h)
@@ -1755,7 +1830,37 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
         }
     }
   }
-  if constexpr (!TCY) {
+  if constexpr (!TCY && NG > 1) {
+    // sums over the row groups: each step exchanges half of the values that are left
+    constexpr int F = 2 * RP;
+    T v[F];
+#pragma unroll
+    for (int s = 0; s < RP; ++s) {
+      v[2 * s] = acc[0][s].re;
+      v[2 * s + 1] = acc[0][s].im;
+    }
+    int base = 0;  // first value of this lane
+#pragma unroll
+    for (int o = 16, n = F; o >= CW; o >>= 1, n = n > 1 ? n / 2 : 1) {
+      if (n > 1) {
+        const bool up = (lane & o) != 0;
+        base += up ? n / 2 : 0;
+#pragma unroll
+        for (int q = 0; q < F / 2; ++q)
+          if (q < n / 2) {
+            const T send = up ? v[q] : v[q + n / 2], keep = up ? v[q + n / 2] : v[q];
+            v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+      } else {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < (F > NG ? F / NG : 1); ++q) {
+      const int e = base + q;
+      reinterpret_cast<T*>(red + (wid * RP + e / 2) * TW + lc)[e & 1] = v[q];  // (equal values where F < NG)
+    }
+  } else if constexpr (!TCY) {
 #pragma unroll
     for (int s = 0; s < RP; ++s)
 #pragma unroll
@@ -1820,12 +1925,12 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
     if (tile >= d.ytiles) continue;
     int s, u;
     tri_index(task, r, s, u);
-    const cx<T>* ys = Yn + s * TW + 32 * h;
-    const cx<T>* yu = Yn + u * TW + 32 * h;
+    const cx<T>* ys = Yn + s * TW + CW * h;
+    const cx<T>* yu = Yn + u * TW + CW * h;
     cx<T> g = {T(0), T(0)};
 #pragma unroll 8
-    for (int c = 0; c < 32; ++c) {
-      const int cc = (c + u) & 31;
+    for (int c = 0; c < CW; ++c) {
+      const int cc = (c + u) & (CW - 1);
       cfmac(g, ys[cc], yu[cc]);
     }
     d.Ag[((size_t)k * d.ytiles + tile) * ntask + task] = cx<double>{(double)g.re, (double)g.im};
@@ -1837,9 +1942,9 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
 #pragma unroll
   for (int h = 0; h < CPL; ++h)
 #pragma unroll
-    for (int s = 0; s < RP; ++s) yv[h][s] = Yn[s * TW + 32 * h + lane];
-  cx<T>* zc = d.Zt + (size_t)k * n2 + j0 + lane;
-  for (int i = wid; i < n1; i += nw) {
+    for (int s = 0; s < RP; ++s) yv[h][s] = Yn[s * TW + 32 * h + lc];
+  cx<T>* zc = d.Zt + (size_t)k * n2 + j0 + lc;
+  for (int i = row0; i < n1; i += nr) {
     cx<T> z[CPL];
 #pragma unroll
     for (int h = 0; h < CPL; ++h) z[h] = cx<T>{T(0), T(0)};
@@ -1861,16 +1966,27 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
 }
 
 // XSH is chosen at launch (d.yx_global == 0 for XSH, TCY never stages).
-template <typename T, int RP, bool TCY = false, bool XSH = !TCY>
+template <typename T, int RP, bool TCY = false, bool XSH = !TCY, int CW = 32>
 __global__ void __launch_bounds__(kYThreads) k_ystep(Dev<T> d) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (converged(d)) return;
-  ystep_impl<T, RP, TCY, XSH && !TCY>(d, smem);
+  ystep_impl<T, RP, TCY, XSH && !TCY, CW>(d, smem);
 }
 
 template <typename T>
-__host__ inline size_t ystep_smem_bytes(int n1, int r, int rp, bool x_in_smem = true, bool tcy = false) {
-  return ystep_gh64_offset<T>(n1, r, rp, x_in_smem, tcy) + (size_t)r * r * sizeof(double);
+__host__ inline size_t ystep_smem_bytes(int n1, int r, int rp, int cw, bool x_in_smem = true, bool tcy = false) {
+  return ystep_gh64_offset<T>(n1, r, rp, x_in_smem, tcy, cw) + (size_t)r * r * sizeof(double);
+}
+
+// Rows per CTA of k_qcon and its threads (a warp per pass of kQRR rows, 8 at
+// most): 32 rows, halved while the grid gives the SMs fewer than two CTAs each
+// and every warp keeps a pass.
+template <typename T>
+inline void qcon_shape(int S, int n1, int rp, int& rows, int& threads) {
+  const int rr = (rp <= 8 && sizeof(T) == 4) ? 2 : 1;
+  rows = 32;
+  while (rows > 4 * rr && S * ((n1 + rows - 1) / rows) < 2 * 152) rows /= 2;
+  threads = 32 * (rows / rr < 8 ? rows / rr : 8);
 }
 
 template <typename T>

@@ -119,6 +119,19 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+// 1/a.  FP64: a correctly rounded FP32 seed and two Newton steps
+// y <- y (2 - a y) (the error squares at each step); FP64 division is slow on
+// this part.  FP32: the IEEE quotient.
+__device__ __forceinline__ double rcp_refined(double a) {
+  const float af = (float)a;
+  if (!(fabsf(af) > 1e-30f && fabsf(af) < 1e30f)) return 1.0 / a;
+  double y = (double)__frcp_rn(af);
+  y = y * fma(-a, y, 2.0);
+  y = y * fma(-a, y, 2.0);
+  return y;
+}
+__device__ __forceinline__ float rcp_refined(float a) { return 1.0f / a; }
+
 // s + c += a b with the rounding errors of the product (FMA) and of the sum
 // (Knuth's two-sum) collected in c: about twice the working precision.
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }

@@ -30,11 +30,11 @@ namespace tc {
 template <typename T>
 using SlabFn = void (*)(Dev<T>, T*, int, int);
 
-template <typename T, int L>
+template <typename T>
 inline void slab_table(SlabFn<T> f[3]) {
-  f[MODE_ITER] = k_slab<T, L, MODE_ITER>;
-  f[MODE_W] = k_slab<T, L, MODE_W>;
-  f[MODE_R] = k_slab<T, L, MODE_R>;
+  f[MODE_ITER] = k_slab<T, MODE_ITER>;
+  f[MODE_W] = k_slab<T, MODE_W>;
+  f[MODE_R] = k_slab<T, MODE_R>;
 }
 
 // Folded-transform slab kernels with TL rows / slices per item (the read-back
@@ -55,40 +55,12 @@ inline SlabFn<T> pick_slab_g(int mode, int tl, bool staged) {
 template <typename T>
 inline SlabFn<T> pick_slab_tile(bool folded, bool staged, int tl) {
   if (folded) return pick_slab_g<T>(MODE_ITER, tl, staged);
-  return tl == 2 ? k_slab<T, 0, MODE_ITER, 2> : tl == 4 ? k_slab<T, 0, MODE_ITER, 4> : k_slab<T, 0, MODE_ITER, 8>;
-}
-
-// Launch shape of the folded-transform slab kernels: two CTAs of 256 threads on
-// an SM where the slab, the coefficients and a stage of one group fit half of
-// its shared memory, else one with twice the threads; as many groups per stage
-// as fit; unstaged where even one does not.  False where the slab itself does
-// not fit (k_slab keeps it in global memory).
-struct SlabGPlan {
-  int threads, sg;
-  size_t smem;
-};
-template <typename T>
-inline bool slab_g_plan(int n2, int n3, int optin, SlabGPlan& pl) {
-  if (n3 > kSlabGMaxN3) return false;
-  const int ngr = (n2 + kGTubes - 1) / kGTubes;
-  const size_t half = (size_t)(optin + kStaticSmemReserve + 1024) / 2 - 1024;  // 1 KB per CTA is the system's
-  for (int pass = 0; pass < 2; ++pass) {
-    const size_t room = pass == 0 ? half : (size_t)optin;
-    for (int sg = ngr; sg >= 1; --sg) {
-      const size_t b = slab_g_layout<T>(n2, n3, sg).total;
-      if (b <= room) {
-        pl = SlabGPlan{pass == 0 ? 256 : kSlabGThreads<T>, sg, b};
-        return true;
-      }
-    }
-  }
-  pl = SlabGPlan{kSlabGThreads<T>, 0, slab_g_layout<T>(n2, n3, 0).total};
-  return pl.smem <= (size_t)optin;
+  return tl == 2 ? k_slab<T, MODE_ITER, 2> : tl == 4 ? k_slab<T, MODE_ITER, 4> : k_slab<T, MODE_ITER, 8>;
 }
 
 template <typename T, int L, int N1, int N2>
-inline void slab_f_table(SlabFn<T> f[3]) {
-  f[MODE_ITER] = k_slab_f<T, L, N1, N2, MODE_ITER>;
+inline void slab_f_table(SlabFn<T> f[3], bool bf16) {
+  f[MODE_ITER] = bf16 ? k_slab_f<T, L, N1, N2, MODE_ITER, true> : k_slab_f<T, L, N1, N2, MODE_ITER>;
   f[MODE_W] = k_slab_f<T, L, N1, N2, MODE_W>;
   f[MODE_R] = k_slab_f<T, L, N1, N2, MODE_R>;
 }
@@ -105,7 +77,7 @@ struct SlabCfg {
 // (defined per translation unit); false when none applies to (n2, n3) within
 // the shared-memory limit optin.
 template <typename T>
-bool pick_slab(int n2, int n3, int optin, SlabCfg<T>& cfg);
+bool pick_slab(int n2, int n3, int optin, bool bf16, SlabCfg<T>& cfg);
 
 template <typename T>
 using YFn = void (*)(Dev<T>);
@@ -117,9 +89,24 @@ inline int pad_rank(int r) {
   return r <= 2 ? 2 : r <= 4 ? 4 : r <= 8 ? 8 : r <= 16 ? 16 : 32;
 }
 
+template <typename T, int CW>
+inline YFn<T> pick_ystep_narrow(int rp, bool xsh) {
+  switch (rp) {
+    case 2: return xsh ? k_ystep<T, 2, false, true, CW> : k_ystep<T, 2, false, false, CW>;
+    case 4: return xsh ? k_ystep<T, 4, false, true, CW> : k_ystep<T, 4, false, false, CW>;
+    case 8: return xsh ? k_ystep<T, 8, false, true, CW> : k_ystep<T, 8, false, false, CW>;
+    case 16: return xsh ? k_ystep<T, 16, false, true, CW> : k_ystep<T, 16, false, false, CW>;
+    default: return xsh ? k_ystep<T, 32, false, true, CW> : k_ystep<T, 32, false, false, CW>;
+  }
+}
+
 // xsh: X~' of the slice staged in shared memory (r n1 fits), else read through L1
 template <typename T>
-inline YFn<T> pick_ystep(int rp, bool xsh = true) {
+inline YFn<T> pick_ystep(int rp, int cw, bool xsh = true) {
+  if constexpr (sizeof(T) == 8) {
+    if (cw == 8) return pick_ystep_narrow<T, 8>(rp, xsh);
+    if (cw == 4) return pick_ystep_narrow<T, 4>(rp, xsh);
+  }
   switch (rp) {
     case 2: return xsh ? k_ystep<T, 2, false, true> : k_ystep<T, 2, false, false>;
     case 4: return xsh ? k_ystep<T, 4, false, true> : k_ystep<T, 4, false, false>;
@@ -200,9 +187,6 @@ inline QFn<T> pick_qcon(int rp) {
 }
 
 template <typename T>
-void upload_twiddles();
-
-template <typename T>
 class Engine final : public EngineBase {
  public:
   ~Engine() override { release(); }
@@ -238,8 +222,6 @@ class Engine final : public EngineBase {
     int optin = 0;
     TC_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device_));
     optin -= kStaticSmemReserve;  // room for the kernels' static shared memory
-    upload_twiddles<T>();
-    TC_CUDA_TRY(cudaGetLastError());
 
     // ---- state buffers -----------------------------------------------------------
     const size_t nx = (size_t)S_ * r_ * n1_, ny = (size_t)S_ * r_ * n2_, nrr = (size_t)S_ * r_ * r_;
@@ -247,7 +229,8 @@ class Engine final : public EngineBase {
     uint32_t* maskbits = alloc<uint32_t>((size_t)n1_ * n3_ * mw_, err);
     cx<T>* Rt = alloc<cx<T>>((size_t)n1_ * S_ * n2_, err);
     cx<T>* Zt = alloc<cx<T>>((size_t)n1_ * S_ * n2_, err);
-    const int ytiles = (n2_ + 31) / 32;
+    ycw_ = ystep_cw<T>(S_, n2_, rp_);
+    const int ytw = ycw_ < 32 ? ycw_ : 32, ytiles = (n2_ + ytw - 1) / ytw;
     cx<double>* Ag = alloc<cx<double>>((size_t)S_ * ytiles * (r_ * (r_ + 1) / 2), err);
     cx<T>* Xt = alloc<cx<T>>(nx, err);
     Q_ = alloc<cx<T>>(nx, err);
@@ -277,7 +260,7 @@ class Engine final : public EngineBase {
 
     // ---- kernel variants and shared memory -------------------------------------------
     SlabCfg<T> cfg{};
-    specialised_ = pick_slab<T>(n2_, n3_, optin, cfg);
+    specialised_ = pick_slab<T>(n2_, n3_, optin, p.precision == TC_BF16, cfg);
     d_.scratch = nullptr;
     if (specialised_) {
       for (int m = 0; m < 3; ++m) slab_[m] = cfg.f[m];
@@ -287,7 +270,7 @@ class Engine final : public EngineBase {
     } else if (SlabGPlan gp; p.precision != TC_BF16 && slab_g_plan<T>(n2_, n3_, optin, gp)) {
       folded_ = true;
       d_.fold_sg = gp.sg;
-      for (int m = 0; m < 3; ++m) slab_[m] = pick_slab_g<T>(m, 4, gp.sg > 0);
+      for (int m = 0; m < 3; ++m) slab_[m] = pick_slab_g<T>(m, n3_ == 7 ? 2 : 4, gp.sg > 0);
       slab_smem_ = gp.smem;
       slab_threads_ = gp.threads;
       slabs_in_smem_ = true;
@@ -295,12 +278,12 @@ class Engine final : public EngineBase {
       if (!err.empty()) return TC_ERR_NOMEM;
       d_.fold = fold_;
     } else {
-      slab_table<T, 0>(slab_);
-      slab_threads_ = 256;
-      SlabLayout lay = slab_layout<T>(n2_, n3_, false, true);
+      slab_table<T>(slab_);
+      slab_threads_ = kSlabThreads;
+      SlabLayout lay = slab_layout<T>(n2_, n3_, true);
       slabs_in_smem_ = lay.total <= (size_t)optin;
       if (!slabs_in_smem_) {
-        lay = slab_layout<T>(n2_, n3_, false, false);
+        lay = slab_layout<T>(n2_, n3_, false);
         T* scratch = alloc<T>(lay.slab_bytes / sizeof(T) * (size_t)n1_ + 16, err);
         if (!err.empty()) return TC_ERR_NOMEM;
         d_.scratch = scratch;
@@ -372,14 +355,14 @@ class Engine final : public EngineBase {
       TC_CUDA_TRY(allow_dynamic_smem((const void*)k_xbc<T>, xbc_smem_));
       TC_CUDA_TRY(allow_dynamic_smem((const void*)k_xg<T>, xg_smem_));
     }
-    ystep_smem_ = ystep_smem_bytes<T>(n1_, r_, rp_);
+    ystep_smem_ = ystep_smem_bytes<T>(n1_, r_, rp_, ycw_);
     d_.yx_global = ystep_smem_ > (size_t)optin ? 1 : 0;
-    if (d_.yx_global) ystep_smem_ = ystep_smem_bytes<T>(n1_, r_, rp_, false);
-    ystep_ = pick_ystep<T>(rp_, !d_.yx_global);
+    if (d_.yx_global) ystep_smem_ = ystep_smem_bytes<T>(n1_, r_, rp_, ycw_, false);
+    ystep_ = pick_ystep<T>(rp_, ycw_, !d_.yx_global);
     qcon_ = pick_qcon<T>(rp_);
     qcon_smem_ = qcon_smem_bytes<T>(n2_, r_, rp_);
-    qgrid_ = dim3(S_, (n1_ + 31) / 32);
-    qthreads_ = kSliceThreads;
+    qcon_shape<T>(S_, n1_, rp_, d_.qrows, qthreads_);
+    qgrid_ = dim3(S_, (n1_ + d_.qrows - 1) / d_.qrows);
     if (mixed_ && rp_ == 32 && pick_tc<T>(p.precision, (p.flags & TC_FLAG_SINGLE_PASS) == 0, tck_)) {
       tcy_ = true;
       qcon_ = tck_.qcon;
@@ -387,7 +370,7 @@ class Engine final : public EngineBase {
       qgrid_ = dim3(S_, (n1_ + 127) / 128);
       qthreads_ = 256;
       ystep_ = k_ystep<T, 32, true>;
-      ystep_smem_ = ystep_smem_bytes<T>(n1_, r_, rp_, false, true);
+      ystep_smem_ = ystep_smem_bytes<T>(n1_, r_, rp_, 32, false, true);
       // split the n1 reduction of D so that the grid covers the SMs about twice
       int nsm = 0;
       TC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device_));
@@ -453,6 +436,7 @@ class Engine final : public EngineBase {
     d_.Zt = Zt;
     d_.Ag = Ag;
     d_.ytiles = ytiles;
+    d_.ytw = ytw;
     d_.Xt = Xt;
     d_.Yt = Yt;
     d_.Dg = Dg;
@@ -516,7 +500,7 @@ class Engine final : public EngineBase {
     k_gram_tiles<T><<<dim3(S_, ytiles), 256, 0, stream_>>>(d_);         // A of the first X-step
     if (xsplit_ || apre_) xa_fn_<<<S_, xa_threads_, xa_smem_, stream_>>>(d_);  // its A^+
     if (folded_) k_fold_tables<T><<<2 * 152, 256, 0, stream_>>>(fold_, twg, n3_);
-    if (!specialised_) {
+    if (!specialised_ && !(folded_ && n3_ == 7)) {  // (four rows and slices: nothing to choose)
       // tile of the generic transform for this shape: each candidate runs the
       // initial slab pass (it only depends on G and Z~0, so every run writes the
       // same R~0), timed twice; the fastest is kept
@@ -918,7 +902,7 @@ class Engine final : public EngineBase {
   // the rest of the iteration; the return value says whether it was, and the
   // caller then joins on ev_join_.  Without one it follows on s.
   bool launch_ystep(cudaStream_t s, cudaStream_t branch = nullptr, bool with_xa = true) {
-    const int tw = 32 * ystep_cpl(rp_);
+    const int tw = ystep_tw(rp_, ycw_);
     dim3 g(S_, (n2_ + tw - 1) / tw);
     if (tcy_) tck_.dcon<<<dim3(S_, (n2_ + 127) / 128, ksplit_), 256, tck_.dsm, s>>>(d_);
     ystep_<<<g, kYThreads, ystep_smem_, s>>>(d_);
@@ -1017,6 +1001,7 @@ class Engine final : public EngineBase {
   bool tcy_ = false;  // tensor-core Y-step (D partials, update, Z~ synthesis)
   TcKernels<T> tck_;
   int ksplit_ = 1;
+  int ycw_ = 32;  // lanes per row group of k_ystep
   cx<T>* Dpart_ = nullptr;
   dim3 qgrid_;
   int qthreads_ = kSliceThreads;

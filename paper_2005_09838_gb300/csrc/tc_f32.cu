@@ -5,20 +5,17 @@
 
 namespace tc {
 
-bool slab_setup_f32_112(int n2, int optin, SlabCfg<float>& cfg);
-bool slab_setup_f32_168(int n2, int optin, SlabCfg<float>& cfg);
+bool slab_setup_f32_112(int n2, int optin, bool bf16, SlabCfg<float>& cfg);
+bool slab_setup_f32_168(int n2, int optin, bool bf16, SlabCfg<float>& cfg);
 
 template <>
-bool pick_slab<float>(int n2, int n3, int optin, SlabCfg<float>& cfg) {
+bool pick_slab<float>(int n2, int n3, int optin, bool bf16, SlabCfg<float>& cfg) {
   switch (n3) {
-    case 112: return slab_setup_f32_112(n2, optin, cfg);
-    case 168: return slab_setup_f32_168(n2, optin, cfg);
+    case 112: return slab_setup_f32_112(n2, optin, bf16, cfg);
+    case 168: return slab_setup_f32_168(n2, optin, bf16, cfg);
     default: return false;
   }
 }
-
-template <>
-void upload_twiddles<float>() {}
 
 template <>
 bool pick_tc<float>(int precision, bool split, TcKernels<float>& k) {

@@ -3,11 +3,11 @@
 
 namespace tc {
 
-bool slab_setup_f32_168(int n2, int optin, SlabCfg<float>& cfg) {
+bool slab_setup_f32_168(int n2, int optin, bool bf16, SlabCfg<float>& cfg) {
   const SlabFLayout lay = slab_f_layout<float>(n2, 168);
   if (lay.total > (size_t)optin) return false;
-  fft::upload_tables<float>();
-  slab_f_table<float, 168, 12, 7>(cfg.f);
+  fft::upload_tables();
+  slab_f_table<float, 168, 12, 7>(cfg.f, bf16);
   cfg.threads = kSlabFThreads;
   cfg.smem = lay.total;
   return true;

@@ -49,8 +49,8 @@ GFn<T> pick_qcon_g(int rp) {
   }
 }
 
-// Slab kernel for MODE_GRAD: the shared-memory transform for n3 in {112, 168}
-// (FP32), the register transform for n3 = 7 (FP64), else the direct DFT.
+// Slab kernel for MODE_GRAD: the shared-memory FFT for n3 in {112, 168} (FP32),
+// else the folded transform, or the generic one past shared memory.
 template <typename T>
 struct GradSlab {
   GSlabFn<T> f = nullptr;
@@ -58,6 +58,8 @@ struct GradSlab {
   size_t smem = 0;
   bool in_smem = true;
   size_t scratch_bytes = 0;
+  bool folded = false;
+  int sg = 0;
 };
 
 template <typename T>
@@ -67,31 +69,29 @@ GradSlab<T> pick_grad_slab(int n2, int n3, int optin) {
     if (n3 == 168 || n3 == 112) {
       const SlabFLayout lay = slab_f_layout<T>(n2, n3);
       if (lay.total <= (size_t)optin) {
-        fft::upload_tables<T>();
+        fft::upload_tables();
         g.f = (n3 == 168) ? k_slab_f<T, 168, 12, 7, MODE_GRAD> : k_slab_f<T, 112, 8, 7, MODE_GRAD>;
         g.threads = kSlabFThreads;
         g.smem = lay.total;
         return g;
       }
     }
-  } else {
-    if (n3 == 7) {
-      const SlabLayout lay = slab_layout<T>(n2, 7, true, true);
-      if (lay.total <= (size_t)optin) {
-        fft::upload_tables<T>();
-        g.f = k_slab<T, 7, MODE_GRAD>;
-        g.threads = std::max(std::min((n2 + 31) / 32 * 32, slab_max_threads(7)), 32);
-        g.smem = lay.total;
-        return g;
-      }
-    }
   }
-  SlabLayout lay = slab_layout<T>(n2, n3, false, true);
-  g.f = k_slab<T, 0, MODE_GRAD>;
-  g.threads = 256;
+  SlabGPlan gp;
+  if (slab_g_plan<T>(n2, n3, optin, gp)) {
+    g.f = gp.sg > 0 ? k_slab_g<T, MODE_GRAD, 4, true> : k_slab_g<T, MODE_GRAD, 4, false>;
+    g.threads = gp.threads;
+    g.smem = gp.smem;
+    g.folded = true;
+    g.sg = gp.sg;
+    return g;
+  }
+  SlabLayout lay = slab_layout<T>(n2, n3, true);
+  g.f = k_slab<T, MODE_GRAD>;
+  g.threads = kSlabThreads;
   if (lay.total > (size_t)optin) {
     g.in_smem = false;
-    lay = slab_layout<T>(n2, n3, false, false);
+    lay = slab_layout<T>(n2, n3, false);
     g.scratch_bytes = lay.slab_bytes;
   }
   g.smem = lay.total;
@@ -153,7 +153,6 @@ struct GradEngine final : tc_grad {
     int optin = 0;
     TCG_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
     optin -= kStaticSmemReserve;  // room for the kernels' static shared memory
-    if constexpr (sizeof(T) == 8) fft::upload_tables<T>();
 
     T* Gint = alloc<T>(N, err);
     uint32_t* maskbits = alloc<uint32_t>((size_t)n1_ * n3_ * mw, err);
@@ -177,9 +176,17 @@ struct GradEngine final : tc_grad {
       if (!err.empty()) return TC_ERR_NOMEM;
       d_.scratch = scratch;
     }
+    cx<T>* fold = nullptr;
+    if (slab_.folded) {
+      fold = alloc<cx<T>>(fold_table_entries(n3_), err);
+      if (!err.empty()) return TC_ERR_NOMEM;
+      d_.fold = fold;
+      d_.fold_sg = slab_.sg;
+    }
     TCG_TRY(allow_dynamic_smem((const void*)slab_.f, slab_.smem));
     qcon_ = pick_qcon_g<T>(rp_);
     dcon_ = pick_dcon<T>(rp_);
+    qcon_shape<T>(S_, n1_, rp_, d_.qrows, qthreads_);
     qsmem_ = qcon_smem_bytes<T>(n2_, r_, rp_);
     dsmem_ = dcon_smem_bytes<T>(n1_, r_, rp_);
     d_.yx_global = dsmem_ > (size_t)optin ? 1 : 0;
@@ -231,6 +238,7 @@ struct GradEngine final : tc_grad {
       dM = static_cast<const uint8_t*>(tM);
     }
     k_pack<T><<<pack_grid(n1_, n2_, n3_), kTileThreads, 0, stream_>>>(dG, dM, Gint, maskbits, n1_, n2_, n3_, mw);
+    if (fold) k_fold_tables<T><<<2 * 152, 256, 0, stream_>>>(fold, twg, n3_);
     const cudaError_t le = cudaGetLastError();
     const cudaError_t se = cudaStreamSynchronize(stream_);
     if (tG) cudaFree(tG);
@@ -269,7 +277,7 @@ struct GradEngine final : tc_grad {
         const size_t tot = (size_t)n1_ * S_ * n2_;
         k_grad_hth<T><<<(unsigned)std::min<size_t>((tot + 255) / 256, 16 * 152), 256, 0, stream_>>>(d_);
       }
-      qcon_<<<dim3(S_, (n1_ + 31) / 32), kSliceThreads, qsmem_, stream_>>>(d_, GX_);  // R~ Y~^H
+      qcon_<<<dim3(S_, (n1_ + d_.qrows - 1) / d_.qrows), qthreads_, qsmem_, stream_>>>(d_, GX_);  // R~ Y~^H
       dcon_<<<dim3(S_, (n2_ + 31) / 32), kYThreads, dsmem_, stream_>>>(d_, GY_);     // X~^H R~
       T* ox = static_cast<T*>(dX);
       T* oy = static_cast<T*>(dY);
@@ -321,6 +329,7 @@ struct GradEngine final : tc_grad {
   GFn<T> qcon_ = nullptr;
   GFn<T> dcon_ = nullptr;
   size_t qsmem_ = 0, dsmem_ = 0;
+  int qthreads_ = kSliceThreads;
   cx<T>* GX_ = nullptr;
   cx<T>* GY_ = nullptr;
   T* xin_ = nullptr;

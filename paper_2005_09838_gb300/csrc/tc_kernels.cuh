@@ -34,8 +34,10 @@ struct Dev {
   cx<T>* Zt;        // [n1][S][n2] Z~ = X~Y~ of the current factors (written by k_ystep)
   cx<T>* Xt;
   cx<T>* Yt;
-  cx<double>* Ag;   // [S][ytiles][r(r+1)/2] partial Grams Y~Y~^H over 32-column tiles
-  int ytiles;       // ceil(n2 / 32)
+  cx<double>* Ag;   // [S][ytiles][r(r+1)/2] partial Grams Y~Y~^H over tiles of ytw columns
+  int ytiles;       // ceil(n2 / ytw)
+  int ytw;          // columns of a tile Gram (32; fewer where k_ystep takes narrow tiles)
+  int qrows;        // rows of R~ per CTA of k_qcon
   cx<T>* Dg;        // [S][r][r] E - G of the Y-step (k_xstep)
   cx<T>* Gp;        // [S][r][r] G^+
   cx<double>* Gp64; // [2][r][r] t G^+ of the real slices (DC, Nyquist) in FP64; FP32 engines only

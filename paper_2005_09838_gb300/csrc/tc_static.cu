@@ -115,9 +115,11 @@ __global__ void k_static_objective(const double* part, const double* part_k, int
   out[0] = 0.5 * sr + 0.5 * mu * sw + 0.5 * rho2 * sk + 0.5 * rho1 * sh / (double)n3;
 }
 
+// cw: lanes per row group of the Y-step (0: ystep_cw's choice; 32, whose tile
+// Grams are the smallest, where that does not fit the scratch).
 template <typename T>
 tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, const void* Y0, const void* X0,
-                     int n_iters, void* W, double* f0, cudaStream_t st) {
+                     int n_iters, void* W, double* f0, cudaStream_t st, int cw = 0) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return sfail(TC_ERR_CUDA, "cudaGetDevice failed");
   unsigned char* base = nullptr;
@@ -133,14 +135,18 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
   const size_t N = (size_t)n1 * n2 * n3;
   const size_t nx = (size_t)S * r * n1, ny = (size_t)S * r * n2, nrr = (size_t)S * r * r;
 
-  SlabLayout lay = slab_layout<T>(n2, n3, false, true);
+  SlabLayout lay = slab_layout<T>(n2, n3, true);
   const bool slabs_in_smem = lay.total <= (size_t)optin;
-  if (!slabs_in_smem) lay = slab_layout<T>(n2, n3, false, false);
+  if (!slabs_in_smem) lay = slab_layout<T>(n2, n3, false);
+  SlabGPlan gp;
+  bool folded = slab_g_plan<T>(n2, n3, optin, gp);
   XLayout xl = xstep_layout_for<T>(n1, n2, r, rp, false, true);
   const bool xsmem = xl.total <= (size_t)optin;
   if (!xsmem) xl = xstep_layout_for<T>(n1, n2, r, rp, false, false);
-  const bool yxg = ystep_smem_bytes<T>(n1, r, rp) > (size_t)optin;
-  const size_t ysm = ystep_smem_bytes<T>(n1, r, rp, !yxg), qsm = qcon_smem_bytes<T>(n2, r, rp);
+  if (cw == 0) cw = ystep_cw<T>(S, n2, rp);
+  const int tw = ystep_tw(rp, cw);
+  const bool yxg = ystep_smem_bytes<T>(n1, r, rp, cw) > (size_t)optin;
+  const size_t ysm = ystep_smem_bytes<T>(n1, r, rp, cw, !yxg), qsm = qcon_smem_bytes<T>(n2, r, rp);
   if (xl.total > (size_t)optin || ysm > (size_t)optin || qsm > (size_t)optin)
     return sfail(TC_ERR_UNSUPPORTED, "shared memory of the slice kernels exceeds the device limit for these sizes");
 
@@ -151,7 +157,8 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
   uint32_t* maskbits = cv.take<uint32_t>((size_t)n1 * n3 * mw);
   d.Rt = cv.take<cx<T>>((size_t)n1 * S * n2);
   d.Zt = cv.take<cx<T>>((size_t)n1 * S * n2);
-  d.ytiles = (n2 + 31) / 32;
+  d.ytw = cw < 32 ? cw : 32;
+  d.ytiles = (n2 + d.ytw - 1) / d.ytw;
   d.Ag = cv.take<cx<double>>((size_t)S * d.ytiles * (r * (r + 1) / 2));
   d.Xt = cv.take<cx<T>>(nx);
   cx<T>* Q = cv.take<cx<T>>(nx);
@@ -168,6 +175,18 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
   double* fout = cv.take<double>(1);
   d.err = cv.take<int>(1);
   d.scratch = slabs_in_smem ? nullptr : cv.take<T>(lay.slab_bytes / sizeof(T) * (size_t)n1 + 16);
+  if (cv.off > kStaticScratchBytes && cw < 32) return run_static<T>(p, G, mask, Y0, X0, n_iters, W, f0, st, 32);
+  // the folded transform's tables take the rest; where that is too small, the
+  // generic transform (which needs none) serves the problem as before
+  cx<T>* fold = nullptr;
+  if (folded && cv.off <= kStaticScratchBytes) {
+    const size_t before = cv.off;
+    fold = cv.take<cx<T>>(fold_table_entries(n3));
+    if (cv.off > kStaticScratchBytes) {
+      cv.off = before;
+      folded = false;
+    }
+  }
   if (cv.off > kStaticScratchBytes) {
     return sfail(TC_ERR_ARG, "problem needs " + std::to_string(cv.off) + " bytes of scratch; the static scratch of " +
                                  "tc_complete_static holds " + std::to_string(kStaticScratchBytes) + " bytes");
@@ -190,19 +209,30 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
   d.rtol = (p.pinv_rtol > 0) ? p.pinv_rtol : default_rtol<T>(r, rp, false);
   d.rtol64 = (p.pinv_rtol > 0) ? p.pinv_rtol : (double)r * std::numeric_limits<double>::epsilon();
 
-  // ---- kernels (generic mode-3 transform) ------------------------------------------------
+  // ---- kernels ---------------------------------------------------------------------------
   SlabFn<T> slab[3];
-  slab_table<T, 0>(slab);
-  YFn<T> ystep = pick_ystep<T>(rp, !yxg);
+  slab_table<T>(slab);
+  size_t slab_smem = lay.total;
+  int slab_threads = kSlabThreads;
+  if (folded) {
+    for (int m = 0; m < 3; ++m) slab[m] = pick_slab_g<T>(m, n3 == 7 ? 2 : 4, gp.sg > 0);
+    slab_smem = gp.smem;
+    slab_threads = gp.threads;
+    d.fold = fold;
+    d.fold_sg = gp.sg;
+  }
+  YFn<T> ystep = pick_ystep<T>(rp, cw, !yxg);
   QFn<T> qcon = pick_qcon<T>(rp);
+  int qthreads = kSliceThreads;
+  qcon_shape<T>(S, n1, rp, d.qrows, qthreads);
   XFn<T> xstep = pick_xstep_for<T>(rp, false);
   const struct {
     const void* fn;
     size_t bytes;
     const char* name;
-  } opt_in[] = {{(const void*)slab[MODE_ITER], lay.total, "slab (iteration)"},
-                {(const void*)slab[MODE_W], lay.total, "slab (W read-back)"},
-                {(const void*)slab[MODE_R], lay.total, "slab (objective)"},
+  } opt_in[] = {{(const void*)slab[MODE_ITER], slab_smem, "slab (iteration)"},
+                {(const void*)slab[MODE_W], slab_smem, "slab (W read-back)"},
+                {(const void*)slab[MODE_R], slab_smem, "slab (objective)"},
                 {(const void*)xstep, xl.total, "X-step"},
                 {(const void*)ystep, ysm, "Y-step"},
                 {(const void*)qcon, qsm, "Q contraction"}};
@@ -222,6 +252,7 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
       return sfail(TC_ERR_CUDA, std::string("clearing the device error flag failed: ") + cudaGetErrorString(e));
   }
   k_static_tables<T><<<3, 256, 0, st>>>(winv, hinv, twg, n1, n2, n3, p.mu, p.rho1, p.rho2);
+  if (folded) k_fold_tables<T><<<2 * 152, 256, 0, st>>>(fold, twg, n3);
   k_pack<T><<<pack_grid(n1, n2, n3), kTileThreads, 0, st>>>(static_cast<const T*>(G), mask, Gint, maskbits, n1, n2, n3, mw);
   k_factor_dft<T><<<fgrid, 256, 0, st>>>(static_cast<const T*>(Y0), d.Yt, n2, r, n3, 1, twg);
   if (X0) {
@@ -233,16 +264,16 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
   }
   k_synth_init<T><<<fgrid, 256, 0, st>>>(d);
   k_gram_tiles<T><<<dim3(S, d.ytiles), 256, 0, st>>>(d);
-  slab[MODE_ITER]<<<n1, 256, lay.total, st>>>(d, nullptr, sis, 1);
+  slab[MODE_ITER]<<<n1, slab_threads, slab_smem, st>>>(d, nullptr, sis, 1);
   for (int it = 0; it < n_iters; ++it) {
-    qcon<<<dim3(S, (n1 + 31) / 32), kSliceThreads, qsm, st>>>(d, Q);
+    qcon<<<dim3(S, (n1 + d.qrows - 1) / d.qrows), qthreads, qsm, st>>>(d, Q);
     xstep<<<S, xstep_threads(rp), xl.total, st>>>(d, Q, xsmem ? 1 : 0);
-    ystep<<<dim3(S, (n2 + 32 * ystep_cpl(rp) - 1) / (32 * ystep_cpl(rp))), kYThreads, ysm, st>>>(d);
-    slab[MODE_ITER]<<<n1, 256, lay.total, st>>>(d, nullptr, sis, 0);
+    ystep<<<dim3(S, (n2 + tw - 1) / tw), kYThreads, ysm, st>>>(d);
+    slab[MODE_ITER]<<<n1, slab_threads, slab_smem, st>>>(d, nullptr, sis, 0);
   }
-  slab[MODE_W]<<<n1, 256, lay.total, st>>>(d, static_cast<T*>(W), sis | (f0 ? 0 : SLAB_NOSUM), 0);
+  slab[MODE_W]<<<n1, slab_threads, slab_smem, st>>>(d, static_cast<T*>(W), sis | (f0 ? 0 : SLAB_NOSUM), 0);
   if (f0) {
-    slab[MODE_R]<<<n1, 256, lay.total, st>>>(d, nullptr, sis, 0);
+    slab[MODE_R]<<<n1, slab_threads, slab_smem, st>>>(d, nullptr, sis, 0);
     k_rho1_term<T><<<dim3(S, kRhoChunks), 256, 0, st>>>(d);
     k_static_objective<<<1, 32, 0, st>>>(d.part, d.part_k, n1, S, n3, p.mu, p.rho1, p.rho2, fout);
   }
