@@ -473,4 +473,27 @@ __global__ void k_gram_tiles(Dev<T> d) {
   }
 }
 
+// Transforms of a factor (n r tubes): the folded product where its tables exist
+// (fold) and fit, else one thread per tube.
+constexpr int kFactorGrid = 4 * 152;
+template <typename T>
+inline cudaError_t allow_fold_dft(int n3) {
+  const cudaError_t e = allow_dynamic_smem((const void*)k_fold_dft<T>, fold_dft_smem<T>(n3));
+  return e != cudaSuccess ? e : allow_dynamic_smem((const void*)k_fold_idft<T>, fold_dft_smem<T>(n3));
+}
+template <typename T>
+inline void launch_factor_dft(const T* in, cx<T>* out, const cx<T>* fold, const cx<T>* twg, int n, int r, int n3,
+                              int transposed, cudaStream_t s) {
+  const unsigned g = (unsigned)(((size_t)n * r + kGTubes<T> - 1) / kGTubes<T>);
+  if (fold) k_fold_dft<T><<<g, kFoldThreads, fold_dft_smem<T>(n3), s>>>(in, out, fold, n, r, n3, transposed);
+  else k_factor_dft<T><<<kFactorGrid, 256, 0, s>>>(in, out, n, r, n3, transposed, twg);
+}
+template <typename T>
+inline void launch_factor_idft(const cx<T>* in, T* out, const cx<T>* fold, const cx<T>* twg, int n, int r, int n3,
+                               int transposed, cudaStream_t s) {
+  const unsigned g = (unsigned)(((size_t)n * r + kGTubes<T> - 1) / kGTubes<T>);
+  if (fold) k_fold_idft<T><<<g, kFoldThreads, fold_dft_smem<T>(n3), s>>>(in, out, fold, n, r, n3, transposed);
+  else k_factor_idft<T><<<kFactorGrid, 256, 0, s>>>(in, out, n, r, n3, transposed, twg);
+}
+
 }  // namespace tc

@@ -7,9 +7,9 @@
 // Sec. 2), i.e. per slice of the half spectrum
 //   dL/dX~_k = E~_k Y~_k^H,  dL/dY~_k = X~_k^H E~_k,
 // E~_k = R~_k + rho1 H^T H Z~_k with R~ = DFT(P_Omega(Z - G)) from the slab
-// kernel (MODE_GRAD) and the stencil k_grad_hth adding the rho1 part in
-// place; the inverse mode-3 DFT brings the gradients back to the spatial
-// factors.
+// kernel (MODE_GRAD) and the rho1 part added in place by k_grad_rho1; the
+// inverse mode-3 DFT brings the gradients back to the spatial factors.  FP32 ranks above 4 take the tiled
+// contractions of k_gemm.cuh, the others those below.
 #pragma once
 
 namespace tc {
@@ -74,26 +74,63 @@ __host__ inline size_t dcon_smem_bytes(int n1, int r, int rp, bool x_in_smem = t
   return ((size_t)(kYThreads / 32) * rp * 32 + (x_in_smem ? (size_t)r * n1 : 0)) * sizeof(cx<T>);
 }
 
-// rho1 part of the gradient: with E = P_Omega(Z - G) + rho1 (H^T H) x_1 Z the
-// spectrum R~ holds DFT3(P_Omega(Z - G)) after the slab kernel; adding
-// rho1 (H^T H Z~)_k to every slice makes the contractions R~Y~^H and X~^H R~
-// that follow give the whole gradient.  (H^T H z)_i = deg_i z_i - z_{i-1} -
-// z_{i+1} along mode 1.  One thread per entry of R~ ([n1][S][n2]).
-template <typename T>
-__global__ void k_grad_hth(Dev<T> d) {
-  const int n1 = d.n1, n2 = d.n2, S = d.S;
-  const size_t rs = (size_t)S * n2, tot = (size_t)n1 * rs;
+// rho1 terms in one pass over Z~: R~ += rho1 H^T H Z~ (with WRITE), so that the
+// contractions R~Y~^H and X~^H R~ that follow give the whole gradient, and the
+// sum ||H Z~_k||^2 of the loss (part_k, as k_rho1_term).  (H^T H z)_i = deg_i z_i
+// - z_{i-1} - z_{i+1} along mode 1.  Grid (S, kRhoChunks): a thread walks down
+// one column of its chunk of rows with the row above and below in registers, so
+// Z~ is read once and R~ once and written once (312 MB at 529 x 288 x 168; as two
+// kernels, one of them a thread per entry reading three rows, 31 + 70 us).
+template <typename T, bool WRITE>
+__global__ void __launch_bounds__(256) k_grad_rho1(Dev<T> d) {
+  __shared__ double part[8];
+  const int k = blockIdx.x, ch = blockIdx.y;
+  const int n1 = d.n1, n2 = d.n2;
+  const size_t rs = (size_t)d.S * n2;
+  const cx<T>* Z = d.Zt + (size_t)k * n2;
+  cx<T>* R = d.Rt + (size_t)k * n2;
+  const bool real = k == 0 || 2 * k == d.n3;
   const T rho1 = d.rho1;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e / rs);
-    const cx<T> z = d.Zt[e];
-    cx<T> h = {T(0), T(0)};
-    if (i > 0) h = h + (z - d.Zt[e - rs]);
-    if (i + 1 < n1) h = h + (z - d.Zt[e + rs]);
-    const int k = (int)((e / n2) % S);
-    cx<T> v = d.Rt[e] + h * rho1;
-    if (k == 0 || 2 * k == d.n3) v.im = T(0);
-    d.Rt[e] = v;
+  const int per = (n1 + kRhoChunks - 1) / kRhoChunks, i0 = min(ch * per, n1), i1 = min(i0 + per, n1);
+  SqSum<T> sum;
+  constexpr int U = 4;  // rows in flight
+  for (int j = threadIdx.x; j < n2 && i0 < i1; j += blockDim.x) {
+    cx<T> cur = Z[(size_t)i0 * rs + j];
+    cx<T> up = {T(0), T(0)};  // z_i - z_{i-1}
+    if (i0 > 0) up = cur - Z[(size_t)(i0 - 1) * rs + j];
+    for (int i = i0; i < i1; i += U) {
+      cx<T> nx[U], rv[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        if (i + q < i1 && i + q + 1 < n1) nx[q] = Z[(size_t)(i + q + 1) * rs + j];
+        if (WRITE && i + q < i1) rv[q] = R[(size_t)(i + q) * rs + j];
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        if (i + q >= i1) break;
+        cx<T> dn = {T(0), T(0)};  // z_{i+1} - z_i
+        if (i + q + 1 < n1) {
+          dn = nx[q] - cur;
+          sum.add(dn.re);
+          sum.add(dn.im);
+        }
+        if (WRITE) {
+          const cx<T> h = up - dn;
+          R[(size_t)(i + q) * rs + j] = cx<T>{fma(h.re, rho1, rv[q].re), real ? T(0) : fma(h.im, rho1, rv[q].im)};
+        }
+        up = dn;
+        cur = nx[q];
+      }
+    }
+  }
+  const double tot = warp_sum(sum.total());
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (lane == 0) part[wid] = tot;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[w];
+    d.part_k[(size_t)k * kRhoChunks + ch] = s;
   }
 }
 

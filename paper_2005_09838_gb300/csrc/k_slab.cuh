@@ -314,19 +314,18 @@ __device__ void wstep_sweeps_seg(ColFn col_of, int LP, const uint32_t* __restric
 //          w_j = e w_{j-1} + f (pivots by the distance from that end: the same
 //          table), so the segment's last entry is (d + c f) / (1 - c e).
 // Fewer than half the instructions of the two sweeps over shared memory (no
-// second pass over the values, the table and the mask).  A segment is a mask
-// word in FP32; in FP64, where a warp instruction holds its scheduler's pipe for
+// second pass over the values, the table and the mask).  FP32 segments of 16 keep
+// the thread within 64 registers; in FP64, where a warp instruction holds its scheduler's pipe for
 // 60 clocks however few lanes take part, shorter ones fill the lanes (121 x 144 x 7:
 // 7 rows are 7 lanes as rows, 126 as segments of 8).
 // ---------------------------------------------------------------------------
 template <typename T>
-constexpr int kWSeg = sizeof(T) == 8 ? 8 : 32;
+constexpr int kWSeg = sizeof(T) == 8 ? 8 : 16;
 
-template <typename T, bool FULL, bool LAST>
+template <typename T, int SEG, bool FULL, bool LAST>
 __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP, const uint32_t* __restrict__ rowm,
                                               int words, int sgm, int qn, int n2, T rho2, const T* __restrict__ wtab,
-                                              T (&v)[kWSeg<T>]) {
-  constexpr int SEG = kWSeg<T>;
+                                              T (&v)[SEG]) {
   const int base = SEG * sgm, bw = base >> 5, bb = base & 31;
   const uint32_t word = rowm[bw], mw = word >> bb;
 #pragma unroll
@@ -348,22 +347,23 @@ __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP,
       }
     }
   }
-  const int cw = ((st == 0) ? 0 : n2) + base - st;  // index base of entries without bits below
+  // table position of the entry: one further per missing entry, the start of the
+  // second table after an observed one
+  const T* tp = wtab + ((st == 0) ? 0 : n2) + base - st;
+  const T* const t1 = wtab + n2;
   T c[SEG];
 #pragma unroll
   for (int q = 0; q < SEG; ++q) {
     if (FULL || q < qn) {
       const bool ob = (mw >> q) & 1u;
-      const uint32_t below = mw & ((1u << q) - 1u);
-      int idx = below ? (n2 - 32 + q + __clz(below)) : (cw + q);
       const bool end = LAST && base + q == n2 - 1;
-      if (end) idx += 4 * n2;
-      const T inv = wtab[idx];
+      const T inv = end ? tp[4 * n2] : *tp;
       // rho2 inv from its table in FP64, whose pipe is the scarce one
-      const T a = (sizeof(T) == 8 && !end) ? wtab[idx + 2 * n2] : rho2 * inv;
+      const T a = (sizeof(T) == 8 && !end) ? tp[2 * n2] : rho2 * inv;
       d = fma(ob ? T(0) : a, d, ob ? v[q] : v[q] * inv);
       v[q] = d;
       c[q] = (ob || end) ? T(0) : a;
+      tp = ob ? t1 : tp + 1;
     }
   }
   T wn = T(0);
@@ -396,10 +396,9 @@ __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP,
 // W-step of every row of the slab: a thread per (row, segment), as many whole
 // rows at a time as the block has threads for; rows at col_of(q) (stride LP
 // along j), their mask words at msk + q words.  Ends with a barrier.
-template <typename T, typename ColFn>
+template <typename T, int SEG, typename ColFn>
 __device__ __forceinline__ void wstep_segments(ColFn col_of, int LP, const uint32_t* __restrict__ msk, int nrows, int n2,
                                                T rho2, const T* __restrict__ wtab) {
-  constexpr int SEG = kWSeg<T>;
   const int words = (n2 + 31) >> 5, segs = (n2 + SEG - 1) / SEG, ql = n2 - SEG * (segs - 1);
   const int rpr = blockDim.x / segs;  // rows per round (the block has at least segs threads)
   const int row = threadIdx.x % rpr, w = threadIdx.x / rpr;
@@ -410,8 +409,8 @@ __device__ __forceinline__ void wstep_segments(ColFn col_of, int LP, const uint3
     if (work) {
       col = col_of(r0 + row);
       const uint32_t* rowm = msk + (size_t)(r0 + row) * words;
-      if (w < segs - 1) wstep_segment<T, true, false>(col, LP, rowm, words, w, SEG, n2, rho2, wtab, v);
-      else wstep_segment<T, false, true>(col, LP, rowm, words, w, ql, n2, rho2, wtab, v);
+      if (w < segs - 1) wstep_segment<T, SEG, true, false>(col, LP, rowm, words, w, SEG, n2, rho2, wtab, v);
+      else wstep_segment<T, SEG, false, true>(col, LP, rowm, words, w, ql, n2, rho2, wtab, v);
     }
     __syncthreads();
     if (work) {

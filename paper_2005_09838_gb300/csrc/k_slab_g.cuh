@@ -20,34 +20,48 @@
 // slot: the transforms read 32 consecutive tubes of a slot and the W-step 32
 // consecutive rows of a tube, both without bank conflicts.
 //
-// Tiles.  A warp computes TL rows (inverse) or slices (forward) of 64 tubes
-// (two per lane; FP64: 32): each pair that is read feeds TL products and each
-// coefficient two.  tc_init times TL = 2, 4, 8 (a larger tile has fewer loads
-// per product, a smaller one fills the warps of small slabs).
+// Tiles.  An SM returns 128 bytes a clock from shared memory, so a pair that a
+// lane reads has to feed several products: a lane computes TL rows (inverse, one
+// parity of slices at a time) or slices (forward) of four tubes, 8 (TL + 4) bytes
+// for 4 TL products; two groups of 16 lanes take neighbouring TL columns of 64
+// tubes (FP64: 32 lanes, one tube each).  tc_init times TL = 2 and 4 (a larger
+// tile has fewer loads per product, a smaller one fills the warps of small slabs).
+// The even and odd sums of a row pair are parked in the slab and unfolded in a
+// pass of their own, which also places G.
 //
-// Staging.  The coefficients of one direction, the spectrum of as many 64-tube
-// groups as fit (all of them for most sizes) and G are copied to shared memory
-// by cp.async, so the transforms read nothing but shared memory: with the
+// Staging.  The coefficients of one direction, and the spectrum of as many 64-tube
+// groups as fit (all of them for most sizes) are copied to shared memory by
+// cp.async, so the transforms read nothing but shared memory: with the
 // spectrum and the coefficients read through L1 and G inside the item's
 // epilogue the inverse took 72K cycles of a 925 x 153 x 92 CTA against 28K for
-// the forward one.  G goes straight to its place in the slab and the inverse
-// stores only the missing entries.  Sizes whose slab leaves no room for the
-// stages take the unstaged form (STAGED = false).
+// the forward one.  Sizes whose slab leaves no room for a stage take the
+// unstaged form (STAGED = false).
 //
 // The modes are those of k_slab.
 #pragma once
 
 namespace tc {
 
-// Threads per CTA at most: 512 leave 128 registers a thread (FP64 values take
-// two each, so half as many threads).
+// Threads per CTA: kSlabGThreads where one CTA fills an SM, kSlabGHalf where two
+// slabs fit.  FP32: 32 warps of 64 registers on an SM either way (16 of 128
+// before: the kernel waits on shared memory and barriers, issue active 38%;
+// 925 x 153 x 92: 162 -> 150 us).  FP64 values take two registers each.
 template <typename T>
-constexpr int kSlabGThreads = sizeof(T) == 8 ? 256 : 512;
-// Tubes per lane (FP64: one, no product is worth a half-empty warp there) and per item.
+constexpr int kSlabGThreads = sizeof(T) == 8 ? 256 : 1024;
 template <typename T>
-constexpr int kTT = sizeof(T) == 8 ? 1 : 2;
+constexpr int kSlabGHalf = sizeof(T) == 8 ? 256 : 512;
+// A warp's item: kLW lanes side by side along the tubes with kTT tubes each (kLW
+// apart), and 32 / kLW groups of lanes with TL columns of the product each.  FP64
+// takes one tube per lane: no product is worth a half-empty warp there.
 template <typename T>
-constexpr int kGTubes = 32 * kTT<T>;
+constexpr int kLW = sizeof(T) == 8 ? 32 : 16;
+template <typename T>
+constexpr int kTT = sizeof(T) == 8 ? 1 : 4;
+template <typename T>
+constexpr int kLG = 32 / kLW<T>;
+template <typename T>
+constexpr int kGTubes = kLW<T> * kTT<T>;  // tubes of an item
+constexpr int kFoldPad = 16;              // columns of the tables, padded: a multiple of kLG TL
 constexpr int kSlabGMaxN3 = 512;      // the tables grow as n3^2
 
 // Pairs of T with packed arithmetic.
@@ -109,23 +123,24 @@ struct Pk<double> {
 struct FoldDims {
   int even, M, h;      // n3 = 2M, or n3 = 2h + 1
   int np;              // pair slots of a tube
-  int nl, nlp;         // rows l of the inverse (the others follow), padded to 8
+  int nl, nlp;         // rows l of the inverse (the others follow), padded
   int kmax;            // slices 1 .. kmax of the inverse loop
-  int nke, nkep, nkt;  // even slices (all slices for odd n3), padded to 8; columns of the forward table
+  int nke, nkep, nkt;  // even slices (all slices for odd n3), padded; columns of the forward table
   int lmax;            // rows 1 .. lmax of the forward loop
 };
 __host__ __device__ inline FoldDims fold_dims(int n3) {
   FoldDims f{};
+  auto pad = [](int n) { return (n + kFoldPad - 1) / kFoldPad * kFoldPad; };
   f.even = (n3 % 2) == 0;
   f.M = n3 / 2;
   f.h = (n3 - 1) / 2;
   f.np = (n3 + 1) / 2;
   f.nl = f.even ? f.M / 2 + 1 : f.h + 1;
-  f.nlp = (f.nl + 7) / 8 * 8;
+  f.nlp = pad(f.nl);
   f.kmax = f.even ? f.M - 1 : f.h;
   f.nke = f.even ? f.M / 2 + 1 : f.h + 1;
-  f.nkep = (f.nke + 7) / 8 * 8;
-  f.nkt = f.even ? f.nkep + ((f.M + 1) / 2 + 7) / 8 * 8 : f.nkep;
+  f.nkep = pad(f.nke);
+  f.nkt = f.even ? f.nkep + pad((f.M + 1) / 2) : f.nkep;
   f.lmax = f.even ? (f.M - 1) / 2 : f.h;
   return f;
 }
@@ -177,9 +192,10 @@ struct SlabGLayout {
 };
 // Tubes per slot of the slab: odd, so that consecutive slots start in other banks.
 __host__ __device__ inline int slab_g_stride(int n2) { return n2 | 1; }
-// Tubes of a stage of sg groups.
+// Row pitch of a stage of sg groups (whole groups: the lanes past n2 read what is
+// there and store nothing).
 template <typename T>
-__host__ __device__ inline int slab_g_width(int n2, int sg) { return sg * kGTubes<T> < n2 ? sg * kGTubes<T> : n2; }
+__host__ __device__ inline int slab_g_width(int sg) { return sg * kGTubes<T>; }
 // sg: 64-tube groups per stage (0: unstaged).
 template <typename T>
 __host__ __device__ inline SlabGLayout slab_g_layout(int n2, int n3, int sg) {
@@ -198,14 +214,15 @@ __host__ __device__ inline SlabGLayout slab_g_layout(int n2, int n3, int sg) {
     off = align_up(off + sizeof(cx<T>) * (ni > nf ? ni : nf), 16);
   }
   L.pairs = off;
-  off = align_up(off + sizeof(cx<T>) * (size_t)((n3 + 1) / 2) * slab_g_stride(n2), 16);
+  // (the last slot's lanes past n2 read up to a group further)
+  off = align_up(off + sizeof(cx<T>) * ((size_t)((n3 + 1) / 2) * slab_g_stride(n2) + kGTubes<T>), 16);
   L.stage = off;
-  off = align_up(off + sizeof(cx<T>) * (size_t)(n3 / 2 + 1) * slab_g_width<T>(n2, sg), 16);
+  off = align_up(off + sizeof(cx<T>) * (size_t)(n3 / 2 + 1) * slab_g_width<T>(sg), 16);
   L.total = off;
   return L;
 }
 
-// Launch shape of the folded-transform slab kernels: two CTAs of 256 threads on
+// Launch shape of the folded-transform slab kernels: two CTAs of kSlabGHalf threads on
 // an SM where the slab, the coefficients and a stage of one group fit half of
 // its shared memory, else one with twice the threads; as many groups per stage
 // as fit; unstaged where even one does not.  False where the slab itself does
@@ -225,7 +242,7 @@ inline bool slab_g_plan(int n2, int n3, int optin, SlabGPlan& pl) {
     for (int sg = ngr; sg >= 1; --sg) {
       const size_t b = slab_g_layout<T>(n2, n3, sg).total;
       if (b <= room) {
-        pl = SlabGPlan{pass == 0 ? 256 : kSlabGThreads<T>, sg, b};
+        pl = SlabGPlan{pass == 0 ? kSlabGHalf<T> : kSlabGThreads<T>, sg, b};
         return true;
       }
     }
@@ -251,130 +268,81 @@ __device__ __forceinline__ int slab_g_off(bool even, int n3, int l, int np2) {
   return (l <= m) ? 2 * np2 * l : 2 * np2 * (n3 - l) + 1;
 }
 
-// One item of the inverse transform: rows l0 .. l0 + TL - 1 (and those that
-// follow from them) of kGTubes<T> tubes.  load(k, j) gives the spectrum pair of
-// slice k in tube j of the lane; E, O receive the sums over even and odd
-// slices (all slices in E for odd n3), slices 0 and n3/2 included with weight 1/2.
-template <typename T, int TL, bool EVEN, bool SH, typename LoadFn>
-__device__ __forceinline__ void fold_inverse(const FoldDims& f, const cx<T>* __restrict__ tab, int l0, LoadFn load,
-                                             typename Pk<T>::V (&E)[TL][kTT<T>],
-                                             typename Pk<T>::V (&O)[EVEN ? TL : 1][kTT<T>]) {
+// acc[i][j] += sum over n rows of x(tube j) * tab[i]: the pair matrix and the
+// table advance by dx and dc pairs per row, tube j is kLW j pairs on.  (Running
+// pointers and one base per operand: with a clamped pointer per tube and indexed
+// rows the loop had ten integer instructions to its sixteen products.)
+template <typename T, int TL, bool SH>
+__device__ __forceinline__ void fold_product(typename Pk<T>::V (&acc)[TL][kTT<T>], const cx<T>* __restrict__ tab, int dc,
+                                             const cx<T>* __restrict__ x, int dx, int n) {
   using P = Pk<T>;
   using V = typename P::V;
+#pragma unroll 2
+  for (int q = 0; q < n; ++q, x += dx, tab += dc) {
+    V v[kTT<T>];
 #pragma unroll
-  for (int j = 0; j < kTT<T>; ++j) {
-    const V x0 = P::mk(T(0.5) * P::un(load(0, j)).re, T(0));
-#pragma unroll
-    for (int i = 0; i < TL; ++i) E[i][j] = x0;
-    if constexpr (EVEN) {
-      const T xm = T(0.5) * P::un(load(f.M, j)).re;
-      const bool modd = f.M & 1;
-#pragma unroll
-      for (int i = 0; i < TL; ++i) {
-        const V a = P::mk(((l0 + i) & 1) ? -xm : xm, T(0));
-        O[i][j] = modd ? a : P::mk(T(0), T(0));
-        if (!modd) E[i][j] = P::add(E[i][j], a);
-      }
-    }
-  }
-  const cx<T>* tl = tab + l0;
-  auto step = [&](int k, const V (&x)[kTT<T>], V (&acc)[TL][kTT<T>]) {
-    const cx<T>* tk = tl + (size_t)k * f.nlp;
+    for (int j = 0; j < kTT<T>; ++j) v[j] = P::lds(x + kLW<T> * j);
 #pragma unroll
     for (int i = 0; i < TL; i += 2) {
       V c0, c1;
-      P::template ld2<SH>(tk + i, c0, c1);
+      P::template ld2<SH>(tab + i, c0, c1);
 #pragma unroll
       for (int j = 0; j < kTT<T>; ++j) {
-        P::fma(acc[i][j], x[j], c0);
-        P::fma(acc[i + 1][j], x[j], c1);
+        P::fma(acc[i][j], v[j], c0);
+        P::fma(acc[i + 1][j], v[j], c1);
       }
-    }
-  };
-  auto acc_of = [&](int odd) -> V(&)[TL][kTT<T>] {
-    if constexpr (EVEN) {
-      if (odd) return O;
-    }
-    return E;
-  };
-  constexpr int U = 4;  // slices whose loads are in flight together (even: parity fixed per position)
-  V xn[U][kTT<T>];
-  int k = 1;
-  const int kend = 1 + f.kmax / U * U;
-  if (k < kend) {
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int j = 0; j < kTT<T>; ++j) xn[u][j] = load(k + u, j);
-  }
-  for (; k < kend; k += U) {
-    V x[U][kTT<T>];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int j = 0; j < kTT<T>; ++j) x[u][j] = xn[u][j];
-    if (k + U < kend) {
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int j = 0; j < kTT<T>; ++j) xn[u][j] = load(k + U + u, j);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) step(k + u, x[u], acc_of((u + 1) & 1));
-  }
-#pragma unroll
-  for (int u = 0; u < U - 1; ++u) {
-    if (k + u <= f.kmax) {
-      V x[kTT<T>];
-#pragma unroll
-      for (int j = 0; j < kTT<T>; ++j) x[j] = load(k + u, j);
-      step(k + u, x, acc_of((u + 1) & 1));
     }
   }
 }
 
-// One item of the forward transform: columns q0 .. q0 + TL - 1 of the forward
-// table (slices of one parity for even n3) of kGTubes<T> tubes, from the folded
-// slab.  acc receives (sum e c, sum o s).
-template <typename T, int TL, bool EVEN, bool SH>
-__device__ __forceinline__ void fold_forward(const FoldDims& f, const cx<T>* __restrict__ tab, int q0,
-                                             const cx<T>* const (&col)[kTT<T>], int np2,
+// One item of the inverse transform: the sums (C, D) over the slices of parity
+// par (all slices for odd n3) at rows l0 .. l0 + TL - 1, slices 0 and n3/2 with
+// weight 1/2.
+// x: the lane's first tube in the staged spectrum [k][ldx].
+template <typename T, int TL, bool EVEN>
+__device__ __forceinline__ void fold_inverse(const FoldDims& f, const cx<T>* __restrict__ tab, int l0, int par,
+                                             const cx<T>* __restrict__ x, int ldx,
                                              typename Pk<T>::V (&acc)[TL][kTT<T>]) {
   using P = Pk<T>;
-  using V = typename P::V;
-  const bool oddk = EVEN && q0 >= f.nkep;
-  const int kk0 = oddk ? q0 - f.nkep : q0;  // k = 2 (kk0 + i) + oddk for even n3
 #pragma unroll
   for (int j = 0; j < kTT<T>; ++j) {
-    const cx<T> s0 = col[j][0];
-    const V a0 = P::mk(EVEN && oddk ? s0.im : s0.re, T(0));
+    const T x0 = (!EVEN || par == 0) ? T(0.5) * x[kLW<T> * j].re : T(0);
+    const T xm = (EVEN && (f.M & 1) == par) ? T(0.5) * x[f.M * ldx + kLW<T> * j].re : T(0);
 #pragma unroll
-    for (int i = 0; i < TL; ++i) acc[i][j] = a0;
-    if (EVEN && (f.M & 1) == 0) {
-      // row M/2: e cos(pi k / 2) on even slices, o sin(pi k / 2) on odd ones
-      const cx<T> sm = col[j][(size_t)(f.M / 2) * np2];
-#pragma unroll
-      for (int i = 0; i < TL; ++i) {
-        const bool neg = (kk0 + i) & 1;
-        const T a = neg ? -sm.re : sm.re, b = neg ? -sm.im : sm.im;
-        acc[i][j] = P::add(acc[i][j], oddk ? P::mk(T(0), b) : P::mk(a, T(0)));
-      }
-    }
+    for (int i = 0; i < TL; ++i) acc[i][j] = P::mk(((l0 + i) & 1) ? x0 - xm : x0 + xm, T(0));
   }
-  // slot l holds the even fold, slot M - l the odd one
-  const int sl = oddk ? f.M : 0, sd = oddk ? -1 : 1;
-  const cx<T>* tq = tab + q0;
-#pragma unroll 4
-  for (int l = 1; l <= f.lmax; ++l) {
-    V x[kTT<T>];
-    const int so = (sl + sd * l) * np2;
+  const int k0 = EVEN ? 2 - par : 1, step = EVEN ? 2 : 1;
+  fold_product<T, TL, true>(acc, tab + l0 + k0 * f.nlp, step * f.nlp, x + k0 * ldx, step * ldx,
+                            (f.kmax - k0 + step) / step);
+}
+// The same from the stored spectrum in global memory (tube j of the lane at z[j],
+// rows n2 apart, plus r[j] where ADD) and the tables there.
+template <typename T, int TL, bool EVEN, bool ADD>
+__device__ __forceinline__ void fold_inverse_global(const FoldDims& f, const cx<T>* __restrict__ tab, int l0, int par,
+                                                    const cx<T>* const (&z)[kTT<T>], const cx<T>* const (&r)[kTT<T>],
+                                                    int n2, typename Pk<T>::V (&acc)[TL][kTT<T>]) {
+  using P = Pk<T>;
+  using V = typename P::V;
+  auto load = [&](int k, int j) -> V {
+    const size_t o = (size_t)k * n2;
+    return ADD ? P::add(P::ldg(z[j] + o), P::ldg(r[j] + o)) : P::ldg(z[j] + o);
+  };
 #pragma unroll
-    for (int j = 0; j < kTT<T>; ++j) x[j] = P::lds(col[j] + so);
-    const cx<T>* tk = tq + (size_t)l * f.nkt;
+  for (int j = 0; j < kTT<T>; ++j) {
+    const T x0 = (!EVEN || par == 0) ? T(0.5) * P::un(load(0, j)).re : T(0);
+    const T xm = (EVEN && (f.M & 1) == par) ? T(0.5) * P::un(load(f.M, j)).re : T(0);
+#pragma unroll
+    for (int i = 0; i < TL; ++i) acc[i][j] = P::mk(((l0 + i) & 1) ? x0 - xm : x0 + xm, T(0));
+  }
+#pragma unroll 2
+  for (int k = EVEN ? 2 - par : 1; k <= f.kmax; k += EVEN ? 2 : 1) {
+    V x[kTT<T>];
+#pragma unroll
+    for (int j = 0; j < kTT<T>; ++j) x[j] = load(k, j);
 #pragma unroll
     for (int i = 0; i < TL; i += 2) {
       V c0, c1;
-      P::template ld2<SH>(tk + i, c0, c1);
+      P::template ld2<false>(tab + l0 + k * f.nlp + i, c0, c1);
 #pragma unroll
       for (int j = 0; j < kTT<T>; ++j) {
         P::fma(acc[i][j], x[j], c0);
@@ -382,6 +350,57 @@ __device__ __forceinline__ void fold_forward(const FoldDims& f, const cx<T>* __r
       }
     }
   }
+}
+
+// Where the sums of row l and parity par go in the slab until all are there: the
+// even slices' to slot l, the odd ones' to slot M - l; rows 0 and M/2, whose
+// sums have one component each, share a slot.
+// (live: one bit per tube of the lane)
+template <typename T, bool EVEN>
+__device__ __forceinline__ void fold_park(const FoldDims& f, cx<T>* col, int np2, int l, int par, uint32_t live,
+                                          const typename Pk<T>::V (&v)[kTT<T>]) {
+  if (EVEN && (l == 0 || 2 * l == f.M)) {
+    T* at = reinterpret_cast<T*>(col + l * np2) + par;
+    const bool re = par == 0 || l == 0;
+#pragma unroll
+    for (int j = 0; j < kTT<T>; ++j) {
+      const cx<T> a = Pk<T>::un(v[j]);
+      if ((live >> j) & 1u) at[2 * kLW<T> * j] = re ? a.re : a.im;
+    }
+  } else {
+    cx<T>* at = col + (EVEN && par ? f.M - l : l) * np2;
+#pragma unroll
+    for (int j = 0; j < kTT<T>; ++j)
+      if ((live >> j) & 1u) at[kLW<T> * j] = Pk<T>::un(v[j]);
+  }
+}
+
+// One item of the forward transform: columns q0 .. q0 + TL - 1 of the forward
+// table (slices of one parity for even n3) of the item's tubes, from the folded
+// slab.  acc receives (sum e c, sum o s).
+template <typename T, int TL, bool EVEN, bool SH>
+__device__ __forceinline__ void fold_forward(const FoldDims& f, const cx<T>* __restrict__ tab, int q0,
+                                             const cx<T>* __restrict__ col, int np2,
+                                             typename Pk<T>::V (&acc)[TL][kTT<T>]) {
+  using P = Pk<T>;
+  const bool oddk = EVEN && q0 >= f.nkep;
+  const int kk0 = oddk ? q0 - f.nkep : q0;  // k = 2 (kk0 + i) + oddk for even n3
+#pragma unroll
+  for (int j = 0; j < kTT<T>; ++j) {
+    const cx<T> s0 = col[kLW<T> * j];
+    const T x0 = EVEN && oddk ? s0.im : s0.re;
+    // row M/2: e cos(pi k / 2) on even slices, o sin(pi k / 2) on odd ones
+    const cx<T> sm = (EVEN && (f.M & 1) == 0) ? col[(f.M / 2) * np2 + kLW<T> * j] : cx<T>{T(0), T(0)};
+    const T a = oddk ? T(0) : sm.re, b = oddk ? sm.im : T(0);
+#pragma unroll
+    for (int i = 0; i < TL; ++i) {
+      const bool neg = (kk0 + i) & 1;
+      acc[i][j] = P::mk(neg ? x0 - a : x0 + a, neg ? -b : b);
+    }
+  }
+  // slot l holds the even fold, slot M - l the odd one
+  const cx<T>* x = col + (oddk ? f.M - 1 : 1) * np2;
+  fold_product<T, TL, SH>(acc, tab + q0 + f.nkt, f.nkt, x, oddk ? -np2 : np2, f.lmax);
 }
 
 template <typename T, int MODE, int TL, bool EVEN, bool STAGED>
@@ -404,7 +423,6 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
   cx<T>* stg = reinterpret_cast<cx<T>*>(smem + lay.stage);
   T* spat = reinterpret_cast<T*>(pairs);
   const int ni = (f.kmax + 1) * f.nlp, nf = (f.lmax + 1) * f.nkt;
-  const cx<T>* tabi = STAGED ? tab : d.fold;
   const cx<T>* tabf = STAGED ? tab : d.fold + ni;
   const cx<T>* zrow = d.Zt + (size_t)i1 * S * n2;
   const cx<T>* rrow = d.Rt + (size_t)i1 * S * n2;
@@ -424,18 +442,15 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
     }
   if (STAGED)
     for (int e = tid; e < ni; e += nt) cp_async_elem(tab + e, d.fold + e);
-  if (NEED_G)
-    for (int l = wid; l < n3; l += nw) {
-      T* row = spat + slab_g_off(EVEN, n3, l, np2);
-      for (int t = lane; t < n2; t += 32) cp_async_elem(row + 2 * t, Gi + (size_t)l * n2 + t);
-    }
+  if (NEED_G)  // G, wanted after the inverse transform, on its way to L2
+    for (int e = 128 / (int)sizeof(T) * tid; e < n3 * n2; e += 128 / (int)sizeof(T) * nt) asm volatile("prefetch.global.L2 [%0];" ::"l"(Gi + e));
 
-  // ---- inverse transform; v = G on the mask, Z elsewhere (MODE_GRAD: Z - G on the
-  // mask, 0 elsewhere) --------------------------------------------------------------------
+  // ---- inverse transform: the sums of every row pair, parked in the slab -------------------
   const int ngr = (n2 + kGTubes<T> - 1) / kGTubes<T>;
   const int gstage = STAGED ? sg : ngr;
-  const int width = slab_g_width<T>(n2, gstage);  // tubes of a full stage, its row stride
-  const T scale = T(2) / T(n3);
+  const int width = slab_g_width<T>(gstage);  // tubes of a full stage, its row stride
+  constexpr int LC = kLG<T> * TL;                 // columns of a warp's item
+  const int lt = lane & (kLW<T> - 1), lg = lane / kLW<T>;
   SqSum<T> gsum;
   for (int g0 = 0; g0 < ngr; g0 += gstage) {
     const int gn = min(gstage, ngr - g0);
@@ -453,77 +468,90 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
     }
     cp_async_wait_all();
     __syncthreads();
-    const int ntile = (f.nl + TL - 1) / TL;
-    for (int e = wid; e < ntile * gn; e += nw) {
-      const int gl = e / ntile, g = g0 + gl, l0 = (e - gl * ntile) * TL;
-      int t[kTT<T>];
-      const cx<T>* zc[kTT<T>];
-      const cx<T>* rc[kTT<T>];
+    const int ntile = (f.nl + LC - 1) / LC, npar = EVEN ? 2 : 1;
+    for (int e = wid; e < npar * ntile * gn; e += nw) {
+      const int gl = e / (npar * ntile), rest = e - gl * npar * ntile, par = rest & (npar - 1);
+      const int g = g0 + gl, l0 = (rest / npar) * LC + lg * TL;
+      const int t0 = g * kGTubes<T> + lt;
+      uint32_t live = 0;
 #pragma unroll
-      for (int j = 0; j < kTT<T>; ++j) {
-        t[j] = g * kGTubes<T> + 32 * j + lane;
-        const int tq = min(t[j], n2 - 1);
-        zc[j] = STAGED ? stg + (tq - g0 * kGTubes<T>) : zrow + tq;
-        rc[j] = rrow + tq;
-      }
-      auto load = [&](int k, int j) -> V {
-        if (STAGED) return P::lds(zc[j] + k * width);
-        const size_t o = (size_t)k * n2;
-        if (MODE == MODE_W) return P::add(P::ldg(zc[j] + o), P::ldg(rc[j] + o));
-        return P::ldg((MODE == MODE_R ? rc[j] : zc[j]) + o);
-      };
-      V E[TL][kTT<T>], O[EVEN ? TL : 1][kTT<T>];
-      fold_inverse<T, TL, EVEN, STAGED>(f, tabi, l0, load, E, O);
-      // value of the row at slab index q (row order), half h of slot p, tube j
-      auto put = [&](T x, int q, T* at, int j) {
-        x *= scale;
-        const bool live = t[j] < n2;
-        if (NEED_G) {
-          const uint32_t w = (g * kTT<T> + j < mw) ? msk[q * mw + g * kTT<T> + j] : 0u;
-          const bool ob = (w >> lane) & 1u;
-          if (MODE == MODE_ITER) {
-            if (live && !ob) *at = x * zfac;
-          } else if (live) {
-            x = ob ? x - *at : T(0);
-            gsum.add(x);
-            *at = x;
-          }
-        } else if (live) {
-          *at = x;
-        }
-      };
-#pragma unroll
-      for (int i = 0; i < TL; ++i) {
-        const int l = l0 + i;
-        if (l >= f.nl) break;
+      for (int j = 0; j < kTT<T>; ++j) live |= (uint32_t)(t0 + kLW<T> * j < n2) << j;
+      V acc[TL][kTT<T>];
+      if constexpr (STAGED) {
+        fold_inverse<T, TL, EVEN>(f, tab, l0, par, stg + t0 - g0 * kGTubes<T>, width, acc);
+      } else {
+        const cx<T>* zc[kTT<T>];
+        const cx<T>* rc[kTT<T>];
 #pragma unroll
         for (int j = 0; j < kTT<T>; ++j) {
-          T* cp = spat + 2 * (l * np2 + t[j]);
-          if constexpr (EVEN) {
-            const cx<T> a = P::un(E[i][j]), b = P::un(O[i][j]);
-            const T cs = a.re + b.re, ds = a.im + b.im, cd = a.re - b.re, dd = a.im - b.im;
-            if (l == 0) {
-              put(cs, 0, cp, j);
-              put(cd, 1, cp + 1, j);
-            } else {
-              put(cs - ds, 2 * l, cp, j);
-              put(cs + ds, 2 * l + 1, cp + 1, j);
-              if (2 * l != f.M) {
-                T* cm = spat + 2 * ((f.M - l) * np2 + t[j]);
-                put(cd + dd, 2 * (f.M - l), cm, j);
-                put(cd - dd, 2 * (f.M - l) + 1, cm + 1, j);
-              }
-            }
-          } else {
-            const cx<T> a = P::un(E[i][j]);
-            if (l == 0) {
-              put(a.re, 0, cp, j);
-            } else {
-              put(a.re - a.im, 2 * l - 1, cp, j);
-              put(a.re + a.im, 2 * l, cp + 1, j);
-            }
+          const int tq = min(t0 + kLW<T> * j, n2 - 1);
+          zc[j] = (MODE == MODE_R ? rrow : zrow) + tq;
+          rc[j] = rrow + tq;
+        }
+        fold_inverse_global<T, TL, EVEN, MODE == MODE_W>(f, d.fold, l0, par, zc, rc, n2, acc);
+      }
+#pragma unroll
+      for (int i = 0; i < TL; ++i) {
+        if (l0 + i >= f.nl) break;
+        fold_park<T, EVEN>(f, pairs + t0, np2, l0 + i, par, live, acc[i]);
+      }
+    }
+  }
+  __syncthreads();
+  // ---- the rows from the sums; v = G on the mask, Z elsewhere (MODE_GRAD: Z - G on the
+  // mask, 0 elsewhere) ------------------------------------------------------------------------
+  {
+    const T fac = (T(2) / T(n3)) * (MODE == MODE_ITER ? zfac : T(1));
+    // (two warps share a slot, 32 tubes in turn)
+    const int nun = EVEN ? f.M / 2 + 1 : f.h + 1;
+    for (int e = wid; e < 2 * nun; e += nw) {
+      const int l = e >> 1;
+      // slots of the item and their rows: slot l = rows (l, r1), slot M - l = rows (r2, r3)
+      const bool two = EVEN && l > 0 && 2 * l != f.M;
+      const int r1 = EVEN ? (l == 0 ? f.M : n3 - l) : (l == 0 ? 0 : n3 - l);
+      const int q0 = EVEN ? 2 * l : (l == 0 ? 0 : 2 * l - 1), q2 = two ? 2 * (f.M - l) : q0;
+      const uint32_t *m0 = msk + q0 * mw, *m2 = msk + q2 * mw;
+      const int first = (EVEN || l > 0) ? mw : 0;  // the second row's words
+      const T *g0 = Gi + l * n2, *g1 = Gi + r1 * n2, *g2 = Gi + (two ? f.M - l : l) * n2, *g3 = Gi + (two ? f.M + l : l) * n2;
+      cx<T>*c0 = pairs + l * np2, *c2 = pairs + (two ? f.M - l : l) * np2;
+#pragma unroll 2
+      for (int t = 32 * (e & 1) + lane; t < n2; t += 64) {
+        T gv[4] = {};
+        uint32_t w[4] = {};
+        if (NEED_G) {
+          const int blk = t >> 5;
+          gv[0] = __ldg(g0 + t), gv[1] = __ldg(g1 + t);
+          w[0] = m0[blk], w[1] = m0[first + blk];
+          if (EVEN) {
+            gv[2] = __ldg(g2 + t), gv[3] = __ldg(g3 + t);
+            w[2] = m2[blk], w[3] = m2[mw + blk];
           }
         }
+        T x[4];
+        const cx<T> a = c0[t];
+        if (EVEN) {
+          const cx<T> b = c2[t];
+          const T cs = a.re + b.re, ds = a.im + b.im, cd = a.re - b.re, dd = a.im - b.im;
+          x[0] = two ? cs - ds : (l == 0 ? a.re + a.im : a.re - a.im);
+          x[1] = two ? cs + ds : (l == 0 ? a.re - a.im : a.re + a.im);
+          x[2] = cd + dd, x[3] = cd - dd;
+        } else {
+          x[0] = l == 0 ? a.re : a.re - a.im;
+          x[1] = l == 0 ? T(0) : a.re + a.im;
+          x[2] = x[3] = T(0);
+        }
+#pragma unroll
+        for (int q = 0; q < (EVEN ? 4 : 2); ++q) {
+          x[q] *= fac;
+          const bool ob = (w[q] >> lane) & 1u;
+          if (MODE == MODE_ITER) x[q] = ob ? gv[q] : x[q];
+          if (MODE == MODE_GRAD) {
+            x[q] = ob ? x[q] - gv[q] : T(0);
+            if ((q < 2 && (EVEN || q == 0 || l > 0)) || two) gsum.add(x[q]);
+          }
+        }
+        c0[t] = cx<T>{x[0], x[1]};
+        if (two) c2[t] = cx<T>{x[2], x[3]};
       }
     }
   }
@@ -565,7 +593,7 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
 
   // ---- W-step -------------------------------------------------------------------------------
   if (wsolve)
-    wstep_segments<T>([&](int q) { return spat + slab_g_off(EVEN, n3, slab_g_row(EVEN, n3, q), np2); }, 2, msk, n3, n2,
+    wstep_segments<T, kWSeg<T>>([&](int q) { return spat + slab_g_off(EVEN, n3, slab_g_row(EVEN, n3, q), np2); }, 2, msk, n3, n2,
                    d.rho2, wtab);
 
   // ---- fold -----------------------------------------------------------------------------------
@@ -593,8 +621,8 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
   const bool zstaged = STAGED && gstage >= ngr;  // the whole spectrum is still staged
   double dw2 = 0.0;
   {
-    const int nte = (f.nke + TL - 1) / TL;                                  // tiles of even (all) slices
-    const int ntile = nte + (EVEN ? ((f.M + 1) / 2 + TL - 1) / TL : 0);
+    const int nte = (f.nke + LC - 1) / LC;                                  // tiles of even (all) slices
+    const int ntile = nte + (EVEN ? ((f.M + 1) / 2 + LC - 1) / LC : 0);
     cx<T>* rt = d.Rt + (size_t)i1 * S * n2;
     const cx<T>* dz = track ? d.dZt + (size_t)i1 * S * n2 : nullptr;
     // the change of W~ (FP64) in a loop of its own: as a predicated part of the
@@ -604,29 +632,34 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
       constexpr bool TRACK = decltype(tr)::value;
       for (int e = wid; e < ntile * ngr; e += nw) {
         const int g = e / ntile, it = e - g * ntile;
-        const int q0 = (it < nte) ? it * TL : f.nkep + (it - nte) * TL;
-        int t[kTT<T>];
-        const cx<T>* col[kTT<T>];
-#pragma unroll
-        for (int j = 0; j < kTT<T>; ++j) {
-          t[j] = g * kGTubes<T> + 32 * j + lane;
-          col[j] = pairs + min(t[j], n2 - 1);
-        }
+        const int q0 = ((it < nte) ? it * LC : f.nkep + (it - nte) * LC) + lg * TL;
+        const int t0 = g * kGTubes<T> + lt;
         V acc[TL][kTT<T>];
-        fold_forward<T, TL, EVEN, STAGED>(f, tabf, q0, col, np2, acc);
+        fold_forward<T, TL, EVEN, STAGED>(f, tabf, q0, pairs + t0, np2, acc);
+        int k = EVEN ? (it < nte ? 2 * q0 : 2 * (q0 - f.nkep) + 1) : q0;
+        int o = k * n2 + t0;
+        const int dk = EVEN ? 2 : 1;
 #pragma unroll
-        for (int i = 0; i < TL; ++i) {
-          const int k = EVEN ? (it < nte ? 2 * (q0 + i) : 2 * (q0 - f.nkep + i) + 1) : q0 + i;
+        for (int i = 0; i < TL; ++i, k += dk, o += dk * n2) {
           if (k >= S) break;
+          const bool real = k == 0 || 2 * k == n3;
+          cx<T> zv[kTT<T>];
+          if (MODE != MODE_GRAD) {
+#pragma unroll
+            for (int j = 0; j < kTT<T>; ++j)
+              if (t0 + kLW<T> * j < n2) {
+                if (STAGED && zstaged) zv[j] = stg[k * width + t0 + kLW<T> * j];
+                else zv[j] = ldg_cx(zrow + o + kLW<T> * j);
+              }
+          }
 #pragma unroll
           for (int j = 0; j < kTT<T>; ++j) {
-            if (t[j] >= n2) continue;
-            const int o = k * n2 + t[j];
+            if (t0 + kLW<T> * j >= n2) break;
             const cx<T> a = P::un(acc[i][j]);
-            cx<T> x = {a.re, (k == 0 || 2 * k == n3) ? T(0) : -a.im};
-            if (MODE != MODE_GRAD) x = x - (zstaged ? stg[o] : ldg_cx(zrow + o));
-            if constexpr (TRACK) dw2 += dw_term(x, rt[o], dz[o], k, n3);
-            rt[o] = x;
+            cx<T> x = {a.re, real ? T(0) : -a.im};
+            if (MODE != MODE_GRAD) x = x - zv[j];
+            if constexpr (TRACK) dw2 += dw_term(x, rt[o + kLW<T> * j], dz[o + kLW<T> * j], k, n3);
+            rt[o + kLW<T> * j] = x;
           }
         }
       }
@@ -644,6 +677,162 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
     block_sum2(g, unused, red);
     if (tid == 0) d.part[(size_t)i1 * 4] = g;
   }
+}
+
+// ---------------------------------------------------------------------------
+// Transforms of the factors with the same products: kGTubes tubes per CTA, the
+// tubes and the coefficients staged in shared memory.  A factor is U = n r tubes,
+// contiguous for every l (and, in the spectrum [S][r][n], for every k); with
+// transposed = 1 (Y: spatial order s fastest) tube u of the spectrum is
+// u = s n + i and of the spatial side s + r i.
+//   k_fold_dft   real [n3][U] -> half spectrum [S][U]
+//   k_fold_idft  half spectrum -> real, 1 / n3 included
+// One thread per tube and four outputs before (k_factor_dft, k_factor_idft, which
+// keep the lengths whose tables do not fit): 80 + 51 and 88 + 65 us for both
+// factors of 529 x 288 x 168, r = 16.
+// ---------------------------------------------------------------------------
+constexpr int kFoldThreads = 256;
+constexpr int kFoldTL = 4;
+
+// Shared bytes: table, then the folded pairs (forward) or the spectrum (inverse).
+template <typename T>
+__host__ __device__ inline size_t fold_dft_smem(int n3) {
+  const FoldDims f = fold_dims(n3);
+  const size_t ni = (size_t)(f.kmax + 1) * f.nlp, nf = (size_t)(f.lmax + 1) * f.nkt;
+  return ((ni > nf ? ni : nf) + (size_t)(n3 / 2 + 1) * (kGTubes<T> + 1)) * sizeof(cx<T>);
+}
+template <typename T>
+inline bool fold_dft_fits(int n3, int optin) {
+  return n3 <= kSlabGMaxN3 && fold_dft_smem<T>(n3) <= (size_t)optin;
+}
+
+template <typename T, bool EVEN>
+__device__ __forceinline__ void fold_dft_impl(const T* __restrict__ in, cx<T>* __restrict__ out,
+                                              const cx<T>* __restrict__ fold, int n, int r, int n3, int transposed,
+                                              unsigned char* smem) {
+  constexpr int TL = kFoldTL, W = kGTubes<T>, LD = W + 1, LC = kLG<T> * TL;
+  using P = Pk<T>;
+  const FoldDims f = fold_dims(n3);
+  const int ni = (f.kmax + 1) * f.nlp, nf = (f.lmax + 1) * f.nkt, S = n3 / 2 + 1;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+  cx<T>* tab = reinterpret_cast<cx<T>*>(smem);
+  cx<T>* pairs = tab + (ni > nf ? ni : nf);
+  const size_t U = (size_t)n * r, u0 = (size_t)blockIdx.x * W;
+  const int tn = (int)(U - u0 < (size_t)W ? U - u0 : (size_t)W);
+  for (int e = tid; e < nf; e += blockDim.x) tab[e] = fold[ni + e];
+  // the rows folded as in the slab kernel
+  const int nfold = EVEN ? f.M / 2 + 1 : f.h + 1;
+  for (int l = wid; l < nfold; l += nw)
+    for (int t = lane; t < tn; t += 32) {
+      const T* x = in + u0 + t;
+      auto row = [&](int q) { return x[(size_t)q * U]; };
+      if (EVEN && l > 0 && 2 * l != f.M) {
+        const T a = row(l), b = row(n3 - l), c = row(f.M - l), e = row(f.M + l);
+        const T ea = a + b, oa = a - b, eb = c + e, ob = c - e;
+        pairs[l * LD + t] = cx<T>{ea + eb, oa - ob};
+        pairs[(f.M - l) * LD + t] = cx<T>{ea - eb, oa + ob};
+      } else if (EVEN) {
+        const T a = row(l), b = row(l == 0 ? f.M : n3 - l);
+        pairs[l * LD + t] = cx<T>{a + b, a - b};
+      } else {
+        const T a = row(l), b = l > 0 ? row(n3 - l) : T(0);
+        pairs[l * LD + t] = l > 0 ? cx<T>{a + b, a - b} : cx<T>{a, T(0)};
+      }
+    }
+  __syncthreads();
+  const int lt = lane & (kLW<T> - 1), lg = lane / kLW<T>;
+  const int nte = (f.nke + LC - 1) / LC, ntile = nte + (EVEN ? ((f.M + 1) / 2 + LC - 1) / LC : 0);
+  for (int it = wid; it < ntile; it += nw) {
+    const int q0 = ((it < nte) ? it * LC : f.nkep + (it - nte) * LC) + lg * TL;
+    typename P::V acc[TL][kTT<T>];
+    fold_forward<T, TL, EVEN, true>(f, tab, q0, pairs + lt, LD, acc);
+#pragma unroll
+    for (int i = 0; i < TL; ++i) {
+      const int k = EVEN ? (it < nte ? 2 * (q0 + i) : 2 * (q0 - f.nkep + i) + 1) : q0 + i;
+      if (k >= S) break;
+#pragma unroll
+      for (int j = 0; j < kTT<T>; ++j) {
+        const int t = kLW<T> * j + lt;
+        if (t >= tn) continue;
+        const size_t u = u0 + t, o = transposed ? (u % r) * n + u / r : u;
+        const cx<T> a = P::un(acc[i][j]);
+        out[(size_t)k * U + o] = cx<T>{a.re, (k == 0 || 2 * k == n3) ? T(0) : -a.im};
+      }
+    }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kFoldThreads) k_fold_dft(const T* __restrict__ in, cx<T>* __restrict__ out,
+                                                           const cx<T>* __restrict__ fold, int n, int r, int n3,
+                                                           int transposed) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (n3 & 1) fold_dft_impl<T, false>(in, out, fold, n, r, n3, transposed, smem);
+  else fold_dft_impl<T, true>(in, out, fold, n, r, n3, transposed, smem);
+}
+
+template <typename T, bool EVEN>
+__device__ __forceinline__ void fold_idft_impl(const cx<T>* __restrict__ in, T* __restrict__ out,
+                                               const cx<T>* __restrict__ fold, int n, int r, int n3, int transposed,
+                                               unsigned char* smem) {
+  constexpr int TL = kFoldTL, W = kGTubes<T>, LC = kLG<T> * TL;
+  using P = Pk<T>;
+  const FoldDims f = fold_dims(n3);
+  const int ni = (f.kmax + 1) * f.nlp, nf = (f.lmax + 1) * f.nkt, S = n3 / 2 + 1;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+  cx<T>* tab = reinterpret_cast<cx<T>*>(smem);
+  cx<T>* spec = tab + (ni > nf ? ni : nf);  // [S][W]
+  const size_t U = (size_t)n * r, u0 = (size_t)blockIdx.x * W;
+  const int tn = (int)(U - u0 < (size_t)W ? U - u0 : (size_t)W);
+  for (int e = tid; e < ni; e += blockDim.x) cp_async_elem(tab + e, fold + e);
+  for (int k = wid; k < S; k += nw)
+    for (int t = lane; t < tn; t += 32) cp_async_elem(spec + k * W + t, in + (size_t)k * U + u0 + t);
+  cp_async_wait_all();
+  __syncthreads();
+  const T scale = T(2) / T(n3);
+  const int lt = lane & (kLW<T> - 1), lg = lane / kLW<T>;
+  for (int lb = wid * LC; lb < f.nl; lb += nw * LC) {
+    const int l0 = lb + lg * TL;
+    typename P::V E[TL][kTT<T>], O[TL][kTT<T>];
+    fold_inverse<T, TL, EVEN>(f, tab, l0, 0, spec + lt, W, E);
+    if (EVEN) fold_inverse<T, TL, EVEN>(f, tab, l0, 1, spec + lt, W, O);
+#pragma unroll
+    for (int i = 0; i < TL; ++i) {
+      const int l = l0 + i;
+      if (l >= f.nl) break;
+#pragma unroll
+      for (int j = 0; j < kTT<T>; ++j) {
+        const int t = kLW<T> * j + lt;
+        if (t >= tn) continue;
+        const size_t u = u0 + t, o = transposed ? (u % n) * r + u / n : u;
+        auto put = [&](int q, T v) { out[(size_t)q * U + o] = v * scale; };
+        const cx<T> a = P::un(E[i][j]);
+        if constexpr (EVEN) {
+          const cx<T> b = P::un(O[i][j]);
+          const T cs = a.re + b.re, ds = a.im + b.im, cd = a.re - b.re, dd = a.im - b.im;
+          put(l, cs - ds);
+          if (l > 0) put(n3 - l, cs + ds);
+          if (l == 0) put(f.M, cd);
+          else if (2 * l != f.M) {
+            put(f.M - l, cd + dd);
+            put(f.M + l, cd - dd);
+          }
+        } else {
+          put(l, a.re - a.im);
+          if (l > 0) put(n3 - l, a.re + a.im);
+        }
+      }
+    }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kFoldThreads) k_fold_idft(const cx<T>* __restrict__ in, T* __restrict__ out,
+                                                            const cx<T>* __restrict__ fold, int n, int r, int n3,
+                                                            int transposed) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (n3 & 1) fold_idft_impl<T, false>(in, out, fold, n, r, n3, transposed, smem);
+  else fold_idft_impl<T, true>(in, out, fold, n, r, n3, transposed, smem);
 }
 
 template <typename T, int MODE, int TL, bool STAGED>

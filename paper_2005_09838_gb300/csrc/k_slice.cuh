@@ -1776,11 +1776,18 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
   // real slices of an FP32 engine: t G^+ in FP64 (k_xstep / k_xc), applied in FP64
   const bool realslice = (k == 0) || (2 * k == d.n3);
   const bool g64 = sizeof(T) == 4 && realslice && d.Gp64 != nullptr;
-  double* gh64 = reinterpret_cast<double*>(smem + ystep_gh64_offset<T>(n1, r, RP, XSH, TCY, CW));
+  // (as FP32 head and tail: the products below are error-free, where an FP64
+  // multiply-add and a conversion per term took the FP64 pipe of the real slices'
+  // CTAs 15 us at r = 32)
+  cx<float>* gh64 = reinterpret_cast<cx<float>*>(smem + ystep_gh64_offset<T>(n1, r, RP, XSH, TCY, CW));
   for (int e = tid; e < rr; e += blockDim.x) {
     Dgs[e] = d.Dg[(size_t)k * rr + e];
     Gh[e] = d.Gp[(size_t)k * rr + e];
-    if (g64) gh64[e] = d.Gp64[(size_t)(k == 0 ? 0 : 1) * rr + e].re;
+    if (g64) {
+      const double g = d.Gp64[(size_t)(k == 0 ? 0 : 1) * rr + e].re;
+      const float h = (float)g;
+      gh64[e] = cx<float>{h, (float)(g - (double)h)};
+    }
   }
   for (int e = tid; e < r * TW; e += blockDim.x) {
     const int s = e / TW, c = e - s * TW;
@@ -1901,9 +1908,14 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
     }
     cx<T> y = Yo[e];
     if (g64) {
-      double yd = (double)y.re;
-      for (int u = 0; u < r; ++u) yd = fma(gh64[s * r + u], (double)Ds[u * TW + c].re, yd);
-      y.re = (T)yd;
+      float h = (float)y.re, l = 0.f;
+      for (int u = 0; u < r; ++u) {
+        const cx<float> g = gh64[s * r + u];
+        const float v = (float)Ds[u * TW + c].re;
+        dot2(h, l, g.re, v);
+        l = fmaf(g.im, v, l);
+      }
+      y.re = (T)(h + l);
     } else {
       for (int u = 0; u < r; ++u) cfma(y, Gh[s * r + u], Ds[u * TW + c]);
     }

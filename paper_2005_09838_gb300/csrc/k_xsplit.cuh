@@ -19,7 +19,6 @@ namespace tc {
 
 constexpr int kXaThreads = 1024;
 constexpr int kXgRows = 64;
-constexpr int kXgLd = kXgRows + 1;  // odd row pitch: conflict-free column reads
 
 template <typename TS>
 __host__ __device__ inline size_t xa_smem_bytes(int r) {
@@ -28,8 +27,8 @@ __host__ __device__ inline size_t xa_smem_bytes(int r) {
 }
 
 template <typename T>
-__host__ __device__ inline size_t xg_smem_bytes(int r) {
-  return 2 * (size_t)r * kXgLd * sizeof(cx<T>);
+__host__ __device__ inline size_t xg_smem_bytes(int rp) {
+  return (2 * (size_t)kXgRows + 1) * (rp + 2) * sizeof(cx<T>);
 }
 
 // ---- A^+ and P of every slice ----------------------------------------------------------
@@ -299,98 +298,135 @@ __global__ void __launch_bounds__(256) k_xbc(Dev<T> d) {
 // Grams are the ill-conditioned ones (the DC slice carries the mean traffic),
 // so they are accumulated with dot2 and the partial is stored as (sum,
 // compensation) in the (re, im) fields.
-template <typename T>
-__global__ void __launch_bounds__(256) k_xg(Dev<T> d) {
+//
+// Complex slices: a thread forms a 4 x 2 tile (2 x 2 for r <= 16) of the three Grams, so each row
+// costs it eight 8-byte loads and 96 multiply-adds (2 x 2 tiles of one Gram per
+// 10 loads before: 47 us on 529 x 96 x 112, r = 32).  Real slices: a thread per
+// entry, an entry's error-free sums being a chain of dependent operations, and
+// kXgReal CTAs per chunk so that every entry has its own thread (those of the
+// 2 x 2 form took four entries in turn and set the kernel's length).  Products
+// of the first two Grams are symmetric, and formed for s <= u only there.
+constexpr int kXgThreads = 128;
+// CTAs per chunk of a real slice, and the grid's x extent: the slices, then the
+// further CTAs of the real ones.
+__host__ __device__ inline int xg_real_ctas(int r) { return (r * r + kXgThreads - 1) / kXgThreads; }
+__host__ __device__ inline int xg_grid_x(int S, int n3, int r) {
+  return S + (xg_real_ctas(r) - 1) * ((n3 % 2 == 0 && n3 > 1) ? 2 : 1);
+}
+constexpr int xg_pitch(int rp) { return rp + 2; }  // complex values per row: 16-byte rows, few staging conflicts
+
+template <typename T, int RP>
+__global__ void __launch_bounds__(kXgThreads) k_xg(Dev<T> d) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (converged(d)) return;
-  const int k = blockIdx.x, c = blockIdx.y, n1 = d.n1, r = d.r, rr = r * r;
-  const int tid = threadIdx.x, i0 = c * kXgRows;
-  cx<T>* gx = reinterpret_cast<cx<T>*>(smem);  // [r][kXgLd] rows i0 .. i0 + kXgRows of X~'
-  cx<T>* go = gx + (size_t)r * kXgLd;          // [r][kXgLd] rows i0 .. of X~' - X~
+  constexpr int LD = xg_pitch(RP);
+  const int n1 = d.n1, r = d.r, rr = r * r, S = d.S, tid = threadIdx.x;
+  const int c = blockIdx.y, i0 = c * kXgRows;
+  int k = blockIdx.x, part = 0;
+  if (k >= S) {  // further CTAs of the real slices
+    const int np = xg_real_ctas(r) - 1, e = k - S;
+    part = 1 + e % np;
+    k = (e / np == 0) ? 0 : S - 1;
+  }
+  cx<T>* gx = reinterpret_cast<cx<T>*>(smem);  // [kXgRows + 1][LD] rows i0 .. i0 + kXgRows of X~'
+  cx<T>* go = gx + (kXgRows + 1) * LD;         // [kXgRows][LD] rows i0 .. of X~' - X~
   // k_xbc left X~' in d.Xt and X~' - X~ in d.Tb when P = I, else X~' in d.Tb
   const bool inplace = d.certA[k] != 0;
   const cx<T>* Xp = (inplace ? d.Xt : d.Tb) + (size_t)k * r * n1;
   const cx<T>* X2 = (inplace ? d.Tb : d.Xt) + (size_t)k * r * n1;
   const int nrow = min(kXgRows + 1, n1 - i0);
-  for (int e = tid; e < r * kXgLd; e += blockDim.x) {
-    const int s = e / kXgLd, ii = e - s * kXgLd;
-    if (ii < nrow) {
-      const cx<T> xp = Xp[(size_t)s * n1 + i0 + ii];
-      gx[e] = xp;
-      if (ii < kXgRows) go[e] = inplace ? X2[(size_t)s * n1 + i0 + ii] : xp - X2[(size_t)s * n1 + i0 + ii];
+  const int w = tid >> 5, lane = tid & 31;
+#pragma unroll 4
+  for (int s = w; s < RP; s += kXgThreads / 32)
+    for (int ii = lane; ii < kXgRows + 1; ii += 32) {
+      cx<T> xp = {T(0), T(0)}, dx = {T(0), T(0)};
+      if (s < r && ii < nrow) {
+        xp = Xp[(size_t)s * n1 + i0 + ii];
+        if (ii < kXgRows) dx = inplace ? X2[(size_t)s * n1 + i0 + ii] : xp - X2[(size_t)s * n1 + i0 + ii];
+      }
+      gx[ii * LD + s] = xp;
+      if (ii < kXgRows) go[ii * LD + s] = dx;
     }
-  }
   __syncthreads();
   const int iend = min(kXgRows, n1 - i0);
   cx<T>* out = d.Gpart + ((size_t)k * d.gch + c) * 3 * rr;
   const bool realslice = (k == 0) || (2 * k == d.n3);
   if (realslice) {
-    for (int task = tid; task < rr; task += blockDim.x) {
-      const int s = task / r, u = task - s * r;
-      const cx<T>* xs = gx + s * kXgLd;
-      const cx<T>* xu = gx + u * kXgLd;
-      const cx<T>* ou = go + u * kXgLd;
-      T s0 = T(0), c0 = T(0), s1 = T(0), c1 = T(0), s2 = T(0), c2 = T(0);
-      for (int ii = 0; ii < iend; ++ii) {
-        const T a = xs[ii].re, b = xu[ii].re;
+    const int task = part * kXgThreads + tid;
+    if (task >= rr) return;
+    const int s = task / r, u = task - s * r;
+    T s0 = T(0), c0 = T(0), s1 = T(0), c1 = T(0), s2 = T(0), c2 = T(0);
+    for (int ii = 0; ii < iend; ++ii) {
+      const T a = gx[ii * LD + s].re, b = gx[ii * LD + u].re;
+      dot2(s2, c2, a, go[ii * LD + u].re);
+      if (s <= u) {
         dot2(s0, c0, a, b);
-        dot2(s2, c2, a, ou[ii].re);
-        if (i0 + ii + 1 < n1) dot2(s1, c1, a - xs[ii + 1].re, b - xu[ii + 1].re);
+        if (i0 + ii + 1 < n1) dot2(s1, c1, a - gx[(ii + 1) * LD + s].re, b - gx[(ii + 1) * LD + u].re);
       }
-      out[task] = cx<T>{s0, c0};
-      out[rr + task] = cx<T>{s1, c1};
-      out[2 * rr + task] = cx<T>{s2, c2};
+    }
+    out[2 * rr + task] = cx<T>{s2, c2};
+    if (s <= u) {
+      out[task] = out[u * r + s] = cx<T>{s0, c0};
+      out[rr + task] = out[rr + u * r + s] = cx<T>{s1, c1};
     }
     return;
   }
-  // a thread takes the pairs {s0, s0 + rb} x {u0, u0 + rb} (rb = ceil(r / 2)):
-  // 10 loads per row feed 12 products, and consecutive threads (consecutive
-  // u0) read consecutive rows of odd pitch, so a half-warp hits distinct banks
-  const int rb = (r + 1) / 2;
-  for (int blk = tid; blk < rb * rb; blk += blockDim.x) {
-    const int s0 = blk / rb, u0 = blk % rb;
-    const int s1 = min(s0 + rb, r - 1), u1 = min(u0 + rb, r - 1);
-    const cx<T>* xs[2] = {gx + s0 * kXgLd, gx + s1 * kXgLd};
-    const cx<T>* xu[2] = {gx + u0 * kXgLd, gx + u1 * kXgLd};
-    const cx<T>* ou[2] = {go + u0 * kXgLd, go + u1 * kXgLd};
-    cx<T> a0[2][2], hh[2][2], dd[2][2];
+  constexpr int TS = RP == 32 ? 4 : 2;             // rows s of a tile (r <= 16: 64 tiles of 2 x 2)
+  constexpr int NU = RP / 2, NT = (RP / TS) * NU;  // threads of the tiles
+  static_assert(NT <= kXgThreads, "one pass");
+  if (tid >= NT) return;
+  const int s0 = TS * (tid / NU), u0 = 2 * (tid % NU);
+  if (s0 >= r || u0 >= r) return;
+  cx<T> a0[TS][2], hh[TS][2], dd[TS][2], a[TS], b[2];
 #pragma unroll
-    for (int x = 0; x < 2; ++x)
+  for (int x = 0; x < TS; ++x) {
+    a[x] = gx[s0 + x];
 #pragma unroll
-      for (int y = 0; y < 2; ++y) a0[x][y] = hh[x][y] = dd[x][y] = cx<T>{T(0), T(0)};
-    for (int ii = 0; ii < iend; ++ii) {
-      const bool nb = i0 + ii + 1 < n1;
-      cx<T> a[2], da[2], b[2], db[2], e[2];
+    for (int y = 0; y < 2; ++y) a0[x][y] = hh[x][y] = dd[x][y] = cx<T>{T(0), T(0)};
+  }
 #pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        a[x] = xs[x][ii];
-        da[x] = nb ? a[x] - xs[x][ii + 1] : cx<T>{T(0), T(0)};
-        b[x] = xu[x][ii];
-        db[x] = nb ? b[x] - xu[x][ii + 1] : cx<T>{T(0), T(0)};
-        e[x] = ou[x][ii];
-      }
+  for (int y = 0; y < 2; ++y) b[y] = gx[u0 + y];
+  for (int ii = 0; ii < iend; ++ii) {
+    const bool nb = i0 + ii + 1 < n1;  // (row n1 is staged as zero)
+    const cx<T>* nx = gx + (ii + 1) * LD;
+    cx<T> an[TS], bn[2], e[2];
 #pragma unroll
-      for (int x = 0; x < 2; ++x)
+    for (int x = 0; x < TS; ++x) an[x] = nx[s0 + x];
 #pragma unroll
-        for (int y = 0; y < 2; ++y) {
-          cfmaconj(a0[x][y], a[x], b[y]);
-          cfmaconj(dd[x][y], a[x], e[y]);
-          cfmaconj(hh[x][y], da[x], db[y]);
-        }
+    for (int y = 0; y < 2; ++y) {
+      bn[y] = nx[u0 + y];
+      e[y] = go[ii * LD + u0 + y];
     }
 #pragma unroll
-    for (int x = 0; x < 2; ++x)
+    for (int x = 0; x < TS; ++x)
 #pragma unroll
       for (int y = 0; y < 2; ++y) {
-        const int s = s0 + x * rb, u = u0 + y * rb;
-        if (s < r && u < r) {
-          const int task = s * r + u;
-          out[task] = a0[x][y];
-          out[rr + task] = hh[x][y];
-          out[2 * rr + task] = dd[x][y];
-        }
+        cfmaconj(a0[x][y], a[x], b[y]);
+        cfmaconj(dd[x][y], a[x], e[y]);
       }
+    if (nb) {
+#pragma unroll
+      for (int x = 0; x < TS; ++x)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) cfmaconj(hh[x][y], a[x] - an[x], b[y] - bn[y]);
+    }
+#pragma unroll
+    for (int x = 0; x < TS; ++x) a[x] = an[x];
+#pragma unroll
+    for (int y = 0; y < 2; ++y) b[y] = bn[y];
   }
+#pragma unroll
+  for (int x = 0; x < TS; ++x)
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      const int s = s0 + x, u = u0 + y;
+      if (s < r && u < r) {
+        const int task = s * r + u;
+        out[task] = a0[x][y];
+        out[rr + task] = hh[x][y];
+        out[2 * rr + task] = dd[x][y];
+      }
+    }
 }
 
 // Sums of the k_xg partials of one Gram entry in chunk order.  FP32 engines:

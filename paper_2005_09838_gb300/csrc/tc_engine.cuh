@@ -43,8 +43,7 @@ template <typename T, bool STAGED>
 inline SlabFn<T> pick_slab_g_st(int mode, int tl) {
   if (mode == MODE_W) return k_slab_g<T, MODE_W, 4, STAGED>;
   if (mode == MODE_R) return k_slab_g<T, MODE_R, 4, STAGED>;
-  return tl == 2 ? k_slab_g<T, MODE_ITER, 2, STAGED>
-                 : tl == 4 ? k_slab_g<T, MODE_ITER, 4, STAGED> : k_slab_g<T, MODE_ITER, 8, STAGED>;
+  return tl == 2 ? k_slab_g<T, MODE_ITER, 2, STAGED> : k_slab_g<T, MODE_ITER, 4, STAGED>;
 }
 template <typename T>
 inline SlabFn<T> pick_slab_g(int mode, int tl, bool staged) {
@@ -151,6 +150,15 @@ inline XFn<T> pick_xstep(int rp) {
   }
 }
 
+// Whether the contractions run in k_gemm.cuh.  At r <= 8 the fused Y-step reads
+// R~ and writes Z~ in one kernel, but its S ceil(n2/64) CTAs each walk all of n1:
+// it keeps short slices in a grid that covers the SMs (us per iteration, fused
+// against tiled: 144x288x168 r = 5 109/119, r = 8 126/125; 200x288x168 r = 8
+// 196/184; 100x100x60 r = 8 62/54; 900x150x90 r = 8 335/261).
+inline bool gemm_pays(int rp, int S, int n1, int n2) {
+  return rp > 8 || (rp == 8 && (n1 >= 192 || S * ((n2 + 63) / 64) < 152));
+}
+
 // Tensor-core Q contraction of the precision form (TC_TF32 / TC_BF16 over
 // FP32 data, r > 16): the kernel and its dynamic shared memory, or nullptr
 // where it is not built (FP64 data).
@@ -170,6 +178,14 @@ struct TcKernels {
 };
 template <typename T>
 bool pick_tc(int precision, bool split, TcKernels<T>& k);
+// Register-tiled contractions of the plain form (k_gemm.cuh); false where they
+// are not built (FP64 data).
+template <typename T>
+bool pick_gemm(int rp, int r, TcKernels<T>& k);
+template <>
+bool pick_gemm<float>(int rp, int r, TcKernels<float>& k);
+template <>
+bool pick_gemm<double>(int rp, int r, TcKernels<double>& k);
 template <>
 bool pick_tc<float>(int precision, bool split, TcKernels<float>& k);
 template <>
@@ -260,23 +276,20 @@ class Engine final : public EngineBase {
 
     // ---- kernel variants and shared memory -------------------------------------------
     SlabCfg<T> cfg{};
-    specialised_ = pick_slab<T>(n2_, n3_, optin, p.precision == TC_BF16, cfg);
+    specialised_ = pick_slab<T>(n2_, n3_, optin, p.precision == TC_BF16 && rp_ == 32, cfg);
     d_.scratch = nullptr;
     if (specialised_) {
       for (int m = 0; m < 3; ++m) slab_[m] = cfg.f[m];
       slab_threads_ = cfg.threads;
       slab_smem_ = cfg.smem;
       slabs_in_smem_ = true;
-    } else if (SlabGPlan gp; p.precision != TC_BF16 && slab_g_plan<T>(n2_, n3_, optin, gp)) {
+    } else if (SlabGPlan gp; !(p.precision == TC_BF16 && rp_ == 32) && slab_g_plan<T>(n2_, n3_, optin, gp)) {
       folded_ = true;
       d_.fold_sg = gp.sg;
       for (int m = 0; m < 3; ++m) slab_[m] = pick_slab_g<T>(m, n3_ == 7 ? 2 : 4, gp.sg > 0);
       slab_smem_ = gp.smem;
       slab_threads_ = gp.threads;
       slabs_in_smem_ = true;
-      fold_ = alloc<cx<T>>(fold_table_entries(n3_), err);
-      if (!err.empty()) return TC_ERR_NOMEM;
-      d_.fold = fold_;
     } else {
       slab_table<T>(slab_);
       slab_threads_ = kSlabThreads;
@@ -292,6 +305,14 @@ class Engine final : public EngineBase {
     }
     for (int m = 0; m < 3; ++m)
       TC_CUDA_TRY(allow_dynamic_smem((const void*)slab_[m], slab_smem_));
+    // folded transforms: the slab's, and the factors' where they fit
+    fold_factors_ = fold_dft_fits<T>(n3_, optin);
+    if (folded_ || fold_factors_) {
+      fold_ = alloc<cx<T>>(fold_table_entries(n3_), err);
+      if (!err.empty()) return TC_ERR_NOMEM;
+      d_.fold = fold_;
+    }
+    if (fold_factors_) TC_CUDA_TRY(allow_fold_dft<T>(n3_));
 
     // precision form: r x r solves in FP64, contractions on the tensor cores for r > 16
     mixed_ = p.precision == TC_TF32 || p.precision == TC_BF16;
@@ -316,7 +337,7 @@ class Engine final : public EngineBase {
     const size_t xa_bytes = (s64 || sizeof(T) == 4) ? xa_smem_bytes<double>(r_) : xa_smem_bytes<T>(r_);
     xsplit_ = (sizeof(T) == 4 ? rp_ >= 16 : rp_ == 32) && xbc_smem_bytes<T>(n1_) <= (size_t)optin &&
               xbg_smem_bytes<T>(r_) <= (size_t)optin &&
-              xa_bytes <= (size_t)optin && xg_smem_bytes<T>(r_) <= (size_t)optin;
+              xa_bytes <= (size_t)optin && xg_smem_bytes<T>(rp_) <= (size_t)optin;
     // one-CTA X-step: A^+ of the next X-step formed by k_xa on a graph branch after
     // each Y-step (beside Z~ synthesis and the slab kernel), off the critical path
     apre_ = !xsplit_ && xa_bytes <= (size_t)optin;
@@ -348,12 +369,13 @@ class Engine final : public EngineBase {
       xc_fn_ = s64 ? k_xc<T, double> : k_xc<T, T>;
       xbg_smem_ = xbg_smem_bytes<T>(r_);
       xbc_smem_ = xbc_smem_bytes<T>(n1_);
-      xg_smem_ = xg_smem_bytes<T>(r_);
+      xg_smem_ = xg_smem_bytes<T>(rp_);
       TC_CUDA_TRY(allow_dynamic_smem((const void*)xa_fn_, xa_smem_));
       TC_CUDA_TRY(allow_dynamic_smem((const void*)xc_fn_, xa_smem_));
       TC_CUDA_TRY(allow_dynamic_smem((const void*)k_xbg<T>, xbg_smem_));
       TC_CUDA_TRY(allow_dynamic_smem((const void*)k_xbc<T>, xbc_smem_));
-      TC_CUDA_TRY(allow_dynamic_smem((const void*)k_xg<T>, xg_smem_));
+      xg_fn_ = rp_ == 32 ? k_xg<T, 32> : k_xg<T, 16>;
+      TC_CUDA_TRY(allow_dynamic_smem((const void*)xg_fn_, xg_smem_));
     }
     ystep_smem_ = ystep_smem_bytes<T>(n1_, r_, rp_, ycw_);
     d_.yx_global = ystep_smem_ > (size_t)optin ? 1 : 0;
@@ -363,25 +385,38 @@ class Engine final : public EngineBase {
     qcon_smem_ = qcon_smem_bytes<T>(n2_, r_, rp_);
     qcon_shape<T>(S_, n1_, rp_, d_.qrows, qthreads_);
     qgrid_ = dim3(S_, (n1_ + d_.qrows - 1) / d_.qrows);
+    int nsm = 0;
+    TC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device_));
     if (mixed_ && rp_ == 32 && pick_tc<T>(p.precision, (p.flags & TC_FLAG_SINGLE_PASS) == 0, tck_)) {
       tcy_ = true;
-      qcon_ = tck_.qcon;
-      qcon_smem_ = tck_.qsm;
       qgrid_ = dim3(S_, (n1_ + 127) / 128);
       qthreads_ = 256;
-      ystep_ = k_ystep<T, 32, true>;
-      ystep_smem_ = ystep_smem_bytes<T>(n1_, r_, rp_, 32, false, true);
       // split the n1 reduction of D so that the grid covers the SMs about twice
-      int nsm = 0;
-      TC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device_));
       const int ntj = (n2_ + 127) / 128;
       ksplit_ = std::max(1, std::min((2 * nsm + S_ * ntj - 1) / (S_ * ntj), (n1_ + 31) / 32));
+      dgrid_ = dim3(S_, ntj, ksplit_);
+      dthreads_ = 256;
+      zgrid_ = dim3(S_, (n1_ + 127) / 128, (n2_ + 63) / 64);
+    } else if (gemm_pays(rp_, S_, n1_, n2_) && pick_gemm<T>(rp_, r_, tck_)) {
+      tcy_ = true;
+      qgrid_ = dim3(S_, (n1_ + kGmTile - 1) / kGmTile);
+      qthreads_ = kGmThreads;
+      ksplit_ = dcon_f_split(S_, n1_, n2_, nsm);
+      dgrid_ = dim3(S_, (n2_ + kGmTile - 1) / kGmTile, ksplit_);
+      dthreads_ = kGmThreads;
+      zgrid_ = dim3(S_, (n1_ + kGmTile - 1) / kGmTile, (n2_ + kGmTile - 1) / kGmTile);
+    }
+    if (tcy_) {
+      qcon_ = tck_.qcon;
+      qcon_smem_ = tck_.qsm;
+      ystep_ = rp_ == 8 ? k_ystep<T, 8, true> : rp_ == 16 ? k_ystep<T, 16, true> : k_ystep<T, 32, true>;
+      ystep_smem_ = ystep_smem_bytes<T>(n1_, r_, rp_, 32, false, true);
       d_.ksplit = ksplit_;
       Dpart_ = alloc<cx<T>>((size_t)S_ * ksplit_ * r_ * n2_, err);
       if (!err.empty()) return TC_ERR_NOMEM;
       d_.Dpart = Dpart_;
       if (tck_.dsm > (size_t)optin || tck_.zsm > (size_t)optin) {
-        err = "shared memory of the tensor-core kernels exceeds the device limit";
+        err = "shared memory of the contraction kernels exceeds the device limit";
         return TC_ERR_UNSUPPORTED;
       }
       TC_CUDA_TRY(allow_dynamic_smem((const void*)tck_.dcon, tck_.dsm));
@@ -489,17 +524,19 @@ class Engine final : public EngineBase {
       }
     }
     k_pack<T><<<pack_grid(n1_, n2_, n3_), kTileThreads, 0, stream_>>>(dG, dM, Gint, maskbits, n1_, n2_, n3_, mw_);
-    const int fgrid = 4 * 152;
-    k_factor_dft<T><<<fgrid, 256, 0, stream_>>>(dY, Yt, n2_, r_, n3_, 1, twg);
+    if (fold_) k_fold_tables<T><<<2 * 152, 256, 0, stream_>>>(fold_, twg, n3_);
+    // (TC_BF16 at r > 16 keeps the former rounding of the start, see kTL)
+    const cx<T>* ffold = fold_factors_ && !(p.precision == TC_BF16 && rp_ == 32) ? fold_ : nullptr;
+    launch_factor_dft<T>(dY, Yt, ffold, twg, n2_, r_, n3_, 1, stream_);
     if (dX) {
-      k_factor_dft<T><<<fgrid, 256, 0, stream_>>>(dX, Xt, n1_, r_, n3_, 0, twg);
+      launch_factor_dft<T>(dX, Xt, ffold, twg, n1_, r_, n3_, 0, stream_);
+      TC_CUDA_TRY(launch_synth(stream_));  // Z~0 = X~0 Y~0
     } else {
-      cudaMemsetAsync(Xt, 0, nx * sizeof(cx<T>), stream_);
+      TC_CUDA_TRY(cudaMemsetAsync(Xt, 0, nx * sizeof(cx<T>), stream_));
+      TC_CUDA_TRY(cudaMemsetAsync(Zt, 0, (size_t)n1_ * S_ * n2_ * sizeof(cx<T>), stream_));
     }
-    k_synth_init<T><<<fgrid, 256, 0, stream_>>>(d_);                    // Z~0 = X~0 Y~0
     k_gram_tiles<T><<<dim3(S_, ytiles), 256, 0, stream_>>>(d_);         // A of the first X-step
     if (xsplit_ || apre_) xa_fn_<<<S_, xa_threads_, xa_smem_, stream_>>>(d_);  // its A^+
-    if (folded_) k_fold_tables<T><<<2 * 152, 256, 0, stream_>>>(fold_, twg, n3_);
     if (!specialised_ && !(folded_ && n3_ == 7)) {  // (four rows and slices: nothing to choose)
       // tile of the generic transform for this shape: each candidate runs the
       // initial slab pass (it only depends on G and Z~0, so every run writes the
@@ -653,9 +690,9 @@ class Engine final : public EngineBase {
         launch_slab(MODE_W, dW, 0, stream_, SLAB_NOSUM);
       }
     }
-    const int fgrid = 4 * 152;
-    if (dXo) k_factor_idft<T><<<fgrid, 256, 0, stream_>>>(d_.Xt, dXo, n1_, r_, n3_, 0, d_.twg);
-    if (dYo) k_factor_idft<T><<<fgrid, 256, 0, stream_>>>(d_.Yt, dYo, n2_, r_, n3_, 1, d_.twg);
+    const cx<T>* ffold = fold_factors_ ? fold_ : nullptr;
+    if (dXo) launch_factor_idft<T>(d_.Xt, dXo, ffold, d_.twg, n1_, r_, n3_, 0, stream_);
+    if (dYo) launch_factor_idft<T>(d_.Yt, dYo, ffold, d_.twg, n2_, r_, n3_, 1, stream_);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && !on_device) {
       if (W) e = cudaMemcpyAsync(W, dW, N * sizeof(T), cudaMemcpyDeviceToHost, stream_);
@@ -848,9 +885,9 @@ class Engine final : public EngineBase {
     TC_CUDA_TRY(cudaEventCreate(&e0));
     TC_CUDA_TRY(cudaEventCreate(&e1));
     float best = 1e30f;
-    int pick = 1;
+    int pick = 0;
     cudaError_t e = cudaSuccess;
-    for (int c = 0; c < 3 && e == cudaSuccess; ++c) {
+    for (int c = 0; c < (folded_ ? 2 : 3) && e == cudaSuccess; ++c) {
       slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[c]);
       e = allow_dynamic_smem((const void*)slab_[MODE_ITER], slab_smem_);
       float ms = 1e30f;
@@ -884,6 +921,13 @@ class Engine final : public EngineBase {
   void launch_slab(int mode, T* Wout, int init, cudaStream_t s, int flags = 0) {
     slab_[mode]<<<n1_, slab_threads_, slab_smem_, s>>>(d_, Wout, flags | (slabs_in_smem_ ? SLAB_IN_SMEM : 0), init);
   }
+  cudaError_t launch_synth(cudaStream_t s) {
+    const size_t sm = zsyn_f_smem<T>(r_);
+    const cudaError_t e = allow_dynamic_smem((const void*)k_zsyn_f<T>, sm);
+    if (e != cudaSuccess) return e;
+    k_zsyn_f<T><<<dim3(S_, (n1_ + kGmTile - 1) / kGmTile, (n2_ + kGmTile - 1) / kGmTile), kGmZThreads, sm, s>>>(d_);
+    return cudaGetLastError();
+  }
   void launch_qcon(cudaStream_t s) { qcon_<<<qgrid_, qthreads_, qcon_smem_, s>>>(d_, Q_); }
   // With the four-kernel X-step, A^+ (k_xa) is formed after every change of Y~
   // (initialisation, Y-step), so the X-step starts with it in place.
@@ -891,7 +935,7 @@ class Engine final : public EngineBase {
     if (xsplit_) {
       k_xbg<T><<<dim3(S_, (n1_ + kXbRows - 1) / kXbRows), 256, xbg_smem_, s>>>(d_, Q_);
       k_xbc<T><<<dim3(S_, (r_ + 7) / 8), 256, xbc_smem_, s>>>(d_);
-      k_xg<T><<<dim3(S_, gch_), 256, xg_smem_, s>>>(d_);
+      xg_fn_<<<dim3(xg_grid_x(S_, n3_, r_), gch_), kXgThreads, xg_smem_, s>>>(d_);
       xc_fn_<<<S_, kXaThreads, xa_smem_, s>>>(d_);
       return;
     }
@@ -904,7 +948,7 @@ class Engine final : public EngineBase {
   bool launch_ystep(cudaStream_t s, cudaStream_t branch = nullptr, bool with_xa = true) {
     const int tw = ystep_tw(rp_, ycw_);
     dim3 g(S_, (n2_ + tw - 1) / tw);
-    if (tcy_) tck_.dcon<<<dim3(S_, (n2_ + 127) / 128, ksplit_), 256, tck_.dsm, s>>>(d_);
+    if (tcy_) tck_.dcon<<<dgrid_, dthreads_, tck_.dsm, s>>>(d_);
     ystep_<<<g, kYThreads, ystep_smem_, s>>>(d_);
     bool forked = false;
     if ((xsplit_ || apre_) && with_xa) {
@@ -916,7 +960,7 @@ class Engine final : public EngineBase {
         xa_fn_<<<S_, xa_threads_, xa_smem_, s>>>(d_);
       }
     }
-    if (tcy_) tck_.zsyn<<<dim3(S_, (n1_ + 127) / 128, (n2_ + 63) / 64), 256, tck_.zsm, s>>>(d_);
+    if (tcy_) tck_.zsyn<<<zgrid_, 256, tck_.zsm, s>>>(d_);
     return forked;
   }
 
@@ -980,6 +1024,7 @@ class Engine final : public EngineBase {
   bool poisoned_ = false;
   bool specialised_ = false;
   bool folded_ = false;  // folded-transform slab kernels (k_slab_g)
+  bool fold_factors_ = false;  // the factors' transforms too
   cx<T>* fold_ = nullptr;
   T* wrows_ = nullptr;   // W in row-major order (allocated by the first read-back)
   bool slabs_in_smem_ = true;
@@ -993,12 +1038,14 @@ class Engine final : public EngineBase {
   cx<T>* rscr_ = nullptr;
   size_t rank_smem_ = 0;
   int xa_threads_ = kXaThreads;
-  YFn<T> xa_fn_ = nullptr, xc_fn_ = nullptr;
+  YFn<T> xa_fn_ = nullptr, xc_fn_ = nullptr, xg_fn_ = nullptr;
   int gch_ = 0;
   size_t xa_smem_ = 0, xbg_smem_ = 0, xbc_smem_ = 0, xg_smem_ = 0;
   cudaStream_t aux_stream_ = nullptr;  // graph branch of k_xa during capture
   cudaEvent_t ev_fork_ = nullptr, ev_join_ = nullptr;
-  bool tcy_ = false;  // tensor-core Y-step (D partials, update, Z~ synthesis)
+  bool tcy_ = false;  // Y-step in three kernels (D partials, update, Z~ synthesis)
+  dim3 dgrid_, zgrid_;
+  int dthreads_ = 256;
   TcKernels<T> tck_;
   int ksplit_ = 1;
   int ycw_ = 32;  // lanes per row group of k_ystep

@@ -43,6 +43,18 @@ bool pick_tc<float>(int precision, bool split, TcKernels<float>& k) {
   return false;
 }
 
+template <>
+bool pick_gemm<float>(int rp, int r, TcKernels<float>& k) {
+  k.zsyn = k_zsyn_f<float>;
+  k.zsm = zsyn_f_smem<float>(r);
+  switch (rp) {
+    case 8: k.qcon = k_qcon_f<8>, k.dcon = k_dcon_f<8>, k.qsm = qcon_f_smem<8>(), k.dsm = dcon_f_smem<8>(); return true;
+    case 16: k.qcon = k_qcon_f<16>, k.dcon = k_dcon_f<16>, k.qsm = qcon_f_smem<16>(), k.dsm = dcon_f_smem<16>(); return true;
+    case 32: k.qcon = k_qcon_f<32>, k.dcon = k_dcon_f<32>, k.qsm = qcon_f_smem<32>(), k.dsm = dcon_f_smem<32>(); return true;
+    default: return false;
+  }
+}
+
 EngineBase* make_engine_f32() { return new Engine<float>(); }
 
 }  // namespace tc

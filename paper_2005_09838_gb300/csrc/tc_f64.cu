@@ -13,6 +13,11 @@ bool pick_tc<double>(int, bool, TcKernels<double>&) {
   return false;
 }
 
+template <>
+bool pick_gemm<double>(int, int, TcKernels<double>&) {
+  return false;
+}
+
 EngineBase* make_engine_f64() { return new Engine<double>(); }
 
 }  // namespace tc

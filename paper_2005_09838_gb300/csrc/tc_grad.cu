@@ -27,6 +27,8 @@ inline int grad_pad_rank(int r) { return r <= 2 ? 2 : r <= 4 ? 4 : r <= 8 ? 8 : 
 
 template <typename T>
 using GFn = void (*)(Dev<T>, cx<T>*);
+template <typename T>
+using GDFn = void (*)(Dev<T>);
 
 template <typename T>
 GFn<T> pick_dcon(int rp) {
@@ -177,26 +179,53 @@ struct GradEngine final : tc_grad {
       d_.scratch = scratch;
     }
     cx<T>* fold = nullptr;
-    if (slab_.folded) {
+    const bool fold_factors = fold_dft_fits<T>(n3_, optin);
+    if (slab_.folded || fold_factors) {
       fold = alloc<cx<T>>(fold_table_entries(n3_), err);
       if (!err.empty()) return TC_ERR_NOMEM;
       d_.fold = fold;
       d_.fold_sg = slab_.sg;
     }
+    if (fold_factors) {
+      TCG_TRY(allow_fold_dft<T>(n3_));
+      ffold_ = fold;
+    }
     TCG_TRY(allow_dynamic_smem((const void*)slab_.f, slab_.smem));
-    qcon_ = pick_qcon_g<T>(rp_);
-    dcon_ = pick_dcon<T>(rp_);
-    qcon_shape<T>(S_, n1_, rp_, d_.qrows, qthreads_);
-    qsmem_ = qcon_smem_bytes<T>(n2_, r_, rp_);
-    dsmem_ = dcon_smem_bytes<T>(n1_, r_, rp_);
-    d_.yx_global = dsmem_ > (size_t)optin ? 1 : 0;
-    if (d_.yx_global) dsmem_ = dcon_smem_bytes<T>(n1_, r_, rp_, false);
+    zsmem_ = zsyn_f_smem<T>(r_);
+    TCG_TRY(allow_dynamic_smem((const void*)k_zsyn_f<T>, zsmem_));
+    if (sizeof(T) == 4 && rp_ >= 8) {
+      if constexpr (sizeof(T) == 4) {
+        int nsm = 0;
+        TCG_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device));
+        d_.ksplit = dcon_f_split(S_, n1_, n2_, nsm);
+        dgrid_ = dim3(S_, (n2_ + kGmTile - 1) / kGmTile, d_.ksplit);
+        d_.Dpart = alloc<cx<T>>((size_t)S_ * d_.ksplit * r_ * n2_, err);
+        if (!err.empty()) return TC_ERR_NOMEM;
+        qgrid_ = dim3(S_, (n1_ + kGmTile - 1) / kGmTile);
+        qthreads_ = kGmThreads;
+        switch (rp_) {
+          case 8: qcon_ = k_qcon_f<8>, dpart_ = k_dcon_f<8>, qsmem_ = qcon_f_smem<8>(), dsmem_ = dcon_f_smem<8>(); break;
+          case 16: qcon_ = k_qcon_f<16>, dpart_ = k_dcon_f<16>, qsmem_ = qcon_f_smem<16>(), dsmem_ = dcon_f_smem<16>(); break;
+          default: qcon_ = k_qcon_f<32>, dpart_ = k_dcon_f<32>, qsmem_ = qcon_f_smem<32>(), dsmem_ = dcon_f_smem<32>();
+        }
+        TCG_TRY(allow_dynamic_smem((const void*)dpart_, dsmem_));
+      }
+    } else {
+      qcon_ = pick_qcon_g<T>(rp_);
+      dcon_ = pick_dcon<T>(rp_);
+      qcon_shape<T>(S_, n1_, rp_, d_.qrows, qthreads_);
+      qgrid_ = dim3(S_, (n1_ + d_.qrows - 1) / d_.qrows);
+      qsmem_ = qcon_smem_bytes<T>(n2_, r_, rp_);
+      dsmem_ = dcon_smem_bytes<T>(n1_, r_, rp_);
+      d_.yx_global = dsmem_ > (size_t)optin ? 1 : 0;
+      if (d_.yx_global) dsmem_ = dcon_smem_bytes<T>(n1_, r_, rp_, false);
+    }
     if (qsmem_ > (size_t)optin || dsmem_ > (size_t)optin) {
       err = "shared memory of the gradient kernels exceeds the device limit for these sizes";
       return TC_ERR_UNSUPPORTED;
     }
     TCG_TRY(allow_dynamic_smem((const void*)qcon_, qsmem_));
-    TCG_TRY(allow_dynamic_smem((const void*)dcon_, dsmem_));
+    if (dcon_) TCG_TRY(allow_dynamic_smem((const void*)dcon_, dsmem_));
 
     std::vector<cx<T>> tw(n3_);
     for (int m = 0; m < n3_; ++m) {
@@ -262,31 +291,30 @@ struct GradEngine final : tc_grad {
       xs = xin_;
       ys = yin_;
     }
-    const int fgrid = 4 * 152;
-    k_factor_dft<T><<<fgrid, 256, 0, stream_>>>(xs, d_.Xt, n1_, r_, n3_, 0, d_.twg);
-    k_factor_dft<T><<<fgrid, 256, 0, stream_>>>(ys, d_.Yt, n2_, r_, n3_, 1, d_.twg);
-    {
-      const size_t tot = (size_t)n1_ * S_ * n2_;
-      k_synth_init<T><<<(unsigned)std::min<size_t>((tot + 255) / 256, 8 * 152), 256, 0, stream_>>>(d_);
-    }
+    launch_factor_dft<T>(xs, d_.Xt, ffold_, d_.twg, n1_, r_, n3_, 0, stream_);
+    launch_factor_dft<T>(ys, d_.Yt, ffold_, d_.twg, n2_, r_, n3_, 1, stream_);
+    k_zsyn_f<T><<<dim3(S_, (n1_ + kGmTile - 1) / kGmTile, (n2_ + kGmTile - 1) / kGmTile), kGmZThreads, zsmem_, stream_>>>(d_);
     slab_.f<<<n1_, slab_.threads, slab_.smem, stream_>>>(d_, nullptr, slab_.in_smem ? 1 : 0, 0);  // R~, ||E||^2
-    if (d_.rho1 != T(0)) k_rho1_term<T><<<dim3(S_, kRhoChunks), 256, 0, stream_>>>(d_);  // ||H Z~_k||^2 from Z~
+    if (d_.rho1 != T(0)) {  // ||H Z~_k||^2, and R~ += rho1 H^T H Z~ where a gradient is wanted
+      if (dX || dY) k_grad_rho1<T, true><<<dim3(S_, kRhoChunks), 256, 0, stream_>>>(d_);
+      else k_grad_rho1<T, false><<<dim3(S_, kRhoChunks), 256, 0, stream_>>>(d_);
+    }
     if (dX || dY) {
-      if (d_.rho1 != T(0)) {
-        // R~ += rho1 H^T H Z~: the contractions below then carry the rho1 term too
-        const size_t tot = (size_t)n1_ * S_ * n2_;
-        k_grad_hth<T><<<(unsigned)std::min<size_t>((tot + 255) / 256, 16 * 152), 256, 0, stream_>>>(d_);
+      if (dX) qcon_<<<qgrid_, qthreads_, qsmem_, stream_>>>(d_, GX_);  // R~Y~^H
+      if (dY && dpart_) {                                              // X~^H R~
+        dpart_<<<dgrid_, kGmThreads, dsmem_, stream_>>>(d_);
+        k_dsum<T><<<dim3((r_ * n2_ + 255) / 256, S_), 256, 0, stream_>>>(d_, GY_);
+      } else if (dY) {
+        dcon_<<<dim3(S_, (n2_ + 31) / 32), kYThreads, dsmem_, stream_>>>(d_, GY_);
       }
-      qcon_<<<dim3(S_, (n1_ + d_.qrows - 1) / d_.qrows), qthreads_, qsmem_, stream_>>>(d_, GX_);  // R~ Y~^H
-      dcon_<<<dim3(S_, (n2_ + 31) / 32), kYThreads, dsmem_, stream_>>>(d_, GY_);     // X~^H R~
       T* ox = static_cast<T*>(dX);
       T* oy = static_cast<T*>(dY);
       if (!on_device) {
         ox = dX ? xin_ : nullptr;
         oy = dY ? yin_ : nullptr;
       }
-      if (ox) k_factor_idft<T><<<fgrid, 256, 0, stream_>>>(GX_, ox, n1_, r_, n3_, 0, d_.twg);
-      if (oy) k_factor_idft<T><<<fgrid, 256, 0, stream_>>>(GY_, oy, n2_, r_, n3_, 1, d_.twg);
+      if (ox) launch_factor_idft<T>(GX_, ox, ffold_, d_.twg, n1_, r_, n3_, 0, stream_);
+      if (oy) launch_factor_idft<T>(GY_, oy, ffold_, d_.twg, n2_, r_, n3_, 1, stream_);
       if (!on_device) {
         if (dX) TCG_TRY(cudaMemcpyAsync(dX, xin_, nx * sizeof(T), cudaMemcpyDeviceToHost, stream_));
         if (dY) TCG_TRY(cudaMemcpyAsync(dY, yin_, ny * sizeof(T), cudaMemcpyDeviceToHost, stream_));
@@ -328,6 +356,10 @@ struct GradEngine final : tc_grad {
   GradSlab<T> slab_;
   GFn<T> qcon_ = nullptr;
   GFn<T> dcon_ = nullptr;
+  GDFn<T> dpart_ = nullptr;  // tiled D (FP32, r > 4)
+  dim3 qgrid_, dgrid_;
+  const cx<T>* ffold_ = nullptr;
+  size_t zsmem_ = 0;
   size_t qsmem_ = 0, dsmem_ = 0;
   int qthreads_ = kSliceThreads;
   cx<T>* GX_ = nullptr;
