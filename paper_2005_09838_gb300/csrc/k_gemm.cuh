@@ -53,8 +53,9 @@ __device__ __forceinline__ void lds_cx4(const cx<double>* p, cx<double> (&v)[4])
 }
 
 // Sums of the KG thread groups, into group 0 (fixed order); red: KG - 1 tiles.
+// pairs: the accumulators are (value, rounding errors) pairs.
 template <int KG>
-__device__ __forceinline__ void group_sum(cx<float> (&acc)[4][4], cx<float>* red, int g, int t, int nt) {
+__device__ __forceinline__ void group_sum(cx<float> (&acc)[4][4], cx<float>* red, int g, int t, int nt, bool pairs) {
   if constexpr (KG > 1) {
     __syncthreads();
     if (g > 0)
@@ -65,7 +66,12 @@ __device__ __forceinline__ void group_sum(cx<float> (&acc)[4][4], cx<float>* red
 #pragma unroll
       for (int q = 1; q < KG; ++q)
 #pragma unroll
-        for (int e = 0; e < 16; ++e) acc[e / 4][e % 4] = acc[e / 4][e % 4] + red[((q - 1) * 16 + e) * nt + t];
+        for (int e = 0; e < 16; ++e) {
+          cx<float>& a = acc[e / 4][e % 4];
+          const cx<float> b = red[((q - 1) * 16 + e) * nt + t];
+          if (pairs) pair_add(a.re, a.im, b.re, b.im);
+          else a = a + b;
+        }
   }
 }
 
@@ -75,14 +81,33 @@ __host__ __device__ constexpr size_t dcon_f_smem() {
   return 2 * (size_t)kGmKC * (kGmTile + RP) * sizeof(cx<float>);
 }
 
-template <int RP>
-__global__ void __launch_bounds__(kGmThreads) k_dcon_f(Dev<float> d) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  if (converged(d)) return;
+// Columns j0 .. j0 + 63 of the partial D of slice k over the z-th of ks ranges of
+// rows, by 128 threads (tid) with dcon_f_smem<RP>() bytes; every thread of the
+// block calls it with the same range.
+//
+// STRIDED: partial w of eight sums the rows i = w mod 8 in increasing order, as the
+// warps of the fused k_ystep do (bit for bit: see Engine::strict_); the thread
+// groups take a partial each in place of sharing one, and z counts the CTAs.
+//
+// Real slices (with d.dpairs): the factors and the residual are real, and D is formed as a
+// compensated sum, (value, rounding errors) in the (re, im) fields.  D of the DC
+// slice is the one sum of the iteration whose rounding matters: it is added to
+// Dg Y~ of nearly the same size, and G^+ multiplies what is left of both by the
+// condition number of the DC Gram.  Rounded to FP32 it alone gave 1.5e-5 of the
+// 1.5e-5 error of X~ and 2.6e-5 of the 2.7e-5 of Y~ after five iterations on
+// 529 x 96 x 112, r = 32; every other sum and stored array together 6e-6.
+constexpr int kDStride = 8;  // partials of the strided form
+template <int RP, bool STRIDED>
+__device__ __forceinline__ void dcon_f_tile(const Dev<float>& d, int k, int j0, int z, int ks, unsigned char* smem,
+                                            int tid) {
   constexpr int SG = GmGroups<RP>::SG, KG = GmGroups<RP>::KG, NTG = 16 * SG;
-  const int k = blockIdx.x, j0 = blockIdx.y * kGmTile, z = blockIdx.z, ks = gridDim.z;
-  const int n1 = d.n1, n2 = d.n2, r = d.r, S = d.S, tid = threadIdx.x;
-  const int per = (n1 + ks - 1) / ks, ib = min(z * per, n1), ie = min(ib + per, n1);
+  const int n1 = d.n1, n2 = d.n2, r = d.r, S = d.S;
+  const bool real = (k == 0 || 2 * k == d.n3) && d.dpairs;
+  const int per = (n1 + ks - 1) / ks;
+  // staged rows ib .. ie - 1; the strided form counts them from 0: kDStride / KG
+  // CTAs share n1 rows, KG of them at a time
+  const int ib = STRIDED ? 0 : min(z * per, n1), ie = STRIDED ? (n1 + kDStride - 1) / kDStride * KG : min(ib + per, n1);
+  auto row_of = [&](int q) { return STRIDED ? kDStride * (q / KG) + z * KG + q % KG : q; };
   cx<float>* Rs = reinterpret_cast<cx<float>*>(smem);        // [2][KC][64]
   cx<float>* Xs = Rs + 2 * kGmKC * kGmTile;                  // [2][KC][RP]
   const int cl = tid & 15, sgi = (tid >> 4) % SG, g = tid / NTG;
@@ -94,24 +119,30 @@ __global__ void __launch_bounds__(kGmThreads) k_dcon_f(Dev<float> d) {
   if (r < RP)
     for (int e = tid; e < 2 * kGmKC * RP; e += kGmThreads)
       if (e % RP >= r) Xs[e] = cx<float>{0.f, 0.f};
+  auto rows_in = [&](int i0) {  // rows of the stage at i0 that exist
+    int nk = min(kGmKC, ie - i0);
+    if (STRIDED)
+      while (nk > 0 && row_of(i0 + nk - 1) >= n1) --nk;
+    return nk;
+  };
   auto stage = [&](int b, int i0) {
-    const int nk = min(kGmKC, ie - i0);
+    const int nk = rows_in(i0);
     cx<float>* rd = Rs + b * kGmKC * kGmTile;
     cx<float>* xd = Xs + b * kGmKC * RP;
     if (vec) {
       for (int e = tid; e < nk * (kGmTile / 2); e += kGmThreads) {
         const int q = e / (kGmTile / 2), c = 2 * (e % (kGmTile / 2));
-        if (c < ncol) cp_async16(rd + q * kGmTile + c, Rb + (size_t)(i0 + q) * rs + c);
+        if (c < ncol) cp_async16(rd + q * kGmTile + c, Rb + (size_t)row_of(i0 + q) * rs + c);
       }
     } else {
       for (int e = tid; e < nk * kGmTile; e += kGmThreads) {
         const int q = e / kGmTile, c = e % kGmTile;
-        if (c < ncol) cp_async_elem(rd + q * kGmTile + c, Rb + (size_t)(i0 + q) * rs + c);
+        if (c < ncol) cp_async_elem(rd + q * kGmTile + c, Rb + (size_t)row_of(i0 + q) * rs + c);
       }
     }
     for (int e = tid; e < r * kGmKC; e += kGmThreads) {
       const int s = e / kGmKC, q = e % kGmKC;
-      if (q < nk) cp_async_elem(xd + q * RP + s, Xb + (size_t)s * n1 + i0 + q);
+      if (q < nk) cp_async_elem(xd + q * RP + s, Xb + (size_t)s * n1 + row_of(i0 + q));
     }
     cp_async_commit();
   };
@@ -130,32 +161,72 @@ __global__ void __launch_bounds__(kGmThreads) k_dcon_f(Dev<float> d) {
     __syncthreads();
     const cx<float>* rd = Rs + b * kGmKC * kGmTile + cl;
     const cx<float>* xd = Xs + b * kGmKC * RP + 4 * sgi;
-    const int nk = min(kGmKC, ie - i0);
+    const int nk = rows_in(i0);
+    if (!STRIDED && real) {
+      // four rows in plain FP32, then one error-free addition: the roundings that
+      // count are those against the whole sum
+      for (int q = g; q < nk; q += 4 * KG) {
+        float p4[4][4];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) p4[e / 4][e % 4] = 0.f;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          const int row = q + w * KG;
+          if (row < nk) {
+            cx<float> x[4];
+            lds_cx4(xd + row * RP, x);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const float v = rd[row * kGmTile + 16 * c].re;
+#pragma unroll
+              for (int p = 0; p < 4; ++p) p4[c][p] = fmaf(x[p].re, v, p4[c][p]);
+            }
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) pair_add(acc[e / 4][e % 4].re, acc[e / 4][e % 4].im, p4[e / 4][e % 4], 0.f);
+      }
+    } else {
 #pragma unroll 4
-    for (int q = g; q < nk; q += KG) {
-      cx<float> x[4], v[4];
-      lds_cx4(xd + q * RP, x);
+      for (int q = g; q < nk; q += KG) {
+        cx<float> x[4], v[4];
+        lds_cx4(xd + q * RP, x);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) v[c] = rd[q * kGmTile + 16 * c];
+        for (int c = 0; c < 4; ++c) v[c] = rd[q * kGmTile + 16 * c];
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+        for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int p = 0; p < 4; ++p) cfmaconj(acc[c][p], x[p], v[c]);
+          for (int p = 0; p < 4; ++p) cfmaconj(acc[c][p], x[p], v[c]);
+      }
     }
     __syncthreads();
   }
-  group_sum<KG>(acc, Rs, g, tid % NTG, NTG);
-  if (g > 0) return;
+  int zp = z;  // partial written
+  if constexpr (STRIDED) {
+    zp = z * KG + g;
+  } else {
+    group_sum<KG>(acc, Rs, g, tid % NTG, NTG, real);
+    if (g > 0) return;
+  }
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
     const int s = 4 * sgi + p;
     if (s >= r) break;
-    cx<float>* o = d.Dpart + (((size_t)k * ks + z) * r + s) * n2 + j0;
+    cx<float>* o = d.Dpart + (((size_t)k * d.ksplit + zp) * r + s) * n2 + j0;
 #pragma unroll
     for (int c = 0; c < 4; ++c)
       if (cl + 16 * c < ncol) o[cl + 16 * c] = acc[c][p];
   }
 }
+
+template <int RP, bool STRIDED = false>
+__global__ void __launch_bounds__(kGmThreads) k_dcon_f(Dev<float> d) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (converged(d)) return;
+  dcon_f_tile<RP, STRIDED>(d, blockIdx.x, blockIdx.y * kGmTile, blockIdx.z, gridDim.z, smem, threadIdx.x);
+}
+
+inline int dcon_f_groups(int rp) { return rp == 8 ? GmGroups<8>::KG : rp == 16 ? GmGroups<16>::KG : GmGroups<32>::KG; }
 
 // Splits of n1: about four CTAs of k_dcon_f per SM, at least 32 rows each.
 inline int dcon_f_split(int S, int n1, int n2, int nsm) {
@@ -228,7 +299,7 @@ __global__ void __launch_bounds__(kGmThreads) k_qcon_f(Dev<float> d, cx<float>* 
     }
     __syncthreads();
   }
-  group_sum<KG>(acc, Rs, g, tid % NTG, NTG);
+  group_sum<KG>(acc, Rs, g, tid % NTG, NTG, false);
   if (g > 0) return;
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
@@ -238,6 +309,71 @@ __global__ void __launch_bounds__(kGmThreads) k_qcon_f(Dev<float> d, cx<float>* 
 #pragma unroll
     for (int c = 0; c < 4; ++c)
       if (rl + 16 * c < nrow) o[rl + 16 * c] = acc[c][p];
+  }
+}
+
+// ---- Q = R~ Y~^H with the lanes along the columns: grid (S, ceil(n1/32)), 256 threads.
+// A warp forms 4 rows x 8 columns of Q, each lane summing the columns j = lane mod
+// 32 in increasing order and the lanes added pairwise (distance 16, 8, .., 1): the
+// order of k_qcon, bit for bit, at 12 loads for 32 complex products where k_qcon
+// has 33 (529 x 96 x 112, r = 32: 53 -> 30 us).
+constexpr int kQlRows = 4, kQlCols = 8;
+template <int RP>
+__global__ void __launch_bounds__(256, 2) k_qcon_l(Dev<float> d, cx<float>* __restrict__ Qout) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (converged(d)) return;
+  constexpr int NS = RP / kQlCols, NR = 8 / NS;  // warps along s, along the rows
+  const int k = blockIdx.x, n1 = d.n1, n2 = d.n2, r = d.r, S = d.S;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  cx<float>* Ys = reinterpret_cast<cx<float>*>(smem);  // [r][n2]
+  const cx<float>* Y = d.Yt + (size_t)k * r * n2;
+  for (int e = tid; e < r * n2; e += 256) cp_async_elem(Ys + e, Y + e);
+  cp_async_wait_all();
+  __syncthreads();
+  const int s0 = (wid % NS) * kQlCols;
+  if (s0 >= r) return;
+  for (int ii = (wid / NS) * kQlRows; ii < 32; ii += NR * kQlRows) {
+    const int i0 = blockIdx.y * 32 + ii;
+    if (i0 >= n1) break;
+    const cx<float>* row[kQlRows];
+#pragma unroll
+    for (int q = 0; q < kQlRows; ++q) row[q] = d.Rt + ((size_t)min(i0 + q, n1 - 1) * S + k) * n2;
+    cx<float> acc[kQlRows][kQlCols], nx[kQlRows];
+#pragma unroll
+    for (int q = 0; q < kQlRows; ++q) {
+      nx[q] = lane < n2 ? ldg_cx(row[q] + lane) : cx<float>{0.f, 0.f};
+#pragma unroll
+      for (int s = 0; s < kQlCols; ++s) acc[q][s] = cx<float>{0.f, 0.f};
+    }
+    for (int j = lane; j < n2; j += 32) {
+      cx<float> v[kQlRows];
+#pragma unroll
+      for (int q = 0; q < kQlRows; ++q) {
+        v[q] = nx[q];
+        if (j + 32 < n2) nx[q] = ldg_cx(row[q] + j + 32);
+      }
+      const cx<float>* yj = Ys + s0 * n2 + j;
+#pragma unroll
+      for (int s = 0; s < kQlCols; ++s) {
+        const cx<float> y = yj[min(s, r - 1 - s0) * n2];
+#pragma unroll
+        for (int q = 0; q < kQlRows; ++q) cfmac(acc[q][s], v[q], y);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < kQlRows; ++q) {
+      float f[2 * kQlCols];
+#pragma unroll
+      for (int s = 0; s < kQlCols; ++s) {
+        f[2 * s] = acc[q][s].re;
+        f[2 * s + 1] = acc[q][s].im;
+      }
+      const float tot = warp_reduce_scatter<float, 2 * kQlCols>(f);
+      const int idx = lane >> 1, s = s0 + idx / 2;
+      if ((lane & 1) == 0 && s < r && i0 + q < n1)
+        reinterpret_cast<float*>(Qout + ((size_t)k * r + s) * n1 + i0 + q)[idx & 1] = tot;
+    }
   }
 }
 
@@ -297,7 +433,7 @@ __global__ void __launch_bounds__(kGmZThreads) k_zsyn_f(Dev<T> d) {
 }
 
 // Sum of the ksplit partials of D (the differentiation form's X~^H R~), real
-// slices with a zero imaginary part.
+// slices from their pairs.
 template <typename T>
 __global__ void __launch_bounds__(256) k_dsum(Dev<T> d, cx<T>* __restrict__ out) {
   const int rn = d.r * d.n2, k = blockIdx.y;
@@ -305,8 +441,12 @@ __global__ void __launch_bounds__(256) k_dsum(Dev<T> d, cx<T>* __restrict__ out)
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < rn; e += gridDim.x * blockDim.x) {
     const cx<T>* p = d.Dpart + (size_t)k * d.ksplit * rn + e;
     cx<T> v = p[0];
-    for (int z = 1; z < d.ksplit; ++z) v = v + p[(size_t)z * rn];
-    if (real) v.im = T(0);
+    for (int z = 1; z < d.ksplit; ++z) {
+      const cx<T> q = p[(size_t)z * rn];
+      if (real) pair_add(v.re, v.im, q.re, q.im);
+      else v = v + q;
+    }
+    if (real) v = cx<T>{v.re + v.im, T(0)};  // (value, rounding errors) pairs
     out[(size_t)k * rn + e] = v;
   }
 }

@@ -31,7 +31,7 @@
 
 namespace tc {
 
-constexpr int kSlabFThreads = 1024;
+constexpr int kSlabFThreads = 512;
 // Items per thread whose global loads are issued together in the first split phase.
 constexpr int kSlabFBatch = 4;
 
@@ -118,10 +118,10 @@ __device__ __forceinline__ cx<T> fwd_split(cx<T> zk, cx<T> zm, int k) {
   return E + cmul(O, fft::tw<T, L, false>(k));
 }
 
-// SEGW: the W-step by wstep_sweeps_seg, bit for bit the sequential sweeps (the
-// TC_BF16 form, see kTL); else one thread per segment (wstep_segments).
-template <typename T, int L, int N1, int N2, int MODE, bool SEGW = false>
-__global__ void __launch_bounds__(SEGW ? kSlabFThreads / 2 : kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
+// The W-step is wstep_sweeps_seg, bit for bit the sequential sweeps
+// (Engine::strict_).
+template <typename T, int L, int N1, int N2, int MODE>
+__global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
   constexpr int M = L / 2;
   static_assert(L % 2 == 0 && M == N1 * N2, "n3 = 2 N1 N2");
   constexpr int LP = slab_f_stride(L);
@@ -303,10 +303,8 @@ __global__ void __launch_bounds__(SEGW ? kSlabFThreads / 2 : kSlabFThreads, 1) k
 
   // ---- W-step ----------------------------------------------------------------------------------
   if (wsolve) {
-    auto col_of = [&](int q) { return buf + q; };
-    // SEGW: rows split into segments so that every thread has one (row, segment)
-    if (SEGW) wstep_sweeps_seg<T>(col_of, LP, msk, stw, L, max(1, nt / L), tid, n2, d.rho2, wtab);
-    else wstep_segments<T, kWSeg<T>>(col_of, LP, msk, L, n2, d.rho2, wtab);
+    // rows split into segments so that every thread has one (row, segment)
+    wstep_sweeps_seg<T>([&](int q) { return buf + q; }, LP, msk, stw, L, max(1, nt / L), tid, n2, d.rho2, wtab);
   }
 
   // ---- C1: forward DFT_N2 over slots N2 k1 + j, twiddle w_M^{k1 q} -----------------------

@@ -1776,17 +1776,20 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
   // real slices of an FP32 engine: t G^+ in FP64 (k_xstep / k_xc), applied in FP64
   const bool realslice = (k == 0) || (2 * k == d.n3);
   const bool g64 = sizeof(T) == 4 && realslice && d.Gp64 != nullptr;
-  // (as FP32 head and tail: the products below are error-free, where an FP64
-  // multiply-add and a conversion per term took the FP64 pipe of the real slices'
-  // CTAs 15 us at r = 32)
-  cx<float>* gh64 = reinterpret_cast<cx<float>*>(smem + ystep_gh64_offset<T>(n1, r, RP, XSH, TCY, CW));
+  // (as FP32 head and tail where D comes as pairs too: the products are error-free,
+  // and an FP64 multiply-add and a conversion per term took the FP64 pipe of the
+  // real slices' CTAs 15 us at r = 32)
+  const bool dreal = g64 && d.dpairs;
+  double* gh64 = reinterpret_cast<double*>(smem + ystep_gh64_offset<T>(n1, r, RP, XSH, TCY, CW));
+  cx<float>* ghp = reinterpret_cast<cx<float>*>(gh64);
   for (int e = tid; e < rr; e += blockDim.x) {
     Dgs[e] = d.Dg[(size_t)k * rr + e];
     Gh[e] = d.Gp[(size_t)k * rr + e];
     if (g64) {
       const double g = d.Gp64[(size_t)(k == 0 ? 0 : 1) * rr + e].re;
       const float h = (float)g;
-      gh64[e] = cx<float>{h, (float)(g - (double)h)};
+      if (dreal) ghp[e] = cx<float>{h, (float)(g - (double)h)};
+      else gh64[e] = g;
     }
   }
   for (int e = tid; e < r * TW; e += blockDim.x) {
@@ -1804,7 +1807,14 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
   for (int h = 0; h < CPL; ++h) live[h] = j0 + 32 * h + lc < n2;
   const cx<T>* rbase = d.Rt + (size_t)k * n2 + j0 + lc;  // + i * S * n2 + 32 h
   const size_t rstride = (size_t)S * n2;
-  if constexpr (!TCY) {
+  // Real slices of an FP32 engine: D as an error-free sum, (value, rounding errors)
+  // in the (re, im) fields (why: dcon_f_tile)
+  auto contract = [&](auto real) {
+    constexpr bool REAL = decltype(real)::value;
+    auto mac = [](cx<T>& a, cx<T> x, cx<T> v) {
+      if constexpr (REAL) dot2(a.re, a.im, x.re, v.re);
+      else cfmaconj(a, x, v);
+    };
     int i = row0;
     for (; i + nr < n1; i += 2 * nr) {
       cx<T> v[2][CPL];
@@ -1820,7 +1830,7 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
           if (s < r) {
             const cx<T> x = Xs[(size_t)s * n1 + i + q * nr];
 #pragma unroll
-            for (int h = 0; h < CPL; ++h) cfmaconj(acc[h][s], x, v[q][h]);
+            for (int h = 0; h < CPL; ++h) mac(acc[h][s], x, v[q][h]);
           }
     }
     for (; i < n1; i += nr) {
@@ -1833,8 +1843,16 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
         if (s < r) {
           const cx<T> x = Xs[(size_t)s * n1 + i];
 #pragma unroll
-          for (int h = 0; h < CPL; ++h) cfmaconj(acc[h][s], x, v[h]);
+          for (int h = 0; h < CPL; ++h) mac(acc[h][s], x, v[h]);
         }
+    }
+  };
+  if constexpr (!TCY) {
+    if constexpr (sizeof(T) == 4) {
+      if (dreal) contract(BoolC<true>{});
+      else contract(BoolC<false>{});
+    } else {
+      contract(BoolC<false>{});
     }
   }
   if constexpr (!TCY && NG > 1) {
@@ -1878,6 +1896,10 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
   for (int e = tid; e < r * TW; e += blockDim.x) {
     const int s = e / TW, c = e - s * TW;
     cx<T> v = {T(0), T(0)};
+    auto add = [&](cx<T> q) {
+      if (dreal) pair_add(v.re, v.im, q.re, q.im);
+      else v = v + q;
+    };
     if constexpr (TCY) {
       if (j0 + c < n2) {
         const cx<T>* dp = d.Dpart + ((size_t)k * d.ksplit * r + s) * n2 + j0 + c;  // + z r n2
@@ -1888,14 +1910,24 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
 #pragma unroll
           for (int w = 0; w < 4; ++w) q[w] = dp[(z + w) * zs];
 #pragma unroll
-          for (int w = 0; w < 4; ++w) v = v + q[w];
+          for (int w = 0; w < 4; ++w) add(q[w]);
         }
-        for (; z < d.ksplit; ++z) v = v + dp[z * zs];
+        for (; z < d.ksplit; ++z) add(dp[z * zs]);
       }
     } else {
-      for (int w = 0; w < nw; ++w) v = v + red[(w * RP + s) * TW + c];
+      for (int w = 0; w < nw; ++w) add(red[(w * RP + s) * TW + c]);
     }
-    for (int u = 0; u < r; ++u) cfma(v, Dgs[s * r + u], Yo[u * TW + c]);
+    if (dreal) {  // the head and tail of the real V
+      for (int u = 0; u < r; ++u) dot2(v.re, v.im, Dgs[s * r + u].re, Yo[u * TW + c].re);
+      const T h = v.re + v.im;
+      v = cx<T>{h, v.im - (h - v.re)};
+    } else {
+      for (int u = 0; u < r; ++u) cfma(v, Dgs[s * r + u], Yo[u * TW + c]);
+    }
+    if (g64 && !dreal) {
+      reinterpret_cast<double*>(Ds)[s * TW + c] = (double)v.re;
+      continue;
+    }
     Ds[s * TW + c] = v;
   }
   __syncthreads();
@@ -1907,15 +1939,21 @@ __device__ __forceinline__ void ystep_impl(const Dev<T>& d, unsigned char* smem)
       continue;
     }
     cx<T> y = Yo[e];
-    if (g64) {
+    if (dreal) {
       float h = (float)y.re, l = 0.f;
       for (int u = 0; u < r; ++u) {
-        const cx<float> g = gh64[s * r + u];
-        const float v = (float)Ds[u * TW + c].re;
-        dot2(h, l, g.re, v);
-        l = fmaf(g.im, v, l);
+        const cx<float> g = ghp[s * r + u];
+        const cx<T> v = Ds[u * TW + c];
+        dot2(h, l, g.re, (float)v.re);
+        l = fmaf(g.im, (float)v.re, fmaf(g.re, (float)v.im, l));
       }
       y.re = (T)(h + l);
+    } else if (g64) {
+      // (FP64 values of V from the (re, im) fields: one conversion each, below)
+      double yd = (double)y.re;
+      const double* vd = reinterpret_cast<const double*>(Ds) + c;
+      for (int u = 0; u < r; ++u) yd = fma(gh64[s * r + u], vd[u * TW], yd);
+      y.re = (T)yd;
     } else {
       for (int u = 0; u < r; ++u) cfma(y, Gh[s * r + u], Ds[u * TW + c]);
     }

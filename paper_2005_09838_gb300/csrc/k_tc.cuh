@@ -318,7 +318,8 @@ __global__ void __launch_bounds__(umma::kTcThreads) k_qcon_tc(Dev<float> d, cx<f
 // ---------------------------------------------------------------------------
 template <int KIND, bool SPLIT>
 __host__ inline size_t dcon_tc_smem() {
-  return qcon_tc_smem<KIND, SPLIT>();
+  const size_t real = 2 * align_up(dcon_f_smem<32>(), 16), tc = qcon_tc_smem<KIND, SPLIT>();
+  return tc > real ? tc : real;
 }
 
 template <int KIND, bool SPLIT>
@@ -326,6 +327,16 @@ __global__ void __launch_bounds__(umma::kTcThreads) k_dcon_tc(Dev<float> d) {
   using namespace umma;
   extern __shared__ __align__(1024) unsigned char smem[];
   if (converged(d)) return;
+  // real slices of the split TF32 form: compensated FP32 sums (see dcon_f_tile), 64
+  // columns to each half of the block
+  if constexpr (KIND == kTF32 && SPLIT) {
+    if (d.dpairs && (blockIdx.x == 0 || 2 * (int)blockIdx.x == d.n3)) {
+      const int half = threadIdx.x / kGmThreads;
+      dcon_f_tile<32, false>(d, blockIdx.x, blockIdx.y * kM + half * kGmTile, blockIdx.z, d.ksplit,
+                      smem + half * align_up(dcon_f_smem<32>(), 16), threadIdx.x % kGmThreads);
+      return;
+    }
+  }
   constexpr uint32_t TA = tile_bytes<KIND>(kM), TB = tile_bytes<KIND>(64);
   unsigned char* Ahi = smem;
   unsigned char* Alo = Ahi + TA;

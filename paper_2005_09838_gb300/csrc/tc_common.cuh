@@ -147,6 +147,15 @@ __device__ __forceinline__ void dot2(T& s, T& c, T a, T b) {
   s = t;
 }
 
+// (s, c) += (s2, c2) for sums kept as value and collected rounding errors.
+template <typename T>
+__device__ __forceinline__ void pair_add(T& s, T& c, T s2, T c2) {
+  const T t = s + s2;
+  const T z = t - s;
+  c += ((s - (t - z)) + (s2 - z)) + c2;
+  s = t;
+}
+
 // Sum of squares of a thread's values to FP64 accuracy.  FP32 values: error-free
 // products and sums on the FP32 pipe (dot2); GB300 issues one FP64 warp
 // instruction per scheduler in about 60 clocks, and the FP64 form (a conversion

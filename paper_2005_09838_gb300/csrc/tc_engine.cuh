@@ -58,8 +58,8 @@ inline SlabFn<T> pick_slab_tile(bool folded, bool staged, int tl) {
 }
 
 template <typename T, int L, int N1, int N2>
-inline void slab_f_table(SlabFn<T> f[3], bool bf16) {
-  f[MODE_ITER] = bf16 ? k_slab_f<T, L, N1, N2, MODE_ITER, true> : k_slab_f<T, L, N1, N2, MODE_ITER>;
+inline void slab_f_table(SlabFn<T> f[3]) {
+  f[MODE_ITER] = k_slab_f<T, L, N1, N2, MODE_ITER>;
   f[MODE_W] = k_slab_f<T, L, N1, N2, MODE_W>;
   f[MODE_R] = k_slab_f<T, L, N1, N2, MODE_R>;
 }
@@ -76,7 +76,7 @@ struct SlabCfg {
 // (defined per translation unit); false when none applies to (n2, n3) within
 // the shared-memory limit optin.
 template <typename T>
-bool pick_slab(int n2, int n3, int optin, bool bf16, SlabCfg<T>& cfg);
+bool pick_slab(int n2, int n3, int optin, SlabCfg<T>& cfg);
 
 template <typename T>
 using YFn = void (*)(Dev<T>);
@@ -181,11 +181,11 @@ bool pick_tc(int precision, bool split, TcKernels<T>& k);
 // Register-tiled contractions of the plain form (k_gemm.cuh); false where they
 // are not built (FP64 data).
 template <typename T>
-bool pick_gemm(int rp, int r, TcKernels<T>& k);
+bool pick_gemm(int rp, int r, int n2, bool strided, TcKernels<T>& k);
 template <>
-bool pick_gemm<float>(int rp, int r, TcKernels<float>& k);
+bool pick_gemm<float>(int rp, int r, int n2, bool strided, TcKernels<float>& k);
 template <>
-bool pick_gemm<double>(int rp, int r, TcKernels<double>& k);
+bool pick_gemm<double>(int rp, int r, int n2, bool strided, TcKernels<double>& k);
 template <>
 bool pick_tc<float>(int precision, bool split, TcKernels<float>& k);
 template <>
@@ -276,7 +276,7 @@ class Engine final : public EngineBase {
 
     // ---- kernel variants and shared memory -------------------------------------------
     SlabCfg<T> cfg{};
-    specialised_ = pick_slab<T>(n2_, n3_, optin, p.precision == TC_BF16 && rp_ == 32, cfg);
+    specialised_ = pick_slab<T>(n2_, n3_, optin, cfg);
     d_.scratch = nullptr;
     if (specialised_) {
       for (int m = 0; m < 3; ++m) slab_[m] = cfg.f[m];
@@ -314,6 +314,7 @@ class Engine final : public EngineBase {
     }
     if (fold_factors_) TC_CUDA_TRY(allow_fold_dft<T>(n3_));
 
+    strict_ = sizeof(T) == 4 && (specialised_ || (p.precision == TC_BF16 && rp_ == 32));
     // precision form: r x r solves in FP64, contractions on the tensor cores for r > 16
     mixed_ = p.precision == TC_TF32 || p.precision == TC_BF16;
     auto xlay = [&](bool in_smem) { return xstep_layout_for<T>(n1_, n2_, r_, rp_, mixed_, in_smem); };
@@ -385,6 +386,8 @@ class Engine final : public EngineBase {
     qcon_smem_ = qcon_smem_bytes<T>(n2_, r_, rp_);
     qcon_shape<T>(S_, n1_, rp_, d_.qrows, qthreads_);
     qgrid_ = dim3(S_, (n1_ + d_.qrows - 1) / d_.qrows);
+    // compensated D on the real slices (the tiled kernels, the fused Y-step, the split TF32 form)
+    d_.dpairs = !strict_ && !(mixed_ && rp_ == 32 && (p.precision == TC_BF16 || (p.flags & TC_FLAG_SINGLE_PASS)));
     int nsm = 0;
     TC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device_));
     if (mixed_ && rp_ == 32 && pick_tc<T>(p.precision, (p.flags & TC_FLAG_SINGLE_PASS) == 0, tck_)) {
@@ -397,12 +400,12 @@ class Engine final : public EngineBase {
       dgrid_ = dim3(S_, ntj, ksplit_);
       dthreads_ = 256;
       zgrid_ = dim3(S_, (n1_ + 127) / 128, (n2_ + 63) / 64);
-    } else if (gemm_pays(rp_, S_, n1_, n2_) && pick_gemm<T>(rp_, r_, tck_)) {
+    } else if (gemm_pays(rp_, S_, n1_, n2_) && pick_gemm<T>(rp_, r_, n2_, strict_, tck_)) {
       tcy_ = true;
-      qgrid_ = dim3(S_, (n1_ + kGmTile - 1) / kGmTile);
-      qthreads_ = kGmThreads;
-      ksplit_ = dcon_f_split(S_, n1_, n2_, nsm);
-      dgrid_ = dim3(S_, (n2_ + kGmTile - 1) / kGmTile, ksplit_);
+      qgrid_ = dim3(S_, (n1_ + 31) / 32);
+      qthreads_ = 256;
+      ksplit_ = strict_ ? kDStride : dcon_f_split(S_, n1_, n2_, nsm);
+      dgrid_ = dim3(S_, (n2_ + kGmTile - 1) / kGmTile, strict_ ? kDStride / dcon_f_groups(rp_) : ksplit_);
       dthreads_ = kGmThreads;
       zgrid_ = dim3(S_, (n1_ + kGmTile - 1) / kGmTile, (n2_ + kGmTile - 1) / kGmTile);
     }
@@ -525,8 +528,7 @@ class Engine final : public EngineBase {
     }
     k_pack<T><<<pack_grid(n1_, n2_, n3_), kTileThreads, 0, stream_>>>(dG, dM, Gint, maskbits, n1_, n2_, n3_, mw_);
     if (fold_) k_fold_tables<T><<<2 * 152, 256, 0, stream_>>>(fold_, twg, n3_);
-    // (TC_BF16 at r > 16 keeps the former rounding of the start, see kTL)
-    const cx<T>* ffold = fold_factors_ && !(p.precision == TC_BF16 && rp_ == 32) ? fold_ : nullptr;
+    const cx<T>* ffold = fold_factors_ && !strict_ ? fold_ : nullptr;
     launch_factor_dft<T>(dY, Yt, ffold, twg, n2_, r_, n3_, 1, stream_);
     if (dX) {
       launch_factor_dft<T>(dX, Xt, ffold, twg, n1_, r_, n3_, 0, stream_);
@@ -1023,6 +1025,13 @@ class Engine final : public EngineBase {
   int n1_ = 0, n2_ = 0, n3_ = 0, r_ = 0, S_ = 0, mw_ = 0, rp_ = 8;
   bool poisoned_ = false;
   bool specialised_ = false;
+  // Sums in the order of the plain kernels (k_factor_dft, k_qcon, the fused k_ystep,
+  // the sequential W-step), bit for bit: an iteration amplifies the rounding of D on
+  // the DC slice by the condition of its Gram (1e-5 of X~ and Y~ at r = 32), so another
+  // order gives other factors at that level.  For the lengths with an FFT, where
+  // nothing is gained by another order, and for TC_BF16 (see kTL).  The other forms
+  // compensate that sum (dcon_f_tile).
+  bool strict_ = false;
   bool folded_ = false;  // folded-transform slab kernels (k_slab_g)
   bool fold_factors_ = false;  // the factors' transforms too
   cx<T>* fold_ = nullptr;

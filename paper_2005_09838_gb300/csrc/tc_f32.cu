@@ -5,14 +5,14 @@
 
 namespace tc {
 
-bool slab_setup_f32_112(int n2, int optin, bool bf16, SlabCfg<float>& cfg);
-bool slab_setup_f32_168(int n2, int optin, bool bf16, SlabCfg<float>& cfg);
+bool slab_setup_f32_112(int n2, int optin, SlabCfg<float>& cfg);
+bool slab_setup_f32_168(int n2, int optin, SlabCfg<float>& cfg);
 
 template <>
-bool pick_slab<float>(int n2, int n3, int optin, bool bf16, SlabCfg<float>& cfg) {
+bool pick_slab<float>(int n2, int n3, int optin, SlabCfg<float>& cfg) {
   switch (n3) {
-    case 112: return slab_setup_f32_112(n2, optin, bf16, cfg);
-    case 168: return slab_setup_f32_168(n2, optin, bf16, cfg);
+    case 112: return slab_setup_f32_112(n2, optin, cfg);
+    case 168: return slab_setup_f32_168(n2, optin, cfg);
     default: return false;
   }
 }
@@ -44,15 +44,17 @@ bool pick_tc<float>(int precision, bool split, TcKernels<float>& k) {
 }
 
 template <>
-bool pick_gemm<float>(int rp, int r, TcKernels<float>& k) {
+bool pick_gemm<float>(int rp, int r, int n2, bool strided, TcKernels<float>& k) {
   k.zsyn = k_zsyn_f<float>;
   k.zsm = zsyn_f_smem<float>(r);
+  k.qsm = qcon_smem_bytes<float>(n2, r, rp);
   switch (rp) {
-    case 8: k.qcon = k_qcon_f<8>, k.dcon = k_dcon_f<8>, k.qsm = qcon_f_smem<8>(), k.dsm = dcon_f_smem<8>(); return true;
-    case 16: k.qcon = k_qcon_f<16>, k.dcon = k_dcon_f<16>, k.qsm = qcon_f_smem<16>(), k.dsm = dcon_f_smem<16>(); return true;
-    case 32: k.qcon = k_qcon_f<32>, k.dcon = k_dcon_f<32>, k.qsm = qcon_f_smem<32>(), k.dsm = dcon_f_smem<32>(); return true;
+    case 8: k.qcon = k_qcon_l<8>, k.dcon = strided ? k_dcon_f<8, true> : k_dcon_f<8>, k.dsm = dcon_f_smem<8>(); break;
+    case 16: k.qcon = k_qcon_l<16>, k.dcon = strided ? k_dcon_f<16, true> : k_dcon_f<16>, k.dsm = dcon_f_smem<16>(); break;
+    case 32: k.qcon = k_qcon_l<32>, k.dcon = strided ? k_dcon_f<32, true> : k_dcon_f<32>, k.dsm = dcon_f_smem<32>(); break;
     default: return false;
   }
+  return true;
 }
 
 EngineBase* make_engine_f32() { return new Engine<float>(); }

@@ -4,7 +4,7 @@
 namespace tc {
 
 template <>
-bool pick_slab<double>(int, int, int, bool, SlabCfg<double>&) {
+bool pick_slab<double>(int, int, int, SlabCfg<double>&) {
   return false;
 }
 
@@ -14,7 +14,7 @@ bool pick_tc<double>(int, bool, TcKernels<double>&) {
 }
 
 template <>
-bool pick_gemm<double>(int, int, TcKernels<double>&) {
+bool pick_gemm<double>(int, int, int, bool, TcKernels<double>&) {
   return false;
 }
 

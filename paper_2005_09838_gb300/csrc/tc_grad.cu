@@ -239,6 +239,7 @@ struct GradEngine final : tc_grad {
     d_.n3 = n3_;
     d_.S = S_;
     d_.r = r_;
+    d_.dpairs = 1;
     d_.mw = mw;
     d_.rho1 = (T)p.rho1;
     d_.G = Gint;

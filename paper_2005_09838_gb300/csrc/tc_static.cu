@@ -192,6 +192,7 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
                                  "tc_complete_static holds " + std::to_string(kStaticScratchBytes) + " bytes");
   }
   d.n1 = n1;
+  d.dpairs = 1;
   d.n2 = n2;
   d.n3 = n3;
   d.S = S;
