@@ -283,12 +283,12 @@ tc_status tc_complete_static(const tc_params* p, const void* G, const uint8_t* m
 
 /* Tile of the mode-3 transform chosen for this context (the library's own
  * tuning, no counterpart in the paper).  Tube lengths other than the ones with
- * dedicated kernels (7, 112, 168 in FP32; 7 in FP64) use a transform written as
+ * a transform of their own (112, 168 in FP32; 7 in FP64) use a transform written as
  * a product with the DFT matrix of Eq. (bar BA-k) / Eq. (barAAk), each work
- * item covering one tube and slab_tile rows (inverse) or slices (forward);
- * tc_init times slab_tile = 2, 4 and 8 on the initial pass (every choice gives
+ * item covering slab_tile rows (inverse) or slices (forward) of some tubes;
+ * tc_init times slab_tile = 2 and 4 on the initial pass (every choice gives
  * the same sums in the same order) and keeps the fastest.
- *   slab_tile : receives the chosen tile, 0 for a dedicated-kernel length.
+ *   slab_tile : receives the chosen tile, 0 for the lengths above.
  * Errors: TC_ERR_ARG. */
 tc_status tc_tile(tc_ctx* c, int32_t* slab_tile);
 

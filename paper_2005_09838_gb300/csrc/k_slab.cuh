@@ -25,7 +25,7 @@ enum SlabFlag : int { SLAB_IN_SMEM = 1, SLAB_WROWS = 2, SLAB_NOSUM = 4 };
 constexpr int kSlabThreads = 256;
 // Rows (inverse) or slices (forward) per item of the generic transform by
 // default; every tile gives the same sums in the same order, and tc_init times
-// 2, 4 and 8 where this kernel runs the iteration.  It runs where k_slab_g does
+// 2 and 4 where this kernel runs the iteration.  It runs where k_slab_g does
 // not hold the slab in shared memory, and for TC_BF16: the split operands of
 // its contractions keep 16 bits, so any other rounding of the transform
 // comes back as other BF16 rounding errors in the factors (3e-5 of Y~ after
@@ -448,8 +448,11 @@ __device__ __forceinline__ double dw_term(cx<T> rnew, cx<T> rold, cx<T> dz, int 
 // Layouts used here: G row-major [i1][n3][n2] and mask words row-major
 // [i1][n3][ceil(n2/32)] (written by k_pack), copied to shared memory.
 // ---------------------------------------------------------------------------
-template <typename T, int MODE, int TL = kTL>
-__global__ void __launch_bounds__(kSlabThreads, 1)
+// NB: CTAs per SM to leave registers for, as many as the slab's shared memory
+// allows (the sweeps alone take 255 registers, one CTA of 8 warps per SM; at 85 and
+// three CTAs the iteration of 435 x 205 x 34 went from 223 to 180 us).
+template <typename T, int MODE, int TL = kTL, int NB = 1>
+__global__ void __launch_bounds__(kSlabThreads, NB)
     k_slab(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
   const int slabs_in_smem = flags & SLAB_IN_SMEM;
   extern __shared__ __align__(16) unsigned char smem[];

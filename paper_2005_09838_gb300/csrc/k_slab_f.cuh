@@ -32,6 +32,9 @@
 namespace tc {
 
 constexpr int kSlabFThreads = 512;
+// The other modes have no W-step and fit 64 registers: twice the threads
+// (MODE_GRAD on 529 x 288 x 168: the call 905 -> 880 us).
+constexpr int kSlabFAux = 1024;
 // Items per thread whose global loads are issued together in the first split phase.
 constexpr int kSlabFBatch = 4;
 
@@ -56,7 +59,7 @@ __host__ __device__ inline SlabFLayout slab_f_layout(int n2, int L) {
   Lo.wtab = off;
   off = align_up(off + sizeof(T) * 6 * (size_t)n2, 16);
   Lo.red = off;
-  off = align_up(off + sizeof(double) * 2 * (kSlabFThreads / 32), 16);
+  off = align_up(off + sizeof(double) * 2 * (kSlabFAux / 32), 16);
   Lo.buf = off;  // [n2][slab_f_stride(L)]
   off = align_up(off + sizeof(T) * (size_t)n2 * slab_f_stride(L), 16);
   Lo.total = off;
@@ -121,7 +124,7 @@ __device__ __forceinline__ cx<T> fwd_split(cx<T> zk, cx<T> zm, int k) {
 // The W-step is wstep_sweeps_seg, bit for bit the sequential sweeps
 // (Engine::strict_).
 template <typename T, int L, int N1, int N2, int MODE>
-__global__ void __launch_bounds__(kSlabFThreads, 1) k_slab_f(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
+__global__ void __launch_bounds__(MODE == MODE_ITER ? kSlabFThreads : kSlabFAux, 1) k_slab_f(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
   constexpr int M = L / 2;
   static_assert(L % 2 == 0 && M == N1 * N2, "n3 = 2 N1 N2");
   constexpr int LP = slab_f_stride(L);

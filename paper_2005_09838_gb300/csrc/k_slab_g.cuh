@@ -691,8 +691,8 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
 // keep the lengths whose tables do not fit): 80 + 51 and 88 + 65 us for both
 // factors of 529 x 288 x 168, r = 16.
 // ---------------------------------------------------------------------------
-constexpr int kFoldThreads = 256;
-constexpr int kFoldTL = 4;
+constexpr int kFoldThreads = 512;
+constexpr int kFoldTL = 2;  // 22 items of the forward transform at n3 = 168 for 16 warps
 
 // Shared bytes: table, then the folded pairs (forward) or the spectrum (inverse).
 template <typename T>

@@ -50,11 +50,14 @@ inline SlabFn<T> pick_slab_g(int mode, int tl, bool staged) {
   return staged ? pick_slab_g_st<T, true>(mode, tl) : pick_slab_g_st<T, false>(mode, tl);
 }
 
-// The iteration's slab kernel with a tile of tl.
+// The iteration's slab kernel with a tile of tl; nb: CTAs of the generic one that
+// an SM's shared memory holds.
 template <typename T>
-inline SlabFn<T> pick_slab_tile(bool folded, bool staged, int tl) {
+inline SlabFn<T> pick_slab_tile(bool folded, bool staged, int tl, int nb) {
   if (folded) return pick_slab_g<T>(MODE_ITER, tl, staged);
-  return tl == 2 ? k_slab<T, MODE_ITER, 2> : tl == 4 ? k_slab<T, MODE_ITER, 4> : k_slab<T, MODE_ITER, 8>;
+  if (sizeof(T) == 4 && nb >= 3) return tl == 2 ? k_slab<T, MODE_ITER, 2, 3> : k_slab<T, MODE_ITER, 4, 3>;
+  if (sizeof(T) == 4 && nb == 2) return tl == 2 ? k_slab<T, MODE_ITER, 2, 2> : k_slab<T, MODE_ITER, 4, 2>;
+  return tl == 2 ? k_slab<T, MODE_ITER, 2> : k_slab<T, MODE_ITER, 4>;
 }
 
 template <typename T, int L, int N1, int N2>
@@ -302,6 +305,7 @@ class Engine final : public EngineBase {
         d_.scratch = scratch;
       }
       slab_smem_ = lay.total;
+      slab_nb_ = (int)((size_t)(optin + kStaticSmemReserve + 1024) / (slab_smem_ + 1024));
     }
     for (int m = 0; m < 3; ++m)
       TC_CUDA_TRY(allow_dynamic_smem((const void*)slab_[m], slab_smem_));
@@ -539,7 +543,7 @@ class Engine final : public EngineBase {
     }
     k_gram_tiles<T><<<dim3(S_, ytiles), 256, 0, stream_>>>(d_);         // A of the first X-step
     if (xsplit_ || apre_) xa_fn_<<<S_, xa_threads_, xa_smem_, stream_>>>(d_);  // its A^+
-    if (!specialised_ && !(folded_ && n3_ == 7)) {  // (four rows and slices: nothing to choose)
+    if (!specialised_ && !(folded_ && sizeof(T) == 8 && n3_ == 7)) {  // (four rows and slices: nothing to choose)
       // tile of the generic transform for this shape: each candidate runs the
       // initial slab pass (it only depends on G and Z~0, so every run writes the
       // same R~0), timed twice; the fastest is kept
@@ -882,15 +886,15 @@ class Engine final : public EngineBase {
   }
 
   tc_status tune_slab_tile(std::string& err) {
-    const int cand[3] = {2, 4, 8};
+    const int cand[2] = {2, 4};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     TC_CUDA_TRY(cudaEventCreate(&e0));
     TC_CUDA_TRY(cudaEventCreate(&e1));
     float best = 1e30f;
     int pick = 0;
     cudaError_t e = cudaSuccess;
-    for (int c = 0; c < (folded_ ? 2 : 3) && e == cudaSuccess; ++c) {
-      slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[c]);
+    for (int c = 0; c < 2 && e == cudaSuccess; ++c) {
+      slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[c], slab_nb_);
       e = allow_dynamic_smem((const void*)slab_[MODE_ITER], slab_smem_);
       float ms = 1e30f;
       for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
@@ -915,13 +919,14 @@ class Engine final : public EngineBase {
       poisoned_ = true;
       return TC_ERR_CUDA;
     }
-    slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[pick]);
+    slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[pick], slab_nb_);
     slab_tile_ = cand[pick];
     return TC_OK;
   }
 
   void launch_slab(int mode, T* Wout, int init, cudaStream_t s, int flags = 0) {
-    slab_[mode]<<<n1_, slab_threads_, slab_smem_, s>>>(d_, Wout, flags | (slabs_in_smem_ ? SLAB_IN_SMEM : 0), init);
+    const int threads = specialised_ && mode != MODE_ITER ? 2 * slab_threads_ : slab_threads_;
+    slab_[mode]<<<n1_, threads, slab_smem_, s>>>(d_, Wout, flags | (slabs_in_smem_ ? SLAB_IN_SMEM : 0), init);
   }
   cudaError_t launch_synth(cudaStream_t s) {
     const size_t sm = zsyn_f_smem<T>(r_);
@@ -1041,6 +1046,7 @@ class Engine final : public EngineBase {
   bool mixed_ = false;
   bool xsplit_ = false;  // X-step as four kernels
   bool apre_ = false;    // one-CTA X-step with A^+ from k_xa on a graph branch
+  int slab_nb_ = 1;      // CTAs of the generic slab kernel that an SM holds
   int slab_tile_ = 0;    // rows / slices per item of the generic transform (0: specialised length)
   int* rk_ = nullptr;    // step 5: slice ranks, counters and work (allocated when the rule is first on)
   int* rcnt_ = nullptr;

@@ -5,6 +5,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
+#include <cstring>
 #include <new>
 #include <string>
 #include <vector>
@@ -73,7 +75,7 @@ GradSlab<T> pick_grad_slab(int n2, int n3, int optin) {
       if (lay.total <= (size_t)optin) {
         fft::upload_tables();
         g.f = (n3 == 168) ? k_slab_f<T, 168, 12, 7, MODE_GRAD> : k_slab_f<T, 112, 8, 7, MODE_GRAD>;
-        g.threads = kSlabFThreads;
+        g.threads = kSlabFAux;
         g.smem = lay.total;
         return g;
       }
@@ -124,6 +126,8 @@ template <typename T>
 struct GradEngine final : tc_grad {
   ~GradEngine() override {
     for (void* q : allocs_) cudaFree(q);
+    if (pinned_) cudaFreeHost(host_);
+    else std::free(host_);
   }
 
   template <typename U>
@@ -165,12 +169,24 @@ struct GradEngine final : tc_grad {
     GX_ = alloc<cx<T>>((size_t)S_ * r_ * n1_, err);
     GY_ = alloc<cx<T>>((size_t)S_ * r_ * n2_, err);
     cx<T>* twg = alloc<cx<T>>((size_t)n3_, err);
-    double* part = alloc<double>((size_t)n1_ * 4, err);
-    double* part_k = alloc<double>((size_t)S_ * kRhoChunks, err);
-    int* derr = alloc<int>(1, err);
+    // the partial sums and the error word of a call lie together, for one copy into
+    // pinned memory
+    const size_t npart = (size_t)n1_ * 4, npk = (size_t)S_ * kRhoChunks;
+    double* part = alloc<double>(npart + npk + 1, err);
     xin_ = alloc<T>((size_t)n1_ * r_ * n3_, err);
     yin_ = alloc<T>((size_t)r_ * n2_ * n3_, err);
     if (!err.empty()) return TC_ERR_NOMEM;
+    pinned_ = cudaMallocHost(&host_, (npart + npk + 1) * sizeof(double)) == cudaSuccess;
+    if (!pinned_) {  // pageable memory serves too
+      cudaGetLastError();
+      host_ = static_cast<double*>(std::malloc((npart + npk + 1) * sizeof(double)));
+      if (!host_) {
+        err = "host allocation failed";
+        return TC_ERR_NOMEM;
+      }
+    }
+    double* part_k = part + npart;
+    int* derr = reinterpret_cast<int*>(part_k + npk);
 
     slab_ = pick_grad_slab<T>(n2_, n3_, optin);
     if (!slab_.in_smem) {
@@ -322,13 +338,12 @@ struct GradEngine final : tc_grad {
       }
     }
     TCG_TRY(cudaGetLastError());
-    std::vector<double> part(4 * (size_t)n1_), pk((size_t)S_ * kRhoChunks);
-    TCG_TRY(cudaMemcpyAsync(part.data(), d_.part, part.size() * sizeof(double), cudaMemcpyDeviceToHost, stream_));
-    if (d_.rho1 != T(0))
-      TCG_TRY(cudaMemcpyAsync(pk.data(), d_.part_k, pk.size() * sizeof(double), cudaMemcpyDeviceToHost, stream_));
-    int herr = 0;
-    TCG_TRY(cudaMemcpyAsync(&herr, d_.err, sizeof(int), cudaMemcpyDeviceToHost, stream_));
+    const size_t npart = (size_t)n1_ * 4, npk = (size_t)S_ * kRhoChunks;
+    TCG_TRY(cudaMemcpyAsync(host_, d_.part, (npart + npk + 1) * sizeof(double), cudaMemcpyDeviceToHost, stream_));
     TCG_TRY(cudaStreamSynchronize(stream_));
+    const double *part = host_, *pk = host_ + npart;
+    int herr = 0;
+    std::memcpy(&herr, pk + npk, sizeof(int));
     if (herr != DEV_OK) {
       err = "device-side check failed (code " + std::to_string(herr) + ")";
       return TC_ERR_CUDA;
@@ -367,6 +382,8 @@ struct GradEngine final : tc_grad {
   cx<T>* GY_ = nullptr;
   T* xin_ = nullptr;
   T* yin_ = nullptr;
+  double* host_ = nullptr;  // partial sums, error word
+  bool pinned_ = false;
   std::vector<void*> allocs_;
 };
 
