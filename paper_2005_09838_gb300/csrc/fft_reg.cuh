@@ -47,6 +47,14 @@ __device__ __forceinline__ cx<T> tw(int m) {
   return INV ? cx<T>{v.re, -v.im} : v;
 }
 
+// The same for 0 <= m < L (no reduction: four integer instructions less per
+// twiddle where m is not a constant).
+template <typename T, int L, bool INV>
+__device__ __forceinline__ cx<T> tw_at(int m) {
+  const cx<T> v = tw_entry<T>(table_offset(L) + m);
+  return INV ? cx<T>{v.re, -v.im} : v;
+}
+
 // Radix-P DFT of P values x[q*xs], q < P, written to o[k*os].
 // TOP is the length of the twiddle table in use (P divides TOP).
 template <typename T, int P, int TOP, bool INV>

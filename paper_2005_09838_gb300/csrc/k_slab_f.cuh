@@ -105,7 +105,7 @@ __device__ __forceinline__ cx<T> inv_split(cx<T> a, cx<T> b, int k) {
   const cx<T> bc = conj(b);
   const cx<T> E = (a + bc) * T(0.5);
   const cx<T> D = (a - bc) * T(0.5);
-  const cx<T> O = (k == 0) ? D : cmul(D, fft::tw<T, L, true>(k));
+  const cx<T> O = (k == 0) ? D : cmul(D, fft::tw_at<T, L, true>(k));
   return cx<T>{E.re - O.im, E.im + O.re};
 }
 
@@ -118,7 +118,7 @@ __device__ __forceinline__ cx<T> fwd_split(cx<T> zk, cx<T> zm, int k) {
   const cx<T> E = (zk + zc) * T(0.5);
   const cx<T> D = (zk - zc) * T(0.5);
   const cx<T> O = {D.im, -D.re};
-  return E + cmul(O, fft::tw<T, L, false>(k));
+  return E + cmul(O, fft::tw_at<T, L, false>(k));
 }
 
 // The W-step is wstep_sweeps_seg, bit for bit the sequential sweeps
@@ -127,6 +127,7 @@ template <typename T, int L, int N1, int N2, int MODE>
 __global__ void __launch_bounds__(MODE == MODE_ITER ? kSlabFThreads : kSlabFAux, 1) k_slab_f(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
   constexpr int M = L / 2;
   static_assert(L % 2 == 0 && M == N1 * N2, "n3 = 2 N1 N2");
+  static_assert(2 * (N1 - 1) * (N2 - 1) < L, "twiddle indices below L");
   constexpr int LP = slab_f_stride(L);
   extern __shared__ __align__(16) unsigned char smem[];
   const int i1 = blockIdx.x;
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(MODE == MODE_ITER ? kSlabFThreads : kSlabFAux,
       fft::CFFT<T, N1, L, true>::run(v, 1, o);
 #pragma unroll
       for (int k1 = 0; k1 < N1; ++k1) {
-        const cx<T> x = (k1 == 0) ? o[0] : cmul(o[k1], fft::tw<T, L, true>(2 * q * k1));
+        const cx<T> x = (k1 == 0) ? o[0] : cmul(o[k1], fft::tw_at<T, L, true>(2 * q * k1));
         st_slot(tb, N2 * k1 + q, x);
       }
     }
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(MODE == MODE_ITER ? kSlabFThreads : kSlabFAux,
       fft::CFFT<T, N2, L, false>::run(v, 1, o);
 #pragma unroll
       for (int q = 0; q < N2; ++q) {
-        const cx<T> x = (q == 0) ? o[0] : cmul(o[q], fft::tw<T, L, false>(2 * k1 * q));
+        const cx<T> x = (q == 0) ? o[0] : cmul(o[q], fft::tw_at<T, L, false>(2 * k1 * q));
         st_slot(tb, q, x);
       }
     }

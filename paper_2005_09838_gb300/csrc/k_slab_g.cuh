@@ -688,8 +688,9 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
 //   k_fold_dft   real [n3][U] -> half spectrum [S][U]
 //   k_fold_idft  half spectrum -> real, 1 / n3 included
 // One thread per tube and four outputs before (k_factor_dft, k_factor_idft, which
-// keep the lengths whose tables do not fit): 80 + 51 and 88 + 65 us for both
-// factors of 529 x 288 x 168, r = 16.
+// keep the lengths whose tables do not fit and the exact order of Engine::strict_):
+// 80 + 51 and 88 + 65 us for both factors of 529 x 288 x 168, r = 16, against
+// 27 + 23 and 18 + 14 here.
 // ---------------------------------------------------------------------------
 constexpr int kFoldThreads = 512;
 constexpr int kFoldTL = 2;  // 22 items of the forward transform at n3 = 168 for 16 warps
