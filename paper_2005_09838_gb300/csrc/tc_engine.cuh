@@ -406,8 +406,9 @@ class Engine final : public EngineBase {
       zgrid_ = dim3(S_, (n1_ + 127) / 128, (n2_ + 63) / 64);
     } else if (gemm_pays(rp_, S_, n1_, n2_) && pick_gemm<T>(rp_, r_, n2_, strict_, tck_)) {
       tcy_ = true;
-      qgrid_ = dim3(S_, (n1_ + 31) / 32);
-      qthreads_ = 256;
+      const bool tiled_q = rp_ == 8 && !strict_;  // k_qcon_f, else k_qcon_l
+      qgrid_ = dim3(S_, tiled_q ? (n1_ + kGmTile - 1) / kGmTile : (n1_ + 31) / 32);
+      qthreads_ = tiled_q ? kGmThreads : 256;
       ksplit_ = strict_ ? kDStride : dcon_f_split(S_, n1_, n2_, nsm);
       dgrid_ = dim3(S_, (n2_ + kGmTile - 1) / kGmTile, strict_ ? kDStride / dcon_f_groups(rp_) : ksplit_);
       dthreads_ = kGmThreads;
