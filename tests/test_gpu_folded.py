@@ -72,3 +72,14 @@ def test_whole_rows_and_weights(rows, weights):
 ])
 def test_large_slabs(shape, precision):
     _check(shape, 2, 0.3, precision, iters=2)
+
+
+@pytest.mark.parametrize("shape,r", [
+    ((70, 65, 112), 12),    # eight strided partials of D, two per CTA; odd n2
+    ((200, 34, 112), 8),    # four per CTA; rows past a multiple of 8
+    ((66, 97, 112), 20),    # one per CTA, r padded
+    ((65, 64, 10), 16),     # contiguous ranges, compensated real slices
+    ((200, 129, 9), 7),     # tiled Q, four groups sharing a sum
+])
+def test_tiled_contractions(shape, r):
+    _check(shape, r, 0.4, "fp32")
