@@ -119,6 +119,23 @@ __host__ __device__ inline void wstep_tables(T* w, int n2, double mu, double rho
   }
 }
 
+// Excess ratios of the same pivots, h = 1 - rho2 inv = g / (rho2 + g) with the
+// excess g = 1 / inv - rho2 of a pivot, [2][n2] by position in the run (run start
+// as in wstep_tables).  g follows g_q = 1 + mu + rho2 g_{q-1} / (rho2 + g_{q-1}):
+// no subtraction, so h keeps its digits however close to 1 rho2 inv is.
+template <typename T>
+__host__ __device__ inline void wstep_excess(T* h, int n2, double mu, double rho2) {
+  const double first[2] = {1.0 + mu, 1.0 + mu + rho2};
+  for (int b = 0; b < 2; ++b) {
+    double prev = 0.0;
+    for (int q = 0; q < n2; ++q) {
+      const double g = (q > 0) ? 1.0 + mu + rho2 * prev : first[b];
+      prev = g / (rho2 + g);
+      h[(size_t)b * n2 + q] = (T)prev;
+    }
+  }
+}
+
 // One mask word (32 entries, fewer in the last word) of the forward sweep.
 // The table index of entry j is inv-table + (j - rs), rs the start of the run
 // holding j: from the mask bits below j (rs = 32 w + 32 - clz(below)) or,
@@ -302,17 +319,22 @@ __device__ void wstep_sweeps_seg(ColFn col_of, int LP, const uint32_t* __restric
 }
 
 // ---------------------------------------------------------------------------
-// W-step of one segment (kWSeg entries, fewer in the last one) of one row, from
-// the slab's values v (G on the mask, Z elsewhere) as they were before any
-// segment was solved: every segment then stands alone, and the caller stores the
-// results once all segments of the row have read.  Inside the segment the sweeps
-// are those of wstep_sweeps, with the values and the backward coefficients in
-// registers.
+// W-step with every segment of a row (kWSeg entries, fewer in the last one) solved
+// on its own by one thread, from the slab's values v (G on the mask, Z elsewhere)
+// as they were before any segment was solved; the caller stores the results once
+// all segments of the row have read.  Inside the segment the sweeps are those of
+// wstep_sweeps, with the values and the backward coefficients in registers.
 //   Left:  d_{base-1} of a run that enters the segment, by the forward
 //          recurrence from the run's start.
 //   Right: a run that goes on past the segment is eliminated from its other end,
 //          w_j = e w_{j-1} + f (pivots by the distance from that end: the same
-//          table), so the segment's last entry is (d + c f) / (1 - c e).
+//          table), so the segment's last entry is (d + c f) / (1 - c e).  c and
+//          e tend to 1 as rho2 grows, so from c e = 1/2 on 1 - c e is formed from the
+//          excess ratios of the two pivots, h_c + c h_e: the difference loses the digits
+//          (FP32, a row of 100 missing entries, mu = 1e-3: 6e-4 of W at rho2 = 1e6
+//          and 3e-2 at 1e8, against 2e-7 and 4e-7 of the sequential sweeps).
+// The excess ratios are the GENERAL form, which the engine takes where rho2 asks for
+// it (wstep_strong).
 // Fewer than half the instructions of the two sweeps over shared memory (no
 // second pass over the values, the table and the mask).  FP32 segments of 16 keep
 // the thread within 64 registers; in FP64, where a warp instruction holds its scheduler's pipe for
@@ -322,22 +344,35 @@ __device__ void wstep_sweeps_seg(ColFn col_of, int LP, const uint32_t* __restric
 template <typename T>
 constexpr int kWSeg = sizeof(T) == 8 ? 8 : 16;
 
-template <typename T, int SEG, bool FULL, bool LAST>
+// Start of the run of missing entries that reaches entry `base` from the left, and
+// end (one past its last entry) of the one that reaches entry j1 - 1 from the right.
+__device__ __forceinline__ int run_start(const uint32_t* __restrict__ rowm, int base, uint32_t word) {
+  int u = base >> 5;  // (word = rowm[u])
+  uint32_t m = word & ((1u << (base & 31)) - 1u);
+  while (m == 0u && u > 0) m = rowm[--u];
+  return m ? 32 * u + 32 - __clz(m) : 0;
+}
+__device__ __forceinline__ int run_end(const uint32_t* __restrict__ rowm, int words, int j1, int n2) {
+  int u = j1 >> 5;
+  uint32_t m = rowm[u] & (0xffffffffu << (j1 & 31));
+  while (m == 0u && u + 1 < words) m = rowm[++u];
+  return m ? 32 * u + __ffs(m) - 1 : n2;
+}
+
+// Whether c e can reach 1/2: the largest coefficient is that of a run's first entry
+// at the row's start, rho2 / (1 + mu + rho2), whose square is below 4/9 up to here.
+inline bool wstep_strong(double mu, double rho2) { return rho2 > 2.0 * (1.0 + mu); }
+// GENERAL: any rho2.
+template <typename T, int SEG, bool FULL, bool LAST, bool GENERAL>
 __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP, const uint32_t* __restrict__ rowm,
-                                              int words, int sgm, int qn, int n2, T rho2, const T* __restrict__ wtab,
-                                              T (&v)[SEG]) {
-  const int base = SEG * sgm, bw = base >> 5, bb = base & 31;
-  const uint32_t word = rowm[bw], mw = word >> bb;
-#pragma unroll
-  for (int q = 0; q < SEG; ++q)
-    if (FULL || q < qn) v[q] = col[(base + q) * LP];
+                                              int words, int sgm, int qn, int n2, T rho2,
+                                              const T* __restrict__ wtab, const T* __restrict__ hex, T (&v)[SEG]) {
+  const int base = SEG * sgm, j1 = base + SEG;
+  const uint32_t word = rowm[base >> 5], mw = word >> (base & 31);
   int st = 0;  // start of the run of missing entries that enters the segment
   T d = T(0);
   if (base > 0) {
-    uint32_t m = word & ((1u << bb) - 1u);
-    int u = bw;
-    while (m == 0u && u > 0) m = rowm[--u];
-    if (m) st = 32 * u + 32 - __clz(m);
+    st = run_start(rowm, base, word);
     if (!(mw & 1u)) {
       if (st > 0) d = col[(st - 1) * LP];
       const T* tb = wtab + (st == 0 ? 0 : n2);
@@ -368,20 +403,21 @@ __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP,
   }
   T wn = T(0);
   if (!LAST && !((mw >> (SEG - 1)) & 1u)) {
-    const int j1 = base + SEG;
-    int u = j1 >> 5;
-    uint32_t m = rowm[u] & (0xffffffffu << (j1 & 31));
-    while (m == 0u && u + 1 < words) m = rowm[++u];
-    const int k = m ? 32 * u + __ffs(m) - 1 : n2;  // next observed entry, or the row's end
-    T x = (k < n2) ? col[k * LP] : T(0), e = T(0);
-    const T* tb = wtab + (k < n2 ? n2 : 0);
+    const int k = run_end(rowm, words, j1, n2);  // next observed entry, or the row's end
+    T x = (k < n2) ? col[k * LP] : T(0);
+    const int tb = k < n2 ? n2 : 0;
     for (int j = k - 1; j >= j1; --j) {
-      const T inv = tb[k - 1 - j];
-      e = rho2 * inv;
-      x = fma(e, x, col[j * LP] * inv);
+      const T inv = wtab[tb + k - 1 - j];
+      x = fma(rho2 * inv, x, col[j * LP] * inv);
     }
     wn = fma(c[SEG - 1], x, v[SEG - 1]);
-    if (k > j1) wn *= rcp_refined(fma(-c[SEG - 1], e, T(1)));
+    if (k > j1) {
+      const int p1 = tb + k - 1 - j1;
+      const T e = rho2 * wtab[p1], ce = c[SEG - 1] * e;
+      // (tp is one past the position of the segment's last entry)
+      wn *= rcp_refined(!GENERAL || ce < T(0.5) ? fma(-c[SEG - 1], e, T(1))
+                                                : fma(c[SEG - 1], hex[p1], hex[tp - 1 - wtab]));
+    }
     v[SEG - 1] = wn;
     c[SEG - 1] = T(0);
   }
@@ -395,22 +431,35 @@ __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP,
 
 // W-step of every row of the slab: a thread per (row, segment), as many whole
 // rows at a time as the block has threads for; rows at col_of(q) (stride LP
-// along j), their mask words at msk + q words.  Ends with a barrier.
-template <typename T, int SEG, typename ColFn>
+// along j), their mask words at msk + q words; hex: [2][n2] excess ratios
+// (wstep_excess; read in the GENERAL form only).  Ends with a barrier.
+template <typename T, int SEG, bool GENERAL, typename ColFn>
 __device__ __forceinline__ void wstep_segments(ColFn col_of, int LP, const uint32_t* __restrict__ msk, int nrows, int n2,
-                                               T rho2, const T* __restrict__ wtab) {
+                                               T rho2, const T* __restrict__ wtab, const T* __restrict__ hex) {
   const int words = (n2 + 31) >> 5, segs = (n2 + SEG - 1) / SEG, ql = n2 - SEG * (segs - 1);
   const int rpr = blockDim.x / segs;  // rows per round (the block has at least segs threads)
   const int row = threadIdx.x % rpr, w = threadIdx.x / rpr;
   for (int r0 = 0; r0 < nrows; r0 += rpr) {
     const bool work = w < segs && r0 + row < nrows;
+    const uint32_t* rowm = msk + (size_t)(r0 + row) * words;
     T v[SEG];
     T* col = nullptr;
     if (work) {
       col = col_of(r0 + row);
-      const uint32_t* rowm = msk + (size_t)(r0 + row) * words;
-      if (w < segs - 1) wstep_segment<T, SEG, true, false>(col, LP, rowm, words, w, SEG, n2, rho2, wtab, v);
-      else wstep_segment<T, SEG, false, true>(col, LP, rowm, words, w, ql, n2, rho2, wtab, v);
+      const T* cb = col + SEG * w * LP;
+      if (w < segs - 1) {
+#pragma unroll
+        for (int q = 0; q < SEG; ++q) v[q] = cb[q * LP];
+      } else {
+#pragma unroll
+        for (int q = 0; q < SEG; ++q)
+          if (q < ql) v[q] = cb[q * LP];
+      }
+    }
+    if (work) {
+      if (w < segs - 1)
+        wstep_segment<T, SEG, true, false, GENERAL>(col, LP, rowm, words, w, SEG, n2, rho2, wtab, hex, v);
+      else wstep_segment<T, SEG, false, true, GENERAL>(col, LP, rowm, words, w, ql, n2, rho2, wtab, hex, v);
     }
     __syncthreads();
     if (work) {

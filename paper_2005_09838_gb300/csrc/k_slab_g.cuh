@@ -403,7 +403,7 @@ __device__ __forceinline__ void fold_forward(const FoldDims& f, const cx<T>* __r
   fold_product<T, TL, SH>(acc, tab + q0 + f.nkt, f.nkt, x, oddk ? -np2 : np2, f.lmax);
 }
 
-template <typename T, int MODE, int TL, bool EVEN, bool STAGED>
+template <typename T, int MODE, int TL, bool EVEN, bool STAGED, bool GENERAL>
 __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wout, int flags, int init,
                                             unsigned char* smem) {
   using P = Pk<T>;
@@ -433,8 +433,11 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
   constexpr bool NEED_G = (MODE == MODE_ITER || MODE == MODE_GRAD);
 
   // ---- masks, W-step table, coefficients, G into its place in the slab ---------------------
+  // (rows 2 and 3 of the table are read in FP64 only; FP32 keeps the excess ratios
+  // in their place)
+  constexpr bool HEX_SH = GENERAL && sizeof(T) == 4;
   if (wsolve)
-    for (int j = tid; j < 6 * n2; j += nt) wtab[j] = d.winv[j];
+    for (int j = tid; j < 6 * n2; j += nt) wtab[j] = HEX_SH && j >= 2 * n2 && j < 4 * n2 ? d.wexc[j - 2 * n2] : d.winv[j];
   if (MODE != MODE_W)
     for (int e = tid; e < n3 * mw; e += nt) {
       const int q = e / mw;
@@ -592,9 +595,10 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
     for (int e = tid; e < nf; e += nt) cp_async_elem(tab + e, d.fold + ni + e);
 
   // ---- W-step -------------------------------------------------------------------------------
-  if (wsolve)
-    wstep_segments<T, kWSeg<T>>([&](int q) { return spat + slab_g_off(EVEN, n3, slab_g_row(EVEN, n3, q), np2); }, 2, msk, n3, n2,
-                   d.rho2, wtab);
+  if (wsolve) {
+    auto col_of = [&](int q) { return spat + slab_g_off(EVEN, n3, slab_g_row(EVEN, n3, q), np2); };
+    wstep_segments<T, kWSeg<T>, GENERAL>(col_of, 2, msk, n3, n2, d.rho2, wtab, HEX_SH ? wtab + 2 * n2 : d.wexc);
+  }
 
   // ---- fold -----------------------------------------------------------------------------------
   {
@@ -836,12 +840,15 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold_idft(const cx<T>* __restr
   else fold_idft_impl<T, true>(in, out, fold, n, r, n3, transposed, smem);
 }
 
-template <typename T, int MODE, int TL, bool STAGED>
-__global__ void __launch_bounds__(kSlabGThreads<T>, 1) k_slab_g(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
+// GENERAL (MODE_ITER): the W-step of strong smoothing (see wstep_segments), chosen by
+// the engine; as a branch of one kernel it cost the plain form 5%
+// (925 x 153 x 92: 150 -> 160 us, in spills).
+template <typename T, int MODE, int TL, bool STAGED, bool GENERAL = false>
+__global__ void __launch_bounds__(kSlabGThreads<T>, GENERAL && sizeof(T) == 8 ? 2 : 1) k_slab_g(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (MODE == MODE_ITER && !init && converged(d)) return;
-  if ((d.n3 & 1) == 0) slab_g_impl<T, MODE, TL, true, STAGED>(d, Wout, flags, init, smem);
-  else slab_g_impl<T, MODE, TL, false, STAGED>(d, Wout, flags, init, smem);
+  if ((d.n3 & 1) == 0) slab_g_impl<T, MODE, TL, true, STAGED, GENERAL>(d, Wout, flags, init, smem);
+  else slab_g_impl<T, MODE, TL, false, STAGED, GENERAL>(d, Wout, flags, init, smem);
 }
 
 }  // namespace tc

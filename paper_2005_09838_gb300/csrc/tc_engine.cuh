@@ -40,21 +40,22 @@ inline void slab_table(SlabFn<T> f[3]) {
 // Folded-transform slab kernels with TL rows / slices per item (the read-back
 // modes, one launch per call, take TL = 4).
 template <typename T, bool STAGED>
-inline SlabFn<T> pick_slab_g_st(int mode, int tl) {
+inline SlabFn<T> pick_slab_g_st(int mode, int tl, bool general) {
   if (mode == MODE_W) return k_slab_g<T, MODE_W, 4, STAGED>;
   if (mode == MODE_R) return k_slab_g<T, MODE_R, 4, STAGED>;
+  if (general) return tl == 2 ? k_slab_g<T, MODE_ITER, 2, STAGED, true> : k_slab_g<T, MODE_ITER, 4, STAGED, true>;
   return tl == 2 ? k_slab_g<T, MODE_ITER, 2, STAGED> : k_slab_g<T, MODE_ITER, 4, STAGED>;
 }
 template <typename T>
-inline SlabFn<T> pick_slab_g(int mode, int tl, bool staged) {
-  return staged ? pick_slab_g_st<T, true>(mode, tl) : pick_slab_g_st<T, false>(mode, tl);
+inline SlabFn<T> pick_slab_g(int mode, int tl, bool staged, bool general) {
+  return staged ? pick_slab_g_st<T, true>(mode, tl, general) : pick_slab_g_st<T, false>(mode, tl, general);
 }
 
 // The iteration's slab kernel with a tile of tl; nb: CTAs of the generic one that
 // an SM's shared memory holds.
 template <typename T>
-inline SlabFn<T> pick_slab_tile(bool folded, bool staged, int tl, int nb) {
-  if (folded) return pick_slab_g<T>(MODE_ITER, tl, staged);
+inline SlabFn<T> pick_slab_tile(bool folded, bool staged, int tl, int nb, bool general) {
+  if (folded) return pick_slab_g<T>(MODE_ITER, tl, staged, general);
   if (sizeof(T) == 4 && nb >= 3) return tl == 2 ? k_slab<T, MODE_ITER, 2, 3> : k_slab<T, MODE_ITER, 4, 3>;
   if (sizeof(T) == 4 && nb == 2) return tl == 2 ? k_slab<T, MODE_ITER, 2, 2> : k_slab<T, MODE_ITER, 4, 2>;
   return tl == 2 ? k_slab<T, MODE_ITER, 2> : k_slab<T, MODE_ITER, 4>;
@@ -288,8 +289,9 @@ class Engine final : public EngineBase {
       slabs_in_smem_ = true;
     } else if (SlabGPlan gp; !(p.precision == TC_BF16 && rp_ == 32) && slab_g_plan<T>(n2_, n3_, optin, gp)) {
       folded_ = true;
+      wgeneral_ = p.rho2 != 0.0 && wstep_strong(p.mu, p.rho2);
       d_.fold_sg = gp.sg;
-      for (int m = 0; m < 3; ++m) slab_[m] = pick_slab_g<T>(m, n3_ == 7 ? 2 : 4, gp.sg > 0);
+      for (int m = 0; m < 3; ++m) slab_[m] = pick_slab_g<T>(m, n3_ == 7 ? 2 : 4, gp.sg > 0, wgeneral_);
       slab_smem_ = gp.smem;
       slab_threads_ = gp.threads;
       slabs_in_smem_ = true;
@@ -316,6 +318,8 @@ class Engine final : public EngineBase {
       if (!err.empty()) return TC_ERR_NOMEM;
       d_.fold = fold_;
     }
+    T* wexc = folded_ ? alloc<T>((size_t)2 * n2_, err) : nullptr;
+    if (!err.empty()) return TC_ERR_NOMEM;
     if (fold_factors_) TC_CUDA_TRY(allow_fold_dft<T>(n3_));
 
     strict_ = sizeof(T) == 4 && (specialised_ || (p.precision == TC_BF16 && rp_ == 32));
@@ -443,6 +447,8 @@ class Engine final : public EngineBase {
       // W-step runs: inverse LU pivots by position in the run
       std::vector<T> w(6 * (size_t)n2_);
       wstep_tables<T>(w.data(), n2_, mu, rho2);
+      std::vector<T> wx(folded_ ? 2 * (size_t)n2_ : 0);
+      if (folded_) wstep_excess<T>(wx.data(), n2_, mu, rho2);
       // H_rho1 = I + rho1 H^T H: diagonal 1 + rho1 deg_i, off-diagonal -rho1
       std::vector<T> h(2 * (size_t)n1_);
       double hi = 0.0;
@@ -459,6 +465,7 @@ class Engine final : public EngineBase {
         tw[m] = cx<T>{(T)std::cos(a), (T)(-std::sin(a))};
       }
       TC_CUDA_TRY(cudaMemcpyAsync(winv, w.data(), w.size() * sizeof(T), cudaMemcpyHostToDevice, stream_));
+      if (folded_) TC_CUDA_TRY(cudaMemcpyAsync(wexc, wx.data(), wx.size() * sizeof(T), cudaMemcpyHostToDevice, stream_));
       TC_CUDA_TRY(cudaMemcpyAsync(hinv, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, stream_));
       TC_CUDA_TRY(cudaMemcpyAsync(twg, tw.data(), tw.size() * sizeof(cx<T>), cudaMemcpyHostToDevice, stream_));
       TC_CUDA_TRY(cudaStreamSynchronize(stream_));  // the host vectors go out of scope
@@ -486,6 +493,7 @@ class Engine final : public EngineBase {
     d_.Gp = Gp;
     d_.Tb = Tb;
     d_.winv = winv;
+    d_.wexc = wexc;
     d_.hinv = hinv;
     d_.twg = twg;
     d_.part = part;
@@ -895,7 +903,7 @@ class Engine final : public EngineBase {
     int pick = 0;
     cudaError_t e = cudaSuccess;
     for (int c = 0; c < 2 && e == cudaSuccess; ++c) {
-      slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[c], slab_nb_);
+      slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[c], slab_nb_, wgeneral_);
       e = allow_dynamic_smem((const void*)slab_[MODE_ITER], slab_smem_);
       float ms = 1e30f;
       for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
@@ -920,7 +928,7 @@ class Engine final : public EngineBase {
       poisoned_ = true;
       return TC_ERR_CUDA;
     }
-    slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[pick], slab_nb_);
+    slab_[MODE_ITER] = pick_slab_tile<T>(folded_, d_.fold_sg > 0, cand[pick], slab_nb_, wgeneral_);
     slab_tile_ = cand[pick];
     return TC_OK;
   }
@@ -1039,6 +1047,7 @@ class Engine final : public EngineBase {
   // compensate that sum (dcon_f_tile).
   bool strict_ = false;
   bool folded_ = false;  // folded-transform slab kernels (k_slab_g)
+  bool wgeneral_ = false;  // with the W-step of strong smoothing
   bool fold_factors_ = false;  // the factors' transforms too
   cx<T>* fold_ = nullptr;
   T* wrows_ = nullptr;   // W in row-major order (allocated by the first read-back)

@@ -44,6 +44,7 @@ struct Dev {
   double rtol64;    // pseudo-inverse cutoff of the FP64-accurate real-slice solves
   cx<T>* Tb;        // [S][3][r][n1] X-step work arrays when shared memory is too small
   const T* winv;    // [6][n2] W-step run tables (wstep_tables)
+  const T* wexc;    // [2][n2] excess ratios of the W-step pivots (wstep_excess; k_slab_g)
   const T* hinv;    // [2][n1] H_rho1 = I + rho1 H^T H: inverse pivots and rho1 * inverse pivots
   const cx<T>* twg; // [n3] exp(-2 pi i m / n3) for the generic transform
   int fold_sg;       // 64-tube groups per stage of k_slab_g (0: unstaged)

@@ -75,7 +75,7 @@ struct Carve {
 // Device-side construction of the FP64 tables (no host buffers): inverse LU
 // pivots of the W-step runs and of H_rho1, and the generic DFT twiddles.
 template <typename T>
-__global__ void k_static_tables(T* winv, T* hinv, cx<T>* twg, int n1, int n2, int n3, double mu, double rho1,
+__global__ void k_static_tables(T* winv, T* wexc, T* hinv, cx<T>* twg, int n1, int n2, int n3, double mu, double rho1,
                                 double rho2) {
   if (blockIdx.x == 0 && threadIdx.x == 0) wstep_tables<T>(winv, n2, mu, rho2);
   if (blockIdx.x == 1 && threadIdx.x == 0) {
@@ -87,6 +87,7 @@ __global__ void k_static_tables(T* winv, T* hinv, cx<T>* twg, int n1, int n2, in
       hinv[n1 + i] = (T)(rho1 * hi);
     }
   }
+  if (blockIdx.x == 3 && threadIdx.x == 0 && wexc) wstep_excess<T>(wexc, n2, mu, rho2);
   if (blockIdx.x == 2) {
     for (int m = threadIdx.x; m < n3; m += blockDim.x) {
       double s, c;
@@ -179,12 +180,16 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
   // the folded transform's tables take the rest; where that is too small, the
   // generic transform (which needs none) serves the problem as before
   cx<T>* fold = nullptr;
+  T* wexc = nullptr;
+  const bool strong = p.rho2 != 0.0 && wstep_strong(p.mu, p.rho2);
   if (folded && cv.off <= kStaticScratchBytes) {
     const size_t before = cv.off;
     fold = cv.take<cx<T>>(fold_table_entries(n3));
+    if (strong) wexc = cv.take<T>((size_t)2 * n2);
     if (cv.off > kStaticScratchBytes) {
       cv.off = before;
       folded = false;
+      wexc = nullptr;
     }
   }
   if (cv.off > kStaticScratchBytes) {
@@ -204,6 +209,7 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
   d.G = Gint;
   d.mask = maskbits;
   d.winv = winv;
+  d.wexc = wexc;
   d.hinv = hinv;
   d.twg = twg;
   d.yx_global = yxg ? 1 : 0;
@@ -216,7 +222,7 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
   size_t slab_smem = lay.total;
   int slab_threads = kSlabThreads;
   if (folded) {
-    for (int m = 0; m < 3; ++m) slab[m] = pick_slab_g<T>(m, n3 == 7 ? 2 : 4, gp.sg > 0);
+    for (int m = 0; m < 3; ++m) slab[m] = pick_slab_g<T>(m, n3 == 7 ? 2 : 4, gp.sg > 0, strong);
     slab_smem = gp.smem;
     slab_threads = gp.threads;
     d.fold = fold;
@@ -252,7 +258,7 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
     if (e != cudaSuccess)
       return sfail(TC_ERR_CUDA, std::string("clearing the device error flag failed: ") + cudaGetErrorString(e));
   }
-  k_static_tables<T><<<3, 256, 0, st>>>(winv, hinv, twg, n1, n2, n3, p.mu, p.rho1, p.rho2);
+  k_static_tables<T><<<4, 256, 0, st>>>(winv, wexc, hinv, twg, n1, n2, n3, p.mu, p.rho1, p.rho2);
   if (folded) k_fold_tables<T><<<2 * 152, 256, 0, st>>>(fold, twg, n3);
   k_pack<T><<<pack_grid(n1, n2, n3), kTileThreads, 0, st>>>(static_cast<const T*>(G), mask, Gint, maskbits, n1, n2, n3, mw);
   k_factor_dft<T><<<fgrid, 256, 0, st>>>(static_cast<const T*>(Y0), d.Yt, n2, r, n3, 1, twg);
