@@ -50,6 +50,24 @@ inline dim3 pack_grid(int n1, int n2, int n3) {
   return dim3((unsigned)(((n1 + 31) / 32) * ((n2 + 31) / 32)), (unsigned)n3);
 }
 
+// Slabs (i1) with a run of kWChoice or more missing entries, counted in *count.
+// Grid n1, a thread per row.
+template <typename T>
+__global__ void __launch_bounds__(128) k_long_runs(const uint32_t* __restrict__ mask, int n2, int n3, int mw, int* count) {
+  bool lng = false;
+  for (int l = threadIdx.x; l < n3; l += blockDim.x) {
+    const uint32_t* row = mask + ((size_t)blockIdx.x * n3 + l) * mw;
+    int run = 0;  // missing entries that end at the word
+    for (int w = 0; w < mw; ++w) {
+      const int nb = min(32, n2 - 32 * w);
+      const uint32_t m = row[w];
+      lng |= run + (m ? __ffs(m) - 1 : nb) >= kWChoice<T>;  // (a run inside the word is shorter)
+      run = m ? nb - 32 + __clz(m) : run + nb;
+    }
+  }
+  if (__syncthreads_or(lng) && threadIdx.x == 0) atomicAdd(count, 1);
+}
+
 // Row-major [i1][i3][i2] -> column-major.
 template <typename T>
 __global__ void __launch_bounds__(kTileThreads) k_unpack(const T* __restrict__ in, T* __restrict__ out, int n1, int n2,

@@ -244,8 +244,14 @@ __device__ void wstep_sweeps(T* __restrict__ col, int LP, const uint32_t* __rest
 //   item: this thread's (row, segment) index, row = item % nrows, segment =
 //         item / nrows; items >= nrows * nseg only join the barriers
 //   col(l): the row's first entry; rows are strided by LP along j
+// SEQ: a row with a run of missing words over more than half of it is left to
+// its first thread and the sequential sweeps: the carries of its segments walk the
+// run at twice their cost per entry (slab kernel with a tenth of the rows missing:
+// 32 x 2000 x 12 FP64 1046 -> 713 us, 702 with all rows sequential; 150 x 205 x 34
+// BF16 61 -> 55; with 85 registers to a thread the sweeps spill: 435 x 205 x 34
+// 108 -> 115, so not there).
 // ---------------------------------------------------------------------------
-template <typename T, typename ColFn>
+template <typename T, bool SEQ, typename ColFn>
 __device__ void wstep_sweeps_seg(ColFn col_of, int LP, const uint32_t* __restrict__ msk, int* __restrict__ stw,
                                  int nrows, int nseg, int item, int n2, T rho2, const T* __restrict__ wtab) {
   const int words = (n2 + 31) >> 5;
@@ -254,10 +260,18 @@ __device__ void wstep_sweeps_seg(ColFn col_of, int LP, const uint32_t* __restric
   const bool active = item < nrows * nseg;
   const int l = active ? item % nrows : 0, sg = active ? item / nrows : 0;
   const int w0 = min(sg * wps, words), w1 = min(w0 + wps, words);
-  const bool work = active && w0 < w1;
   T* col = col_of(l);
   const uint32_t* rowm = msk + (size_t)l * ((n2 + 31) >> 5);
   int* rowst = stw + (size_t)l * ((n2 + 31) >> 5);
+  bool seq = false;
+  if (SEQ && nseg > 1 && active) {
+    for (int w = 0, run = 0; w < words; ++w) {
+      run = rowm[w] ? 0 : run + 1;
+      seq |= 2 * run > words;
+    }
+    if (seq && sg == 0) wstep_sweeps<T>(col, LP, rowm, rowst, n2, rho2, wtab);
+  }
+  const bool work = active && w0 < w1 && !seq;
   auto bit = [&](int j) { return (rowm[j >> 5] >> (j & 31)) & 1u; };
 
   // ---- forward carry: d_{j0 - 1} and the run start entering word w0 -------------------
@@ -333,8 +347,19 @@ __device__ void wstep_sweeps_seg(ColFn col_of, int LP, const uint32_t* __restric
 //          excess ratios of the two pivots, h_c + c h_e: the difference loses the digits
 //          (FP32, a row of 100 missing entries, mu = 1e-3: 6e-4 of W at rho2 = 1e6
 //          and 3e-2 at 1e8, against 2e-7 and 4e-7 of the sequential sweeps).
-// The excess ratios are the GENERAL form, which the engine takes where rho2 asks for
-// it (wstep_strong).
+// Both walk the run's entries, a few for scattered observations.  In a run of
+// kWLong entries or more (a row or day without data) every segment that lies in
+// it whole first leaves its part of the two recurrences, d -> a d + b, in its own
+// slots of the slab (its values are in registers), and the walks take a segment
+// per step: a row of n2 missing entries costs each of its threads some n2 / kWSeg
+// steps, where walking the entries cost them n2 (slab kernel with a tenth of the
+// rows missing: 60 x 144 x 30 FP64 194 -> 92 us, 32 x 3000 x 10 FP32 272 -> 84; with
+// none 70 and 48).
+// The further barrier, the values held across it and the excess ratios are the
+// GENERAL form, 5% of the slab kernel where no run is long.  The engine takes it
+// where rho2 asks for it (wstep_strong) or at least a quarter of the slabs have a
+// run of kWChoice entries, which masks with 10% or more observed at random don't
+// (FP32; FP64, where a step is the dearer, has it earlier).
 // Fewer than half the instructions of the two sweeps over shared memory (no
 // second pass over the values, the table and the mask).  FP32 segments of 16 keep
 // the thread within 64 registers; in FP64, where a warp instruction holds its scheduler's pipe for
@@ -343,6 +368,10 @@ __device__ void wstep_sweeps_seg(ColFn col_of, int LP, const uint32_t* __restric
 // ---------------------------------------------------------------------------
 template <typename T>
 constexpr int kWSeg = sizeof(T) == 8 ? 8 : 16;
+template <typename T>
+constexpr int kWLong = 4 * kWSeg<T>;
+template <typename T>
+constexpr int kWChoice = sizeof(T) == 8 ? 64 : 192;
 
 // Start of the run of missing entries that reaches entry `base` from the left, and
 // end (one past its last entry) of the one that reaches entry j1 - 1 from the right.
@@ -359,16 +388,44 @@ __device__ __forceinline__ int run_end(const uint32_t* __restrict__ rowm, int wo
   return m ? 32 * u + __ffs(m) - 1 : n2;
 }
 
+// A whole segment inside a long run: the forward recurrence over it as d -> a d + b
+// in its first two slots, the one from the run's other end in the next two.
+template <typename T, int SEG>
+__device__ __forceinline__ void wstep_publish(T* __restrict__ col, int LP, int base, int st, int k, int n2, T rho2,
+                                              const T* __restrict__ wtab, const T (&v)[SEG]) {
+  const T* tf = wtab + (st == 0 ? 0 : n2) + base - st;
+  const T* tr = wtab + (k < n2 ? n2 : 0) + k - 1 - base;
+  T a = T(1), b = T(0), e = T(1), f = T(0);
+#pragma unroll
+  for (int q = 0; q < SEG; ++q) {
+    const T inv = tf[q], c = rho2 * inv;
+    a *= c;
+    b = fma(c, b, v[q] * inv);
+  }
+#pragma unroll
+  for (int q = SEG - 1; q >= 0; --q) {
+    const T inv = tr[-q], c = rho2 * inv;
+    e *= c;
+    f = fma(c, f, v[q] * inv);
+  }
+  T* o = col + base * LP;
+  o[0] = a;
+  o[LP] = b;
+  o[2 * LP] = e;
+  o[3 * LP] = f;
+}
+
 // Whether c e can reach 1/2: the largest coefficient is that of a run's first entry
 // at the row's start, rho2 / (1 + mu + rho2), whose square is below 4/9 up to here.
 inline bool wstep_strong(double mu, double rho2) { return rho2 > 2.0 * (1.0 + mu); }
-// GENERAL: any rho2.
+// GENERAL: the whole segments of long runs have published theirs; any rho2.
 template <typename T, int SEG, bool FULL, bool LAST, bool GENERAL>
 __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP, const uint32_t* __restrict__ rowm,
-                                              int words, int sgm, int qn, int n2, T rho2,
+                                              int words, int segs, int sgm, int qn, int n2, T rho2,
                                               const T* __restrict__ wtab, const T* __restrict__ hex, T (&v)[SEG]) {
   const int base = SEG * sgm, j1 = base + SEG;
   const uint32_t word = rowm[base >> 5], mw = word >> (base & 31);
+  const uint32_t mb = mw & ((1u << SEG) - 1u);  // (bits past n2 are 0)
   int st = 0;  // start of the run of missing entries that enters the segment
   T d = T(0);
   if (base > 0) {
@@ -376,10 +433,17 @@ __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP,
     if (!(mw & 1u)) {
       if (st > 0) d = col[(st - 1) * LP];
       const T* tb = wtab + (st == 0 ? 0 : n2);
-      for (int j = st; j < base; ++j) {
+      int jf = base;  // entries up to here, then segments
+      if (GENERAL && base - st >= SEG) {
+        const int k = mb ? base + __ffs(mb) - 1 : (LAST ? n2 : run_end(rowm, words, j1, n2));
+        if (k - st >= kWLong<T>) jf = (st + SEG - 1) / SEG * SEG;
+      }
+      for (int j = st; j < jf; ++j) {
         const T inv = tb[j - st];
         d = fma(rho2 * inv, d, col[j * LP] * inv);
       }
+      if (GENERAL)
+        for (int j = jf; j < base; j += SEG) d = fma(col[j * LP], d, col[(j + 1) * LP]);
     }
   }
   // table position of the entry: one further per missing entry, the start of the
@@ -406,10 +470,17 @@ __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP,
     const int k = run_end(rowm, words, j1, n2);  // next observed entry, or the row's end
     T x = (k < n2) ? col[k * LP] : T(0);
     const int tb = k < n2 ? n2 : 0;
-    for (int j = k - 1; j >= j1; --j) {
+    int jl = j1;  // entries down to here, then segments
+    if (GENERAL && k - j1 >= SEG) {
+      const int s0 = mb ? base + 32 - __clz(mb) : st;
+      if (k - s0 >= kWLong<T>) jl = max(j1, min(k / SEG, segs - 1) * SEG);
+    }
+    for (int j = k - 1; j >= jl; --j) {
       const T inv = wtab[tb + k - 1 - j];
       x = fma(rho2 * inv, x, col[j * LP] * inv);
     }
+    if (GENERAL)
+      for (int j = jl - SEG; j >= j1; j -= SEG) x = fma(col[(j + 2) * LP], x, col[(j + 3) * LP]);
     wn = fma(c[SEG - 1], x, v[SEG - 1]);
     if (k > j1) {
       const int p1 = tb + k - 1 - j1;
@@ -456,10 +527,19 @@ __device__ __forceinline__ void wstep_segments(ColFn col_of, int LP, const uint3
           if (q < ql) v[q] = cb[q * LP];
       }
     }
+    if constexpr (GENERAL) {
+      const int base = SEG * w;
+      const uint32_t word = work ? rowm[base >> 5] : 0u;
+      if (work && w < segs - 1 && ((word >> (base & 31)) & ((1u << SEG) - 1u)) == 0u) {
+        const int st = run_start(rowm, base, word), k = run_end(rowm, words, base + SEG, n2);
+        if (k - st >= kWLong<T>) wstep_publish<T, SEG>(col, LP, base, st, k, n2, rho2, wtab, v);
+      }
+      __syncthreads();
+    }
     if (work) {
       if (w < segs - 1)
-        wstep_segment<T, SEG, true, false, GENERAL>(col, LP, rowm, words, w, SEG, n2, rho2, wtab, hex, v);
-      else wstep_segment<T, SEG, false, true, GENERAL>(col, LP, rowm, words, w, ql, n2, rho2, wtab, hex, v);
+        wstep_segment<T, SEG, true, false, GENERAL>(col, LP, rowm, words, segs, w, SEG, n2, rho2, wtab, hex, v);
+      else wstep_segment<T, SEG, false, true, GENERAL>(col, LP, rowm, words, segs, w, ql, n2, rho2, wtab, hex, v);
     }
     __syncthreads();
     if (work) {
@@ -633,7 +713,7 @@ __global__ void __launch_bounds__(kSlabThreads, NB)
   }
   if (wsolve) {
     if (n3 <= nt) {  // every thread one (row, segment)
-      wstep_sweeps_seg<T>([&](int l) { return spat + l; }, LP, msk, stw, n3, nt / n3, tid, n2, d.rho2, wtab);
+      wstep_sweeps_seg<T, (NB <= 2)>([&](int l) { return spat + l; }, LP, msk, stw, n3, nt / n3, tid, n2, d.rho2, wtab);
     } else {
       for (int l = tid; l < n3; l += nt)
         wstep_sweeps<T>(spat + l, LP, msk + l * mwords, stw + l * mwords, n2, d.rho2, wtab);

@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(MODE == MODE_ITER ? kSlabFThreads : kSlabFAux,
   // ---- W-step ----------------------------------------------------------------------------------
   if (wsolve) {
     // rows split into segments so that every thread has one (row, segment)
-    wstep_sweeps_seg<T>([&](int q) { return buf + q; }, LP, msk, stw, L, max(1, nt / L), tid, n2, d.rho2, wtab);
+    wstep_sweeps_seg<T, false>([&](int q) { return buf + q; }, LP, msk, stw, L, max(1, nt / L), tid, n2, d.rho2, wtab);
   }
 
   // ---- C1: forward DFT_N2 over slots N2 k1 + j, twiddle w_M^{k1 q} -----------------------

@@ -840,9 +840,9 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold_idft(const cx<T>* __restr
   else fold_idft_impl<T, true>(in, out, fold, n, r, n3, transposed, smem);
 }
 
-// GENERAL (MODE_ITER): the W-step of strong smoothing (see wstep_segments), chosen by
-// the engine; as a branch of one kernel it cost the plain form 5%
-// (925 x 153 x 92: 150 -> 160 us, in spills).
+// GENERAL (MODE_ITER): the W-step of long runs and strong smoothing (see
+// wstep_segments), chosen by the engine; as a branch of one kernel it cost the plain
+// form 5% (925 x 153 x 92: 150 -> 160 us, in spills).
 template <typename T, int MODE, int TL, bool STAGED, bool GENERAL = false>
 __global__ void __launch_bounds__(kSlabGThreads<T>, GENERAL && sizeof(T) == 8 ? 2 : 1) k_slab_g(Dev<T> d, T* __restrict__ Wout, int flags, int init) {
   extern __shared__ __align__(16) unsigned char smem[];

@@ -265,7 +265,7 @@ class Engine final : public EngineBase {
     cx<T>* twg = alloc<cx<T>>((size_t)n3_, err);
     double* part = alloc<double>((size_t)n1_ * 4, err);
     double* part_k = alloc<double>((size_t)S_ * kRhoChunks, err);
-    int* derr = alloc<int>(1, err);
+    int* derr = alloc<int>(2, err);  // error word, slabs with a long run of missing entries
     // stopping test (eps > 0): change maxima, flag, counter; |dW| partial sums; Z~ changes
     unsigned long long* conv = nullptr;
     double* part_dw = nullptr;
@@ -512,7 +512,7 @@ class Engine final : public EngineBase {
     d_.part_dw = part_dw;
     d_.dZt = dZt;
     d_.eps = p.eps;
-    TC_CUDA_TRY(cudaMemsetAsync(derr, 0, sizeof(int), stream_));
+    TC_CUDA_TRY(cudaMemsetAsync(derr, 0, 2 * sizeof(int), stream_));
 
     // ---- inputs --------------------------------------------------------------------------
     const T* dG = static_cast<const T*>(G);
@@ -540,6 +540,8 @@ class Engine final : public EngineBase {
       }
     }
     k_pack<T><<<pack_grid(n1_, n2_, n3_), kTileThreads, 0, stream_>>>(dG, dM, Gint, maskbits, n1_, n2_, n3_, mw_);
+    if (folded_ && !wgeneral_ && p.rho2 != 0.0 && n2_ >= kWChoice<T>)
+      k_long_runs<T><<<n1_, 128, 0, stream_>>>(maskbits, n2_, n3_, mw_, derr + 1);
     if (fold_) k_fold_tables<T><<<2 * 152, 256, 0, stream_>>>(fold_, twg, n3_);
     const cx<T>* ffold = fold_factors_ && !strict_ ? fold_ : nullptr;
     launch_factor_dft<T>(dY, Yt, ffold, twg, n2_, r_, n3_, 1, stream_);
@@ -568,8 +570,14 @@ class Engine final : public EngineBase {
       poisoned_ = true;
       return TC_ERR_CUDA;
     }
-    tc_status st = check_dev_err(err);
+    int lrows = 0;  // slabs with a long run
+    tc_status st = check_dev_err(err, &lrows);
     if (st != TC_OK) return st;
+    if (folded_ && !wgeneral_ && 4 * (long long)lrows >= n1_ && lrows > 0) {
+      wgeneral_ = true;
+      slab_[MODE_ITER] = pick_slab_g<T>(MODE_ITER, slab_tile_ > 0 ? slab_tile_ : 2, d_.fold_sg > 0, true);
+      TC_CUDA_TRY(allow_dynamic_smem((const void*)slab_[MODE_ITER], slab_smem_));
+    }
     // the iteration graph is built and uploaded here, so that tc_iterate only
     // launches it
     st = capture(err);
@@ -1019,12 +1027,14 @@ class Engine final : public EngineBase {
     return TC_OK;
   }
 
-  tc_status check_dev_err(std::string& err) {
-    int h = 0;
-    TC_CUDA_TRY(cudaMemcpyAsync(&h, d_.err, sizeof(int), cudaMemcpyDeviceToHost, stream_));
+  // second: receives the word after the error word
+  tc_status check_dev_err(std::string& err, int* second = nullptr) {
+    int h[2] = {0, 0};
+    TC_CUDA_TRY(cudaMemcpyAsync(h, d_.err, (second ? 2 : 1) * sizeof(int), cudaMemcpyDeviceToHost, stream_));
     TC_CUDA_TRY(cudaStreamSynchronize(stream_));
-    if (h != DEV_OK) {
-      err = "device-side check failed (code " + std::to_string(h) + ")";
+    if (second) *second = h[1];
+    if (h[0] != DEV_OK) {
+      err = "device-side check failed (code " + std::to_string(h[0]) + ")";
       poisoned_ = true;
       return TC_ERR_CUDA;
     }
@@ -1047,7 +1057,7 @@ class Engine final : public EngineBase {
   // compensate that sum (dcon_f_tile).
   bool strict_ = false;
   bool folded_ = false;  // folded-transform slab kernels (k_slab_g)
-  bool wgeneral_ = false;  // with the W-step of strong smoothing
+  bool wgeneral_ = false;  // with the W-step of long runs and strong smoothing
   bool fold_factors_ = false;  // the factors' transforms too
   cx<T>* fold_ = nullptr;
   T* wrows_ = nullptr;   // W in row-major order (allocated by the first read-back)

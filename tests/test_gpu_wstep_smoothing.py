@@ -40,3 +40,28 @@ def test_missing_rows(n3, rho2):
     for i in (0, 1, slice(None)):
         rel = np.linalg.norm(got["W"][i] - ref["W"][i]) / np.linalg.norm(ref["W"][i])
         assert rel <= 1e-5, (i, rel)
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-10), ("fp32", 1e-5)])
+@pytest.mark.parametrize("rho2", [0.1, 3.0])
+@pytest.mark.parametrize("n2", [128, 129, 175, 200])
+def test_runs_around_segment_edges(n2, rho2, precision, tol):
+    # runs of missing entries from every offset within two segments, of lengths
+    # around those from which the segments of a run are taken whole, and in a third
+    # of the slabs a row without data
+    from paper_2005_09838_gb300 import api
+    w = wl.custom(48, n2, 9, 2, 0.5, seed=8320 + n2, iters=2)
+    inst = wl.generate(w)
+    lengths = (15, 16, 17, 31, 32, 33, 47, 63, 64, 65, 80, 96, n2)
+    for i in range(48):
+        for l in range(9):
+            n = n2 if l == 4 and i % 3 == 0 else lengths[(9 * i + l) % len(lengths)]
+            a = i if i < 40 and n < n2 else max(0, n2 - n)  # (the last slabs: runs that end with the row)
+            inst["mask"][i, a:a + n, l] = False
+    inst["G"] = np.where(inst["mask"], inst["M"], 0.0)
+    if precision == "fp32":
+        inst = wl.as_precision(inst, np.float32)
+    ref = O.tctf2r(inst["G"], inst["mask"], 2, 1e-3, 1e-3, rho2, inst["Y0"], iters=2)
+    got = api.complete(inst["G"], inst["mask"], inst["Y0"], 2, 2, 1e-3, 1e-3, rho2, precision)
+    rel = np.linalg.norm(got["W"] - ref["W"]) / np.linalg.norm(ref["W"])
+    assert rel <= tol, rel
