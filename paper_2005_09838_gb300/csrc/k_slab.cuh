@@ -578,8 +578,10 @@ __device__ __forceinline__ double dw_term(cx<T> rnew, cx<T> rold, cx<T> dz, int 
 // [i1][n3][ceil(n2/32)] (written by k_pack), copied to shared memory.
 // ---------------------------------------------------------------------------
 // NB: CTAs per SM to leave registers for, as many as the slab's shared memory
-// allows (the sweeps alone take 255 registers, one CTA of 8 warps per SM; at 85 and
-// three CTAs the iteration of 435 x 205 x 34 went from 223 to 180 us).
+// and the grid allow (the sweeps alone take 255 registers, one CTA of 8 warps per SM;
+// at 85 and three CTAs the iteration of 435 x 205 x 34 went from 223 to 180 us, but
+// with fewer slabs than that the smaller budget only costs: 64 x 600 x 112 FP32
+// 767 -> 806 us, 300 x 205 x 34 BF16 145 -> 161).
 template <typename T, int MODE, int TL = kTL, int NB = 1>
 __global__ void __launch_bounds__(kSlabThreads, NB)
     k_slab(Dev<T> d, T* __restrict__ Wout, int flags, int init) {

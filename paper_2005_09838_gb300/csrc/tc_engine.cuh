@@ -239,7 +239,8 @@ class Engine final : public EngineBase {
     rp_ = pad_rank<T>(r_);
     const size_t N = (size_t)n1_ * n2_ * n3_;
     TC_CUDA_TRY(cudaGetDevice(&device_));
-    int optin = 0;
+    int optin = 0, nsm = 0;
+    TC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device_));
     TC_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device_));
     optin -= kStaticSmemReserve;  // room for the kernels' static shared memory
 
@@ -307,7 +308,8 @@ class Engine final : public EngineBase {
         d_.scratch = scratch;
       }
       slab_smem_ = lay.total;
-      slab_nb_ = (int)((size_t)(optin + kStaticSmemReserve + 1024) / (slab_smem_ + 1024));
+      // CTAs that an SM's shared memory holds and that the grid gives it
+      slab_nb_ = std::min((int)((size_t)(optin + kStaticSmemReserve + 1024) / (slab_smem_ + 1024)), (n1_ + nsm - 1) / nsm);
     }
     for (int m = 0; m < 3; ++m)
       TC_CUDA_TRY(allow_dynamic_smem((const void*)slab_[m], slab_smem_));
@@ -396,8 +398,6 @@ class Engine final : public EngineBase {
     qgrid_ = dim3(S_, (n1_ + d_.qrows - 1) / d_.qrows);
     // compensated D on the real slices (the tiled kernels, the fused Y-step, the split TF32 form)
     d_.dpairs = !strict_ && !(mixed_ && rp_ == 32 && (p.precision == TC_BF16 || (p.flags & TC_FLAG_SINGLE_PASS)));
-    int nsm = 0;
-    TC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device_));
     if (mixed_ && rp_ == 32 && pick_tc<T>(p.precision, (p.flags & TC_FLAG_SINGLE_PASS) == 0, tck_)) {
       tcy_ = true;
       qgrid_ = dim3(S_, (n1_ + 127) / 128);
