@@ -236,7 +236,13 @@ __global__ void __launch_bounds__(256) k_rho1_term(Dev<T> d) {
   const int n1 = d.n1, n2 = d.n2;
   const size_t rs = (size_t)d.S * n2;  // distance between rows i and i + 1 of slice k
   const cx<T>* Z = d.Zt + (size_t)k * n2;
+  // (FP64: squares and sums with their rounding errors)
+  SqSum<T> sum;
   T s = T(0), c = T(0);
+  auto add = [&](T v) {
+    if constexpr (sizeof(T) == 4) sum.add(v);
+    else dot2(s, c, v, v);
+  };
   const int nd = n1 > 1 ? n1 - 1 : 0, per = (nd + kRhoChunks - 1) / kRhoChunks;
   const int i0 = min(ch * per, nd), i1 = min(i0 + per, nd);
   // a thread walks down column j through the chunk's rows, keeping the previous
@@ -251,27 +257,27 @@ __global__ void __launch_bounds__(256) k_rho1_term(Dev<T> d) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const cx<T> a = nx[q] - prev;
-        dot2(s, c, a.re, a.re);
-        dot2(s, c, a.im, a.im);
+        add(a.re);
+        add(a.im);
         prev = nx[q];
       }
     }
     for (; i < i1; ++i) {
       const cx<T> cur = Z[(size_t)(i + 1) * rs + j];
       const cx<T> a = cur - prev;
-      dot2(s, c, a.re, a.re);
-      dot2(s, c, a.im, a.im);
+      add(a.re);
+      add(a.im);
       prev = cur;
     }
   }
-  double tot_d = warp_sum((double)s + (double)c);
+  double tot_d = warp_sum(sum.total() + ((double)s + (double)c));
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (lane == 0) part[wid] = tot_d;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double sum = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += part[w];
-    d.part_k[(size_t)k * kRhoChunks + ch] = sum;
+    double tot = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += part[w];
+    d.part_k[(size_t)k * kRhoChunks + ch] = tot;
   }
 }
 

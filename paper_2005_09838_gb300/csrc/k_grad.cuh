@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(256) k_grad_rho1(Dev<T> d) {
   const bool real = k == 0 || 2 * k == d.n3;
   const T rho1 = d.rho1;
   const int per = (n1 + kRhoChunks - 1) / kRhoChunks, i0 = min(ch * per, n1), i1 = min(i0 + per, n1);
-  SqSum<T> sum;
+  T s = T(0), c = T(0);  // (dot2, as in k_rho1_term)
   constexpr int U = 4;  // rows in flight
   for (int j = threadIdx.x; j < n2 && i0 < i1; j += blockDim.x) {
     cx<T> cur = Z[(size_t)i0 * rs + j];
@@ -111,8 +111,8 @@ __global__ void __launch_bounds__(256) k_grad_rho1(Dev<T> d) {
         cx<T> dn = {T(0), T(0)};  // z_{i+1} - z_i
         if (i + q + 1 < n1) {
           dn = nx[q] - cur;
-          sum.add(dn.re);
-          sum.add(dn.im);
+          dot2(s, c, dn.re, dn.re);
+          dot2(s, c, dn.im, dn.im);
         }
         if (WRITE) {
           const cx<T> h = up - dn;
@@ -123,14 +123,14 @@ __global__ void __launch_bounds__(256) k_grad_rho1(Dev<T> d) {
       }
     }
   }
-  const double tot = warp_sum(sum.total());
+  const double tot = warp_sum((double)s + (double)c);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (lane == 0) part[wid] = tot;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[w];
-    d.part_k[(size_t)k * kRhoChunks + ch] = s;
+    double sum = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += part[w];
+    d.part_k[(size_t)k * kRhoChunks + ch] = sum;
   }
 }
 

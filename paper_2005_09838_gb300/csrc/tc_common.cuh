@@ -156,27 +156,66 @@ __device__ __forceinline__ void pair_add(T& s, T& c, T s2, T c2) {
   s = t;
 }
 
-// Sum of squares of a thread's values to FP64 accuracy.  FP32 values: error-free
-// products and sums on the FP32 pipe (dot2); GB300 issues one FP64 warp
-// instruction per scheduler in about 60 clocks, and the FP64 form (a conversion
-// and a multiply-add per value) took more than half of the read-back kernels.
+// (s, e) <- s + a and the rounding error of it (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float& s, float a) {
+  const float t = s + a, z = t - s, e = (s - (t - z)) + (a - z);
+  s = t;
+  return e;
+}
+
+// The FP64 form of an FP32 term of SqSum, out of line: GB300 issues one FP64 warp
+// instruction per scheduler in about 60 clocks, predicated off or not, and a call
+// is not turned into predicated code.
+static __device__ __noinline__ double sq_diff64(double s, float a, float b) {
+  const double v = (double)a - (double)b;
+  return fma(v, v, s);
+}
+
+// Sum of squares of a thread's values, no less accurate than FP64 additions.
+// FP32 values within 2^+-48 (and 0): every square is taken with its rounding error
+// and added without one to three FP32 words (error some 2^-70 of the sum), on the
+// FP32 pipe; an FP64 conversion and multiply-add per value took more than half of
+// the read-back kernels.  Outside that range a square or its rounding error could
+// leave FP32's: those terms are added in FP64.
 template <typename T>
 struct SqSum {
-  T s = T(0), c = T(0);
-  __device__ __forceinline__ void add(T v) {
-    if constexpr (sizeof(T) == 8) s = fma(v, v, s);
-    else dot2(s, c, v, v);
+  T s = T(0);
+  __device__ __forceinline__ void add(T v) { s = fma(v, v, s); }
+  __device__ __forceinline__ void add_diff(T a, T b) { add(a - b); }
+  __device__ __forceinline__ double total() const { return s; }
+};
+template <>
+struct SqSum<float> {
+  float s = 0.f, c = 0.f, e = 0.f;
+  double far = 0.0;
+  __device__ __forceinline__ static bool near(float v) {
+    const float m = fabsf(v);
+    return (m >= 0x1p-48f && m <= 0x1p48f) || m == 0.f;
   }
-  // (a - b)^2, the difference not rounded
-  __device__ __forceinline__ void add_diff(T a, T b) {
-    const T h = a - b;
-    add(h);
-    if constexpr (sizeof(T) == 4) {
-      const T z = h - a;
-      c = fma(T(2) * h, (a - (h - z)) - (b + z), c);
+  __device__ __forceinline__ void term(float a) { e += two_sum(c, a); }  // a: of the size of a rounding error
+  __device__ __forceinline__ void add(float v) {
+    if (near(v)) {
+      const float p = mul_rn(v, v), pe = fmaf(v, v, -p);
+      term(two_sum(s, p));
+      term(pe);
+    } else {
+      far = sq_diff64(far, v, 0.f);
     }
   }
-  __device__ __forceinline__ double total() const { return (double)s + (double)c; }
+  // (a - b)^2 of the difference as it is, not rounded: h + z
+  __device__ __forceinline__ void add_diff(float a, float b) {
+    const float h = a - b;
+    if (near(h)) {
+      const float w = h - a, z = (a - (h - w)) - (b + w);
+      const float q = mul_rn(2.f * h, z), qe = fmaf(2.f * h, z, -q);
+      add(h);
+      term(q);
+      e += fmaf(z, z, qe);
+    } else {
+      far = sq_diff64(far, a, b);
+    }
+  }
+  __device__ __forceinline__ double total() const { return (double)s + (double)c + (double)e + far; }
 };
 
 // A truth value as a type, for generic lambdas.
