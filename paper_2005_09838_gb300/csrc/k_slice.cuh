@@ -1555,8 +1555,11 @@ __global__ void __launch_bounds__(xstep_threads(RP), 1) k_xstep(Dev<T> d, const 
   // Dg = -X~'^H ((X~' - X~) + rho1 H^T H X~'), the right factors formed once per entry
   // (over Q and X~, both done with): four FP64 operations per product of either where
   // the form below takes sixteen for the three sums (121 x 144 x 7, r = 4: 41 -> 30 us
-  // for the whole X-step)
-  if (sizeof(T) == 8 && arrays_in_smem) {
+  // for the whole X-step).  A stencil of smooth columns cancels where their
+  // differences do not: its rounding errors, rho1 times as large as those of X~'^H X~',
+  // are no more than them up to rho1 = 1 (n1 = 60, r = 3 and 4: the error of X~'Y~'
+  // doubles at rho1 = 1e4 and more), and the form below takes over.
+  if (sizeof(T) == 8 && arrays_in_smem && rho1 <= T(1)) {
     for (int e = tid; e < r * n1; e += blockDim.x) {
       const int s = e / n1, i = e - s * n1;
       const cx<T> x = Ts[e], h = hth_at(Ts + (size_t)s * n1, i, n1);
