@@ -68,10 +68,10 @@ __global__ void __launch_bounds__(128) k_long_runs(const uint32_t* __restrict__ 
   if (__syncthreads_or(lng) && threadIdx.x == 0) atomicAdd(count, 1);
 }
 
-// Row-major [i1][i3][i2] -> column-major.
+// Row-major [i1][i3][i2] of n1 rows i1 -> column-major with ld of them.
 template <typename T>
-__global__ void __launch_bounds__(kTileThreads) k_unpack(const T* __restrict__ in, T* __restrict__ out, int n1, int n2,
-                                                         int n3) {
+__global__ void __launch_bounds__(kTileThreads) k_unpack(const T* __restrict__ in, T* __restrict__ out, int n1, int ld,
+                                                         int n2, int n3) {
   __shared__ T g[32][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nt2 = (n2 + 31) / 32;
   const int l = blockIdx.y, i0 = (blockIdx.x / nt2) * 32, t0 = (blockIdx.x % nt2) * 32;
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kTileThreads) k_unpack(const T* __restrict__ i
 #pragma unroll
   for (int q = w; q < 32; q += kTileThreads / 32)
     if (i0 + lane < n1 && t0 + q < n2)
-      out[(size_t)(i0 + lane) + (size_t)n1 * ((size_t)(t0 + q) + (size_t)n2 * l)] = g[lane][q];
+      out[(size_t)(i0 + lane) + (size_t)ld * ((size_t)(t0 + q) + (size_t)n2 * l)] = g[lane][q];
 }
 
 // Direct DFT (Eq. (bar BA-k), forward sign convention of the library) of a

@@ -17,7 +17,7 @@ enum SlabMode : int { MODE_ITER = 0, MODE_W = 1, MODE_R = 2, MODE_GRAD = 3 };
 // Launch flags of the slab kernels: the slab lives in shared memory (else in
 // d.scratch; k_slab only), and MODE_W writes Wout in the row-major order
 // [i1][i3][i2] (one CTA then writes whole rows; k_unpack brings it to the
-// caller's column-major order) instead of the column-major one.
+// caller's column-major order; not k_slab) instead of the column-major one.
 // SLAB_NOSUM: MODE_W forms no sums.
 enum SlabFlag : int { SLAB_IN_SMEM = 1, SLAB_WROWS = 2, SLAB_NOSUM = 4 };
 
@@ -695,10 +695,7 @@ __global__ void __launch_bounds__(kSlabThreads, NB)
       if (sums) sa.add(v);
       if (MODE == MODE_W) {
         if (sums && j + 1 < n2) sb.add_diff(v, spat[(j + 1) * LP + l]);
-        if (Wout) {
-          if (flags & SLAB_WROWS) Wout[((size_t)i1 * n3 + l) * n2 + j] = v;
-          else Wout[(size_t)i1 + (size_t)n1 * ((size_t)j + (size_t)n2 * l)] = v;
-        }
+        if (Wout) Wout[(size_t)i1 + (size_t)n1 * ((size_t)j + (size_t)n2 * l)] = v;
       } else {
         if ((msk[l * mwords + (j >> 5)] >> (j & 31)) & 1u) sb.add(v);
       }

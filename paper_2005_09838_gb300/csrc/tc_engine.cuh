@@ -206,6 +206,12 @@ inline QFn<T> pick_qcon(int rp) {
   }
 }
 
+// Row buffer of tc_result: its size (925 x 153 x 92 in one part 143 us, in parts of
+// 32 MiB 173, without the buffer 159; 529 x 288 x 168 205, 232 and 241), and the bytes of
+// W from which it pays (16 x 48 x 7 38 us with, 33 without; 121 x 144 x 7 FP64 39 and 35; 64 x
+// 96 x 60, 1.4 MB, 41 and 42).
+constexpr size_t kRowsBytes = size_t(128) << 20, kRowsMin = size_t(1) << 20;
+
 template <typename T>
 class Engine final : public EngineBase {
  public:
@@ -313,6 +319,16 @@ class Engine final : public EngineBase {
     }
     for (int m = 0; m < 3; ++m)
       TC_CUDA_TRY(allow_dynamic_smem((const void*)slab_[m], slab_smem_));
+    // read-back of W: rows of whole waves of slabs, up to kRowsBytes (a wave is some 35 MB
+    // at most).  None for small tensors, where the transpose is a launch more, nor for
+    // k_slab, whose rows are no nearer the order of its threads than the caller's; nor
+    // where there is no room.
+    if ((specialised_ || folded_) && N * sizeof(T) >= kRowsMin) {
+      const size_t wave = (size_t)nsm * n2_ * n3_ * sizeof(T);
+      nwrows_ = (int)std::min<size_t>((size_t)n1_, nsm * std::max<size_t>(1, kRowsBytes / wave));
+      std::string full;
+      wrows_ = alloc<T>((size_t)nwrows_ * n2_ * n3_, full);
+    }
     // folded transforms: the slab's, and the factors' where they fit
     fold_factors_ = fold_dft_fits<T>(n3_, optin);
     if (folded_ || fold_factors_) {
@@ -700,15 +716,14 @@ class Engine final : public EngineBase {
       return TC_ERR_NOMEM;
     }
     if (dW) {
-      // rows into a buffer of the context's own, then one transpose; straight into
-      // the caller's order where there is no room for the buffer
-      if (!wrows_) {
-        std::string full;
-        wrows_ = alloc<T>(N, full);
-      }
+      // rows of some slabs at a time into the context's buffer, then a transpose;
+      // straight into the caller's order without one
       if (wrows_) {
-        launch_slab(MODE_W, wrows_, 0, stream_, SLAB_WROWS | SLAB_NOSUM);
-        k_unpack<T><<<pack_grid(n1_, n2_, n3_), kTileThreads, 0, stream_>>>(wrows_, dW, n1_, n2_, n3_);
+        for (int i0 = 0; i0 < n1_; i0 += nwrows_) {
+          const int ni = std::min(nwrows_, n1_ - i0);
+          launch_slab_rows(i0, ni, wrows_, stream_);
+          k_unpack<T><<<pack_grid(ni, n2_, n3_), kTileThreads, 0, stream_>>>(wrows_, dW + i0, ni, n1_, n2_, n3_);
+        }
       } else {
         launch_slab(MODE_W, dW, 0, stream_, SLAB_NOSUM);
       }
@@ -945,6 +960,14 @@ class Engine final : public EngineBase {
     const int threads = specialised_ && mode != MODE_ITER ? 2 * slab_threads_ : slab_threads_;
     slab_[mode]<<<n1_, threads, slab_smem_, s>>>(d_, Wout, flags | (slabs_in_smem_ ? SLAB_IN_SMEM : 0), init);
   }
+  // W of slabs i0 .. i0 + ni - 1 as rows
+  void launch_slab_rows(int i0, int ni, T* rows, cudaStream_t s) {
+    Dev<T> d = d_;
+    d.Zt += (size_t)i0 * S_ * n2_;
+    d.Rt += (size_t)i0 * S_ * n2_;
+    const int threads = specialised_ ? 2 * slab_threads_ : slab_threads_;
+    slab_[MODE_W]<<<ni, threads, slab_smem_, s>>>(d, rows, SLAB_WROWS | SLAB_NOSUM | (slabs_in_smem_ ? SLAB_IN_SMEM : 0), 0);
+  }
   cudaError_t launch_synth(cudaStream_t s) {
     const size_t sm = zsyn_f_smem<T>(r_);
     const cudaError_t e = allow_dynamic_smem((const void*)k_zsyn_f<T>, sm);
@@ -1060,7 +1083,8 @@ class Engine final : public EngineBase {
   bool wgeneral_ = false;  // with the W-step of long runs and strong smoothing
   bool fold_factors_ = false;  // the factors' transforms too
   cx<T>* fold_ = nullptr;
-  T* wrows_ = nullptr;   // W in row-major order (allocated by the first read-back)
+  T* wrows_ = nullptr;   // W of nwrows_ slabs in row-major order
+  int nwrows_ = 0;
   bool slabs_in_smem_ = true;
   bool xarrays_in_smem_ = true;
   bool mixed_ = false;
