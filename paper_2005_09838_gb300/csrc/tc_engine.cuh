@@ -247,6 +247,7 @@ class Engine final : public EngineBase {
     TC_CUDA_TRY(cudaGetDevice(&device_));
     int optin = 0, nsm = 0;
     TC_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device_));
+    nsm_ = nsm;
     TC_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device_));
     optin -= kStaticSmemReserve;  // room for the kernels' static shared memory
 
@@ -956,8 +957,16 @@ class Engine final : public EngineBase {
     return TC_OK;
   }
 
+  // Threads of the read-back modes, which have no W-step: twice those of the iteration
+  // for the FFT lengths; for many small FP64 slabs half of them, so that an SM holds
+  // more of the CTAs (read-back and objective of 2000 x 48 x 7 68 -> 59 and 252 -> 216 us,
+  // 400 x 144 x 7 49 -> 45 and 122 -> 110; 1000 x 100 x 30 would go from 154 to 170).
+  int readback_threads() const {
+    if (specialised_) return 2 * slab_threads_;
+    return sizeof(T) == 8 && folded_ && n1_ > 2 * nsm_ && n2_ * n3_ <= 1024 ? slab_threads_ / 2 : slab_threads_;
+  }
   void launch_slab(int mode, T* Wout, int init, cudaStream_t s, int flags = 0) {
-    const int threads = specialised_ && mode != MODE_ITER ? 2 * slab_threads_ : slab_threads_;
+    const int threads = mode != MODE_ITER ? readback_threads() : slab_threads_;
     slab_[mode]<<<n1_, threads, slab_smem_, s>>>(d_, Wout, flags | (slabs_in_smem_ ? SLAB_IN_SMEM : 0), init);
   }
   // W of slabs i0 .. i0 + ni - 1 as rows
@@ -965,8 +974,7 @@ class Engine final : public EngineBase {
     Dev<T> d = d_;
     d.Zt += (size_t)i0 * S_ * n2_;
     d.Rt += (size_t)i0 * S_ * n2_;
-    const int threads = specialised_ ? 2 * slab_threads_ : slab_threads_;
-    slab_[MODE_W]<<<ni, threads, slab_smem_, s>>>(d, rows, SLAB_WROWS | SLAB_NOSUM | (slabs_in_smem_ ? SLAB_IN_SMEM : 0), 0);
+    slab_[MODE_W]<<<ni, readback_threads(), slab_smem_, s>>>(d, rows, SLAB_WROWS | SLAB_NOSUM | (slabs_in_smem_ ? SLAB_IN_SMEM : 0), 0);
   }
   cudaError_t launch_synth(cudaStream_t s) {
     const size_t sm = zsyn_f_smem<T>(r_);
@@ -1085,6 +1093,7 @@ class Engine final : public EngineBase {
   cx<T>* fold_ = nullptr;
   T* wrows_ = nullptr;   // W of nwrows_ slabs in row-major order
   int nwrows_ = 0;
+  int nsm_ = 152;        // SMs of the device
   bool slabs_in_smem_ = true;
   bool xarrays_in_smem_ = true;
   bool mixed_ = false;

@@ -35,3 +35,15 @@ def test_read_back_allocates_nothing(shape):
         assert torch.cuda.mem_get_info()[0] == free
     # fully observed: W is G, up to the transform there and back (FP32 parity tolerance)
     assert float((W - G).norm()) <= 1e-5 * float(G.norm())
+
+
+def test_many_small_fp64_slabs():
+    # more than two slabs per SM: the read-back kernels run with half the threads
+    import workloads as wl
+    from oracle import method as O
+    from paper_2005_09838_gb300 import api
+    inst = wl.generate(wl.custom(310, 20, 7, 2, 0.5, seed=8700, iters=2))
+    ref = O.tctf2r(inst["G"], inst["mask"], 2, 1e-3, 1e-3, 1e-1, inst["Y0"], iters=2)
+    got = api.complete(inst["G"], inst["mask"], inst["Y0"], 2, 2, 1e-3, 1e-3, 1e-1, "fp64")
+    assert np.linalg.norm(got["W"] - ref["W"]) <= 1e-10 * np.linalg.norm(ref["W"])
+    assert abs(got["f0"] - ref["f0"]) <= 1e-10 * abs(ref["f0"])
