@@ -154,13 +154,17 @@ inline XFn<T> pick_xstep(int rp) {
   }
 }
 
-// Whether the contractions run in k_gemm.cuh.  At r <= 8 the fused Y-step reads
-// R~ and writes Z~ in one kernel, but its S ceil(n2/64) CTAs each walk all of n1:
-// it keeps short slices in a grid that covers the SMs (us per iteration, fused
-// against tiled: 144x288x168 r = 5 109/119, r = 8 126/125; 200x288x168 r = 8
-// 196/184; 100x100x60 r = 8 62/54; 900x150x90 r = 8 335/261).
+// Whether the contractions run in k_gemm.cuh.  The fused Y-step is one kernel for
+// three, which decides slices of few rows (us per iteration, fused against tiled:
+// r = 6 and 8 20x200x28 41/49, 44/49, 24x96x60 39/45, 41/47, 48x60x28 39/43, 41/43,
+// 64x96x60 45/47, 49/49, 96x96x28 47/45, 52/49; r = 12 to 20 24x36x112 60/62, 68/70, 85/88,
+// 48x60x28 64/60, 74/68, 80/74).  At r <= 8 it also reads R~ and writes Z~ in one pass, but
+// its S ceil(n2/64) CTAs each walk all of n1: it keeps short slices in a grid that
+// covers the SMs (144x288x168 r = 5 109/119, r = 8 126/125; 200x288x168 r = 8 196/184;
+// 100x100x60 r = 8 62/54; 900x150x90 r = 8 335/261).
 inline bool gemm_pays(int rp, int S, int n1, int n2) {
-  return rp > 8 || (rp == 8 && (n1 >= 192 || S * ((n2 + 63) / 64) < 152));
+  if (rp > 8) return n1 >= 32;
+  return rp == 8 && (n1 >= 192 || (n1 >= 80 && S * ((n2 + 63) / 64) < 152));
 }
 
 // Tensor-core Q contraction of the precision form (TC_TF32 / TC_BF16 over
