@@ -282,13 +282,15 @@ tc_status tc_complete_static(const tc_params* p, const void* G, const uint8_t* m
                              const void* X0, int32_t n_iters, void* W, double* f0, void* cuda_stream);
 
 /* Tile of the mode-3 transform chosen for this context (the library's own
- * tuning, no counterpart in the paper).  Tube lengths other than the ones with
- * a transform of their own (112, 168 in FP32; 7 in FP64) use a transform written as
- * a product with the DFT matrix of Eq. (bar BA-k) / Eq. (barAAk), each work
- * item covering slab_tile rows (inverse) or slices (forward) of some tubes;
- * tc_init times slab_tile = 2 and 4 on the initial pass (every choice gives
- * the same sums in the same order) and keeps the fastest.
- *   slab_tile : receives the chosen tile, 0 for the lengths above.
+ * tuning, no counterpart in the paper).  Tube lengths without an FFT of their
+ * own (112 and 168 in FP32 have one) use a transform written as a product with
+ * the DFT matrix of Eq. (bar BA-k) / Eq. (barAAk), each work item covering
+ * slab_tile rows (inverse) or slices (forward) of some tubes; tc_init times
+ * slab_tile = 2 and 4 on the initial pass (every choice gives the same sums in
+ * the same order) and keeps the fastest.
+ *   slab_tile : receives the chosen tile, 0 where none is timed: the lengths with
+ *               an FFT, and in FP64 odd lengths up to 7 (one item is the whole
+ *               transform of its tubes).
  * Errors: TC_ERR_ARG. */
 tc_status tc_tile(tc_ctx* c, int32_t* slab_tile);
 

@@ -251,6 +251,27 @@ inline bool slab_g_plan(int n2, int n3, int optin, SlabGPlan& pl) {
   return pl.smem <= (size_t)optin;
 }
 
+// Items of the inverse transform per group of kGTubes tubes with TL = 4 columns a lane.
+template <typename T>
+inline int fold_items(int n3) {
+  const FoldDims f = fold_dims(n3);
+  return (f.even ? 2 : 1) * ((f.nl + 4 * kLG<T> - 1) / (4 * kLG<T>));
+}
+// Tile where none is timed: TL = 2, twice the items, where the CTA has a warp for each
+// of them (us per iteration of tc_complete_static, TL = 4 and 2: 16 x 48 x 9 FP64 53.0, 50.9,
+// 30 x 90 x 9 FP32 44.3, 42.8; with more items than warps 60 x 90 x 14 FP64 77.4, 79.9).
+template <typename T>
+inline int fold_tile(int n2, int n3, int threads) {
+  return 64 * fold_items<T>(n3) * ((n2 + kGTubes<T> - 1) / kGTubes<T>) <= threads ? 2 : 4;
+}
+// Whether tc_init times the tiles.  In FP64 the pipe is the bound at either, so where
+// one item at TL = 4 is the whole transform of its tubes (odd n3 up to 7) TL = 2
+// spreads it over more lanes' warps and there is nothing to choose.
+template <typename T>
+inline bool fold_timed(int n3) {
+  return sizeof(T) == 4 || fold_items<T>(n3) > 1;
+}
+
 // Row l of the q-th row in slab order (slot by slot), 0 <= q < n3, and the
 // position of row l in the slab, in units of T.
 __device__ __forceinline__ int slab_g_row(bool even, int n3, int q) {

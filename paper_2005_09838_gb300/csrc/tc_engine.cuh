@@ -303,7 +303,8 @@ class Engine final : public EngineBase {
       folded_ = true;
       wgeneral_ = p.rho2 != 0.0 && wstep_strong(p.mu, p.rho2);
       d_.fold_sg = gp.sg;
-      for (int m = 0; m < 3; ++m) slab_[m] = pick_slab_g<T>(m, n3_ == 7 ? 2 : 4, gp.sg > 0, wgeneral_);
+      fold_tl_ = fold_timed<T>(n3_) ? fold_tile<T>(n2_, n3_, gp.threads) : 2;
+      for (int m = 0; m < 3; ++m) slab_[m] = pick_slab_g<T>(m, fold_tl_, gp.sg > 0, wgeneral_);
       slab_smem_ = gp.smem;
       slab_threads_ = gp.threads;
       slabs_in_smem_ = true;
@@ -575,7 +576,7 @@ class Engine final : public EngineBase {
     }
     k_gram_tiles<T><<<dim3(S_, ytiles), 256, 0, stream_>>>(d_);         // A of the first X-step
     if (xsplit_ || apre_) xa_fn_<<<S_, xa_threads_, xa_smem_, stream_>>>(d_);  // its A^+
-    if (!specialised_ && !(folded_ && sizeof(T) == 8 && n3_ == 7)) {  // (four rows and slices: nothing to choose)
+    if (!specialised_ && (!folded_ || fold_timed<T>(n3_))) {
       // tile of the generic transform for this shape: each candidate runs the
       // initial slab pass (it only depends on G and Z~0, so every run writes the
       // same R~0), timed twice; the fastest is kept
@@ -596,7 +597,7 @@ class Engine final : public EngineBase {
     if (st != TC_OK) return st;
     if (folded_ && !wgeneral_ && 4 * (long long)lrows >= n1_ && lrows > 0) {
       wgeneral_ = true;
-      slab_[MODE_ITER] = pick_slab_g<T>(MODE_ITER, slab_tile_ > 0 ? slab_tile_ : 2, d_.fold_sg > 0, true);
+      slab_[MODE_ITER] = pick_slab_g<T>(MODE_ITER, slab_tile_ > 0 ? slab_tile_ : fold_tl_, d_.fold_sg > 0, true);
       TC_CUDA_TRY(allow_dynamic_smem((const void*)slab_[MODE_ITER], slab_smem_));
     }
     // the iteration graph is built and uploaded here, so that tc_iterate only
@@ -1104,7 +1105,8 @@ class Engine final : public EngineBase {
   bool xsplit_ = false;  // X-step as four kernels
   bool apre_ = false;    // one-CTA X-step with A^+ from k_xa on a graph branch
   int slab_nb_ = 1;      // CTAs of the generic slab kernel that an SM holds
-  int slab_tile_ = 0;    // rows / slices per item of the generic transform (0: specialised length)
+  int slab_tile_ = 0;    // rows / slices per item of the generic transform (0: not timed)
+  int fold_tl_ = 4;      // the same of the folded one before it is timed
   int* rk_ = nullptr;    // step 5: slice ranks, counters and work (allocated when the rule is first on)
   int* rcnt_ = nullptr;
   cx<T>* rscr_ = nullptr;

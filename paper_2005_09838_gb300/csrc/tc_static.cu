@@ -222,7 +222,8 @@ tc_status run_static(const tc_params& p, const void* G, const uint8_t* mask, con
   size_t slab_smem = lay.total;
   int slab_threads = kSlabThreads;
   if (folded) {
-    for (int m = 0; m < 3; ++m) slab[m] = pick_slab_g<T>(m, n3 == 7 ? 2 : 4, gp.sg > 0, strong);
+    const int tl = fold_timed<T>(n3) ? fold_tile<T>(n2, n3, gp.threads) : 2;
+    for (int m = 0; m < 3; ++m) slab[m] = pick_slab_g<T>(m, tl, gp.sg > 0, strong);
     slab_smem = gp.smem;
     slab_threads = gp.threads;
     d.fold = fold;

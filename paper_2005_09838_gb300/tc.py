@@ -179,8 +179,8 @@ class Completion:
         _check(self._lib.tc_rank_rule(self._ctx, float(tol), int(patience)))
 
     def tile(self) -> int:
-        """Tile of the generic-length transform chosen at init (tc_tile; 0 for a
-        dedicated-kernel length)."""
+        """Tile of the generic-length transform chosen at init (tc_tile; 0 where
+        none is timed)."""
         t = ctypes.c_int32(0)
         _check(self._lib.tc_tile(self._ctx, ctypes.byref(t)))
         return t.value
