@@ -468,7 +468,7 @@ __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP,
   T wn = T(0);
   if (!LAST && !((mw >> (SEG - 1)) & 1u)) {
     const int k = run_end(rowm, words, j1, n2);  // next observed entry, or the row's end
-    T x = (k < n2) ? col[k * LP] : T(0);
+    T x = (k < n2) ? col[k * LP] : T(0), e = T(0);
     const int tb = k < n2 ? n2 : 0;
     int jl = j1;  // entries down to here, then segments
     if (GENERAL && k - j1 >= SEG) {
@@ -477,14 +477,16 @@ __device__ __forceinline__ void wstep_segment(const T* __restrict__ col, int LP,
     }
     for (int j = k - 1; j >= jl; --j) {
       const T inv = wtab[tb + k - 1 - j];
-      x = fma(rho2 * inv, x, col[j * LP] * inv);
+      e = rho2 * inv;
+      x = fma(e, x, col[j * LP] * inv);
     }
     if (GENERAL)
       for (int j = jl - SEG; j >= j1; j -= SEG) x = fma(col[(j + 2) * LP], x, col[(j + 3) * LP]);
     wn = fma(c[SEG - 1], x, v[SEG - 1]);
     if (k > j1) {
       const int p1 = tb + k - 1 - j1;
-      const T e = rho2 * wtab[p1], ce = c[SEG - 1] * e;
+      if (GENERAL) e = rho2 * wtab[p1];
+      const T ce = c[SEG - 1] * e;
       // (tp is one past the position of the segment's last entry)
       wn *= rcp_refined(!GENERAL || ce < T(0.5) ? fma(-c[SEG - 1], e, T(1))
                                                 : fma(c[SEG - 1], hex[p1], hex[tp - 1 - wtab]));

@@ -193,27 +193,27 @@ struct SqSum<float> {
     return (m >= 0x1p-48f && m <= 0x1p48f) || m == 0.f;
   }
   __device__ __forceinline__ void term(float a) { e += two_sum(c, a); }  // a: of the size of a rounding error
+  __device__ __forceinline__ void square(float v) {
+    const float p = mul_rn(v, v), pe = fmaf(v, v, -p);
+    term(two_sum(s, p));
+    term(pe);
+  }
+  // (the plain terms outside the branch: the sums of several values interleave)
   __device__ __forceinline__ void add(float v) {
-    if (near(v)) {
-      const float p = mul_rn(v, v), pe = fmaf(v, v, -p);
-      term(two_sum(s, p));
-      term(pe);
-    } else {
-      far = sq_diff64(far, v, 0.f);
-    }
+    const bool nr = near(v);
+    square(nr ? v : 0.f);
+    if (!nr) far = sq_diff64(far, v, 0.f);
   }
   // (a - b)^2 of the difference as it is, not rounded: h + z
   __device__ __forceinline__ void add_diff(float a, float b) {
-    const float h = a - b;
-    if (near(h)) {
-      const float w = h - a, z = (a - (h - w)) - (b + w);
-      const float q = mul_rn(2.f * h, z), qe = fmaf(2.f * h, z, -q);
-      add(h);
-      term(q);
-      e += fmaf(z, z, qe);
-    } else {
-      far = sq_diff64(far, a, b);
-    }
+    const bool nr = near(a - b);
+    const float a1 = nr ? a : 0.f, b1 = nr ? b : 0.f, h = a1 - b1;
+    const float w = h - a1, z = (a1 - (h - w)) - (b1 + w);
+    const float q = mul_rn(2.f * h, z), qe = fmaf(2.f * h, z, -q);
+    square(h);
+    term(q);
+    e += fmaf(z, z, qe);
+    if (!nr) far = sq_diff64(far, a, b);
   }
   __device__ __forceinline__ double total() const { return (double)s + (double)c + (double)e + far; }
 };
