@@ -985,7 +985,9 @@ class Engine final : public EngineBase {
     const size_t sm = zsyn_f_smem<T>(r_);
     const cudaError_t e = allow_dynamic_smem((const void*)k_zsyn_f<T>, sm);
     if (e != cudaSuccess) return e;
-    k_zsyn_f<T><<<dim3(S_, (n1_ + kGmTile - 1) / kGmTile, (n2_ + kGmTile - 1) / kGmTile), kGmZThreads, sm, s>>>(d_);
+    Dev<T> d = d_;
+    d.dZt = nullptr;  // no Z~ to take a change from yet
+    k_zsyn_f<T><<<dim3(S_, (n1_ + kGmTile - 1) / kGmTile, (n2_ + kGmTile - 1) / kGmTile), kGmZThreads, sm, s>>>(d);
     return cudaGetLastError();
   }
   void launch_qcon(cudaStream_t s) { qcon_<<<qgrid_, qthreads_, qcon_smem_, s>>>(d_, Q_); }
@@ -1024,23 +1026,12 @@ class Engine final : public EngineBase {
     return forked;
   }
 
-  // One TCTF2R iteration: Q = R~Y~^H, X-step (+ Y-step r x r work), Y-step,
-  // then the slab kernel (Z, W-step, R~).
   // Step 5 (rank vector): the rank kernel, then the tile Grams of Y~ and A^+ of
   // the next X-step again (the rank kernel may have rotated Y~).
   void launch_rank(cudaStream_t s) {
     k_rank<T><<<S_, 256, rank_smem_, s>>>(d_);
     k_gram_tiles<T><<<dim3(S_, d_.ytiles), 256, 0, s>>>(d_);
     if (xsplit_ || apre_) xa_fn_<<<S_, xa_threads_, xa_smem_, s>>>(d_);
-  }
-
-  void launch_iteration(cudaStream_t s) {
-    launch_qcon(s);
-    launch_xstep(s);
-    launch_ystep(s);
-    launch_slab(MODE_ITER, nullptr, 0, s);
-    if (d_.rk) launch_rank(s);
-    if (d_.conv) k_check<T><<<1, 32, 0, s>>>(d_);  // step 6
   }
 
   tc_status read_conv(unsigned long long* h, std::string& err) {
