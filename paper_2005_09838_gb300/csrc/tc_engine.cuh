@@ -346,9 +346,10 @@ class Engine final : public EngineBase {
     if (!err.empty()) return TC_ERR_NOMEM;
     if (fold_factors_) TC_CUDA_TRY(allow_fold_dft<T>(n3_));
 
-    strict_ = sizeof(T) == 4 && (specialised_ || (p.precision == TC_BF16 && rp_ == 32));
     // precision form: r x r solves in FP64, contractions on the tensor cores for r > 16
     mixed_ = p.precision == TC_TF32 || p.precision == TC_BF16;
+    strict_ = sizeof(T) == 4 && ((specialised_ && (rp_ <= 8 || (mixed_ && rp_ == 32))) ||
+                                 (p.precision == TC_BF16 && rp_ == 32));
     auto xlay = [&](bool in_smem) { return xstep_layout_for<T>(n1_, n2_, r_, rp_, mixed_, in_smem); };
     XLayout xl = xlay(true);
     xarrays_in_smem_ = xl.total <= (size_t)optin;
@@ -1076,12 +1077,14 @@ class Engine final : public EngineBase {
   int n1_ = 0, n2_ = 0, n3_ = 0, r_ = 0, S_ = 0, mw_ = 0, rp_ = 8;
   bool poisoned_ = false;
   bool specialised_ = false;
-  // Sums in the order of the plain kernels (k_factor_dft, k_qcon, the fused k_ystep,
-  // the sequential W-step), bit for bit: an iteration amplifies the rounding of D on
-  // the DC slice by the condition of its Gram (1e-5 of X~ and Y~ at r = 32), so another
-  // order gives other factors at that level.  For the lengths with an FFT, where
-  // nothing is gained by another order, and for TC_BF16 (see kTL).  The other forms
-  // compensate that sum (dcon_f_tile).
+  // Sums in the order of the plain kernels (k_factor_dft, k_qcon, the fused k_ystep), D
+  // on the real slices uncompensated: an iteration amplifies its rounding on the DC slice
+  // by the condition of its Gram.  For TC_BF16 at r > 16 (see kTL), and at the lengths
+  // with an FFT where the compensated sum (dcon_f_tile), in the two real slices' CTAs
+  // alone, sets the length of the Y-step: r <= 8 (144 x 288 x 168 r = 8, 10 iterations,
+  // 1368 us and 3.4e-6 of the factors; compensated 1397 us and 1.7e-6) and the tensor-core
+  // contractions (529 x 96 x 112 TF32 1289 us and 1.0e-5; 1314 us and 2.1e-6).  All other
+  // forms compensate it (529 x 96 x 112 FP32 1457 us and 1.1e-5; 1460 us and 1.4e-6).
   bool strict_ = false;
   bool folded_ = false;  // folded-transform slab kernels (k_slab_g)
   bool wgeneral_ = false;  // with the W-step of long runs and strong smoothing

@@ -48,15 +48,17 @@ bool pick_gemm<float>(int rp, int r, int n2, bool strided, TcKernels<float>& k) 
   k.zsyn = k_zsyn_f<float>;
   k.zsm = zsyn_f_smem<float>(r);
   k.qsm = qcon_smem_bytes<float>(n2, r, rp);
-  if (rp == 8 && !strided) {  // (tiled Q is the faster one at r <= 8: 20 against 26 us on 925 x 153 x 92)
+  // (tiled Q is the faster one at r <= 8: 20 against 26 us on 925 x 153 x 92)
+  if (rp == 8 && !strided) {
     k.qcon = k_qcon_f<8>, k.dcon = k_dcon_f<8>, k.qsm = qcon_f_smem<8>(), k.dsm = dcon_f_smem<8>();
-    return true;
-  }
-  switch (rp) {
-    case 8: k.qcon = k_qcon_l<8>, k.dcon = k_dcon_f<8, true>, k.dsm = dcon_f_smem<8>(); break;
-    case 16: k.qcon = k_qcon_l<16>, k.dcon = strided ? k_dcon_f<16, true> : k_dcon_f<16>, k.dsm = dcon_f_smem<16>(); break;
-    case 32: k.qcon = k_qcon_l<32>, k.dcon = strided ? k_dcon_f<32, true> : k_dcon_f<32>, k.dsm = dcon_f_smem<32>(); break;
-    default: return false;
+  } else if (rp == 8) {
+    k.qcon = k_qcon_l<8>, k.dcon = k_dcon_f<8, true>, k.dsm = dcon_f_smem<8>();
+  } else if (rp == 16 && !strided) {
+    k.qcon = k_qcon_l<16>, k.dcon = k_dcon_f<16>, k.dsm = dcon_f_smem<16>();
+  } else if (rp == 32 && !strided) {
+    k.qcon = k_qcon_l<32>, k.dcon = k_dcon_f<32>, k.dsm = dcon_f_smem<32>();
+  } else {
+    return false;
   }
   return true;
 }
