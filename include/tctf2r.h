@@ -109,7 +109,8 @@ typedef struct tc_ctx tc_ctx;
  *   inputs_on_device : 1 if G, mask, Y0, X0 are device pointers on the current
  *            device, 0 if they are host pointers
  *   cuda_stream : cudaStream_t to order all work on (NULL = legacy default)
- * Device memory of the context is allocated here (cudaMalloc) and released by
+ * Device memory of the context is allocated here (cudaMalloc; among it up to
+ * 128 MiB for tc_result, which does without where there is no room) and released by
  * tc_free; the CUDA graph of one iteration is captured and uploaded here too,
  * so tc_iterate only launches it.  Synchronises the stream before returning.
  * Errors: TC_ERR_ARG for invalid sizes/parameters/NULL inputs, TC_ERR_NOMEM,
@@ -129,8 +130,9 @@ tc_status tc_init(tc_ctx** out, const tc_params* p, const void* G, const uint8_t
  * Errors: TC_ERR_ARG (n_iters < 0), TC_ERR_CUDA, TC_ERR_STATE. */
 tc_status tc_iterate(tc_ctx* c, int32_t n_iters, int32_t* done);
 
-/* Objective f0 of Eq. (TETP-optim) at the current iterate (X, Y, W), reduced in
- * FP64, and optionally ||P_Omega(X*Y - G)||_F.  Synchronises the stream.
+/* Objective f0 of Eq. (TETP-optim) at the current iterate (X, Y, W), and
+ * optionally ||P_Omega(X*Y - G)||_F; the sums of squares have at least the
+ * accuracy and the range of FP64.  Synchronises the stream.
  *   f0        : receives f0 (required)
  *   resid_obs : receives the observed-entry residual norm (may be NULL)
  * Errors: TC_ERR_ARG, TC_ERR_CUDA, TC_ERR_NUMERIC (non-finite f0), TC_ERR_STATE. */
@@ -238,7 +240,9 @@ tc_status tc_batch_free(tc_batch* b);
  * tc_grad_init: p gives n1, n2, n3, r, rho1 and precision (TC_FP64 or TC_FP32;
  *   mu, rho2, step, eps are not used); G and mask as for tc_init (copied).
  * tc_grad_eval: X, Y in the precision's type, column-major (i1 fastest) like
- *   X0, Y0 of tc_init; loss receives L in FP64 (required); dX, dY receive the
+ *   X0, Y0 of tc_init; loss receives L in FP64 (required; its rho1 term is summed as FP32
+ *   values with their rounding errors in TC_FP32, so it overflows with the squares of
+ *   the differences of Z past 1e38); dX, dY receive the
  *   gradients in the layouts of X, Y (each may be NULL: then it is not
  *   formed).  on_device selects device or host buffers for X, Y, dX, dY.
  *   Synchronises the stream.  Errors: TC_ERR_ARG, TC_ERR_CUDA,

@@ -86,7 +86,7 @@ __host__ __device__ constexpr size_t dcon_f_smem() {
 // block calls it with the same range.
 //
 // STRIDED: partial w of eight sums the rows i = w mod 8 in increasing order, as the
-// warps of the fused k_ystep do (bit for bit: see Engine::strict_); the thread
+// warps of the fused k_ystep do (bit for bit: see Engine::strict_, r <= 8); the thread
 // groups take a partial each in place of sharing one, and z counts the CTAs.
 //
 // Real slices (with d.dpairs): the factors and the residual are real, and D is formed as a
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kGmThreads) k_qcon_f(Dev<float> d, cx<float>* 
 // A warp forms 4 rows x 8 columns of Q, each lane summing the columns j = lane mod
 // 32 in increasing order and the lanes added pairwise (distance 16, 8, .., 1): the
 // order of k_qcon, bit for bit, at 12 loads for 32 complex products where k_qcon
-// has 33 (529 x 96 x 112, r = 32: 53 -> 30 us).
+// has 33 (529 x 96 x 112, r = 32: 53 -> 41 us).
 constexpr int kQlRows = 4, kQlCols = 8;
 template <int RP>
 __global__ void __launch_bounds__(256, 2) k_qcon_l(Dev<float> d, cx<float>* __restrict__ Qout) {
