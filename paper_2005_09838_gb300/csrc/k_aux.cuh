@@ -236,49 +236,56 @@ __global__ void __launch_bounds__(256) k_rho1_term(Dev<T> d) {
   const int n1 = d.n1, n2 = d.n2;
   const size_t rs = (size_t)d.S * n2;  // distance between rows i and i + 1 of slice k
   const cx<T>* Z = d.Zt + (size_t)k * n2;
-  // (FP64: squares and sums with their rounding errors)
-  SqSum<T> sum;
-  T s = T(0), c = T(0);
-  auto add = [&](T v) {
-    if constexpr (sizeof(T) == 4) sum.add(v);
-    else dot2(s, c, v, v);
-  };
   const int nd = n1 > 1 ? n1 - 1 : 0, per = (nd + kRhoChunks - 1) / kRhoChunks;
   const int i0 = min(ch * per, nd), i1 = min(i0 + per, nd);
   // a thread walks down column j through the chunk's rows, keeping the previous
   // row's value, so each entry is read once; four rows are loaded at a time
-  for (int j = threadIdx.x; j < n2 && i0 < i1; j += blockDim.x) {
-    cx<T> prev = Z[(size_t)i0 * rs + j];
-    int i = i0;
-    for (; i + 4 <= i1; i += 4) {
-      cx<T> nx[4];
+  auto walk = [&](auto& sum) {
+    for (int j = threadIdx.x; j < n2 && i0 < i1; j += blockDim.x) {
+      cx<T> prev = Z[(size_t)i0 * rs + j];
+      int i = i0;
+      for (; i + 4 <= i1; i += 4) {
+        cx<T> nx[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) nx[q] = Z[(size_t)(i + 1 + q) * rs + j];
+        for (int q = 0; q < 4; ++q) nx[q] = Z[(size_t)(i + 1 + q) * rs + j];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const cx<T> a = nx[q] - prev;
-        add(a.re);
-        add(a.im);
-        prev = nx[q];
+        for (int q = 0; q < 4; ++q) {
+          const cx<T> a = nx[q] - prev;
+          sum.add(a.re);
+          sum.add(a.im);
+          prev = nx[q];
+        }
+      }
+      for (; i < i1; ++i) {
+        const cx<T> cur = Z[(size_t)(i + 1) * rs + j];
+        const cx<T> a = cur - prev;
+        sum.add(a.re);
+        sum.add(a.im);
+        prev = cur;
       }
     }
-    for (; i < i1; ++i) {
-      const cx<T> cur = Z[(size_t)(i + 1) * rs + j];
-      const cx<T> a = cur - prev;
-      add(a.re);
-      add(a.im);
-      prev = cur;
-    }
-  }
-  double tot_d = warp_sum(sum.total() + ((double)s + (double)c));
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) part[wid] = tot_d;
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  };
+  auto block_total = [&](double v) {  // valid in thread 0
+    v = warp_sum(v);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __syncthreads();
+    if (lane == 0) part[wid] = v;
+    __syncthreads();
     double tot = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += part[w];
-    d.part_k[(size_t)k * kRhoChunks + ch] = tot;
+    if (threadIdx.x == 0)
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += part[w];
+    return tot;
+  };
+  // (FP64: squares and sums with their rounding errors)
+  std::conditional_t<sizeof(T) == 4, SqSum<T>, SqPair<T>> sum;
+  walk(sum);
+  double tot = block_total(sum.total());
+  if (sq_again<T>(tot, sum.nonzero())) {
+    SqSum64 s64;
+    walk(s64);
+    tot = block_total(s64.s);
   }
+  if (threadIdx.x == 0) d.part_k[(size_t)k * kRhoChunks + ch] = tot;
 }
 
 // ---------------------------------------------------------------------------

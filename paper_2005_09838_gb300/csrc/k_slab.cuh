@@ -686,25 +686,50 @@ __global__ void __launch_bounds__(kSlabThreads, NB)
     }
   }
   __syncthreads();
+  if (MODE == MODE_GRAD) {
+    double g = gsum.total(), unused = 0.0;
+    block_sum2(g, unused, red);
+    if (sq_again<T>(g, gsum.nonzero())) {
+      SqSum64 g64;
+      for (int e = tid; e < n2 * n3; e += nt) g64.add(spat[(e / n3) * LP + e % n3]);
+      g = g64.s;
+      block_sum2(g, unused, red);
+    }
+    if (tid == 0) d.part[(size_t)i1 * 4] = g;
+  }
 
   // ---- phase B: rows ------------------------------------------------------
   if (MODE == MODE_W || MODE == MODE_R) {
     const bool sums = MODE == MODE_R || !(flags & SLAB_NOSUM);
-    SqSum<T> sa, sb;
-    for (int e = tid; e < n2 * n3; e += nt) {
-      const int j = e / n3, l = e - j * n3;
-      const T v = spat[j * LP + l];
-      if (sums) sa.add(v);
-      if (MODE == MODE_W) {
-        if (sums && j + 1 < n2) sb.add_diff(v, spat[(j + 1) * LP + l]);
-        if (Wout) Wout[(size_t)i1 + (size_t)n1 * ((size_t)j + (size_t)n2 * l)] = v;
-      } else {
-        if ((msk[l * mwords + (j >> 5)] >> (j & 31)) & 1u) sb.add(v);
+    if (MODE == MODE_W && Wout)
+      for (int e = tid; e < n2 * n3; e += nt) {
+        const int j = e / n3, l = e - j * n3;
+        Wout[(size_t)i1 + (size_t)n1 * ((size_t)j + (size_t)n2 * l)] = spat[j * LP + l];
       }
-    }
     if (!sums) return;
+    auto walk = [&](auto& sa, auto& sb) {
+      for (int e = tid; e < n2 * n3; e += nt) {
+        const int j = e / n3, l = e - j * n3;
+        const T v = spat[j * LP + l];
+        sa.add(v);
+        if (MODE == MODE_W) {
+          if (j + 1 < n2) sb.add_diff(v, spat[(j + 1) * LP + l]);
+        } else {
+          if ((msk[l * mwords + (j >> 5)] >> (j & 31)) & 1u) sb.add(v);
+        }
+      }
+    };
+    SqSum<T> sa, sb;
+    walk(sa, sb);
     double a = sa.total(), b = sb.total();
     block_sum2(a, b, red);
+    const bool again_a = sq_again<T>(a, sa.nonzero()), again_b = sq_again<T>(b, sb.nonzero());
+    if (again_a || again_b) {
+      SqSum64 a64, b64;
+      walk(a64, b64);
+      a = a64.s, b = b64.s;
+      block_sum2(a, b, red);
+    }
     if (tid == 0) {
       const int o = (MODE == MODE_W) ? 2 : 0;
       d.part[(size_t)i1 * 4 + o] = a;
@@ -779,11 +804,6 @@ __global__ void __launch_bounds__(kSlabThreads, NB)
     double unused = 0.0;
     block_sum2(dw2, unused, red);
     if (tid == 0) d.part_dw[i1] = dw2;
-  }
-  if (MODE == MODE_GRAD) {
-    double g = gsum.total(), unused = 0.0;
-    block_sum2(g, unused, red);
-    if (tid == 0) d.part[(size_t)i1 * 4] = g;
   }
 }
 

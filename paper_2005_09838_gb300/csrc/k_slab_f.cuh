@@ -274,29 +274,53 @@ __global__ void __launch_bounds__(MODE == MODE_ITER ? kSlabFThreads : kSlabFAux,
     }
   }
   __syncthreads();
+  if (MODE == MODE_GRAD) {
+    double g = gsum.total(), unused = 0.0;
+    block_sum2(g, unused, red);
+    if (sq_again<T>(g, gsum.nonzero())) {
+      SqSum64 g64;
+      for (int e = tid; e < L * n2; e += nt) g64.add(buf[(size_t)(e / L) * LP + e % L]);
+      g = g64.s;
+      block_sum2(g, unused, red);
+    }
+    if (tid == 0) d.part[(size_t)i1 * 4] = g;
+  }
 
   // ---- partial sums of the read-back modes ----------------------------------------------
   if (MODE == MODE_W || MODE == MODE_R) {
     const bool sums = MODE == MODE_R || !(flags & SLAB_NOSUM);
-    SqSum<T> sa, sb;
-    for (int e = tid; e < L * n2; e += nt) {
-      const int l = e / n2, t = e - l * n2;
-      const int off = slab_f_off<N1, N2>(l);
-      const T v = buf[(size_t)t * LP + off];
-      if (sums) sa.add(v);
-      if (MODE == MODE_W) {
-        if (sums && t + 1 < n2) sb.add_diff(v, buf[(size_t)(t + 1) * LP + off]);
-        if (Wout) {
-          if (flags & SLAB_WROWS) Wout[((size_t)i1 * L + l) * n2 + t] = v;
-          else Wout[(size_t)i1 + (size_t)n1 * ((size_t)t + (size_t)n2 * l)] = v;
-        }
-      } else {
-        if ((msk[off * mw + (t >> 5)] >> (t & 31)) & 1u) sb.add(v);
+    if (MODE == MODE_W && Wout)
+      for (int e = tid; e < L * n2; e += nt) {
+        const int l = e / n2, t = e - l * n2;
+        const T v = buf[(size_t)t * LP + slab_f_off<N1, N2>(l)];
+        if (flags & SLAB_WROWS) Wout[((size_t)i1 * L + l) * n2 + t] = v;
+        else Wout[(size_t)i1 + (size_t)n1 * ((size_t)t + (size_t)n2 * l)] = v;
       }
-    }
     if (!sums) return;
+    auto walk = [&](auto& sa, auto& sb) {
+      for (int e = tid; e < L * n2; e += nt) {
+        const int l = e / n2, t = e - l * n2;
+        const int off = slab_f_off<N1, N2>(l);
+        const T v = buf[(size_t)t * LP + off];
+        sa.add(v);
+        if (MODE == MODE_W) {
+          if (t + 1 < n2) sb.add_diff(v, buf[(size_t)(t + 1) * LP + off]);
+        } else {
+          if ((msk[off * mw + (t >> 5)] >> (t & 31)) & 1u) sb.add(v);
+        }
+      }
+    };
+    SqSum<T> sa, sb;
+    walk(sa, sb);
     double a = sa.total(), b = sb.total();
     block_sum2(a, b, red);
+    const bool again_a = sq_again<T>(a, sa.nonzero()), again_b = sq_again<T>(b, sb.nonzero());
+    if (again_a || again_b) {
+      SqSum64 a64, b64;
+      walk(a64, b64);
+      a = a64.s, b = b64.s;
+      block_sum2(a, b, red);
+    }
     if (tid == 0) {
       const int o = (MODE == MODE_W) ? 2 : 0;
       d.part[(size_t)i1 * 4 + o] = a;
@@ -389,11 +413,6 @@ __global__ void __launch_bounds__(MODE == MODE_ITER ? kSlabFThreads : kSlabFAux,
     double unused = 0.0;
     block_sum2(dw2, unused, red);
     if (tid == 0) d.part_dw[i1] = dw2;
-  }
-  if (MODE == MODE_GRAD) {
-    double g = gsum.total(), unused = 0.0;
-    block_sum2(g, unused, red);
-    if (tid == 0) d.part[(size_t)i1 * 4] = g;
   }
 }
 

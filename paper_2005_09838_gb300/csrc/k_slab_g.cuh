@@ -580,31 +580,57 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
     }
   }
   __syncthreads();
+  if (MODE == MODE_GRAD) {
+    double g = gsum.total(), unused = 0.0;
+    block_sum2(g, unused, red);
+    if (sq_again<T>(g, gsum.nonzero())) {
+      SqSum64 g64;
+      for (int l = wid; l < n3; l += nw)
+        for (int t = lane; t < n2; t += 32) g64.add(spat[slab_g_off(EVEN, n3, l, np2) + 2 * t]);
+      g = g64.s;
+      block_sum2(g, unused, red);
+    }
+    if (tid == 0) d.part[(size_t)i1 * 4] = g;
+  }
 
   // ---- read-back modes: partial sums, optional copy of W ----------------------------------
   if (MODE == MODE_W || MODE == MODE_R) {
     const bool sums = MODE == MODE_R || !(flags & SLAB_NOSUM);
-    SqSum<T> sa, sb;
-    for (int q = wid; q < n3; q += nw) {
-      const int l = slab_g_row(EVEN, n3, q);
-      const T* row = spat + slab_g_off(EVEN, n3, l, np2);
-      for (int t = lane; t < n2; t += 32) {
-        const T v = row[2 * t];
-        if (sums) sa.add(v);
-        if (MODE == MODE_W) {
-          if (sums && t + 1 < n2) sb.add_diff(v, row[2 * (t + 1)]);
-          if (Wout) {
-            if (flags & SLAB_WROWS) Wout[((size_t)i1 * n3 + l) * n2 + t] = v;
-            else Wout[(size_t)i1 + (size_t)n1 * ((size_t)t + (size_t)n2 * l)] = v;
-          }
-        } else {
-          if ((msk[q * mw + (t >> 5)] >> lane) & 1u) sb.add(v);
+    if (MODE == MODE_W && Wout)
+      for (int q = wid; q < n3; q += nw) {
+        const int l = slab_g_row(EVEN, n3, q);
+        const T* row = spat + slab_g_off(EVEN, n3, l, np2);
+        for (int t = lane; t < n2; t += 32) {
+          if (flags & SLAB_WROWS) Wout[((size_t)i1 * n3 + l) * n2 + t] = row[2 * t];
+          else Wout[(size_t)i1 + (size_t)n1 * ((size_t)t + (size_t)n2 * l)] = row[2 * t];
         }
       }
-    }
     if (!sums) return;
+    auto walk = [&](auto& sa, auto& sb) {
+      for (int q = wid; q < n3; q += nw) {
+        const T* row = spat + slab_g_off(EVEN, n3, slab_g_row(EVEN, n3, q), np2);
+        for (int t = lane; t < n2; t += 32) {
+          const T v = row[2 * t];
+          sa.add(v);
+          if (MODE == MODE_W) {
+            if (t + 1 < n2) sb.add_diff(v, row[2 * (t + 1)]);
+          } else {
+            if ((msk[q * mw + (t >> 5)] >> lane) & 1u) sb.add(v);
+          }
+        }
+      }
+    };
+    SqSum<T> sa, sb;
+    walk(sa, sb);
     double a = sa.total(), b = sb.total();
     block_sum2(a, b, red);
+    const bool again_a = sq_again<T>(a, sa.nonzero()), again_b = sq_again<T>(b, sb.nonzero());
+    if (again_a || again_b) {
+      SqSum64 a64, b64;
+      walk(a64, b64);
+      a = a64.s, b = b64.s;
+      block_sum2(a, b, red);
+    }
     if (tid == 0) {
       const int o = (MODE == MODE_W) ? 2 : 0;
       d.part[(size_t)i1 * 4 + o] = a;
@@ -696,11 +722,6 @@ __device__ __forceinline__ void slab_g_impl(const Dev<T>& d, T* __restrict__ Wou
     double unused = 0.0;
     block_sum2(dw2, unused, red);
     if (tid == 0) d.part_dw[i1] = dw2;
-  }
-  if (MODE == MODE_GRAD) {
-    double g = gsum.total(), unused = 0.0;
-    block_sum2(g, unused, red);
-    if (tid == 0) d.part[(size_t)i1 * 4] = g;
   }
 }
 

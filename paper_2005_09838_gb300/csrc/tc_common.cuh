@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <mutex>
+#include <type_traits>
 
 namespace tc {
 
@@ -163,59 +164,74 @@ __device__ __forceinline__ float two_sum(float& s, float a) {
   return e;
 }
 
-// The FP64 form of an FP32 term of SqSum, out of line: GB300 issues one FP64 warp
-// instruction per scheduler in about 60 clocks, predicated off or not, and a call
-// is not turned into predicated code.
-static __device__ __noinline__ double sq_diff64(double s, float a, float b) {
-  const double v = (double)a - (double)b;
-  return fma(v, v, s);
-}
-
-// Sum of squares of a thread's values, no less accurate than FP64 additions.
-// FP32 values within 2^+-48 (and 0): every square is taken with its rounding error
-// and added without one to three FP32 words (error some 2^-70 of the sum), on the
-// FP32 pipe; an FP64 conversion and multiply-add per value took more than half of
-// the read-back kernels.  Outside that range a square or its rounding error could
-// leave FP32's: those terms are added in FP64.
+// Sum of squares of a thread's values, no less accurate than FP64 additions.  FP32: every
+// square is taken with its rounding error and added without one to three FP32 words
+// (error some 2^-70 of the sum), on the FP32 pipe; GB300 issues one FP64 warp
+// instruction per scheduler in about 60 clocks, and an FP64 conversion and
+// multiply-add per value took more than half of the read-back kernels.  Squares past
+// FP32's range make the sum infinite or NaN, and squares or rounding errors below it
+// are at most 2^-149 each, so the block's sum tells whether it stands (sq_again); where
+// it does not, the kernel sums its block again with SqSum64.  (Objective of 144 x 288 x
+// 168 147 us, gradient call of 300 x 150 x 92 130, of 529 x 288 x 168 427; with every value
+// tested and the far ones added in FP64 on the spot 161, 137, 430; with one error word,
+// which keeps 2^-43 of a long sum and fails outside 2^+-63, 135, 130, 414.)
 template <typename T>
 struct SqSum {
   T s = T(0);
   __device__ __forceinline__ void add(T v) { s = fma(v, v, s); }
   __device__ __forceinline__ void add_diff(T a, T b) { add(a - b); }
+  __device__ __forceinline__ bool nonzero() const { return false; }
   __device__ __forceinline__ double total() const { return s; }
 };
 template <>
 struct SqSum<float> {
   float s = 0.f, c = 0.f, e = 0.f;
-  double far = 0.0;
-  __device__ __forceinline__ static bool near(float v) {
-    const float m = fabsf(v);
-    return (m >= 0x1p-48f && m <= 0x1p48f) || m == 0.f;
-  }
+  unsigned any = 0;  // bits of the values
   __device__ __forceinline__ void term(float a) { e += two_sum(c, a); }  // a: of the size of a rounding error
-  __device__ __forceinline__ void square(float v) {
+  __device__ __forceinline__ void add(float v) {
+    any |= __float_as_uint(v);
     const float p = mul_rn(v, v), pe = fmaf(v, v, -p);
     term(two_sum(s, p));
     term(pe);
   }
-  // (the plain terms outside the branch: the sums of several values interleave)
-  __device__ __forceinline__ void add(float v) {
-    const bool nr = near(v);
-    square(nr ? v : 0.f);
-    if (!nr) far = sq_diff64(far, v, 0.f);
-  }
   // (a - b)^2 of the difference as it is, not rounded: h + z
   __device__ __forceinline__ void add_diff(float a, float b) {
-    const bool nr = near(a - b);
-    const float a1 = nr ? a : 0.f, b1 = nr ? b : 0.f, h = a1 - b1;
-    const float w = h - a1, z = (a1 - (h - w)) - (b1 + w);
+    const float h = a - b, w = h - a, z = (a - (h - w)) - (b + w);
     const float q = mul_rn(2.f * h, z), qe = fmaf(2.f * h, z, -q);
-    square(h);
+    add(h);
     term(q);
     e += fmaf(z, z, qe);
-    if (!nr) far = sq_diff64(far, a, b);
   }
-  __device__ __forceinline__ double total() const { return (double)s + (double)c + (double)e + far; }
+  __device__ __forceinline__ bool nonzero() const { return (any << 1) != 0; }
+  __device__ __forceinline__ double total() const { return (double)s + (double)c + (double)e; }
+};
+// Whether the block has to sum again: total (valid in thread 0) of the threads' SqSum
+// is outside the range in which they are exact, though some value is not 0.  Below
+// 2^20 values the underflows are 2^-129, 2^-49 of the smallest sum that stands.
+template <typename T>
+__device__ __forceinline__ bool sq_again(double total, bool nonzero) {
+  if (sizeof(T) == 8) return false;
+  const bool any = __syncthreads_or(nonzero);
+  return __syncthreads_or(any && threadIdx.x == 0 && !(total >= 0x1p-80 && total <= 1e300));
+}
+struct SqSum64 {
+  double s = 0.0;
+  template <typename T>
+  __device__ __forceinline__ void add(T v) {
+    s = fma((double)v, (double)v, s);
+  }
+  template <typename T>
+  __device__ __forceinline__ void add_diff(T a, T b) {
+    add((double)a - (double)b);
+  }
+};
+// Sum of values and rounding errors in the working precision.
+template <typename T>
+struct SqPair {
+  T s = T(0), c = T(0);
+  __device__ __forceinline__ void add(T v) { dot2(s, c, v, v); }
+  __device__ __forceinline__ bool nonzero() const { return false; }
+  __device__ __forceinline__ double total() const { return (double)s + (double)c; }
 };
 
 // A truth value as a type, for generic lambdas.
