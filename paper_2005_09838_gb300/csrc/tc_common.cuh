@@ -206,13 +206,14 @@ struct SqSum<float> {
   __device__ __forceinline__ double total() const { return (double)s + (double)c + (double)e; }
 };
 // Whether the block has to sum again: total (valid in thread 0) of the threads' SqSum
-// is outside the range in which they are exact, though some value is not 0.  Below
-// 2^20 values the underflows are 2^-129, 2^-49 of the smallest sum that stands.
+// is outside the range in which they are exact, though some value is not 0.  A slab has
+// at most 2^24 values, whose underflows (a few of 2^-149 each) come to 2^-123 at most,
+// 2^-59 of the smallest sum that stands.
 template <typename T>
 __device__ __forceinline__ bool sq_again(double total, bool nonzero) {
   if (sizeof(T) == 8) return false;
   const bool any = __syncthreads_or(nonzero);
-  return __syncthreads_or(any && threadIdx.x == 0 && !(total >= 0x1p-80 && total <= 1e300));
+  return __syncthreads_or(any && threadIdx.x == 0 && !(total >= 0x1p-64 && total <= 1e300));
 }
 struct SqSum64 {
   double s = 0.0;
