@@ -226,7 +226,7 @@ __global__ void k_check(Dev<T> d) {
 // factors; equal to tr((H X~)^H (H X~) Y~ Y~^H).  Grid (S, kRhoChunks): CTA
 // (k, c) streams chunk c of the slice's row differences (coalesced along n2)
 // and writes part_k[k kRhoChunks + c]; squares are summed error-free per thread
-// (dot2) and the thread totals added in FP64 in a fixed order.
+// (SqSum; FP64 dot2) and the thread totals added in FP64 in a fixed order.
 constexpr int kRhoChunks = 16;
 
 template <typename T>
